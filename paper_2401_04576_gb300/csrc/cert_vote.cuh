@@ -1,0 +1,161 @@
+// Voting with certified FP32 decisions (certified.cuh) on the device data layout: the votes of
+// the FP64 (K = 64) or outward FP32 (K = 32) interval program, most of them decided by bare FP32
+// end points and one error bound per (parent cell, hit).
+#pragma once
+#include "certified.cuh"
+#include "kernels.cuh"
+
+namespace apo {
+
+template <int K> struct RefOf { using T = double; };   // the program whose votes K decides
+template <> struct RefOf<32> { using T = float; };
+
+// The reference's sign and guard tests of a cell: its precision's omega interval.  Returns
+// whether the cell is mirrored (omega < 0); *guard: omega reaches 0, every hit votes.
+template <int K> __device__ __forceinline__ bool omega_sign(IV<double> W, bool *guard) {
+    const IV<typename RefOf<K>::T> w = to_prec<typename RefOf<K>::T>(W);
+    const bool mir = lt0(w.hi);
+    *guard = mir ? false : !gt0(w.lo);
+    return mir;
+}
+
+template <int Q> __device__ __forceinline__ cert::X<Q> cx(IV<double> a) { return cert::mk<Q>(a.lo, a.hi); }
+template <int Q> __device__ __forceinline__ cert::X<Q> cxm(IV<double> a, bool mir) {
+    return mir ? cert::mk<Q>(-a.hi, -a.lo) : cert::mk<Q>(a.lo, a.hi);
+}
+template <int Q> __device__ __forceinline__ cert::CellX<Q> cert_cell(const Cell<double> &c, bool mir) {
+    return cert::CellX<Q>{cxm<Q>(c.D, mir), cxm<Q>(c.S0, mir), cx<Q>(c.C0), cxm<Q>(c.W, mir), cx<Q>(c.Z), cx<Q>(c.L)};
+}
+template <int Q> __device__ __forceinline__ cert::HitX<Q> cert_hit(const void *rec, bool mir) {
+    const HitRecF &r = *reinterpret_cast<const HitRecF *>(rec);
+    cert::HitX<Q> h;
+    h.x0 = cert::sc<Q>(r.lo[0]);
+    h.y0 = cert::sc<Q>(mir ? -r.lo[1] : r.lo[1]);
+    h.sph = cert::sc<Q>(r.lo[2]);
+    h.cph = cert::sc<Q>(mir ? -r.lo[3] : r.lo[3]);
+    h.t = cert::sc<Q>(r.lo[4]);
+    h.spt = cert::sc<Q>(r.lo[5]);
+    h.cpt = cert::sc<Q>(mir ? -r.lo[6] : r.lo[6]);
+    h.t2 = cert::sc<Q>(r.lo[7]);
+    h.d = cert::point(cert::sc<Q>(r.lo[8]));
+    return h;
+}
+
+__device__ __forceinline__ IV<double> hull2(IV<double> a, IV<double> b) { return {mn(a.lo, b.lo), mx(a.hi, b.hi)}; }
+// the smallest box around cells [i0, i1] of axis a (edges ascend along an axis)
+__device__ __forceinline__ IV<double> edge_span(const DevGeom &g, int a, int level, int i0, int i1) {
+    return hull2(edge(g, a, level, i0), edge(g, a, level, i1));
+}
+
+// The test of one hit on a parent cell: -1 when no cell inside it gets the hit's vote, else the
+// error bound its cells share (NaN: they cannot be decided by one).  Not inlined: its registers
+// stay out of the callers' loops.
+template <int K>
+__device__ __noinline__ float parent_error(const DevGeom &g, IV<double> D, IV<double> S0, IV<double> C0,
+                                           IV<double> W, IV<double> Z, IV<double> L, const void *rec) {
+    bool guard;
+    const bool mir = omega_sign<K>(W, &guard);
+    if (guard) return NAN;
+    const cert::Eval<K> x = cert::eval(cert_cell<K>(Cell<double>{D, S0, C0, W, Z, L}, mir), cert_hit<K>(rec, mir));
+    const float e = cert::bound(x);
+    return cert::verdict(x, g.k.outgoing != 0, e) == cert::kNo ? -1.f : e;
+}
+
+// Hits no parent could decide for a cell, one by one: the cell's own evaluation with errors,
+// then the reference program.  mask: tan(lambda) cells l0 + bit in question; returns those that
+// vote.  Not inlined: about one pair in 10^4 comes here,
+// and its registers stay out of the callers' loops.
+template <int K>
+__device__ __noinline__ uint32_t resolve(const DevGeom &g, int level, int d, int p, int w, int z, int l0,
+                                         uint32_t mask, const HitRecD *hd, const HitRecF *hf) {
+    using T = typename RefOf<K>::T;
+    Cell<double> c{edge(g, 0, level, d), sin_phi0(g, level, p), cos_phi0(g, level, p), edge(g, 2, level, w),
+                   edge(g, 3, level, z), {0.0, 0.0}};
+    bool guard;
+    const bool mir = omega_sign<K>(c.W, &guard);
+    const cert::HitX<K> h = cert_hit<K>(hf, mir);
+    uint32_t yes = 0;
+    while (mask) {
+        const int b = __ffs(mask) - 1;
+        mask &= mask - 1;
+        c.L = edge(g, 4, level, l0 + b);
+        const cert::Eval<K> ev = cert::eval(cert_cell<K>(c, mir), h);
+        int v = cert::verdict(ev, g.k.outgoing != 0, cert::bound(ev));
+        if (guard) v = cert::kUnknown;
+        if (v == cert::kUnknown) {
+            const Cell<T> ct{to_prec<T>(c.D), to_prec<T>(c.S0), to_prec<T>(c.C0),
+                             to_prec<T>(c.W), to_prec<T>(c.Z), to_prec<T>(c.L)};
+            const void *rec = K == 64 ? static_cast<const void *>(hd) : static_cast<const void *>(hf);
+            v = vote_pair<T>(ct, load_hit<T>(rec), g.k) ? cert::kYes : cert::kNo;
+        }
+        if (v == cert::kYes) yes |= 1u << b;
+    }
+    return yes;
+}
+
+// A block's undecided (thread, hit) pairs, resolved together so that whole warps do that work.
+// Threads push at most kCertStep pairs between block barriers, where the queue is drained if it
+// could overflow in the next step (and at the end); so no push is ever refused.
+constexpr int kCertStep = 4, kCertDrain = 256;
+template <int NT> struct CertQueue {
+    static constexpr int cap = kCertDrain + kCertStep * NT;
+    uint32_t n, pad[3];
+    uint32_t id[cap];     // thread | hit << 16
+    uint32_t mask[cap];   // tan(lambda) bits in question, then those that vote
+    __device__ __forceinline__ void push(int tid, int h, uint32_t m) {
+        const uint32_t s = atomicAdd(&n, 1u);
+        if (s >= (uint32_t)cap) return;   // cannot happen; never write past the arrays
+        id[s] = (uint32_t)tid | ((uint32_t)h << 16);
+        mask[s] = m;
+    }
+};
+
+// The votes of one tan(lambda) interval for a prefix and error bound e: the signs of L and of
+// the wire's t are made known where they can be, by the reflection z -> -z of cell and wire,
+// which changes no end point ((L, t) -> (-L, -t)).
+__device__ __forceinline__ int cert_tail(const cert::PreX<0> &p, cert::X<0> L, const cert::HitX<0> &h,
+                                         cert::X<0> R, cert::X<0> W, float e) {
+    cert::X<0> Gp, Gm;
+    const bool lpos = L.lo >= 0.f;
+    if (lpos || L.hi <= 0.f) {
+        cert::HitX<0> hr = h;
+        if (!lpos) { L = cert::neg(L); hr.t = cert::neg(h.t); }
+        if (hr.t.v >= 0.f) cert::tail<1, 1>(p, L, hr, R, W, Gp, Gm);
+        else cert::tail<1, -1>(p, L, hr, R, W, Gp, Gm);
+    } else {
+        cert::tail<0, 0>(p, L, h, R, W, Gp, Gm);
+    }
+    return cert::decide(Gp, Gm, e);
+}
+
+// The direction condition for a prefix: kNo refuses every vote, kUnknown leaves it open.
+__device__ __forceinline__ int cert_direction(const cert::PreX<0> &p, bool outgoing, float e) {
+    if (!outgoing) return cert::kYes;
+    return p.wt.hi < -e ? cert::kNo : (p.wt.hi >= e ? cert::kYes : cert::kUnknown);
+}
+
+// Bit-sliced vote counters: bit l of plane q is bit q of counter l (counts <= 256: 9 planes);
+// adding a mask of votes is a ripple-carry add.
+struct VotePlanes {
+    uint32_t pl[9];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int q = 0; q < 9; q++) pl[q] = 0u;
+    }
+    __device__ __forceinline__ void add(uint32_t m) {
+#pragma unroll
+        for (int q = 0; q < 9; q++) {
+            const uint32_t c = pl[q] & m;
+            pl[q] ^= m;
+            m = c;
+        }
+    }
+    __device__ __forceinline__ int get(int l) const {
+        int v = 0;
+#pragma unroll
+        for (int q = 0; q < 9; q++) v |= (int)((pl[q] >> l) & 1u) << q;
+        return v;
+    }
+};
+
+}  // namespace apo

@@ -7,6 +7,7 @@
 #include <cstdint>
 
 #include "../../include/apo.h"
+#include "cert_vote.cuh"
 #include "kernels.cuh"
 
 namespace apo {
@@ -180,17 +181,14 @@ void launch_stage(const DevGeom &g, int n_events, const int32_t *offsets, const 
 }
 
 // ---------------------------------------------------------------------------------------
-// Coarse-grid voting.  Block = (event, phi0 bin p, omega bin w); thread = (d0 bin, z0 bin);
-// each thread loops over the tan(lambda) bins, reusing the tan(lambda)-free prefix of the
-// program.  Before that, every hit is tested once on the block's parent cell (all d0, z0,
-// tan(lambda) bins joined): interval operations are inclusion-isotonic and the guards only
-// fire on a parent when they fire on a child, so a hit that fails there fails on every
-// child cell; skipping it leaves every vote unchanged.
-// Modes: FP32 intervals; FP64 intervals; FP64 intervals evaluated only where the FP32
-// program votes (FP32 intervals contain the FP64 ones, so an FP32 "no" is an FP64 "no":
-// the votes are those of the plain FP64 program).
-// Writes votes[e][lin], lin = d + Bd (p + Bp (w + Bw (z + Bz l))), and the per-event
-// histogram of vote counts.
+// Coarse-grid voting.  A tile is the (d0, z0) cells of one (phi0 bin, omega bin), in two parts
+// when they exceed a block; thread = (d0 bin, z0 bin), looping over the tan(lambda) bins, which
+// share the tan(lambda)-free prefix of the program.  Before that, every hit is tested once on
+// the tile's parent cell (all its d0, z0, tan(lambda) bins joined): interval operations are
+// inclusion-isotonic and the guards only fire on a parent when they fire on a child, so a hit
+// that fails there fails on every child cell; skipping it leaves every vote unchanged.
+// Writes votes[e][lin], lin = d + Bd (p + Bp (w + Bw (z + Bz l))), or each tile's K best cells,
+// and the per-event histogram of vote counts.
 // ---------------------------------------------------------------------------------------
 enum : int { kModeF32 = 0, kModeF64 = 1, kModeF64Filtered = 2, kModeF64Exact = 3 };
 // precisions a mode evaluates: FP64 intervals (all but FP32), FP32 intervals (FP32 and the
@@ -201,229 +199,15 @@ template <int MODE> struct ModeOf {
     static constexpr bool exact = MODE == kModeF64Exact;
 };
 
-template <int MODE> struct CoarseSmem {
-    static constexpr bool k64 = ModeOf<MODE>::k64, k32 = ModeOf<MODE>::k32;
-    static constexpr size_t hits64 = 0;
-    static constexpr size_t hits32 = k64 ? kHitCap * 80 : 0;
-    static constexpr size_t hist = hits32 + (k32 ? kHitCap * 80 : 0);
-    static constexpr size_t mask = hist + kHistBins * 4 + 12;
-    static constexpr size_t bar = mask + 32;
-    static constexpr size_t L64 = bar + 8;
-    __host__ __device__ static size_t L32(int Bl) { return L64 + 16 * Bl; }
-    __host__ __device__ static size_t total(int Bl, int) { return L32(Bl) + 8 * Bl + 16; }
-};
-
-// The FP32 coarse kernel splits each tile's (d0, z0) cells over APO_F32_COARSE_SPLIT
-// blocks, and asks the compiler for APO_F32_COARSE_MIN_BLOCKS resident blocks per SM (it
-// caps registers at 64K / (threads x this)); the FP64 kernels are bound by the FP64 pipe.
-#ifndef APO_F32_COARSE_SPLIT
-#define APO_F32_COARSE_SPLIT 1
-#endif
-#ifndef APO_F32_COARSE_MIN_BLOCKS
-#define APO_F32_COARSE_MIN_BLOCKS (3 * APO_F32_COARSE_SPLIT)
-#endif
-// The FP64 modes split each (phi0, omega) tile's (d0, z0) cells over APO_F64_COARSE_SPLIT
-// blocks (consecutive ranges of the d0-fastest index): smaller blocks with the same register
-// budget let more warps share an SM, which hides more FP64 latency.
-#ifndef APO_F64_COARSE_SPLIT
-#define APO_F64_COARSE_SPLIT 2
-#endif
-#ifndef APO_F64_COARSE_MIN_BLOCKS
-#define APO_F64_COARSE_MIN_BLOCKS (APO_F64_COARSE_SPLIT == 1 ? 1 : 3)
-#endif
-template <int MODE> struct CoarseShape {
-    static constexpr int split = MODE == kModeF32 ? APO_F32_COARSE_SPLIT : APO_F64_COARSE_SPLIT;
-    static constexpr int threads = 256 / split;
-    static constexpr int min_blocks = MODE == kModeF32 ? APO_F32_COARSE_MIN_BLOCKS : APO_F64_COARSE_MIN_BLOCKS;
-};
-
-// One block's work: part `part` (of `split`) of the (phi0 bin p, omega bin w) tile of event
-// ev; votes to vo (the event's level-0 votes), the histogram added to hist_e.  Shared by
-// k_vote_coarse (one tile per block) and the persistent batch kernel (tiles in a loop);
-// any block size of at least one warp works (threads past the part's cells idle).
-template <int MODE>
-__device__ __forceinline__ void coarse_block(const DevGeom &g, int ev, int split, int part, int p, int w,
-                                             const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
-                                             const uint32_t *active, int32_t *vo, uint32_t *hist_e,
-                                             unsigned *status, unsigned long long *ctr, unsigned char *smem,
-                                             uint64_t *cand_k = nullptr, int32_t *cand_v = nullptr, int K = 0) {
-    using S = CoarseSmem<MODE>;
-    constexpr bool k64 = S::k64, k32 = S::k32;
-    const int Bd = g.bins[0], Bz = g.bins[3], Bl = g.bins[4];
-    const int ntile = Bd * Bz;                    // (d0, z0) cells of one (phi0, omega) tile
-    const int per = (ntile + split - 1) / split;  // of them in this block
-    const int nthr = blockDim.x;
-    const int tid = threadIdx.x;
-    const int c0 = part * per, c1 = c0 + per < ntile ? c0 + per : ntile;   // this block's cells
-    const bool has_cell = c0 + tid < c1;
-    unsigned char *h64s = smem + S::hits64;
-    unsigned char *h32s = smem + S::hits32;
-    uint32_t *hist_s = reinterpret_cast<uint32_t *>(smem + S::hist);
-    uint32_t *mask_s = reinterpret_cast<uint32_t *>(smem + S::mask);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + S::bar);
-    IV<double> *L64 = reinterpret_cast<IV<double> *>(smem + S::L64);
-    IV<float> *L32 = reinterpret_cast<IV<float> *>(smem + S::L32(Bl));
-
-    int nh = n_hits[ev];
-    if (nh < 0) nh = 0;
-    for (int i = tid; i < kHistBins; i += nthr) hist_s[i] = 0;
-    if (tid < 8) mask_s[tid] = 0;
-    for (int l = tid; l < Bl; l += nthr) {
-        IV<double> el = edge(g, 4, 0, l);
-        L64[l] = el;
-        L32[l] = to_prec<float>(el);
-    }
-    const unsigned bytes = (unsigned)nh * 80u;
-    bool ok = stage_to_smem(h64s, hd + (long long)ev * kHitCap, k64 ? bytes : 0u, h32s,
-                            hf + (long long)ev * kHitCap, k32 ? bytes : 0u, bar, status);
-    __syncthreads();
-    if (tid == 0) mbar_inval(bar);   // the barrier's memory may be set up again by a later call
-    if (!ok) nh = 0;
-
-    const SeriesConsts &k = g.k;
-    const IV<double> S0 = sin_phi0(g, 0, p), C0 = cos_phi0(g, 0, p), W = edge(g, 2, 0, w);
-    unsigned n_par32 = 0, n_pre32 = 0, n_tail32 = 0, n_par64 = 0, n_pre64 = 0, n_tail64 = 0;
-    // parent cell test, one hit per thread
-    {
-        IV<double> D0 = edge(g, 0, 0, c1 - c0 >= Bd ? 0 : c0 % Bd);
-        IV<double> D1 = edge(g, 0, 0, c1 - c0 >= Bd ? Bd - 1 : (c1 - 1) % Bd);
-        if (c0 / Bd != (c1 - 1) / Bd) { D0 = edge(g, 0, 0, 0); D1 = edge(g, 0, 0, Bd - 1); }
-        IV<double> Z0 = edge(g, 3, 0, c0 / Bd), Z1 = edge(g, 3, 0, (c1 - 1) / Bd);
-        IV<double> L0 = edge(g, 4, 0, 0), L1 = edge(g, 4, 0, Bl - 1);
-        Cell<double> par{{D0.lo, D1.hi}, S0, C0, W, {Z0.lo, Z1.hi}, {L0.lo, L1.hi}};
-        Cell<float> par32{to_prec<float>(par.D), to_prec<float>(S0), to_prec<float>(C0),
-                          to_prec<float>(W), to_prec<float>(par.Z), to_prec<float>(par.L)};
-        const uint32_t *act = active ? active + (long long)ev * 8 : nullptr;
-        auto parent_vote = [&](int h) -> bool {
-            if (h >= nh || (act && !((act[h >> 5] >> (h & 31)) & 1u))) return false;
-            bool v = true;
-            if (k32) { v = vote_pair<float>(par32, load_hit<float>(h32s + h * 80), k); n_par32++; }
-            if (k64 && v) {
-                v = ModeOf<MODE>::exact ? vote_pair_exact(par, load_hit<double>(h64s + h * 80), k)
-                                        : vote_pair<double>(par, load_hit<double>(h64s + h * 80), k);
-                n_par64++;
-            }
-            return v;
-        };
-        const int lane = tid & 31, warp = tid >> 5, nfull = nthr >> 5;
-        if (nfull > 0) {   // full warps take 32 hits each; the warp ballot is the mask word
-            if (warp < nfull)
-                for (int base = warp * 32; base < nh; base += nfull * 32) {
-                    unsigned m = __ballot_sync(0xffffffffu, parent_vote(base + lane));
-                    if (lane == 0) mask_s[base >> 5] = m;
-                }
-        } else {
-            for (int h = tid; h < nh; h += nthr)
-                if (parent_vote(h)) atomicOr(&mask_s[h >> 5], 1u << (h & 31));
-        }
-    }
-    __syncthreads();
-
-    const int cell = has_cell ? c0 + tid : c0;   // threads past the block's cells idle
-    const int d = cell % Bd, z = cell / Bd;
-    Cell<double> c{edge(g, 0, 0, d), S0, C0, W, edge(g, 3, 0, z), L64[0]};
-    Cell<float> c32{to_prec<float>(c.D), to_prec<float>(S0), to_prec<float>(C0), to_prec<float>(W),
-                    to_prec<float>(c.Z), L32[0]};
-    const bool mir = mirror_cell(c);
-    mirror_cell(c32);
-    const bool wguard = !gt0(c.W.lo) || !gt0(c32.W.lo);
-    const IV<double> R = recip(c.W);
-    const IV<float> R32 = recip(c32.W);
-    const unsigned all = Bl >= 32 ? 0xffffffffu : ((1u << Bl) - 1u);
-    // The Bl vote counters of this thread, bit-sliced: bit l of plane k is bit k of counter
-    // l (counts <= 256 need 9 planes).  Adding a mask of votes is a ripple-carry add.
-    uint32_t pl[9];
-#pragma unroll
-    for (int q = 0; q < 9; q++) pl[q] = 0u;
-    auto add_votes = [&](uint32_t m) {
-#pragma unroll
-        for (int q = 0; q < 9; q++) {
-            const uint32_t c = pl[q] & m;
-            pl[q] ^= m;
-            m = c;
-        }
-    };
-    for (int wd = 0; wd < 8 && has_cell; wd++) {
-        uint32_t m = mask_s[wd];
-        while (m) {
-            int h = wd * 32 + __ffs(m) - 1;
-            m &= m - 1;
-            if (wguard) {
-                add_votes(all);
-                continue;
-            }
-            // tan(lambda) bins still in question after the FP32 program
-            unsigned lm = all;
-            if (k32) {
-                Hit<float> h32 = load_hit<float>(h32s + h * 80);
-                if (mir) mirror_hit(h32);
-                Pre<float> p32 = prefix<float>(c32, h32, k);
-                n_pre32++;
-                if (p32.novote) {
-                    lm = 0;
-                } else if (!p32.guard) {
-                    lm = 0;
-                    n_tail32 += Bl;
-                    // sign of the wire's stereo tangent (0: unknown)
-                    const int tsg = h32.t.lo >= 0.f ? 1 : (h32.t.hi <= 0.f ? -1 : 0);
-#pragma unroll 1
-                    for (int l = 0; l < Bl; l++) {
-                        const IV<float> Ll = L32[l];
-                        bool tv;
-                        if (MODE == kModeF32) {
-                            // The block's threads share the bin and the hit: uniform branches
-                            // on the signs of L and t.  A bin with L <= 0 is evaluated
-                            // reflected, (L, t) -> (-L, -t), which gives the same vote, so the
-                            // tail always sees L >= 0 and a known sign of t.  (In the filtered
-                            // FP64 mode the extra FP32 tails cost more code than they save.)
-                            const bool lpos = Ll.lo >= 0.f, lneg = Ll.hi <= 0.f;
-                            const int ts = lpos ? tsg : (lneg ? -tsg : 0);
-                            Hit<float> hr = h32;
-                            if (!lpos) hr.t = neg(h32.t);
-                            const IV<float> Lr = lpos ? Ll : neg(Ll);
-                            tv = ts > 0 ? tail<float, 1, false, 1>(p32, Lr, hr, R32, c32.W, k)
-                               : ts < 0 ? tail<float, 1, false, -1>(p32, Lr, hr, R32, c32.W, k)
-                                        : tail<float, 0>(p32, Ll, h32, R32, c32.W, k);
-                        } else {
-                            tv = tail<float>(p32, Ll, h32, R32, c32.W, k);
-                        }
-                        if (tv) lm |= 1u << l;
-                    }
-                }
-                if (!k64) {
-                    add_votes(lm);
-                    continue;
-                }
-            }
-            if (!lm) continue;
-            Hit<double> h64 = load_hit<double>(h64s + h * 80);
-            if (mir) mirror_hit(h64);
-            Pre<double> p64 = prefix<double>(c, h64, k);
-            n_pre64++;
-            if (p64.novote) continue;
-            if (p64.guard) {
-                add_votes(all);
-                continue;
-            }
-            uint32_t v64 = 0;
-            while (lm) {
-                int l = __ffs(lm) - 1;
-                lm &= lm - 1;
-                n_tail64++;
-                const bool tv = ModeOf<MODE>::exact ? tail_exact(p64, L64[l], h64, R, c.W, k)
-                                                    : tail<double>(p64, L64[l], h64, R, c.W, k);
-                if (tv) v64 |= 1u << l;
-            }
-            add_votes(v64);
-        }
-    }
-    const int Bp = g.bins[1], Bw = g.bins[2];
-    auto vote_of = [&](int l) {
-        int v = 0;
-#pragma unroll
-        for (int q = 0; q < 9; q++) v |= (int)((pl[q] >> l) & 1u) << q;
-        return v;
-    };
+// The end of a coarse block: each thread's Bl vote counts (its cell (d, p, w, z), every
+// tan(lambda) bin) to vo or, with cand_k, the block's K best cells; the histogram added to hist_e
+// (may be null).  hist_s: kHistBins zeros in shared memory.
+__device__ __forceinline__ void coarse_output(const DevGeom &g, const VotePlanes &pl, bool has_cell, int d, int p,
+                                              int w, int z, uint32_t *hist_s, uint32_t *hist_e, int32_t *vo,
+                                              uint64_t *cand_k, int32_t *cand_v, int K) {
+    const int Bd = g.bins[0], Bp = g.bins[1], Bw = g.bins[2], Bz = g.bins[3], Bl = g.bins[4];
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    auto vote_of = [&](int l) { return pl.get(l); };
     for (int l = 0; l < Bl && has_cell; l++) {
         const int v = vote_of(l);
         if (!cand_k) {
@@ -433,7 +217,7 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, int ev, int split
         atomicAdd(&hist_s[v], 1u);
     }
     __syncthreads();
-    for (int i = tid; i < kHistBins; i += nthr)
+    for (int i = tid; i < kHistBins && hist_e; i += nthr)
         if (hist_s[i]) atomicAdd(&hist_e[i], hist_s[i]);
     if (cand_k) {
         // The part's K best cells by (votes desc, key asc), from its own histogram: every
@@ -545,39 +329,300 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, int ev, int split
             cand_v[i] = -1;
         }
     }
-    if (ctr) {   // work counters (diagnostics): FP64 parent / prefix / tail, -, FP32 ones
-        unsigned long long v[6] = {n_par64, n_pre64, n_tail64, n_par32, n_pre32, n_tail32};
-        const int slot[6] = {0, 1, 2, 4, 5, 6};
+}
+
+// Adds a thread's six work counts to the diagnostic counters: whole FP64 evaluations (with
+// certified decisions: pairs left undecided), FP64 prefixes, FP64 tails, then the FP32 ones.
+__device__ __forceinline__ void add_counts(unsigned long long *ctr, const unsigned (&cnt)[6]) {
+    if (!ctr) return;
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const int slot[6] = {0, 1, 2, 4, 5, 6};
 #pragma unroll
-        for (int i = 0; i < 6; i++) {
-            unsigned long long x = v[i];
-            if (nthr - (tid & ~31) >= 32) {   // a full warp: reduce, one add per warp
-                for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-                if ((tid & 31) == 0 && x) atomicAdd(&ctr[slot[i]], x);
-            } else if (x) {                   // the lanes of a partial last warp add their own
-                atomicAdd(&ctr[slot[i]], x);
-            }
+    for (int i = 0; i < 6; i++) {
+        unsigned long long x = cnt[i];
+        if (nthr - (tid & ~31) >= 32) {   // a full warp: reduce, one add per warp
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+            if ((tid & 31) == 0 && x) atomicAdd(&ctr[slot[i]], x);
+        } else if (x) {                   // the lanes of a partial last warp add their own
+            atomicAdd(&ctr[slot[i]], x);
         }
     }
+}
+
+// FP64 (K = 64) and outward FP32 (K = 32) voting, decided by certified FP32 end points.
+// Phase 1: the parent test, one (tile, hit) per thread, gives the mask of hits that can vote and
+// the error bound that every cell of the tile shares.  Phase 2: the bare end points per
+// (cell, hit), bit-sliced counters; the undecided pairs are queued and resolved in whole warps.
+// What bounds it: FP32 issue.  The FP64 pipe (about 1.7 directed operations per clock and SM)
+// evaluated every pair before; now about one pair in 10^4 reaches it.
+//
+// A block is 128 threads.  Grids with few (d0, z0) cells put `tiles` of them in one block (full
+// votes only: the K best are kept per tile), so that its warps stay full.
+constexpr int kCoarseThreads = 128, kCoarseMaxTiles = 16;
+struct CoarsePlan {
+    int parts, per, tiles;   // parts of a (phi0, omega) tile, cells of a part, tiles per block
+    long long n_tiles;       // of one event
+};
+__host__ __device__ inline CoarsePlan coarse_plan(const DevGeom &g, bool lists) {
+    CoarsePlan P;
+    const int n = g.bins[0] * g.bins[3];
+    P.parts = (n + kCoarseThreads - 1) / kCoarseThreads;
+    P.per = (n + P.parts - 1) / P.parts;
+    const int fit = kCoarseThreads / P.per;
+    P.tiles = lists ? 1 : (fit < 1 ? 1 : (fit > kCoarseMaxTiles ? kCoarseMaxTiles : fit));
+    P.n_tiles = (long long)P.parts * g.bins[1] * g.bins[2];
+    return P;
+}
+
+struct CoarseSmem {   // of a cert coarse block; every offset a multiple of 16
+    static constexpr size_t hits = 0;
+    static constexpr size_t queue = kHitCap * 80;
+    static constexpr size_t hist = queue + ((sizeof(CertQueue<kCoarseThreads>) + 15) & ~size_t(15));
+    static constexpr size_t bar = hist + ((kHistBins * 4 + 15) & ~size_t(15));
+    static constexpr size_t L = bar + 16;
+    __host__ __device__ static size_t mask(int Bl) { return L + ((8 * (size_t)Bl + 15) & ~size_t(15)); }
+    __host__ __device__ static size_t err(int Bl, int tiles) { return mask(Bl) + 32 * (size_t)tiles; }
+    __host__ __device__ static size_t total(int Bl, int tiles) { return err(Bl, tiles) + sizeof(float) * kHitCap * (size_t)tiles; }
+};
+
+template <int K>
+__device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan &P, int ev, long long tile0,
+                                             const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
+                                             const uint32_t *active, int32_t *vo, uint32_t *hist_e,
+                                             unsigned *status, unsigned long long *ctr, unsigned char *smem,
+                                             uint64_t *cand_k = nullptr, int32_t *cand_v = nullptr, int Kc = 0) {
+    const int Bd = g.bins[0], Bp = g.bins[1], Bz = g.bins[3], Bl = g.bins[4];
+    const int ntile = Bd * Bz, nthr = blockDim.x, tid = threadIdx.x;
+    unsigned char *hs = smem + CoarseSmem::hits;
+    CertQueue<kCoarseThreads> &q = *reinterpret_cast<CertQueue<kCoarseThreads> *>(smem + CoarseSmem::queue);
+    uint32_t *hist_s = reinterpret_cast<uint32_t *>(smem + CoarseSmem::hist);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + CoarseSmem::bar);
+    float2 *Ls = reinterpret_cast<float2 *>(smem + CoarseSmem::L);
+    uint32_t *mask_s = reinterpret_cast<uint32_t *>(smem + CoarseSmem::mask(Bl));
+    float *err_s = reinterpret_cast<float *>(smem + CoarseSmem::err(Bl, P.tiles));
+    const bool outgoing = g.k.outgoing != 0;
+
+    int nh = n_hits[ev];
+    if (nh < 0) nh = 0;
+    for (int i = tid; i < kHistBins; i += nthr) hist_s[i] = 0;
+    for (int i = tid; i < 8 * P.tiles; i += nthr) mask_s[i] = 0;
+    for (int l = tid; l < Bl; l += nthr) {
+        const cert::X<0> x = cx<0>(edge(g, 4, 0, l));
+        Ls[l] = make_float2(x.lo, x.hi);
+    }
+    if (tid == 0) q.n = 0;
+    const bool ok = stage_to_smem(hs, hf + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr, nullptr, 0u, bar,
+                                  status);
+    __syncthreads();
+    if (tid == 0) mbar_inval(bar);   // the barrier's memory may be set up again by a later call
+    if (!ok) nh = 0;
+    unsigned cnt[6] = {0, 0, 0, 0, 0, 0};
+
+    // the parent tests: a warp's 32 items are one word of one tile's hit mask
+    const uint32_t *act = active ? active + (long long)ev * 8 : nullptr;
+    const int nw = (nh + 31) >> 5;
+    for (int i = tid; i < P.tiles * nw * 32; i += nthr) {
+        const int tl = i / (nw * 32), h = i - tl * nw * 32;
+        const long long t = tile0 + tl;
+        bool keep = h < nh && t < P.n_tiles && (!act || ((act[h >> 5] >> (h & 31)) & 1u));
+        float e = NAN;
+        if (keep) {
+            const int part = (int)(t % P.parts), pw = (int)(t / P.parts), p = pw % Bp, w = pw / Bp;
+            const int c0 = part * P.per, c1 = c0 + P.per < ntile ? c0 + P.per : ntile;
+            const bool row = c0 / Bd == (c1 - 1) / Bd;   // cells of one z0 bin
+            e = parent_error<K>(g, edge_span(g, 0, 0, row ? c0 % Bd : 0, row ? (c1 - 1) % Bd : Bd - 1),
+                                sin_phi0(g, 0, p), cos_phi0(g, 0, p), edge(g, 2, 0, w),
+                                edge_span(g, 3, 0, c0 / Bd, (c1 - 1) / Bd), edge_span(g, 4, 0, 0, Bl - 1),
+                                hs + h * 80);
+            keep = !(e < 0.f);
+            cnt[3]++;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        if ((tid & 31) == 0) mask_s[tl * 8 + (h >> 5)] = m;
+        err_s[tl * kHitCap + h] = e;
+    }
+    __syncthreads();
+
+    const int tl = tid / P.per;
+    const long long t = tile0 + tl;
+    const int part = (int)(t % P.parts), pw = (int)(t / P.parts);
+    const int cell = part * P.per + (tid - tl * P.per);
+    const bool has_cell = tl < P.tiles && t < P.n_tiles && cell < ntile;
+    const int p = has_cell ? pw % Bp : 0, w = has_cell ? pw / Bp : 0;
+    const int d = has_cell ? cell % Bd : 0, z = has_cell ? cell / Bd : 0;
+    VotePlanes pl;
+    pl.clear();
+    const unsigned all = Bl >= 32 ? 0xffffffffu : ((1u << Bl) - 1u);
+    const Cell<double> c64{edge(g, 0, 0, d), sin_phi0(g, 0, p), cos_phi0(g, 0, p), edge(g, 2, 0, w),
+                           edge(g, 3, 0, z), {0.0, 0.0}};
+    bool guard;
+    const bool mir = omega_sign<K>(c64.W, &guard);
+    const cert::CellX<0> c = cert_cell<0>(c64, mir);
+    const cert::X<0> R = cert::recip(c.W);
+    int wd = -1;
+    uint32_t m = 0;
+    bool left = has_cell;
+    while (__syncthreads_or(left)) {
+        for (int step = 0; step < kCertStep && left; step++) {
+            while (!m && ++wd < nw) m = mask_s[tl * 8 + wd];
+            if (!m) { left = false; break; }
+            const int h = wd * 32 + __ffs(m) - 1;
+            m &= m - 1;
+            if (guard) { pl.add(all); continue; }
+            const float e = err_s[tl * kHitCap + h];
+            uint32_t yes = 0, unk = all;
+            if (e < 1e30f) {
+                const cert::HitX<0> hx = cert_hit<0>(hs + h * 80, mir);
+                const cert::PreX<0> pre = cert::prefix(c, hx);
+                cnt[4]++;
+                const int dir = cert_direction(pre, outgoing, e);
+                if (dir == cert::kNo) continue;
+                if (dir == cert::kYes) {
+                    unk = 0;
+                    cnt[5] += Bl;
+#pragma unroll 1
+                    for (int l = 0; l < Bl; l++) {
+                        const float2 L = Ls[l];
+                        const int v = cert_tail(pre, cert::X<0>{L.x, L.y, 0.f}, hx, R, c.W, e);
+                        yes |= (uint32_t)(v == cert::kYes) << l;
+                        unk |= (uint32_t)(v == cert::kUnknown) << l;
+                    }
+                }
+            }
+            if (unk) {
+                cnt[0] += __popc(unk);
+                q.push(tid, h, unk);
+            }
+            pl.add(yes);
+        }
+        __syncthreads();
+        const int nq = (int)q.n;
+        if (nq > kCertDrain || !__syncthreads_or(left)) {
+            for (int i = tid; i < nq; i += nthr) {   // any thread's pair: its cell from its number
+                const int ot = (int)(q.id[i] & 0xffffu), oh = (int)(q.id[i] >> 16), otl = ot / P.per;
+                const long long u = tile0 + otl;
+                const int oc = (int)(u % P.parts) * P.per + (ot - otl * P.per), opw = (int)(u / P.parts);
+                q.mask[i] = resolve<K>(g, 0, oc % Bd, opw % Bp, opw / Bp, oc / Bd, 0, q.mask[i],
+                                       hd + (long long)ev * kHitCap + oh, hf + (long long)ev * kHitCap + oh);
+            }
+            __syncthreads();
+            for (int i = 0; i < nq; i++)
+                if ((int)(q.id[i] & 0xffffu) == tid) pl.add(q.mask[i]);
+            __syncthreads();
+            if (tid == 0) q.n = 0;
+        }
+    }
+    coarse_output(g, pl, has_cell, d, p, w, z, hist_s, hist_e, vo, cand_k, cand_v, Kc);
+    add_counts(ctr, cnt);
     __syncthreads();   // shared memory is reused by the caller's next step
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(CoarseShape<MODE>::threads, CoarseShape<MODE>::min_blocks)
-k_vote_coarse(DevGeom g, int ev0, const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
+// Resident blocks per SM the compiler plans for: caps registers at 64K / (128 x this).
+#ifndef APO_COARSE_MIN_BLOCKS
+#define APO_COARSE_MIN_BLOCKS 4
+#endif
+template <int K>
+__global__ void __launch_bounds__(kCoarseThreads, APO_COARSE_MIN_BLOCKS)
+k_vote_coarse(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
               const uint32_t *active, int32_t *votes, uint32_t *hist, unsigned *status,
-              unsigned long long *ctr, uint64_t *cand_k, int32_t *cand_v, int K) {
+              unsigned long long *ctr, uint64_t *cand_k, int32_t *cand_v, int Kc) {
     extern __shared__ __align__(16) unsigned char smem[];
-    constexpr int split = CoarseShape<MODE>::split;
     const int e = blockIdx.y;
-    const int part = blockIdx.x % split, pw = blockIdx.x / split;
-    const int p = pw % g.bins[1], w = pw / g.bins[1];
     const long long ncell = (long long)g.bins[0] * g.bins[1] * g.bins[2] * g.bins[3] * g.bins[4];
-    // candidates: K slots per block, the blocks of an event in blockIdx.x order
-    const long long co = ((long long)e * gridDim.x + blockIdx.x) * K;
-    coarse_block<MODE>(g, ev0 + e, split, part, p, w, hd, hf, n_hits, active,
-                       votes ? votes + (long long)e * ncell : nullptr, hist + (long long)e * kHistBins, status,
-                       ctr, smem, cand_k ? cand_k + co : nullptr, cand_v ? cand_v + co : nullptr, K);
+    // candidates: Kc slots per block (one tile), the blocks of an event in blockIdx.x order
+    const long long co = ((long long)e * gridDim.x + blockIdx.x) * Kc;
+    coarse_block<K>(g, P, ev0 + e, (long long)blockIdx.x * P.tiles, hd, hf, n_hits, active,
+                    votes ? votes + (long long)e * ncell : nullptr,
+                    hist ? hist + (long long)e * kHistBins : nullptr, status, ctr, smem,
+                    cand_k ? cand_k + co : nullptr, cand_v ? cand_v + co : nullptr, Kc);
+}
+
+// The exact-phase program on the coarse grid: FP64, the same tiles in blocks of at most 128
+// threads, one tile each.
+struct ExactSmem {
+    static constexpr size_t hits = 0;
+    static constexpr size_t hist = kHitCap * 80;
+    static constexpr size_t mask = hist + ((kHistBins * 4 + 15) & ~size_t(15));
+    static constexpr size_t bar = mask + 32;
+    static constexpr size_t L = bar + 16;
+    __host__ __device__ static size_t total(int Bl) { return L + 16 * (size_t)Bl; }
+};
+
+__global__ void __launch_bounds__(kCoarseThreads, 3)
+k_vote_coarse_exact(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const int32_t *n_hits, const uint32_t *active,
+                    int32_t *votes, uint32_t *hist, unsigned *status, unsigned long long *ctr, uint64_t *cand_k,
+                    int32_t *cand_v, int Kc) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int e = blockIdx.y, ev = ev0 + e;
+    const int part = blockIdx.x % P.parts, pw = blockIdx.x / P.parts;
+    const int Bd = g.bins[0], Bz = g.bins[3], Bl = g.bins[4], p = pw % g.bins[1], w = pw / g.bins[1];
+    const int ntile = Bd * Bz, nthr = blockDim.x, tid = threadIdx.x;
+    const int c0 = part * P.per, c1 = c0 + P.per < ntile ? c0 + P.per : ntile;   // this block's cells
+    const bool has_cell = c0 + tid < c1;
+    unsigned char *hs = smem + ExactSmem::hits;
+    uint32_t *hist_s = reinterpret_cast<uint32_t *>(smem + ExactSmem::hist);
+    uint32_t *mask_s = reinterpret_cast<uint32_t *>(smem + ExactSmem::mask);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + ExactSmem::bar);
+    IV<double> *Ls = reinterpret_cast<IV<double> *>(smem + ExactSmem::L);
+    int nh = n_hits[ev];
+    if (nh < 0) nh = 0;
+    for (int i = tid; i < kHistBins; i += nthr) hist_s[i] = 0;
+    if (tid < 8) mask_s[tid] = 0;
+    for (int l = tid; l < Bl; l += nthr) Ls[l] = edge(g, 4, 0, l);
+    const bool ok = stage_to_smem(hs, hd + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr, nullptr, 0u, bar,
+                                  status);
+    __syncthreads();
+    if (!ok) nh = 0;
+    const SeriesConsts &k = g.k;
+    const IV<double> S0 = sin_phi0(g, 0, p), C0 = cos_phi0(g, 0, p), W = edge(g, 2, 0, w);
+    unsigned cnt[6] = {0, 0, 0, 0, 0, 0};
+    const uint32_t *act = active ? active + (long long)ev * 8 : nullptr;
+    {
+        const bool row = c0 / Bd == (c1 - 1) / Bd;   // cells of one z0 bin
+        const Cell<double> par{edge_span(g, 0, 0, row ? c0 % Bd : 0, row ? (c1 - 1) % Bd : Bd - 1), S0, C0, W,
+                               edge_span(g, 3, 0, c0 / Bd, (c1 - 1) / Bd), edge_span(g, 4, 0, 0, Bl - 1)};
+        for (int h = tid; h < nh; h += nthr) {
+            if (act && !((act[h >> 5] >> (h & 31)) & 1u)) continue;
+            cnt[0]++;
+            if (vote_pair_exact(par, load_hit<double>(hs + h * 80), k)) atomicOr(&mask_s[h >> 5], 1u << (h & 31));
+        }
+    }
+    __syncthreads();
+    const int cell = has_cell ? c0 + tid : c0;   // threads past the block's cells idle
+    const int d = cell % Bd, z = cell / Bd;
+    Cell<double> c{edge(g, 0, 0, d), S0, C0, W, edge(g, 3, 0, z), Ls[0]};
+    const bool mir = mirror_cell(c);
+    const bool wguard = !gt0(c.W.lo);
+    const IV<double> R = recip(c.W);
+    const unsigned all = Bl >= 32 ? 0xffffffffu : ((1u << Bl) - 1u);
+    VotePlanes pl;
+    pl.clear();
+    for (int wd = 0; wd < 8 && has_cell; wd++) {
+        uint32_t m = mask_s[wd];
+        while (m) {
+            const int h = wd * 32 + __ffs(m) - 1;
+            m &= m - 1;
+            if (wguard) { pl.add(all); continue; }
+            Hit<double> hx = load_hit<double>(hs + h * 80);
+            if (mir) mirror_hit(hx);
+            const Pre<double> pre = prefix<double>(c, hx, k);
+            cnt[1]++;
+            if (pre.novote) continue;
+            if (pre.guard) { pl.add(all); continue; }
+            uint32_t v = 0;
+#pragma unroll 1
+            for (int l = 0; l < Bl; l++)
+                if (tail_exact(pre, Ls[l], hx, R, c.W, k)) v |= 1u << l;
+            cnt[2] += Bl;
+            pl.add(v);
+        }
+    }
+    const long long ncell = (long long)ntile * g.bins[1] * g.bins[2] * Bl;
+    const long long co = ((long long)e * gridDim.x + blockIdx.x) * Kc;
+    coarse_output(g, pl, has_cell, d, p, w, z, hist_s, hist + (long long)e * kHistBins,
+                  votes ? votes + (long long)e * ncell : nullptr, cand_k ? cand_k + co : nullptr,
+                  cand_v ? cand_v + co : nullptr, Kc);
+    add_counts(ctr, cnt);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -765,8 +810,7 @@ static void launch_cells_mid(const DevGeom &g, int n_ev, const HitRecD *hd, cons
 
 // Raises the dynamic shared-memory limit of a kernel once per process (the attribute is a
 // property of the function; setting it outside any stream capture keeps captures clean).
-static bool g_attr_coarse[4] = {false, false, false, false}, g_attr_cells[4] = {false, false, false, false},
-            g_attr_children[4] = {false, false, false, false};
+static bool g_attr_cells[4] = {false, false, false, false};
 
 template <typename K> static void smem_limit_once(K kernel, bool &flag) {
     if (!flag) {
@@ -775,46 +819,34 @@ template <typename K> static void smem_limit_once(K kernel, bool &flag) {
     }
 }
 
-template <int MODE> static void launch_coarse_mode(const DevGeom &g, int ev0, int n_ev, const HitRecD *hd,
-                                                  const HitRecF *hf, const int32_t *n_hits,
-                                                  const uint32_t *active, int32_t *votes,
-                                                  uint32_t *hist, unsigned *status, cudaStream_t s,
-                                                  unsigned long long *ctr, uint64_t *cand_k,
-                                                  int32_t *cand_v, int K) {
-    smem_limit_once(k_vote_coarse<MODE>, g_attr_coarse[MODE]);
-    constexpr int split = CoarseShape<MODE>::split;
-    dim3 grid(g.bins[1] * g.bins[2] * split, n_ev);
-    const int nthr = (g.bins[0] * g.bins[3] + split - 1) / split;
-    size_t sm = CoarseSmem<MODE>::total(g.bins[4], nthr);
-    k_vote_coarse<MODE><<<grid, nthr, sm, s>>>(g, ev0, hd, hf, n_hits, active, votes, hist, status, ctr,
-                                                cand_k, cand_v, K);
+template <int K> static void launch_coarse_cert(const DevGeom &g, int ev0, int n_ev, const HitRecD *hd,
+                                               const HitRecF *hf, const int32_t *n_hits, const uint32_t *active,
+                                               int32_t *votes, uint32_t *hist, unsigned *status, cudaStream_t s,
+                                               unsigned long long *ctr, uint64_t *cand_k, int32_t *cand_v, int Kc) {
+    const CoarsePlan P = coarse_plan(g, cand_k != nullptr);
+    dim3 grid((unsigned)((P.n_tiles + P.tiles - 1) / P.tiles), n_ev);
+    k_vote_coarse<K><<<grid, kCoarseThreads, CoarseSmem::total(g.bins[4], P.tiles), s>>>(
+        g, P, ev0, hd, hf, n_hits, active, votes, hist, status, ctr, cand_k, cand_v, Kc);
 }
 
-int coarse_lists(const DevGeom &g, int prec) {
-    const int split = (prec == APO_F32 || prec == APO_F64_MID) ? CoarseShape<kModeF32>::split
-                                                                : CoarseShape<kModeF64>::split;
-    return g.bins[1] * g.bins[2] * split;
-}
+int coarse_lists(const DevGeom &g, int) { return (int)coarse_plan(g, true).n_tiles; }
 
 void launch_vote_coarse(const DevGeom &g, int prec, int ev0, int n_ev, const HitRecD *hd,
                         const HitRecF *hf, const int32_t *n_hits, int32_t *votes, uint32_t *hist,
                         unsigned *status, cudaStream_t s, unsigned long long *ctr,
                         const uint32_t *active, uint64_t *cand_k, int32_t *cand_v, int K) {
     if (n_ev <= 0) return;
-    if (prec == APO_F64_MID)
+    if (prec == APO_F64_MID) {
         launch_coarse_mid(g, ev0, n_ev, hd, n_hits, active, votes, hist, status, s, ctr);
-    else if (prec == APO_F64_EXACT)
-        launch_coarse_mode<kModeF64Exact>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr,
-                                              cand_k, cand_v, K);
-    else if (prec == APO_F32)
-        launch_coarse_mode<kModeF32>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr,
-                                              cand_k, cand_v, K);
-    else if (prec == APO_F64_FILTERED)
-        launch_coarse_mode<kModeF64Filtered>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr,
-                                              cand_k, cand_v, K);
-    else
-        launch_coarse_mode<kModeF64>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr,
-                                              cand_k, cand_v, K);
+    } else if (prec == APO_F64_EXACT) {
+        const CoarsePlan P = coarse_plan(g, true);
+        k_vote_coarse_exact<<<dim3((unsigned)P.n_tiles, n_ev), P.per, ExactSmem::total(g.bins[4]), s>>>(
+            g, P, ev0, hd, n_hits, active, votes, hist, status, ctr, cand_k, cand_v, K);
+    } else if (prec == APO_F32) {
+        launch_coarse_cert<32>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K);
+    } else {   // APO_F64 and APO_F64_FILTERED: the same votes, the same kernel
+        launch_coarse_cert<64>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K);
+    }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1083,9 +1115,9 @@ void launch_vote_children(const DevGeom &g, int prec, int n_ev, const HitRecD *h
 // Sets every vote kernel's dynamic shared-memory limit now, outside any stream capture.
 void init_kernel_attributes() {
     const int lim = 96 * 1024;   // on the current device, every time a geometry is created there
-    cudaFuncSetAttribute(k_vote_coarse<kModeF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_coarse<kModeF64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_coarse<kModeF64Filtered>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_vote_coarse<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_vote_coarse<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_vote_coarse_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_cells<kModeF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_cells<kModeF64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_cells<kModeF64Filtered>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
@@ -1095,11 +1127,10 @@ void init_kernel_attributes() {
     cudaFuncSetAttribute(k_vote_children<kModeF64, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_children<kModeF64Filtered, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_children<kModeF64Filtered, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_coarse<kModeF64Exact>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_cells<kModeF64Exact>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_children<kModeF64Exact, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_children<kModeF64Exact, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    for (int i = 0; i < 4; i++) g_attr_coarse[i] = g_attr_cells[i] = g_attr_children[i] = true;
+    for (int i = 0; i < 4; i++) g_attr_cells[i] = true;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1535,16 +1566,11 @@ void launch_estimate_mask(const DevGeom &g, int n_ev, const uint64_t *keys, cons
 // pull new ones, and no launch boundary waits for the slowest event of a level.  The only
 // device waits are the bounded waits of the hit staging.
 // ---------------------------------------------------------------------------------------
-template <int MODE> __device__ __noinline__ void persist_coarse(const DevGeom &g, const PersistArgs &A, int e,
-                                                                   int32_t *vo, uint32_t *hist_b,
-                                                                   unsigned char *smem) {
-    const int split = (g.bins[0] * g.bins[3] + blockDim.x - 1) / blockDim.x;
-    const int ntiles = g.bins[1] * g.bins[2] * split;
-    for (int t = 0; t < ntiles; t++) {
-        const int part = t % split, pw = t / split;
-        coarse_block<MODE>(g, e, split, part, pw % g.bins[1], pw / g.bins[1], A.hd, A.hf, A.n_hits,
-                           A.active, vo, hist_b, A.status, nullptr, smem);
-    }
+template <int K> __device__ __noinline__ void persist_coarse(const DevGeom &g, const PersistArgs &A, int e,
+                                                                int32_t *vo, uint32_t *hist_b, unsigned char *smem) {
+    const CoarsePlan P = coarse_plan(g, false);
+    for (long long t = 0; t < P.n_tiles; t += P.tiles)
+        coarse_block<K>(g, P, e, t, A.hd, A.hf, A.n_hits, A.active, vo, hist_b, A.status, nullptr, smem);
 }
 
 template <int MODE> __device__ __noinline__ void persist_children(const DevGeom &g, const PersistArgs &A, int e,
@@ -1588,11 +1614,8 @@ __global__ void __launch_bounds__(128, 3) k_solve_persistent(DevGeom g, PersistA
             if (A.done[e]) break;
             for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist_b[i] = 0u;
             __syncthreads();
-            switch (A.mode[0]) {
-                case kModeF32: persist_coarse<kModeF32>(g, A, e, vo, hist_b, smem); break;
-                case kModeF64Filtered: persist_coarse<kModeF64Filtered>(g, A, e, vo, hist_b, smem); break;
-                default: persist_coarse<kModeF64>(g, A, e, vo, hist_b, smem); break;
-            }
+            if (A.mode[0] == kModeF32) persist_coarse<32>(g, A, e, vo, hist_b, smem);
+            else persist_coarse<64>(g, A, e, vo, hist_b, smem);
             __threadfence_block();
             __syncthreads();
             select_coarse_block(g, vo, hist_b, K, A.fk + (long long)e * K, A.fv + (long long)e * K);
@@ -1618,7 +1641,7 @@ static_assert(kPersistF32 == kModeF32 && kPersistF64 == kModeF64 && kPersistF64F
               "persistent launch modes");
 
 size_t persist_smem_bytes(const DevGeom &g) {
-    size_t a = CoarseSmem<kModeF64Filtered>::total(g.bins[4], 128);
+    size_t a = CoarseSmem::total(g.bins[4], coarse_plan(g, false).tiles);
     size_t b = 2 * kHitCap * 80 + 16;
     size_t c = kSortMax * sizeof(uint64_t) + kEstChunk * 5 * sizeof(double);
     size_t m = a > b ? a : b;
