@@ -32,7 +32,7 @@
 #ifdef __CUDACC__
 #define APO_CERT __device__ __forceinline__
 #else
-#define APO_CERT static inline
+#define APO_CERT inline
 #endif
 
 namespace apo {

@@ -523,7 +523,7 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan 
 #endif
 template <int K>
 __global__ void __launch_bounds__(kCoarseThreads, APO_COARSE_MIN_BLOCKS)
-k_vote_coarse(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
+k_vote_coarse(const __grid_constant__ DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
               const uint32_t *active, int32_t *votes, uint32_t *hist, unsigned *status,
               unsigned long long *ctr, uint64_t *cand_k, int32_t *cand_v, int Kc) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -924,106 +924,207 @@ k_vote_cells(DevGeom g, const HitRecD *hd, const HitRecF *hf, const int32_t *n_h
 
 // Children of kept cells, two per thread: the children 2 idx + bit of a parent that differ
 // only in the tan(lambda) bit share every tan(lambda)-free step of the program, so one
-// prefix per hit serves both tails (same operations as evaluating them apart).
-// One thread's pair j of an event: children 2 idx + bit of parent j / 16 for the bit pattern
-// b = j % 16 on d0 .. z0, with tan(lambda) bit 0 and 1 (slots 32 (j / 16) + b and + 16 of the
-// event's outputs).  h64s / h32s: the event's hits staged in shared memory; parents_e,
-// out_keys_e, out_votes_e: the event's arrays.
-template <int MODE>
-__device__ __forceinline__ void children_pair(const DevGeom &g, const unsigned char *h64s,
-                                              const unsigned char *h32s, int nh, const uint32_t *act,
-                                              int level, const uint64_t *parents_e, long long j,
-                                              uint64_t *out_keys_e, int32_t *out_votes_e) {
-    constexpr bool k64 = ModeOf<MODE>::k64, k32 = ModeOf<MODE>::k32;
-    const int b = (int)(j % 16);
-    int idx[5];
-    unpack_key(g, parents_e[j / 16], idx);
+// prefix per hit serves both tails.  Pair j of an event: children 2 idx + bit of parent j / 16
+// for the bit pattern b = j % 16 on d0 .. z0, with tan(lambda) bit 0 and 1 (slots
+// 32 (j / 16) + b and + 16 of the event's outputs).
+__device__ __forceinline__ void pair_index(const DevGeom &g, uint64_t parent, int b, int idx[5]) {
+    unpack_key(g, parent, idx);
 #pragma unroll
     for (int a = 0; a < 4; a++) idx[a] = 2 * idx[a] + ((b >> a) & 1);
-    const int l0 = 2 * idx[4];                    // tan(lambda) bit 0 / 1 of the pair
-    idx[4] = l0;
+    idx[4] = 2 * idx[4];   // tan(lambda) bit 0
+}
+__device__ __forceinline__ void pair_store(const DevGeom &g, const int idx[5], long long j, int v0, int v1,
+                                           uint64_t *out_keys_e, int32_t *out_votes_e) {
     const uint64_t key0 = pack_key(g, idx);
-    const uint64_t key1 = key0 + (1ULL << g.key_shift[4]);
-    Cell<double> c{edge(g, 0, level, idx[0]), sin_phi0(g, level, idx[1]), cos_phi0(g, level, idx[1]),
-                   edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, l0)};
-    const IV<double> L1 = edge(g, 4, level, l0 + 1);
-    Cell<float> c32{to_prec<float>(c.D), to_prec<float>(c.S0), to_prec<float>(c.C0),
-                    to_prec<float>(c.W), to_prec<float>(c.Z), to_prec<float>(c.L)};
-    const IV<float> L1f = to_prec<float>(L1);
-    const bool mir = mirror_cell(c);
-    mirror_cell(c32);
-    const bool wguard = !gt0(c.W.lo) || !gt0(c32.W.lo);
-    const IV<double> R = recip(c.W);
-    const IV<float> R32 = recip(c32.W);
-    const SeriesConsts &k = g.k;
-    int v0 = 0, v1 = 0;
-    for (int h = 0; h < nh; h++) {
-        if (act && !((act[h >> 5] >> (h & 31)) & 1u)) continue;
-        if (wguard) { v0++; v1++; continue; }
-        unsigned lm = 3u;
-        if (k32) {
-            Hit<float> h32 = load_hit<float>(h32s + h * 80);
-            if (mir) mirror_hit(h32);
-            Pre<float> p32 = prefix<float>(c32, h32, k);
-            if (p32.novote) {
-                lm = 0u;
-            } else if (!p32.guard) {
-                lm = (tail<float>(p32, c32.L, h32, R32, c32.W, k) ? 1u : 0u) |
-                     (tail<float>(p32, L1f, h32, R32, c32.W, k) ? 2u : 0u);
-            }
-            if (!k64) { v0 += lm & 1u; v1 += lm >> 1; continue; }
-            if (!lm) continue;
-        }
-        Hit<double> h64 = load_hit<double>(h64s + h * 80);
-        if (mir) mirror_hit(h64);
-        Pre<double> p64 = prefix<double>(c, h64, k);
-        if (p64.novote) continue;
-        if (p64.guard) { v0++; v1++; continue; }
-        if (ModeOf<MODE>::exact) {
-            if ((lm & 1u) && tail_exact(p64, c.L, h64, R, c.W, k)) v0++;
-            if ((lm & 2u) && tail_exact(p64, L1, h64, R, c.W, k)) v1++;
-        } else {
-            if ((lm & 1u) && tail<double>(p64, c.L, h64, R, c.W, k)) v0++;
-            if ((lm & 2u) && tail<double>(p64, L1, h64, R, c.W, k)) v1++;
-        }
-    }
-    // output order: child b at 32 j' + b, child b + 16 at 32 j' + b + 16 (j' = parent)
-    const long long o = (j / 16) * 32 + b;
+    const long long o = (j / 16) * 32 + j % 16;
     out_keys_e[o] = key0;
     out_votes_e[o] = v0;
-    out_keys_e[o + 16] = key1;
+    out_keys_e[o + 16] = key0 + (1ULL << g.key_shift[4]);
     out_votes_e[o + 16] = v1;
 }
 
-// NT: threads per block, 256 or 128; the 128-thread form asks for three resident blocks
-// per SM (12 warps), which the FP64 modes' register count otherwise limits to 8 warps.
-template <int MODE, int NT>
-__global__ void __launch_bounds__(NT, NT == 128 ? 3 : 1)
-k_vote_children(DevGeom g, const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
+// FP64 (K = 64) and outward FP32 (K = 32) votes of the children, decided by certified FP32 end
+// points (see coarse_block): one evaluation with errors per (parent, hit) gives the bound that
+// the parent's 32 children share, and drops the hits that none of them can get.  FP32 issue
+// bounds it; before, every child hit that passed an FP32 test was evaluated on the FP64 pipe.
+// A block takes 8 parents.
+constexpr int kChildThreads = 128, kChildParents = kChildThreads / 16;
+struct ChildSmem {
+    static constexpr size_t hits = 0;
+    static constexpr size_t queue = kHitCap * 80;
+    static constexpr size_t err = queue + ((sizeof(CertQueue<kChildThreads>) + 15) & ~size_t(15));
+    static constexpr size_t mask = err + sizeof(float) * kHitCap * kChildParents;
+    static constexpr size_t bar = mask + 32 * kChildParents;
+    static constexpr size_t total = bar + 16;
+};
+
+// Pairs [j0, j0 + 128) of one event, those below n_pairs; hits staged at ChildSmem::hits.
+template <int K>
+__device__ __forceinline__ void children_block(const DevGeom &g, unsigned char *smem, int nh, const uint32_t *act,
+                                               int level, const uint64_t *parents_e, long long j0, long long n_pairs,
+                                               const HitRecD *hd_e, const HitRecF *hf_e, uint64_t *out_keys_e,
+                                               int32_t *out_votes_e) {
+    unsigned char *hs = smem + ChildSmem::hits;
+    CertQueue<kChildThreads> &q = *reinterpret_cast<CertQueue<kChildThreads> *>(smem + ChildSmem::queue);
+    float *err_s = reinterpret_cast<float *>(smem + ChildSmem::err);
+    uint32_t *mask_s = reinterpret_cast<uint32_t *>(smem + ChildSmem::mask);
+    const int tid = threadIdx.x;
+    const bool outgoing = g.k.outgoing != 0;
+    for (int i = tid; i < 8 * kChildParents; i += kChildThreads) mask_s[i] = 0u;
+    if (tid == 0) q.n = 0;
+    __syncthreads();
+    const long long p0 = j0 / 16, n_par = n_pairs / 16 - p0;   // parents from p0 on
+    const int np = n_par < kChildParents ? (int)n_par : kChildParents;
+    for (int i = tid; i < np * nh; i += kChildThreads) {
+        const int pl = i / nh, h = i - pl * nh;
+        if (act && !((act[h >> 5] >> (h & 31)) & 1u)) continue;
+        int x[5];
+        unpack_key(g, parents_e[p0 + pl], x);
+#pragma unroll
+        for (int a = 0; a < 5; a++) x[a] *= 2;
+        const float e = parent_error<K>(g, edge_span(g, 0, level, x[0], x[0] + 1),
+                                        hull2(sin_phi0(g, level, x[1]), sin_phi0(g, level, x[1] + 1)),
+                                        hull2(cos_phi0(g, level, x[1]), cos_phi0(g, level, x[1] + 1)),
+                                        edge_span(g, 2, level, x[2], x[2] + 1), edge_span(g, 3, level, x[3], x[3] + 1),
+                                        edge_span(g, 4, level, x[4], x[4] + 1), hs + h * 80);
+        err_s[pl * kHitCap + h] = e;
+        if (!(e < 0.f)) atomicOr(&mask_s[pl * 8 + (h >> 5)], 1u << (h & 31));
+    }
+    __syncthreads();
+    const long long j = j0 + tid;
+    const int pl = tid / 16;
+    const bool has = j < n_pairs;
+    int idx[5] = {0, 0, 0, 0, 0};
+    if (has) pair_index(g, parents_e[j / 16], (int)(j % 16), idx);
+    const Cell<double> c64{edge(g, 0, level, idx[0]), sin_phi0(g, level, idx[1]), cos_phi0(g, level, idx[1]),
+                           edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
+    bool guard;
+    const bool mir = omega_sign<K>(c64.W, &guard);
+    const cert::CellX<0> c = cert_cell<0>(c64, mir);
+    const cert::X<0> R = cert::recip(c.W), L1 = cx<0>(edge(g, 4, level, idx[4] + 1));
+    const int nw = (nh + 31) >> 5;
+    int v0 = 0, v1 = 0, wd = -1;
+    uint32_t m = 0;
+    bool left = has;
+    while (__syncthreads_or(left)) {
+        for (int step = 0; step < kCertStep && left; step++) {
+            while (!m && ++wd < nw) m = mask_s[pl * 8 + wd];
+            if (!m) { left = false; break; }
+            const int h = wd * 32 + __ffs(m) - 1;
+            m &= m - 1;
+            if (guard) { v0++; v1++; continue; }
+            const float e = err_s[pl * kHitCap + h];
+            uint32_t unk = 3u;
+            if (e < 1e30f) {
+                const cert::HitX<0> hx = cert_hit<0>(hs + h * 80, mir);
+                const cert::PreX<0> pre = cert::prefix(c, hx);
+                const int dir = cert_direction(pre, outgoing, e);
+                if (dir == cert::kNo) continue;
+                if (dir == cert::kYes) {
+                    unk = 0;
+#pragma unroll 1
+                    for (int b = 0; b < 2; b++) {
+                        const int v = cert_tail(pre, b ? L1 : c.L, hx, R, c.W, e);
+                        if (v == cert::kYes) { if (b) v1++; else v0++; }
+                        unk |= (uint32_t)(v == cert::kUnknown) << b;
+                    }
+                }
+            }
+            if (unk) q.push(tid, h, unk);
+        }
+        __syncthreads();
+        const int nq = (int)q.n;
+        if (nq > kCertDrain || !__syncthreads_or(left)) {
+            for (int i = tid; i < nq; i += kChildThreads) {
+                const long long oj = j0 + (q.id[i] & 0xffffu);
+                const int oh = (int)(q.id[i] >> 16);
+                int x[5];
+                pair_index(g, parents_e[oj / 16], (int)(oj % 16), x);
+                q.mask[i] = resolve<K>(g, level, x[0], x[1], x[2], x[3], x[4], q.mask[i], hd_e + oh, hf_e + oh);
+            }
+            __syncthreads();
+            for (int i = 0; i < nq; i++)
+                if ((int)(q.id[i] & 0xffffu) == tid) {
+                    v0 += q.mask[i] & 1u;
+                    v1 += (q.mask[i] >> 1) & 1u;
+                }
+            __syncthreads();
+            if (tid == 0) q.n = 0;
+        }
+    }
+    if (has) pair_store(g, idx, j, v0, v1, out_keys_e, out_votes_e);
+}
+
+#ifndef APO_CHILD_MIN_BLOCKS
+#define APO_CHILD_MIN_BLOCKS 4
+#endif
+template <int K>
+__global__ void __launch_bounds__(kChildThreads, APO_CHILD_MIN_BLOCKS)
+k_vote_children(const __grid_constant__ DevGeom g, const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
                 const uint32_t *active, int level, const uint64_t *parents, int n_par,
                 const int32_t *n_valid, uint64_t *out_keys, int32_t *out_votes, unsigned *status) {
-    constexpr bool k64 = ModeOf<MODE>::k64, k32 = ModeOf<MODE>::k32;
     extern __shared__ __align__(16) unsigned char smem[];
-    unsigned char *h64s = smem;
-    unsigned char *h32s = smem + (k64 ? kHitCap * 80 : 0);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + (k64 ? kHitCap * 80 : 0) + (k32 ? kHitCap * 80 : 0));
     const int ev = blockIdx.y;
     // n_valid (may be null): parents 0 .. n_valid[ev] - 1 of the event's n_par slots are
     // real; a block past them has nothing to do (the condition is uniform in the block)
     const long long n_here = n_valid ? (long long)n_valid[ev] : (long long)n_par;
+    const long long j0 = (long long)blockIdx.x * kChildThreads;
+    if (j0 >= n_here * 16) return;
+    int nh = n_hits[ev];
+    if (nh < 0) nh = 0;
+    const bool ok = stage_to_smem(smem + ChildSmem::hits, hf + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr,
+                                  nullptr, 0u, reinterpret_cast<uint64_t *>(smem + ChildSmem::bar), status);
+    __syncthreads();
+    if (!ok) nh = 0;
+    children_block<K>(g, smem, nh, active ? active + (long long)ev * 8 : nullptr, level,
+                      parents + (long long)ev * n_par, j0, n_here * 16, hd + (long long)ev * kHitCap,
+                      hf + (long long)ev * kHitCap, out_keys + (long long)ev * n_par * 32,
+                      out_votes + (long long)ev * n_par * 32);
+}
+
+// The exact-phase program on children, FP64.  NT: threads per block, 256 or 128; the 128-thread
+// form asks for three resident blocks per SM (12 warps), which the register count otherwise
+// limits to 8 warps.
+template <int NT>
+__global__ void __launch_bounds__(NT, NT == 128 ? 3 : 1)
+k_vote_children_exact(DevGeom g, const HitRecD *hd, const int32_t *n_hits, const uint32_t *active, int level,
+                      const uint64_t *parents, int n_par, const int32_t *n_valid, uint64_t *out_keys,
+                      int32_t *out_votes, unsigned *status) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kHitCap * 80);
+    const int ev = blockIdx.y;
+    const long long n_here = n_valid ? (long long)n_valid[ev] : (long long)n_par;
     if ((long long)blockIdx.x * blockDim.x >= n_here * 16) return;
     int nh = n_hits[ev];
     if (nh < 0) nh = 0;
-    const unsigned bytes = (unsigned)nh * 80u;
-    bool ok = stage_to_smem(h64s, hd + (long long)ev * kHitCap, k64 ? bytes : 0u, h32s,
-                            hf + (long long)ev * kHitCap, k32 ? bytes : 0u, bar, status);
+    const bool ok = stage_to_smem(smem, hd + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr, nullptr, 0u, bar,
+                                  status);
     __syncthreads();
     if (!ok) nh = 0;
     const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_here * 16) return;
-    children_pair<MODE>(g, h64s, h32s, nh, active ? active + (long long)ev * 8 : nullptr, level,
-                        parents + (long long)ev * n_par, j, out_keys + (long long)ev * n_par * 32,
-                        out_votes + (long long)ev * n_par * 32);
+    const uint32_t *act = active ? active + (long long)ev * 8 : nullptr;
+    int idx[5];
+    pair_index(g, parents[(long long)ev * n_par + j / 16], (int)(j % 16), idx);
+    Cell<double> c{edge(g, 0, level, idx[0]), sin_phi0(g, level, idx[1]), cos_phi0(g, level, idx[1]),
+                   edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
+    const IV<double> L1 = edge(g, 4, level, idx[4] + 1);
+    const bool mir = mirror_cell(c);
+    const bool wguard = !gt0(c.W.lo);
+    const IV<double> R = recip(c.W);
+    int v0 = 0, v1 = 0;
+    for (int h = 0; h < nh; h++) {
+        if (act && !((act[h >> 5] >> (h & 31)) & 1u)) continue;
+        if (wguard) { v0++; v1++; continue; }
+        Hit<double> hx = load_hit<double>(smem + h * 80);
+        if (mir) mirror_hit(hx);
+        const Pre<double> pre = prefix<double>(c, hx, g.k);
+        if (pre.novote) continue;
+        if (pre.guard) { v0++; v1++; continue; }
+        if (tail_exact(pre, c.L, hx, R, c.W, g.k)) v0++;
+        if (tail_exact(pre, L1, hx, R, c.W, g.k)) v1++;
+    }
+    pair_store(g, idx, j, v0, v1, out_keys + (long long)ev * n_par * 32, out_votes + (long long)ev * n_par * 32);
 }
 
 template <int MODE>
@@ -1070,20 +1171,14 @@ void launch_vote_keys(const DevGeom &g, int prec, int n_ev, const HitRecD *hd, c
                  nullptr, s);
 }
 
-template <int MODE>
-static void launch_children_mode(const DevGeom &g, int n_ev, const HitRecD *hd, const HitRecF *hf,
-                                 const int32_t *n_hits, const uint32_t *active, int level,
-                                 const uint64_t *parents, int n_par, const int32_t *n_valid,
-                                 uint64_t *out_keys, int32_t *out_votes, cudaStream_t s, int block) {
-    size_t sm = (ModeOf<MODE>::k64 ? kHitCap * 80 : 0) + (ModeOf<MODE>::k32 ? kHitCap * 80 : 0) + 16;
-    dim3 grid((unsigned)(((long long)n_par * 16 + block - 1) / block), n_ev);
-    if (block == 128) {
-        k_vote_children<MODE, 128><<<grid, 128, sm, s>>>(g, hd, hf, n_hits, active, level, parents, n_par,
-                                                         n_valid, out_keys, out_votes, nullptr);
-    } else {
-        k_vote_children<MODE, 256><<<grid, 256, sm, s>>>(g, hd, hf, n_hits, active, level, parents, n_par,
-                                                         n_valid, out_keys, out_votes, nullptr);
-    }
+template <int K>
+static void launch_children_cert(const DevGeom &g, int n_ev, const HitRecD *hd, const HitRecF *hf,
+                                 const int32_t *n_hits, const uint32_t *active, int level, const uint64_t *parents,
+                                 int n_par, const int32_t *n_valid, uint64_t *out_keys, int32_t *out_votes,
+                                 cudaStream_t s) {
+    dim3 grid((unsigned)(((long long)n_par + kChildParents - 1) / kChildParents), n_ev);
+    k_vote_children<K><<<grid, kChildThreads, ChildSmem::total, s>>>(g, hd, hf, n_hits, active, level, parents, n_par,
+                                                                     n_valid, out_keys, out_votes, nullptr);
 }
 
 void launch_vote_children(const DevGeom &g, int prec, int n_ev, const HitRecD *hd,
@@ -1092,24 +1187,26 @@ void launch_vote_children(const DevGeom &g, int prec, int n_ev, const HitRecD *h
                           int32_t *child_votes, cudaStream_t s, const uint32_t *active, int block,
                           const int32_t *n_valid) {
     if (n_ev <= 0 || n_par <= 0) return;
-    if (block != 128) block = 256;
+    if (block != 128) block = 256;   // of the midpoint and exact-phase kernels
     if (prec == APO_F64_MID) {   // children in the order of k_vote_children: 32 per parent
         launch_cells_mid(g, n_ev, hd, n_hits, active, child_level, nullptr, parents, (long long)n_par * 32,
                          child_keys, child_votes, nullptr, s, block);
-        return;
+    } else if (prec == APO_F64_EXACT) {
+        const size_t sm = kHitCap * 80 + 16;
+        dim3 grid((unsigned)(((long long)n_par * 16 + block - 1) / block), n_ev);
+        if (block == 128)
+            k_vote_children_exact<128><<<grid, 128, sm, s>>>(g, hd, n_hits, active, child_level, parents, n_par, n_valid,
+                                                             child_keys, child_votes, nullptr);
+        else
+            k_vote_children_exact<256><<<grid, 256, sm, s>>>(g, hd, n_hits, active, child_level, parents, n_par, n_valid,
+                                                             child_keys, child_votes, nullptr);
+    } else if (prec == APO_F32) {
+        launch_children_cert<32>(g, n_ev, hd, hf, n_hits, active, child_level, parents, n_par, n_valid, child_keys,
+                                 child_votes, s);
+    } else {   // APO_F64 and APO_F64_FILTERED: the same votes, the same kernel
+        launch_children_cert<64>(g, n_ev, hd, hf, n_hits, active, child_level, parents, n_par, n_valid, child_keys,
+                                 child_votes, s);
     }
-    if (prec == APO_F64_EXACT)
-        launch_children_mode<kModeF64Exact>(g, n_ev, hd, hf, n_hits, active, child_level, parents, n_par,
-                                            n_valid, child_keys, child_votes, s, block);
-    else if (prec == APO_F32)
-        launch_children_mode<kModeF32>(g, n_ev, hd, hf, n_hits, active, child_level, parents, n_par,
-                                       n_valid, child_keys, child_votes, s, block);
-    else if (prec == APO_F64_FILTERED)
-        launch_children_mode<kModeF64Filtered>(g, n_ev, hd, hf, n_hits, active, child_level, parents, n_par,
-                                               n_valid, child_keys, child_votes, s, block);
-    else
-        launch_children_mode<kModeF64>(g, n_ev, hd, hf, n_hits, active, child_level, parents, n_par,
-                                       n_valid, child_keys, child_votes, s, block);
 }
 
 // Sets every vote kernel's dynamic shared-memory limit now, outside any stream capture.
@@ -1121,15 +1218,11 @@ void init_kernel_attributes() {
     cudaFuncSetAttribute(k_vote_cells<kModeF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_cells<kModeF64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_cells<kModeF64Filtered>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_children<kModeF32, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_children<kModeF32, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_children<kModeF64, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_children<kModeF64, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_children<kModeF64Filtered, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_children<kModeF64Filtered, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_vote_children<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_vote_children<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_vote_children_exact<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_vote_children_exact<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_cells<kModeF64Exact>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_children<kModeF64Exact, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_children<kModeF64Exact, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     for (int i = 0; i < 4; i++) g_attr_cells[i] = true;
 }
 
@@ -1573,29 +1666,26 @@ template <int K> __device__ __noinline__ void persist_coarse(const DevGeom &g, c
         coarse_block<K>(g, P, e, t, A.hd, A.hf, A.n_hits, A.active, vo, hist_b, A.status, nullptr, smem);
 }
 
-template <int MODE> __device__ __noinline__ void persist_children(const DevGeom &g, const PersistArgs &A, int e,
-                                                                     int level, unsigned char *smem) {
-    constexpr bool k64 = ModeOf<MODE>::k64, k32 = ModeOf<MODE>::k32;
-    unsigned char *h64s = smem;
-    unsigned char *h32s = smem + (k64 ? kHitCap * 80 : 0);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + (k64 ? kHitCap * 80 : 0) + (k32 ? kHitCap * 80 : 0));
+template <int K> __device__ __noinline__ void persist_children(const DevGeom &g, const PersistArgs &A, int e,
+                                                               int level, unsigned char *smem) {
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + ChildSmem::bar);
+    const HitRecF *hf_e = A.hf + (long long)e * kHitCap;
     int nh = A.n_hits[e];
     if (nh < 0) nh = 0;
-    const unsigned bytes = (unsigned)nh * 80u;
-    bool ok = stage_to_smem(h64s, A.hd + (long long)e * kHitCap, k64 ? bytes : 0u, h32s,
-                            A.hf + (long long)e * kHitCap, k32 ? bytes : 0u, bar, A.status);
+    const bool ok = stage_to_smem(smem + ChildSmem::hits, hf_e, (unsigned)nh * 80u, nullptr, nullptr, 0u, bar, A.status);
     __syncthreads();
     if (threadIdx.x == 0) mbar_inval(bar);
     if (!ok) nh = 0;
-    const int K = g.topk;
-    const uint32_t *act = A.active + (long long)e * 8;
-    for (long long j = threadIdx.x; j < (long long)K * 16; j += blockDim.x)
-        children_pair<MODE>(g, h64s, h32s, nh, act, level, A.fk + (long long)e * K, j,
-                            A.ck + (long long)e * K * 32, A.cv + (long long)e * K * 32);
-    __syncthreads();
+    const int Kp = g.topk;
+    for (long long j0 = 0; j0 < (long long)Kp * 16; j0 += kChildThreads) {
+        children_block<K>(g, smem, nh, A.active + (long long)e * 8, level, A.fk + (long long)e * Kp, j0,
+                          (long long)Kp * 16, A.hd + (long long)e * kHitCap, hf_e, A.ck + (long long)e * Kp * 32,
+                          A.cv + (long long)e * Kp * 32);
+        __syncthreads();   // the masks and bounds are rewritten by the next pairs
+    }
 }
 
-__global__ void __launch_bounds__(128, 3) k_solve_persistent(DevGeom g, PersistArgs A) {
+__global__ void __launch_bounds__(128, 3) k_solve_persistent(const __grid_constant__ DevGeom g, const __grid_constant__ PersistArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_e;
     const int lv = g.levels, K = g.topk;
@@ -1620,11 +1710,8 @@ __global__ void __launch_bounds__(128, 3) k_solve_persistent(DevGeom g, PersistA
             __syncthreads();
             select_coarse_block(g, vo, hist_b, K, A.fk + (long long)e * K, A.fv + (long long)e * K);
             for (int lev = 1; lev <= lv; lev++) {
-                switch (A.mode[lev]) {
-                    case kModeF32: persist_children<kModeF32>(g, A, e, lev, smem); break;
-                    case kModeF64Filtered: persist_children<kModeF64Filtered>(g, A, e, lev, smem); break;
-                    default: persist_children<kModeF64>(g, A, e, lev, smem); break;
-                }
+                if (A.mode[lev] == kModeF32) persist_children<32>(g, A, e, lev, smem);
+                else persist_children<64>(g, A, e, lev, smem);
                 topk_block(A.ck + (long long)e * K * 32, A.cv + (long long)e * K * 32, K * 32, K,
                            A.fk + (long long)e * K, A.fv + (long long)e * K, s_sort);
             }
@@ -1642,7 +1729,7 @@ static_assert(kPersistF32 == kModeF32 && kPersistF64 == kModeF64 && kPersistF64F
 
 size_t persist_smem_bytes(const DevGeom &g) {
     size_t a = CoarseSmem::total(g.bins[4], coarse_plan(g, false).tiles);
-    size_t b = 2 * kHitCap * 80 + 16;
+    size_t b = ChildSmem::total;
     size_t c = kSortMax * sizeof(uint64_t) + kEstChunk * 5 * sizeof(double);
     size_t m = a > b ? a : b;
     return m > c ? m : c;
