@@ -501,7 +501,7 @@ struct NvtxRange {
 };
 
 // The max-set schedule (APO_SCHED_MAXSET) for every chunk of events: level-0 voting of the
-// whole grid (one thread per cell), then per level the selection of whole vote groups and
+// whole grid, then per level the selection of whole vote groups and
 // the voting of the kept cells' children, until each event's search has ended.
 template <typename PrecAt>
 int enqueue_maxset(const apo_geometry *g, const apo_hits *hits, const apo_solve_opts *o, const DevGeom *gl,
@@ -573,9 +573,9 @@ int enqueue_maxset(const apo_geometry *g, const apo_hits *hits, const apo_solve_
         for (int r = 0; r < mt; r++) {
             A.round = r;
             CU(cudaMemsetAsync(stop, 0, sizeof(int32_t) * (size_t)n, s));
-            // level 0: every cell of the grid, one thread each, in linear (= key) order
-            launch_vote_keys(gl[0], prec_at(0), n, hde, hfe, nhe, 0, nullptr, g->n_coarse, votes, s, act);
-            if ((rc = check_launch("vote_coarse_cells"))) return rc;
+            // level 0: every cell's vote, in linear (= key) order
+            launch_vote_coarse(gl[0], prec_at(0), 0, n, hde, hfe, nhe, votes, nullptr, status, s, nullptr, act);
+            if ((rc = check_launch("vote_coarse"))) return rc;
             A.level = 0;
             A.prec = prec_at(0) & ~APO_OUTGOING;
             A.votes = votes;
@@ -657,7 +657,7 @@ int enqueue_solve(const apo_geometry *g, const apo_hits *hits, const apo_solve_o
         A.min_votes = o->min_votes;
         A.width = width;
         auto mode_of = [](int p) {
-            return p == APO_F32 ? kPersistF32 : (p == APO_F64_FILTERED ? kPersistF64Filtered : kPersistF64);
+            return p == APO_F32 ? kPersistF32 : kPersistF64;   // APO_F64_FILTERED votes as APO_F64
         };
         for (int lev = 0; lev <= lv; lev++) A.mode[lev] = mode_of(prec_at(lev));
         A.hd = hd;

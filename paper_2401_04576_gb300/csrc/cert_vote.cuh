@@ -93,6 +93,52 @@ __device__ __noinline__ uint32_t resolve(const DevGeom &g, int level, int d, int
     return yes;
 }
 
+// The reference's own evaluation of one pair, out of the callers' registers.
+template <typename T>
+__device__ __noinline__ bool vote_reference(const DevGeom &g, const Cell<double> &c, const Hit<T> &h) {
+    const Cell<T> ct{to_prec<T>(c.D), to_prec<T>(c.S0), to_prec<T>(c.C0),
+                     to_prec<T>(c.W), to_prec<T>(c.Z), to_prec<T>(c.L)};
+    return vote_pair<T>(ct, h, g.k);
+}
+
+// The vote of a staged hit for one cell (not mirrored), by the pair's own bound.
+template <int K>
+__device__ __forceinline__ bool vote_single(const DevGeom &g, const Cell<double> &c, const HitRecD *hd,
+                                            const HitRecF *hf) {
+    using T = typename RefOf<K>::T;
+    bool guard;
+    const bool mir = omega_sign<K>(c.W, &guard);
+    if (guard) return true;
+    const cert::Eval<K> x = cert::eval(cert_cell<K>(c, mir), cert_hit<K>(hf, mir));
+    const int v = cert::verdict(x, g.k.outgoing != 0, cert::bound(x));
+    if (v != cert::kUnknown) return v == cert::kYes;
+    const void *rec = K == 64 ? static_cast<const void *>(hd) : static_cast<const void *>(hf);
+    return vote_reference<T>(g, c, load_hit<T>(rec));
+}
+
+// The FP64 vote of a staged hit for one cell with its drift widened to [max(rd(d - width), 0),
+// ru(d + width)] (the hit finding), by the pair's own bound.
+__device__ __forceinline__ bool vote_widened(const DevGeom &g, const Cell<double> &c, const HitRecD *hd,
+                                             double width) {
+    Hit<double> h = load_hit<double>(hd);
+    const double d = h.d.lo, dlo = __dsub_rd(d, width);
+    h.d = {gt0(dlo) ? dlo : 0.0, __dadd_ru(d, width)};
+    bool guard;
+    const bool mir = omega_sign<64>(c.W, &guard);
+    if (guard) return true;
+    cert::HitX<64> hx;
+    const IV<double> *f = &h.x0;
+    cert::Sc<64> *s = &hx.x0;
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+        s[i] = cert::sc<64>(__double2float_rd((mir && (i == 1 || i == 3 || i == 6)) ? -f[i].lo : f[i].lo));
+    hx.d = cx<64>(h.d);
+    const cert::Eval<64> x = cert::eval(cert_cell<64>(c, mir), hx);
+    const int v = cert::verdict(x, g.k.outgoing != 0, cert::bound(x));
+    if (v != cert::kUnknown) return v == cert::kYes;
+    return vote_reference<double>(g, c, h);
+}
+
 // A block's undecided (thread, hit) pairs, resolved together so that whole warps do that work.
 // Threads push at most kCertStep pairs between block barriers, where the queue is drained if it
 // could overflow in the next step (and at the end); so no push is ever refused.

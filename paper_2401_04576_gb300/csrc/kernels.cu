@@ -190,15 +190,6 @@ void launch_stage(const DevGeom &g, int n_events, const int32_t *offsets, const 
 // Writes votes[e][lin], lin = d + Bd (p + Bp (w + Bw (z + Bz l))), or each tile's K best cells,
 // and the per-event histogram of vote counts.
 // ---------------------------------------------------------------------------------------
-enum : int { kModeF32 = 0, kModeF64 = 1, kModeF64Filtered = 2, kModeF64Exact = 3 };
-// precisions a mode evaluates: FP64 intervals (all but FP32), FP32 intervals (FP32 and the
-// FP32-first filter); kModeF64Exact uses the exact-phase program for its FP64 steps
-template <int MODE> struct ModeOf {
-    static constexpr bool k64 = MODE != kModeF32;
-    static constexpr bool k32 = MODE == kModeF32 || MODE == kModeF64Filtered;
-    static constexpr bool exact = MODE == kModeF64Exact;
-};
-
 // The end of a coarse block: each thread's Bl vote counts (its cell (d, p, w, z), every
 // tan(lambda) bin) to vo or, with cand_k, the block's K best cells; the histogram added to hist_e
 // (may be null).  hist_s: kHistBins zeros in shared memory.
@@ -619,7 +610,7 @@ k_vote_coarse_exact(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const i
     }
     const long long ncell = (long long)ntile * g.bins[1] * g.bins[2] * Bl;
     const long long co = ((long long)e * gridDim.x + blockIdx.x) * Kc;
-    coarse_output(g, pl, has_cell, d, p, w, z, hist_s, hist + (long long)e * kHistBins,
+    coarse_output(g, pl, has_cell, d, p, w, z, hist_s, hist ? hist + (long long)e * kHistBins : nullptr,
                   votes ? votes + (long long)e * ncell : nullptr, cand_k ? cand_k + co : nullptr,
                   cand_v ? cand_v + co : nullptr, Kc);
     add_counts(ctr, cnt);
@@ -715,7 +706,7 @@ k_vote_coarse_mid(DevGeom g, int ev0, const HitRecD *hd, const int32_t *n_hits,
         atomicAdd(&hist_s[v], 1u);
     }
     __syncthreads();
-    for (int i = tid; i < kHistBins; i += nthr)
+    for (int i = tid; i < kHistBins && hist; i += nthr)
         if (hist_s[i]) atomicAdd(&hist[(long long)e * kHistBins + i], hist_s[i]);
     if (ctr) {   // work counters (diagnostics): midpoint prefixes / tails in the FP64 slots
         unsigned long long v[2] = {n_pre, n_tail};
@@ -808,17 +799,6 @@ static void launch_cells_mid(const DevGeom &g, int n_ev, const HitRecD *hd, cons
                                                             n_per_ev, out_keys, out_votes, status);
 }
 
-// Raises the dynamic shared-memory limit of a kernel once per process (the attribute is a
-// property of the function; setting it outside any stream capture keeps captures clean).
-static bool g_attr_cells[4] = {false, false, false, false};
-
-template <typename K> static void smem_limit_once(K kernel, bool &flag) {
-    if (!flag) {
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-        flag = true;
-    }
-}
-
 template <int K> static void launch_coarse_cert(const DevGeom &g, int ev0, int n_ev, const HitRecD *hd,
                                                const HitRecF *hf, const int32_t *n_hits, const uint32_t *active,
                                                int32_t *votes, uint32_t *hist, unsigned *status, cudaStream_t s,
@@ -850,76 +830,152 @@ void launch_vote_coarse(const DevGeom &g, int prec, int ev0, int n_ev, const Hit
 }
 
 // ---------------------------------------------------------------------------------------
-// Voting of explicit cells: either given keys (keys != nullptr, n_per_ev per event) or the
-// 32 children of each parent key (parents != nullptr).  Thread = one cell, looping over
-// all hits of its event; child keys are written out when parents are given.
+// Voting of explicit cells given by keys, one per thread, looping over all hits of its event.
+// The cell of a key: false when the key lies outside the level's grid.
 // ---------------------------------------------------------------------------------------
-template <int MODE>
-__global__ void __launch_bounds__(256)
-k_vote_cells(DevGeom g, const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
-             const uint32_t *active, int level, const uint64_t *keys, const uint64_t *parents,
-             long long n_per_ev, uint64_t *out_keys, int32_t *out_votes, unsigned *status) {
-    constexpr bool k64 = ModeOf<MODE>::k64, k32 = ModeOf<MODE>::k32;
-    extern __shared__ __align__(16) unsigned char smem[];
-    unsigned char *h64s = smem;
-    unsigned char *h32s = smem + (k64 ? kHitCap * 80 : 0);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + (k64 ? kHitCap * 80 : 0) + (k32 ? kHitCap * 80 : 0));
-    const int ev = blockIdx.y;
-    int nh = n_hits[ev];
-    if (nh < 0) nh = 0;
-    const unsigned bytes = (unsigned)nh * 80u;
-    bool ok = stage_to_smem(h64s, hd + (long long)ev * kHitCap, k64 ? bytes : 0u, h32s,
-                            hf + (long long)ev * kHitCap, k32 ? bytes : 0u, bar, status);
-    __syncthreads();
-    if (!ok) nh = 0;
-    long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n_per_ev) return;
-    uint64_t key;
-    if (parents) {
-        uint64_t pk = parents[(long long)ev * (n_per_ev / 32) + j / 32];
-        int idx[5], b = (int)(j % 32);
-        unpack_key(g, pk, idx);
-#pragma unroll
-        for (int a = 0; a < 5; a++) idx[a] = 2 * idx[a] + ((b >> a) & 1);
-        key = pack_key(g, idx);
-    } else if (keys) {
-        key = keys[(long long)ev * n_per_ev + j];
-    } else {   // the level-0 grid in linear order (d0 fastest)
-        int idx[5];
-        long long r = j;
-#pragma unroll
-        for (int a = 0; a < 5; a++) { idx[a] = (int)(r % g.bins[a]); r /= g.bins[a]; }
-        key = pack_key(g, idx);
-    }
-    int idx[5];
+__device__ __forceinline__ bool key_cell(const DevGeom &g, int level, uint64_t key, int idx[5], Cell<double> &c) {
     unpack_key(g, key, idx);
-    long long o = (long long)ev * n_per_ev + j;
     bool valid = true;
 #pragma unroll
     for (int a = 0; a < 5; a++) valid = valid && idx[a] < (g.bins[a] << level);
-    if (!valid) {   // a key outside the grid of this level: no lookup, vote count -1
-        out_votes[o] = -1;
-        if (out_keys) out_keys[o] = key;
-        return;
-    }
-    Cell<double> c{edge(g, 0, level, idx[0]), sin_phi0(g, level, idx[1]), cos_phi0(g, level, idx[1]),
-                   edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
-    Cell<float> c32{to_prec<float>(c.D), to_prec<float>(c.S0), to_prec<float>(c.C0),
-                    to_prec<float>(c.W), to_prec<float>(c.Z), to_prec<float>(c.L)};
-    const SeriesConsts &k = g.k;
+    if (valid)
+        c = Cell<double>{edge(g, 0, level, idx[0]), sin_phi0(g, level, idx[1]), cos_phi0(g, level, idx[1]),
+                         edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
+    return valid;
+}
+__device__ __forceinline__ IV<double> warp_hull(IV<double> a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        a = hull2(a, IV<double>{__shfl_xor_sync(0xffffffffu, a.lo, o), __shfl_xor_sync(0xffffffffu, a.hi, o)});
+    return a;
+}
+
+// FP64 (K = 64) and outward FP32 (K = 32) votes, decided by certified FP32 end points (see
+// coarse_block).  The parent is the smallest box around the warp's 32 cells: for the 32 children
+// of one cell, as apo_refine lists them, that cell; for scattered keys it is wide, its bound
+// decides little, and the pairs are evaluated one by one with their own bounds.
+constexpr int kCellsThreads = 128;
+struct CellsSmem {
+    static constexpr size_t hits = 0;
+    static constexpr size_t queue = kHitCap * 80;
+    static constexpr size_t err = queue + ((sizeof(CertQueue<kCellsThreads>) + 15) & ~size_t(15));
+    static constexpr size_t mask = err + sizeof(float) * kHitCap * (kCellsThreads / 32);
+    static constexpr size_t bar = mask + 32 * (kCellsThreads / 32);
+    static constexpr size_t total = bar + 16;
+};
+template <int K>
+__global__ void __launch_bounds__(kCellsThreads, 4)
+k_vote_cells(const __grid_constant__ DevGeom g, const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
+             const uint32_t *active, int level, const uint64_t *keys, long long n_per_ev, int32_t *out_votes,
+             unsigned *status) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned char *hs = smem + CellsSmem::hits;
+    CertQueue<kCellsThreads> &q = *reinterpret_cast<CertQueue<kCellsThreads> *>(smem + CellsSmem::queue);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, ev = blockIdx.y;
+    float *err_w = reinterpret_cast<float *>(smem + CellsSmem::err) + wid * kHitCap;
+    uint32_t *mask_w = reinterpret_cast<uint32_t *>(smem + CellsSmem::mask) + wid * 8;
+    const bool outgoing = g.k.outgoing != 0;
+    int nh = n_hits[ev];
+    if (nh < 0) nh = 0;
+    if (tid == 0) q.n = 0;
+    const bool ok = stage_to_smem(hs, hf + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr, nullptr, 0u,
+                                  reinterpret_cast<uint64_t *>(smem + CellsSmem::bar), status);
+    __syncthreads();
+    if (!ok) nh = 0;
+    const int nw = (nh + 31) >> 5;
     const uint32_t *act = active ? active + (long long)ev * 8 : nullptr;
-    int v = 0;
-    for (int h = 0; h < nh; h++) {
-        if (act && !((act[h >> 5] >> (h & 31)) & 1u)) continue;
-        bool vt = true;
-        if (k32) vt = vote_pair<float>(c32, load_hit<float>(h32s + h * 80), k);
-        if (k64 && vt)
-            vt = ModeOf<MODE>::exact ? vote_pair_exact(c, load_hit<double>(h64s + h * 80), k)
-                                     : vote_pair<double>(c, load_hit<double>(h64s + h * 80), k);
-        v += vt ? 1 : 0;
+    const long long j0 = (long long)blockIdx.x * kCellsThreads, j = j0 + tid;
+    const uint64_t *keys_e = keys + (long long)ev * n_per_ev;
+    const IV<double> none{1e300, -1e300};
+    Cell<double> c64{none, none, none, none, none, none};
+    int idx[5] = {0, 0, 0, 0, 0};
+    const bool in = j < n_per_ev, has = in && key_cell(g, level, keys_e[j], idx, c64);
+    {   // the warp's parent, one hit per lane
+        const bool any = __any_sync(0xffffffffu, has);
+        const IV<double> D = warp_hull(c64.D), S0 = warp_hull(c64.S0), C0 = warp_hull(c64.C0), W = warp_hull(c64.W),
+                         Z = warp_hull(c64.Z), L = warp_hull(c64.L);
+        for (int h = lane; h < nw * 32; h += 32) {
+            bool keep = any && h < nh && (!act || ((act[h >> 5] >> (h & 31)) & 1u));
+            if (keep) {
+                const float e = parent_error<K>(g, D, S0, C0, W, Z, L, hs + h * 80);
+                err_w[h] = e;
+                keep = !(e < 0.f);
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (lane == 0) mask_w[h >> 5] = m;
+        }
+        __syncwarp();
     }
-    out_votes[o] = v;
-    if (out_keys) out_keys[o] = key;
+    bool guard;
+    const bool mir = omega_sign<K>(c64.W, &guard);
+    const cert::CellX<0> c = cert_cell<0>(c64, mir);
+    const cert::X<0> R = cert::recip(c.W);
+    int v = 0, wd = -1;
+    uint32_t m = 0;
+    bool left = has;
+    while (__syncthreads_or(left)) {
+        for (int step = 0; step < kCertStep && left; step++) {
+            while (!m && ++wd < nw) m = mask_w[wd];
+            if (!m) { left = false; break; }
+            const int h = wd * 32 + __ffs(m) - 1;
+            m &= m - 1;
+            if (guard) { v++; continue; }
+            const float e = err_w[h];
+            int r = cert::kUnknown;
+            if (e < 1e30f) {
+                const cert::HitX<0> hx = cert_hit<0>(hs + h * 80, mir);
+                const cert::PreX<0> pre = cert::prefix(c, hx);
+                r = cert_direction(pre, outgoing, e);
+                if (r == cert::kYes) r = cert_tail(pre, c.L, hx, R, c.W, e);
+            }
+            v += r == cert::kYes;
+            if (r == cert::kUnknown) q.push(tid, h, 1u);
+        }
+        __syncthreads();
+        const int nq = (int)q.n;
+        if (nq > kCertDrain || !__syncthreads_or(left)) {
+            for (int i = tid; i < nq; i += kCellsThreads) {
+                const int oh = (int)(q.id[i] >> 16);
+                int x[5];
+                unpack_key(g, keys_e[j0 + (q.id[i] & 0xffffu)], x);
+                q.mask[i] = resolve<K>(g, level, x[0], x[1], x[2], x[3], x[4], 1u, hd + (long long)ev * kHitCap + oh,
+                                       hf + (long long)ev * kHitCap + oh);
+            }
+            __syncthreads();
+            for (int i = 0; i < nq; i++)
+                if ((int)(q.id[i] & 0xffffu) == tid) v += q.mask[i] & 1u;
+            __syncthreads();
+            if (tid == 0) q.n = 0;
+        }
+    }
+    if (in) out_votes[(long long)ev * n_per_ev + j] = has ? v : -1;   // -1: a key outside the level's grid
+}
+
+// The exact-phase program on explicit cells, FP64.
+__global__ void __launch_bounds__(256)
+k_vote_cells_exact(DevGeom g, const HitRecD *hd, const int32_t *n_hits, const uint32_t *active, int level,
+                   const uint64_t *keys, long long n_per_ev, int32_t *out_votes, unsigned *status) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int ev = blockIdx.y;
+    int nh = n_hits[ev];
+    if (nh < 0) nh = 0;
+    const bool ok = stage_to_smem(smem, hd + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr, nullptr, 0u,
+                                  reinterpret_cast<uint64_t *>(smem + kHitCap * 80), status);
+    __syncthreads();
+    if (!ok) nh = 0;
+    const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n_per_ev) return;
+    const uint32_t *act = active ? active + (long long)ev * 8 : nullptr;
+    int idx[5], v = -1;   // -1: a key outside the level's grid
+    Cell<double> c;
+    if (key_cell(g, level, keys[(long long)ev * n_per_ev + j], idx, c)) {
+        v = 0;
+        for (int h = 0; h < nh; h++) {
+            if (act && !((act[h >> 5] >> (h & 31)) & 1u)) continue;
+            v += vote_pair_exact(c, load_hit<double>(smem + h * 80), g.k) ? 1 : 0;
+        }
+    }
+    out_votes[(long long)ev * n_per_ev + j] = v;
 }
 
 // Children of kept cells, two per thread: the children 2 idx + bit of a parent that differ
@@ -1127,48 +1183,23 @@ k_vote_children_exact(DevGeom g, const HitRecD *hd, const int32_t *n_hits, const
     pair_store(g, idx, j, v0, v1, out_keys + (long long)ev * n_par * 32, out_votes + (long long)ev * n_par * 32);
 }
 
-template <int MODE>
-static void launch_cells_mode(const DevGeom &g, int n_ev, const HitRecD *hd, const HitRecF *hf,
-                              const int32_t *n_hits, const uint32_t *active, int level,
-                              const uint64_t *keys, const uint64_t *parents, long long n_per_ev,
-                              uint64_t *out_keys, int32_t *out_votes, unsigned *status, cudaStream_t s,
-                              int block) {
-    smem_limit_once(k_vote_cells<MODE>, g_attr_cells[MODE]);
-    size_t sm = (ModeOf<MODE>::k64 ? kHitCap * 80 : 0) + (ModeOf<MODE>::k32 ? kHitCap * 80 : 0) + 16;
-    dim3 grid((unsigned)((n_per_ev + block - 1) / block), n_ev);
-    k_vote_cells<MODE><<<grid, block, sm, s>>>(g, hd, hf, n_hits, active, level, keys, parents, n_per_ev,
-                                                out_keys, out_votes, status);
-}
-
-static void launch_cells(const DevGeom &g, int prec, int n_ev, const HitRecD *hd, const HitRecF *hf,
-                         const int32_t *n_hits, const uint32_t *active, int level,
-                         const uint64_t *keys, const uint64_t *parents, long long n_per_ev,
-                         uint64_t *out_keys, int32_t *out_votes, unsigned *status, cudaStream_t s,
-                         int block = 256) {
-    if (block != 128) block = 256;
-    if (prec == APO_F64_MID)
-        launch_cells_mid(g, n_ev, hd, n_hits, active, level, keys, parents, n_per_ev, out_keys, out_votes,
-                         status, s, block);
-    else if (prec == APO_F64_EXACT)
-        launch_cells_mode<kModeF64Exact>(g, n_ev, hd, hf, n_hits, active, level, keys, parents, n_per_ev,
-                                         out_keys, out_votes, status, s, block);
-    else if (prec == APO_F32)
-        launch_cells_mode<kModeF32>(g, n_ev, hd, hf, n_hits, active, level, keys, parents, n_per_ev,
-                                    out_keys, out_votes, status, s, block);
-    else if (prec == APO_F64_FILTERED)
-        launch_cells_mode<kModeF64Filtered>(g, n_ev, hd, hf, n_hits, active, level, keys, parents,
-                                            n_per_ev, out_keys, out_votes, status, s, block);
-    else
-        launch_cells_mode<kModeF64>(g, n_ev, hd, hf, n_hits, active, level, keys, parents, n_per_ev,
-                                    out_keys, out_votes, status, s, block);
-}
-
 void launch_vote_keys(const DevGeom &g, int prec, int n_ev, const HitRecD *hd, const HitRecF *hf,
                       const int32_t *n_hits, int level, const uint64_t *keys, long long n_per_ev,
                       int32_t *votes, cudaStream_t s, const uint32_t *active) {
     if (n_ev <= 0 || n_per_ev <= 0) return;
-    launch_cells(g, prec, n_ev, hd, hf, n_hits, active, level, keys, nullptr, n_per_ev, nullptr, votes,
-                 nullptr, s);
+    dim3 grid((unsigned)((n_per_ev + kCellsThreads - 1) / kCellsThreads), n_ev);
+    if (prec == APO_F64_MID) {
+        launch_cells_mid(g, n_ev, hd, n_hits, active, level, keys, nullptr, n_per_ev, nullptr, votes, nullptr, s, 256);
+    } else if (prec == APO_F64_EXACT) {
+        k_vote_cells_exact<<<dim3((unsigned)((n_per_ev + 255) / 256), n_ev), 256, kHitCap * 80 + 16, s>>>(
+            g, hd, n_hits, active, level, keys, n_per_ev, votes, nullptr);
+    } else if (prec == APO_F32) {
+        k_vote_cells<32><<<grid, kCellsThreads, CellsSmem::total, s>>>(g, hd, hf, n_hits, active, level, keys, n_per_ev,
+                                                                       votes, nullptr);
+    } else {   // APO_F64 and APO_F64_FILTERED: the same votes, the same kernel
+        k_vote_cells<64><<<grid, kCellsThreads, CellsSmem::total, s>>>(g, hd, hf, n_hits, active, level, keys, n_per_ev,
+                                                                       votes, nullptr);
+    }
 }
 
 template <int K>
@@ -1215,15 +1246,12 @@ void init_kernel_attributes() {
     cudaFuncSetAttribute(k_vote_coarse<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_coarse<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_coarse_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_cells<kModeF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_cells<kModeF64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_cells<kModeF64Filtered>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_children<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_children<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_children_exact<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_children_exact<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_vote_cells<kModeF64Exact>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    for (int i = 0; i < 4; i++) g_attr_cells[i] = true;
+    cudaFuncSetAttribute(k_vote_cells<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_vote_cells<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1592,7 +1620,6 @@ __device__ __forceinline__ void estimate_mask_block(const DevGeom &g, const uint
         __syncthreads();
         return;
     }
-    const SeriesConsts &k = g.k;
     const long long pairs = (long long)m * nh;
     for (long long q = tid; q < pairs; q += blockDim.x) {
         const int j = (int)(q / nh), i = (int)(q % nh);
@@ -1602,11 +1629,7 @@ __device__ __forceinline__ void estimate_mask_block(const DevGeom &g, const uint
         unpack_key(g, s[j] & kKeyMask, idx);
         Cell<double> c{edge(g, 0, level, idx[0]), sin_phi0(g, level, idx[1]), cos_phi0(g, level, idx[1]),
                        edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
-        Hit<double> h = load_hit<double>(hd_e + i);
-        const double d = h.d.lo;
-        const double dlo = __dsub_rd(d, width);
-        h.d = {gt0(dlo) ? dlo : 0.0, __dadd_ru(d, width)};
-        if (vote_pair<double>(c, h, k)) atomicAnd(&act1[i >> 5], ~(1u << (i & 31)));
+        if (vote_widened(g, c, hd_e + i, width)) atomicAnd(&act1[i >> 5], ~(1u << (i & 31)));
     }
     __syncthreads();
     if (tid < 8) active_e[tid] = act1[tid];
@@ -1623,7 +1646,7 @@ __device__ __forceinline__ void estimate_mask_block(const DevGeom &g, const uint
 }
 
 __global__ void __launch_bounds__(256)
-k_estimate_mask(DevGeom g, const uint64_t *keys, const int32_t *votes, int n_in, int level,
+k_estimate_mask(const __grid_constant__ DevGeom g, const uint64_t *keys, const int32_t *votes, int n_in, int level,
                 const int32_t *n_hits, uint32_t *active, int32_t *done, const HitRecD *hd,
                 int round, int max_tracks, int min_votes, double width, apo_track *out,
                 int32_t *n_tracks, const int32_t *offsets, int32_t *hit_track) {
@@ -1704,13 +1727,13 @@ __global__ void __launch_bounds__(128, 3) k_solve_persistent(const __grid_consta
             if (A.done[e]) break;
             for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist_b[i] = 0u;
             __syncthreads();
-            if (A.mode[0] == kModeF32) persist_coarse<32>(g, A, e, vo, hist_b, smem);
+            if (A.mode[0] == kPersistF32) persist_coarse<32>(g, A, e, vo, hist_b, smem);
             else persist_coarse<64>(g, A, e, vo, hist_b, smem);
             __threadfence_block();
             __syncthreads();
             select_coarse_block(g, vo, hist_b, K, A.fk + (long long)e * K, A.fv + (long long)e * K);
             for (int lev = 1; lev <= lv; lev++) {
-                if (A.mode[lev] == kModeF32) persist_children<32>(g, A, e, lev, smem);
+                if (A.mode[lev] == kPersistF32) persist_children<32>(g, A, e, lev, smem);
                 else persist_children<64>(g, A, e, lev, smem);
                 topk_block(A.ck + (long long)e * K * 32, A.cv + (long long)e * K * 32, K * 32, K,
                            A.fk + (long long)e * K, A.fv + (long long)e * K, s_sort);
@@ -1723,9 +1746,6 @@ __global__ void __launch_bounds__(128, 3) k_solve_persistent(const __grid_consta
         }
     }
 }
-
-static_assert(kPersistF32 == kModeF32 && kPersistF64 == kModeF64 && kPersistF64Filtered == kModeF64Filtered,
-              "persistent launch modes");
 
 size_t persist_smem_bytes(const DevGeom &g) {
     size_t a = CoarseSmem::total(g.bins[4], coarse_plan(g, false).tiles);

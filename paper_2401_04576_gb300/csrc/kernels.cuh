@@ -190,9 +190,9 @@ struct MaxsetArgs {
 };
 // Persistent batch search (kernels.cu): the top-K schedule with multi-track rounds, every
 // event's whole search in one block, blocks pulling events from next_event (zeroed by the
-// host).  mode[L]: the vote kernel mode of level L (FP32, FP64 or FP32-filtered FP64).
+// host).  mode[L]: the votes of level L (FP32 or FP64).
 // votes / hist: per-block scratch (blocks x level-0 cells, blocks x kHistBins).
-enum : int { kPersistF32 = 0, kPersistF64 = 1, kPersistF64Filtered = 2 };   // the vote kernel modes
+enum : int { kPersistF32 = 0, kPersistF64 = 1 };   // the votes of a level
 struct PersistArgs {
     int n_events, max_tracks, min_votes;
     double width;

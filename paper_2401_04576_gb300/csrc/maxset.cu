@@ -24,6 +24,7 @@
 
 #include <climits>
 
+#include "cert_vote.cuh"
 #include "kernels.cuh"
 
 namespace apo {
@@ -51,36 +52,13 @@ __device__ __forceinline__ Cell<double> cell_at(const DevGeom &g, int level, con
                         edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
 }
 
-__device__ __forceinline__ Cell<float> cell32(const Cell<double> &c) {
-    return Cell<float>{to_prec<float>(c.D), to_prec<float>(c.S0), to_prec<float>(c.C0), to_prec<float>(c.W),
-                       to_prec<float>(c.Z), to_prec<float>(c.L)};
-}
-
 // The vote of staged hit i for a cell at the level's precision code, as the voting
-// kernels count it (FP32 cells are the FP64 edges rounded outward; the FP32-filtered mode
-// votes as FP64).  FP64 (expansion) votes are decided by the FP32 program first: its
-// intervals contain the FP64 ones, so an FP32 refusal is an FP64 refusal.
-__device__ __forceinline__ bool vote_at(const DevGeom &g, int prec, const Cell<double> &c, const HitRecD *hd,
-                                        const HitRecF *hf, int i) {
-    if (prec == APO_F32) return vote_pair<float>(cell32(c), load_hit<float>(hf + i), g.k);
+// kernels count it (FP32 cells are the FP64 edges rounded outward).
+__device__ __noinline__ bool vote_at(const DevGeom &g, int prec, const Cell<double> &c, const HitRecD *hd,
+                                     const HitRecF *hf, int i) {
+    if (prec == APO_F32) return vote_single<32>(g, c, hd + i, hf + i);
     if (prec == APO_F64_EXACT) return vote_pair_exact(c, load_hit<double>(hd + i), g.k);
-    if (!vote_pair<float>(cell32(c), load_hit<float>(hf + i), g.k)) return false;
-    return vote_pair<double>(c, load_hit<double>(hd + i), g.k);
-}
-
-// The FP64 vote of staged hit i for a cell with its drift widened to [max(rd(d - width),
-// 0), ru(d + width)] (the hit finding), decided by the FP32 program on the outward-rounded
-// FP32 copy of that interval first.
-__device__ __forceinline__ bool vote_widened(const DevGeom &g, const Cell<double> &c, const Cell<float> &c32,
-                                             const HitRecD *hd, const HitRecF *hf, int i, double width) {
-    Hit<double> h = load_hit<double>(hd + i);
-    const double d = h.d.lo;
-    const double dlo = __dsub_rd(d, width);
-    h.d = {gt0(dlo) ? dlo : 0.0, __dadd_ru(d, width)};
-    Hit<float> h32 = load_hit<float>(hf + i);
-    h32.d = {__double2float_rd(h.d.lo), __double2float_ru(h.d.hi)};
-    if (!vote_pair<float>(c32, h32, g.k)) return false;
-    return vote_pair<double>(c, h, g.k);
+    return vote_single<64>(g, c, hd + i, hf + i);
 }
 
 // Estimate from per-axis index counters (off[a] .. off[a + 1] - 1 hold axis a's bins at
@@ -119,7 +97,7 @@ __device__ __forceinline__ void ordered_estimate(const DevGeom &g, int level, in
 }
 
 __global__ void __launch_bounds__(kMsThreads)
-k_maxset_select(DevGeom g, MaxsetArgs A) {
+k_maxset_select(const __grid_constant__ DevGeom g, const __grid_constant__ MaxsetArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t *cnt = reinterpret_cast<uint32_t *>(smem);    // per-axis index counters
     __shared__ uint32_t hist[kHistBins];
@@ -331,7 +309,7 @@ constexpr int kTfThreads = 192;  // the step's end: one warp per axis for the es
 // shared memory, the queue is tested one cell per thread, and the hit finding runs over
 // the (track cell, hit) pairs one pair per thread, so that whole warps do the votes.
 __global__ void __launch_bounds__(kTsThreads, 3)
-k_track_cells(DevGeom g, MaxsetArgs A) {
+k_track_cells(const __grid_constant__ DevGeom g, const __grid_constant__ MaxsetArgs A) {
     const int e = blockIdx.y, tid = threadIdx.x;
     TrackStep &ts = A.ts[e];
     if (!ts.flag) return;
@@ -404,7 +382,7 @@ k_track_cells(DevGeom g, MaxsetArgs A) {
             int idx[5];
             cell_index(g, ke, base + s_t[q], idx);
             const Cell<double> c = cell_at(g, A.level, idx);
-            if (vote_widened(g, c, cell32(c), hde, hfe, i, A.width)) atomicOr(&ts.take[i >> 5], bit);
+            if (vote_widened(g, c, hde + i, A.width)) atomicOr(&ts.take[i >> 5], bit);
         }
         __syncthreads();   // the queues are refilled by the next chunk
     }
