@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/apo4.h"
+#include "cert4.cuh"
 #include "fourd.cuh"
 #include "kernels.cuh"
 
@@ -194,41 +195,115 @@ __device__ __forceinline__ Col4<T> column4(const Iter4 &it, const double *le, co
     return c;
 }
 
+// ---------------------------------------------------------------------------------------
+// The votes (of the program in T) are decided by certified FP32 values (cert4.cuh).  Per
+// (column, hit) one evaluation with errors over the z0 voxels gives the bound that
+// all its (voxel, sign) pairs share (over each half of the z0 voxels where the whole range decides
+// nothing); the pairs left undecided are queued and evaluated by the program itself in whole warps.
+// FP32 issue bounds it; evaluating every pair was bound by the FP64 pipe, and in FP32 by the
+// instructions of correctly rounded quotients and roots.
+// ---------------------------------------------------------------------------------------
+constexpr int k4Threads = 128, k4Drain = 128, k4Queue = k4Drain + k4Threads;
+
+template <int K> __device__ __forceinline__ cert::X<K> wide(float v) {   // a value rounded to v
+    return cert::point(cert::sc<K>(v));
+}
+template <int K> __device__ __forceinline__ cert::X<K> wide(float lo, float hi) {
+    cert::X<K> r;
+    r.lo = lo;
+    r.hi = hi;
+    r.e = 2.f * cert::rnd<K>(cert::mag2(lo, hi)) + cert::kTiny;
+    return r;
+}
+template <int K> __device__ __forceinline__ cert::X<K> wide(cert::X<0> x) { return wide<K>(x.lo, x.hi); }
+
+// bound4 from the child's own FP32 values; out of the callers' registers
+template <int K>
+__device__ __noinline__ cert::Bound4 column_bound(cert::Col4X<cert::Pt> m, cert::Box4X<0> b, float zc0, float zc1,
+                                                  float z0, float z1, const cert::Hit4X<cert::Pt> *hp) {
+    cert::Col4X<cert::X<K>> M;
+    cert::Hit4X<cert::X<K>> H;
+    const cert::Pt *src = &m.xc, *hs = &hp->x0;
+    cert::X<K> *dst = &M.xc, *hd = &H.x0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) dst[i] = wide<K>(src[i].v);
+#pragma unroll
+    for (int i = 0; i < 9; i++) hd[i] = wide<K>(hs[i].v);
+    M.ion.e *= 2.f;   // an approximate reciprocal
+    return cert::bound4<K>(M, cert::Box4X<K>{wide<K>(b.X_), wide<K>(b.Y_), wide<K>(b.dR)}, wide<K>(zc0, zc1),
+                           wide<K>(z0, z1), H);
+}
+
+// The program's votes of one (column, hit) for the z0 voxels b0 (tan(lambda) > 0) and b1 (< 0).
 template <typename T>
-__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 3 : 5)
-k4_vote(Iter4 it, int ev0, const int32_t *n_hits, const HitRecD *hd, const uint32_t *active,
-        const double *lo, const double *ref, int32_t *votes, int32_t *vmax, int sign_only) {
-    __shared__ HitP<T> s_h[kHitCap];
-    __shared__ HitI<T> s_w[kHitCap];
-    __shared__ T s_zc[32];
-    __shared__ IV<T> s_z[32];
+__device__ __noinline__ uint2 resolve4(const Iter4 &it, const double *le, const double *rf, long long col,
+                                       const HitRecD *rec, uint32_t b0, uint32_t b1) {
+    const Col4<T> c = column4<T>(it, le, rf, col);
+    const HitP<T> h = hit_point<T>(*rec);
+    const HitI<T> w = hit_iv<T>(*rec);
+    uint2 yes = make_uint2(0u, 0u);
+    uint32_t m = b0 | b1;
+    while (m) {
+        const int iz = __ffs(m) - 1;
+        const uint32_t bit = 1u << iz;
+        m &= m - 1;
+        const double zl = edge4(le[3], iz, it.w[3]), zh = edge4(le[3], iz + 1, it.w[3]);
+        const Pre4<T> pre = prefix4<T>(c.m, rn<T>(mid4(zl, zh)), h);
+        if (pre.guard) {
+            yes.x |= b0 & bit;
+            yes.y |= b1 & bit;
+            continue;
+        }
+        const IV<T> A2 = a2_4<T>(c.X, c.Y, box_iv<T>(zl, zh), w);
+#pragma unroll 1
+        for (int s = 0; s < 2; s++) {
+            if (!((s ? b1 : b0) & bit)) continue;
+            if (pair4<T>(c.m, pre, s ? -1 : 1, h, A2, c.Rv)) { if (s) yes.y |= bit; else yes.x |= bit; }
+        }
+    }
+    return yes;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(k4Threads, 4)
+k4_vote(const __grid_constant__ Iter4 it, int ev0, const int32_t *n_hits, const HitRecD *hd,
+             const uint32_t *active, const double *lo, const double *ref, int32_t *votes, int32_t *vmax,
+             int sign_only) {
+    constexpr int K = sizeof(T) == 8 ? 64 : 32;
+    __shared__ cert::Hit4X<cert::Pt> s_h[kHitCap];
+    __shared__ unsigned char s_i[kHitCap];
+    __shared__ float s_zc[32];
+    __shared__ float2 s_z[32];
     __shared__ short s_col[kTile4];
-    __shared__ int s_n, s_np, s_vmax[2];
+    __shared__ uint32_t q_id[k4Queue], q_b0[k4Queue], q_b1[k4Queue];
+    __shared__ int s_n, s_np, s_nq, s_vmax[2];
     const int el = blockIdx.y, e = ev0 + el, tid = threadIdx.x;
     int nh = n_hits[e];
     if (nh < 0) nh = 0;
-    if (tid == 0) { s_n = 0; s_np = 0; s_vmax[0] = s_vmax[1] = 0; }
+    if (tid == 0) { s_n = 0; s_np = 0; s_nq = 0; s_vmax[0] = s_vmax[1] = 0; }
     __syncthreads();
     const uint32_t *act = active + (long long)e * 8;
-    for (int i = tid; i < nh; i += blockDim.x) {
+    const HitRecD *hde = hd + (long long)e * kHitCap;
+    for (int i = tid; i < nh; i += k4Threads) {
         if (!((act[i >> 5] >> (i & 31)) & 1u)) continue;
-        const HitRecD r = hd[(long long)e * kHitCap + i];
         const int j = atomicAdd(&s_n, 1);
-        s_h[j] = hit_point<T>(r);
-        s_w[j] = hit_iv<T>(r);
+        cert::Pt *f = &s_h[j].x0;
+#pragma unroll
+        for (int k = 0; k < 9; k++) f[k].v = (float)hde[i].v[k];
+        s_i[j] = (unsigned char)i;
     }
     const double *le = lo + (long long)e * 4;
-    for (int iz = tid; iz < it.n[3]; iz += blockDim.x) {
+    for (int iz = tid; iz < it.n[3]; iz += k4Threads) {
         const double zl = edge4(le[3], iz, it.w[3]), zh = edge4(le[3], iz + 1, it.w[3]);
-        s_zc[iz] = rn<T>(mid4(zl, zh));
-        s_z[iz] = box_iv<T>(zl, zh);
+        s_zc[iz] = (float)mid4(zl, zh);
+        s_z[iz] = make_float2((float)zl, (float)zh);
     }
     const double *rf = ref + (long long)e * 2;
     const int nz = it.n[3];
     int32_t *vo = votes + (long long)el * 2 * it.nvox;
     const long long col0 = (long long)blockIdx.x * kTile4;
     // disk pre-filter of the tile; failing columns get zero votes
-    for (int k = tid; k < kTile4; k += blockDim.x) {
+    for (int k = tid; k < kTile4; k += k4Threads) {
         const long long col = col0 + k;
         if (col >= it.ncol) break;
         const Col4<T> c = column4<T>(it, le, rf, col);
@@ -242,38 +317,105 @@ k4_vote(Iter4 it, int ev0, const int32_t *n_hits, const HitRecD *hd, const uint3
     }
     __syncthreads();
     const int na = s_n, np = s_np;
+    const uint32_t allz = nz >= 32 ? 0xffffffffu : ((1u << nz) - 1u);
+    const uint32_t all0 = sign_only == 1 ? 0u : allz, all1 = sign_only == 0 ? 0u : allz;
     int mx[2] = {0, 0};
-    for (int i = tid; i < np; i += blockDim.x) {
-        const long long col = col0 + s_col[i];
-        const Col4<T> c = column4<T>(it, le, rf, col);
+    for (int base = 0; base < np; base += k4Threads) {
+        const bool has = base + tid < np;
+        const long long col = col0 + s_col[has ? base + tid : 0];
+        const Col4<T> cd = column4<T>(it, le, rf, col);
+        const T cR = cd.m.R;
+        const cert::Col4X<cert::Pt> m{{(float)cd.m.xc}, {(float)cd.m.yc}, {(float)cR}, {(float)cd.m.aL}, {(float)cd.m.ox},
+                                      {(float)cd.m.oy}, {cert::rcp_a((float)cd.m.on)}, {(float)cd.m.psi_ref}};
+        const cert::Box4X<0> b{cert::mk<0>(cd.X.lo, cd.X.hi), cert::mk<0>(cd.Y.lo, cd.Y.hi),
+                               cert::mk<0>((double)cd.Rv.lo - (double)cR, (double)cd.Rv.hi - (double)cR)};
+        const bool guard = cd.m.guard;
         uint32_t pl[2][9];
 #pragma unroll
         for (int s = 0; s < 2; s++)
 #pragma unroll
             for (int q = 0; q < 9; q++) pl[s][q] = 0u;
-        auto add_votes = [&](int s, uint32_t m) {
+        auto add_votes = [&](int s, uint32_t v) {
 #pragma unroll
             for (int q = 0; q < 9; q++) {
-                const uint32_t cy = pl[s][q] & m;
-                pl[s][q] ^= m;
-                m = cy;
+                const uint32_t cy = pl[s][q] & v;
+                pl[s][q] ^= v;
+                v = cy;
             }
         };
-        for (int j = 0; j < na; j++) {
-            const HitP<T> h = s_h[j];
-            const HitI<T> wi = s_w[j];
-            uint32_t b0 = 0, b1 = 0;
-            for (int iz = 0; iz < nz; iz++) {
-                const Pre4<T> pre = prefix4<T>(c.m, s_zc[iz], h);
-                if (pre.guard) { b0 |= 1u << iz; b1 |= 1u << iz; continue; }
-                const IV<T> A2 = a2_4<T>(c.X, c.Y, s_z[iz], wi);
-                if (sign_only != 1 && pair4<T>(c.m, pre, 1, h, A2, c.Rv)) b0 |= 1u << iz;
-                if (sign_only != 0 && pair4<T>(c.m, pre, -1, h, A2, c.Rv)) b1 |= 1u << iz;
+        for (int j = 0; j < na; j++) {   // at most one queue entry per thread and hit
+            if (has) {
+                uint32_t b0 = 0, b1 = 0, u0 = 0, u1 = 0;
+                if (guard) {
+                    b0 = all0;
+                    b1 = all1;
+                } else {
+                    const int half = (nz + 1) >> 1;
+                    cert::Bound4 e0 = column_bound<K>(m, b, s_zc[0], s_zc[nz - 1], s_z[0].x, s_z[nz - 1].y, s_h + j), e1 = e0;
+                    if (!(e0.e < 1e30f) && nz > 1) {
+                        e0 = column_bound<K>(m, b, s_zc[0], s_zc[half - 1], s_z[0].x, s_z[half - 1].y, s_h + j);
+                        e1 = column_bound<K>(m, b, s_zc[half], s_zc[nz - 1], s_z[half].x, s_z[nz - 1].y, s_h + j);
+                    }
+                    const cert::Hit4X<cert::Pt> h = s_h[j];
+#pragma unroll 1
+                    for (int iz = 0; iz < nz; iz++) {
+                        const uint32_t bit = 1u << iz;
+                        const float e = iz < half ? e0.e : e1.e, eps = iz < half ? e0.eps : e1.eps;
+                        bool bad = true;
+                        if (e < 1e30f) {
+                            cert::Pt dx, dy;
+                            cert::wire4x(m, cert::Pt{s_zc[iz]}, h, dx, dy);
+                            cert::Pre4X<cert::Pt> pre = cert::prefix4x(dx, dy, h);
+                            pre.psi = cert::psi4(m, dx, dy, pre.iRA, eps, bad);
+                            pre.Rpsi = cert::mul(m.R, pre.psi);
+                            if (!bad) {
+                                const float2 z = s_z[iz];
+                                const cert::X<0> A2 = cert::a2_4x<0, cert::Pt>(b, cert::X<0>{z.x, z.y, 0.f}, h);
+#pragma unroll 1
+                                for (int s = 0; s < 2; s++) {
+                                    if (sign_only == 1 - s) continue;
+                                    const int v = cert::vote4x(pre, m, s ? cert::neg(m.aL) : m.aL, h, A2, b.dR, e);
+                                    const uint32_t y = v == cert::kYes ? bit : 0u, u = v == cert::kUnknown ? bit : 0u;
+                                    if (s) { b1 |= y; u1 |= u; } else { b0 |= y; u0 |= u; }
+                                }
+                            }
+                        }
+                        if (bad) { u0 |= all0 & bit; u1 |= all1 & bit; }
+                    }
+                    if (u0 | u1) {
+                        const int k = atomicAdd(&s_nq, 1);
+                        if (k < k4Queue) {   // always: the queue is drained before it could fill
+                            q_id[k] = (uint32_t)tid | ((uint32_t)j << 16);
+                            q_b0[k] = u0;
+                            q_b1[k] = u1;
+                        }
+                    }
+                }
+                add_votes(0, b0);
+                add_votes(1, b1);
             }
-            add_votes(0, b0);
-            add_votes(1, b1);
+            __syncthreads();
+            const int nq = s_nq;
+            __syncthreads();
+            if (nq > k4Drain || (j + 1 == na && nq > 0)) {
+                for (int i = tid; i < nq; i += k4Threads) {
+                    const long long oc = col0 + s_col[base + (int)(q_id[i] & 0xffffu)];
+                    const uint2 y = resolve4<T>(it, le, rf, oc, hde + s_i[q_id[i] >> 16], q_b0[i], q_b1[i]);
+                    q_b0[i] = y.x;
+                    q_b1[i] = y.y;
+                }
+                __syncthreads();
+                for (int i = 0; i < nq; i++)
+                    if ((int)(q_id[i] & 0xffffu) == tid) {
+                        add_votes(0, q_b0[i]);
+                        add_votes(1, q_b1[i]);
+                    }
+                __syncthreads();
+                if (tid == 0) s_nq = 0;
+                __syncthreads();
+            }
         }
-        for (int s = 0; s < 2; s++) {
+        for (int s = 0; s < 2 && has; s++) {
             if (sign_only >= 0 && s != sign_only) continue;
             for (int iz = 0; iz < nz; iz++) {
                 int v = 0;
@@ -511,7 +653,7 @@ void launch_vote4(const Iter4 &it, int ev0, int n, const int32_t *nh, const HitR
                   const uint32_t *active, const double *lo, const double *ref, int32_t *votes,
                   int32_t *vmax, cudaStream_t s, int sign_only = -1) {
     dim3 grid((unsigned)((it.ncol + kTile4 - 1) / kTile4), n);
-    k4_vote<T><<<grid, 128, 0, s>>>(it, ev0, nh, hd, active, lo, ref, votes, vmax, sign_only);
+    k4_vote<T><<<grid, k4Threads, 0, s>>>(it, ev0, nh, hd, active, lo, ref, votes, vmax, sign_only);
 }
 
 void launch_stats4(const Iter4 &it, int ev0, int n, const int32_t *votes, const int32_t *vmax,
