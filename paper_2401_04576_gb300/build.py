@@ -13,8 +13,8 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libapo.so")
 SOURCES = ["kernels.cu", "apo_abi.cu", "diag.cu", "apo_noalloc.cu", "apo_serve.cu", "apo4.cu",
            "maxset.cu"]
-HEADERS = ["interval.cuh", "ipipe.cuh", "vote_program.cuh", "certified.cuh", "cert_point.cuh", "cert_vote.cuh",
-           "cert4.cuh", "kernels.cuh", "fourd.cuh"]
+HEADERS = ["interval.cuh", "ipipe.cuh", "vote_program.cuh", "certified.cuh", "cert_point.cuh", "cert_mid.cuh",
+           "cert_vote.cuh", "cert4.cuh", "kernels.cuh", "fourd.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xptxas", "-v",
          "--expt-relaxed-constexpr"]

@@ -1,13 +1,16 @@
-// Voting with certified FP32 decisions (certified.cuh) on the device data layout: the votes of
-// the FP64 (K = 64) or outward FP32 (K = 32) interval program, most of them decided by bare FP32
-// end points and one error bound per (parent cell, hit).
+// Voting with certified FP32 decisions (certified.cuh, cert_mid.cuh) on the device data layout: the
+// votes of the FP64 (K = 64) or outward FP32 (K = 32) interval program or of the midpoint form,
+// most of them decided by bare FP32 values and one error bound per (parent cell, hit).
 #pragma once
+#include "cert_mid.cuh"
 #include "certified.cuh"
 #include "kernels.cuh"
 
 namespace apo {
 
-template <int K> struct RefOf { using T = double; };   // the program whose votes K decides
+// The program whose votes K decides: 64 and 32 as above, kMid the midpoint form (FP64).
+constexpr int kMid = 1;
+template <int K> struct RefOf { using T = double; };
 template <> struct RefOf<32> { using T = float; };
 
 // The reference's sign and guard tests of a cell: its precision's omega interval.  Returns
@@ -61,6 +64,46 @@ __device__ __noinline__ float parent_error(const DevGeom &g, IV<double> D, IV<do
     return cert::verdict(x, g.k.outgoing != 0, e) == cert::kNo ? -1.f : e;
 }
 
+// The midpoint form's: (Sc, Cc) the sin / cos of the phi0 centres inside (their range); the other
+// centres lie in their cells.
+template <int K>
+__device__ __noinline__ float parent_error_mid(IV<double> D, IV<double> S0, IV<double> C0, IV<double> W, IV<double> Z,
+                                               IV<double> L, IV<double> Sc, IV<double> Cc, const void *rec) {
+    using N = cert::X<64>;
+    bool guard;
+    const bool mir = omega_sign<64>(W, &guard);
+    if (guard) return NAN;
+    const cert::CellX<64> c = cert_cell<64>(Cell<double>{D, S0, C0, W, Z, L}, mir);
+    const cert::HitX<64> hx = cert_hit<64>(rec, mir);
+    const cert::MidHit<N> h{cert::point(hx.x0), cert::point(hx.y0), cert::point(hx.sph), cert::point(hx.cph),
+                            cert::point(hx.t), cert::point(hx.spt), cert::point(hx.cpt), cert::point(hx.t2), hx.d};
+    const cert::MidCell<N> m{c.D, cxm<64>(Sc, mir), cx<64>(Cc), c.W, c.Z, cert::recip(c.W)};
+    N Gp, Gm;
+    cert::mid_tail<64, N>(cert::mid_prefix<64, N>(c, m, h), c.L, m, h, c.W, Gp, Gm);
+    // 1 %: the FP64 program's own distance from the real values
+    const float e = (Gp.e < 1e30f && Gm.e < 1e30f) ? 1.01f * fmaxf(Gp.e, Gm.e) : NAN;
+    return cert::decide(Gp, Gm, e) == cert::kNo ? -1.f : e;
+}
+
+// The parent of cells [i0, i1] per axis at `level` (ends included).
+template <int K>
+__device__ __forceinline__ float parent_span(const DevGeom &g, int level, const int (&i0)[5], const int (&i1)[5],
+                                             const void *rec) {
+    const IV<double> D = edge_span(g, 0, level, i0[0], i1[0]), W = edge_span(g, 2, level, i0[2], i1[2]),
+                     Z = edge_span(g, 3, level, i0[3], i1[3]), L = edge_span(g, 4, level, i0[4], i1[4]),
+                     S0 = hull2(sin_phi0(g, level, i0[1]), sin_phi0(g, level, i1[1])),
+                     C0 = hull2(cos_phi0(g, level, i0[1]), cos_phi0(g, level, i1[1]));
+    if constexpr (K == kMid) {
+        double s0, c0, s1, c1;
+        sincos_phi0_centre(g, level, i0[1], s0, c0);
+        sincos_phi0_centre(g, level, i1[1], s1, c1);
+        return parent_error_mid<K>(D, S0, C0, W, Z, L, IV<double>{mn(s0, s1), mx(s0, s1)}, IV<double>{mn(c0, c1), mx(c0, c1)},
+                                rec);
+    } else {
+        return parent_error<K>(g, D, S0, C0, W, Z, L, rec);
+    }
+}
+
 // Hits no parent could decide for a cell, one by one: the cell's own evaluation with errors,
 // then the reference program.  mask: tan(lambda) cells l0 + bit in question; returns those that
 // vote.  Not inlined: about one pair in 10^4 comes here,
@@ -68,29 +111,43 @@ __device__ __noinline__ float parent_error(const DevGeom &g, IV<double> D, IV<do
 template <int K>
 __device__ __noinline__ uint32_t resolve(const DevGeom &g, int level, int d, int p, int w, int z, int l0,
                                          uint32_t mask, const HitRecD *hd, const HitRecF *hf) {
-    using T = typename RefOf<K>::T;
     Cell<double> c{edge(g, 0, level, d), sin_phi0(g, level, p), cos_phi0(g, level, p), edge(g, 2, level, w),
                    edge(g, 3, level, z), {0.0, 0.0}};
-    bool guard;
-    const bool mir = omega_sign<K>(c.W, &guard);
-    const cert::HitX<K> h = cert_hit<K>(hf, mir);
     uint32_t yes = 0;
-    while (mask) {
-        const int b = __ffs(mask) - 1;
-        mask &= mask - 1;
-        c.L = edge(g, 4, level, l0 + b);
-        const cert::Eval<K> ev = cert::eval(cert_cell<K>(c, mir), h);
-        int v = cert::verdict(ev, g.k.outgoing != 0, cert::bound(ev));
-        if (guard) v = cert::kUnknown;
-        if (v == cert::kUnknown) {
-            const Cell<T> ct{to_prec<T>(c.D), to_prec<T>(c.S0), to_prec<T>(c.C0),
-                             to_prec<T>(c.W), to_prec<T>(c.Z), to_prec<T>(c.L)};
-            const void *rec = K == 64 ? static_cast<const void *>(hd) : static_cast<const void *>(hf);
-            v = vote_pair<T>(ct, load_hit<T>(rec), g.k) ? cert::kYes : cert::kNo;
+    if constexpr (K == kMid) {   // the midpoint form's own evaluation
+        MidCentre m;
+        sincos_phi0_centre(g, level, p, m.S0, m.C0);
+        m.D = pt::centre(c.D);
+        m.W = pt::centre(c.W);
+        m.Z = pt::centre(c.Z);
+        while (mask) {
+            const int b = __ffs(mask) - 1;
+            mask &= mask - 1;
+            if (mid_vote_pair(c, m, pt::centre(edge(g, 4, level, l0 + b)), load_hit<double>(hd))) yes |= 1u << b;
         }
-        if (v == cert::kYes) yes |= 1u << b;
+        return yes;
+    } else {
+        using T = typename RefOf<K>::T;
+        bool guard;
+        const bool mir = omega_sign<K>(c.W, &guard);
+        const cert::HitX<K> h = cert_hit<K>(hf, mir);
+        while (mask) {
+            const int b = __ffs(mask) - 1;
+            mask &= mask - 1;
+            c.L = edge(g, 4, level, l0 + b);
+            const cert::Eval<K> ev = cert::eval(cert_cell<K>(c, mir), h);
+            int v = cert::verdict(ev, g.k.outgoing != 0, cert::bound(ev));
+            if (guard) v = cert::kUnknown;
+            if (v == cert::kUnknown) {
+                const Cell<T> ct{to_prec<T>(c.D), to_prec<T>(c.S0), to_prec<T>(c.C0),
+                                 to_prec<T>(c.W), to_prec<T>(c.Z), to_prec<T>(c.L)};
+                const void *rec = K == 64 ? static_cast<const void *>(hd) : static_cast<const void *>(hf);
+                v = vote_pair<T>(ct, load_hit<T>(rec), g.k) ? cert::kYes : cert::kNo;
+            }
+            if (v == cert::kYes) yes |= 1u << b;
+        }
+        return yes;
     }
-    return yes;
 }
 
 // The reference's own evaluation of one pair, out of the callers' registers.
@@ -179,6 +236,54 @@ __device__ __forceinline__ int cert_direction(const cert::PreX<0> &p, bool outgo
     if (!outgoing) return cert::kYes;
     return p.wt.hi < -e ? cert::kNo : (p.wt.hi >= e ? cert::kYes : cert::kUnknown);
 }
+
+// One cell's evaluation per program: what a thread keeps of its cell, the tan(lambda)-free part per
+// hit, and one tan(lambda) cell's vote with the parent's error bound e.  L: the cell's end points,
+// or (midpoint form) its centre in .x.
+template <int K> struct Prog {
+    struct CellT { cert::CellX<0> c; cert::X<0> R; };
+    using HitT = cert::HitX<0>;
+    using Pre = cert::PreX<0>;
+    static __device__ __forceinline__ CellT cell(const DevGeom &, int, int, const Cell<double> &c, bool mir) {
+        const cert::CellX<0> x = cert_cell<0>(c, mir);
+        return CellT{x, cert::recip(x.W)};
+    }
+    static __device__ __forceinline__ float2 tanl(IV<double> L) { return make_float2((float)L.lo, (float)L.hi); }
+    static __device__ __forceinline__ HitT hit(const void *rec, bool mir) { return cert_hit<0>(rec, mir); }
+    static __device__ __forceinline__ Pre prefix(const CellT &c, const HitT &h) { return cert::prefix(c.c, h); }
+    static __device__ __forceinline__ int direction(const Pre &p, bool outgoing, float e) {
+        return cert_direction(p, outgoing, e);
+    }
+    static __device__ __forceinline__ int vote(const Pre &p, float2 L, const CellT &c, const HitT &h, float e) {
+        return cert_tail(p, cert::X<0>{L.x, L.y, 0.f}, h, c.R, c.c.W, e);
+    }
+};
+template <> struct Prog<kMid> {
+    struct CellT { cert::CellX<0> c; cert::MidCell<cert::Pt> m; };
+    using HitT = cert::MidHit<cert::Pt>;
+    using Pre = cert::MidPreX<0, cert::Pt>;
+    static __device__ __forceinline__ CellT cell(const DevGeom &g, int level, int p, const Cell<double> &c, bool mir) {
+        double s, co;
+        sincos_phi0_centre(g, level, p, s, co);
+        const float sg = mir ? -1.f : 1.f, W = sg * (float)pt::centre(c.W);
+        return CellT{cert_cell<0>(c, mir), {{sg * (float)pt::centre(c.D)}, {sg * (float)s}, {(float)co}, {W},
+                                            {(float)pt::centre(c.Z)}, {cert::rcp_a(W)}}};
+    }
+    static __device__ __forceinline__ float2 tanl(IV<double> L) { return make_float2((float)pt::centre(L), 0.f); }
+    static __device__ __forceinline__ HitT hit(const void *rec, bool mir) {
+        const cert::HitX<0> h = cert_hit<0>(rec, mir);
+        return HitT{{h.x0.v}, {h.y0.v}, {h.sph.v}, {h.cph.v}, {h.t.v}, {h.spt.v}, {h.cpt.v}, {h.t2.v}, {h.d.lo}};
+    }
+    static __device__ __forceinline__ Pre prefix(const CellT &c, const HitT &h) {
+        return cert::mid_prefix<0, cert::Pt>(c.c, c.m, h);
+    }
+    static __device__ __forceinline__ int direction(const Pre &, bool, float) { return cert::kYes; }
+    static __device__ __forceinline__ int vote(const Pre &p, float2 L, const CellT &c, const HitT &h, float e) {
+        cert::X<0> Gp, Gm;
+        cert::mid_tail<0, cert::Pt>(p, cert::Pt{L.x}, c.m, h, c.c.W, Gp, Gm);
+        return cert::decide(Gp, Gm, e);
+    }
+};
 
 // Bit-sliced vote counters: bit l of plane q is bit q of counter l (counts <= 256: 9 planes);
 // adding a mask of votes is a ripple-carry add.

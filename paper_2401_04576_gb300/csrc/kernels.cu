@@ -340,7 +340,7 @@ __device__ __forceinline__ void add_counts(unsigned long long *ctr, const unsign
     }
 }
 
-// FP64 (K = 64) and outward FP32 (K = 32) voting, decided by certified FP32 end points.
+// FP64 (K = 64), outward FP32 (K = 32) and midpoint-form voting, decided by certified FP32 values.
 // Phase 1: the parent test, one (tile, hit) per thread, gives the mask of hits that can vote and
 // the error bound that every cell of the tile shares.  Phase 2: the bare end points per
 // (cell, hit), bit-sliced counters; the undecided pairs are queued and resolved in whole warps.
@@ -397,10 +397,7 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan 
     if (nh < 0) nh = 0;
     for (int i = tid; i < kHistBins; i += nthr) hist_s[i] = 0;
     for (int i = tid; i < 8 * P.tiles; i += nthr) mask_s[i] = 0;
-    for (int l = tid; l < Bl; l += nthr) {
-        const cert::X<0> x = cx<0>(edge(g, 4, 0, l));
-        Ls[l] = make_float2(x.lo, x.hi);
-    }
+    for (int l = tid; l < Bl; l += nthr) Ls[l] = Prog<K>::tanl(edge(g, 4, 0, l));
     if (tid == 0) q.n = 0;
     const bool ok = stage_to_smem(hs, hf + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr, nullptr, 0u, bar,
                                   status);
@@ -421,10 +418,9 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan 
             const int part = (int)(t % P.parts), pw = (int)(t / P.parts), p = pw % Bp, w = pw / Bp;
             const int c0 = part * P.per, c1 = c0 + P.per < ntile ? c0 + P.per : ntile;
             const bool row = c0 / Bd == (c1 - 1) / Bd;   // cells of one z0 bin
-            e = parent_error<K>(g, edge_span(g, 0, 0, row ? c0 % Bd : 0, row ? (c1 - 1) % Bd : Bd - 1),
-                                sin_phi0(g, 0, p), cos_phi0(g, 0, p), edge(g, 2, 0, w),
-                                edge_span(g, 3, 0, c0 / Bd, (c1 - 1) / Bd), edge_span(g, 4, 0, 0, Bl - 1),
-                                hs + h * 80);
+            const int i0[5] = {row ? c0 % Bd : 0, p, w, c0 / Bd, 0};
+            const int i1[5] = {row ? (c1 - 1) % Bd : Bd - 1, p, w, (c1 - 1) / Bd, Bl - 1};
+            e = parent_span<K>(g, 0, i0, i1, hs + h * 80);
             keep = !(e < 0.f);
             cnt[3]++;
         }
@@ -448,8 +444,7 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan 
                            edge(g, 3, 0, z), {0.0, 0.0}};
     bool guard;
     const bool mir = omega_sign<K>(c64.W, &guard);
-    const cert::CellX<0> c = cert_cell<0>(c64, mir);
-    const cert::X<0> R = cert::recip(c.W);
+    const typename Prog<K>::CellT c = Prog<K>::cell(g, 0, p, c64, mir);
     int wd = -1;
     uint32_t m = 0;
     bool left = has_cell;
@@ -463,18 +458,17 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan 
             const float e = err_s[tl * kHitCap + h];
             uint32_t yes = 0, unk = all;
             if (e < 1e30f) {
-                const cert::HitX<0> hx = cert_hit<0>(hs + h * 80, mir);
-                const cert::PreX<0> pre = cert::prefix(c, hx);
+                const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
+                const typename Prog<K>::Pre pre = Prog<K>::prefix(c, hx);
                 cnt[4]++;
-                const int dir = cert_direction(pre, outgoing, e);
+                const int dir = Prog<K>::direction(pre, outgoing, e);
                 if (dir == cert::kNo) continue;
                 if (dir == cert::kYes) {
                     unk = 0;
                     cnt[5] += Bl;
 #pragma unroll 1
                     for (int l = 0; l < Bl; l++) {
-                        const float2 L = Ls[l];
-                        const int v = cert_tail(pre, cert::X<0>{L.x, L.y, 0.f}, hx, R, c.W, e);
+                        const int v = Prog<K>::vote(pre, Ls[l], c, hx, e);
                         yes |= (uint32_t)(v == cert::kYes) << l;
                         unk |= (uint32_t)(v == cert::kUnknown) << l;
                     }
@@ -618,117 +612,13 @@ k_vote_coarse_exact(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const i
 
 // ---------------------------------------------------------------------------------------
 // Midpoint-form voting (APO_F64_MID, Section 3.1's variant with the quantities of d^Ax at
-// the voxel centre).  Coarse grid: the same block / thread layout as k_vote_coarse, the
-// tan(lambda)-free part shared by the tan(lambda) bins, bit-sliced counters; there is no
-// parent-cell test, because the midpoint form is not inclusion-isotonic (a parent's
-// centre says nothing about its children's centres).
+// the voxel centre) of explicit cells; level 0 and bisected cells are coarse_block<kMid> and
+// children_block<kMid>.
 // ---------------------------------------------------------------------------------------
-struct MidSmem {
-    static constexpr size_t hits = 0;
-    static constexpr size_t hist = kHitCap * 80;
-    static constexpr size_t bar = hist + ((kHistBins * 4 + 15) & ~size_t(15));
-    static constexpr size_t Lc = bar + 16;
-    __host__ __device__ static size_t total(int Bl) { return Lc + 8 * Bl; }
-};
-
-__global__ void __launch_bounds__(256)
-k_vote_coarse_mid(DevGeom g, int ev0, const HitRecD *hd, const int32_t *n_hits,
-                  const uint32_t *active, int32_t *votes, uint32_t *hist, unsigned *status,
-                  unsigned long long *ctr) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int Bd = g.bins[0], Bp = g.bins[1], Bw = g.bins[2], Bz = g.bins[3], Bl = g.bins[4];
-    const int nthr = Bd * Bz;
-    const int e = blockIdx.y, ev = ev0 + e;
-    const int p = blockIdx.x % Bp, w = blockIdx.x / Bp;
-    const int tid = threadIdx.x;
-    unsigned char *hs = smem + MidSmem::hits;
-    uint32_t *hist_s = reinterpret_cast<uint32_t *>(smem + MidSmem::hist);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + MidSmem::bar);
-    double *Lc = reinterpret_cast<double *>(smem + MidSmem::Lc);
-
-    int nh = n_hits[ev];
-    if (nh < 0) nh = 0;
-    for (int i = tid; i < kHistBins; i += nthr) hist_s[i] = 0;
-    for (int l = tid; l < Bl; l += nthr) Lc[l] = pt::centre(edge(g, 4, 0, l));
-    bool ok = stage_to_smem(hs, hd + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr, nullptr, 0u,
-                            bar, status);
-    __syncthreads();
-    if (!ok) nh = 0;
-
-    const int d = tid % Bd, z = tid / Bd;
-    Cell<double> c{edge(g, 0, 0, d), sin_phi0(g, 0, p), cos_phi0(g, 0, p), edge(g, 2, 0, w),
-                   edge(g, 3, 0, z), {0.0, 0.0}};
-    MidCentre m;
-    sincos_phi0_centre(g, 0, p, m.S0, m.C0);
-    m.D = pt::centre(c.D);
-    m.W = pt::centre(c.W);
-    m.Z = pt::centre(c.Z);
-    const bool mir = mirror_cell(c);
-    if (mir) { m.D = -m.D; m.S0 = -m.S0; m.W = -m.W; }
-    const bool wguard = le0(c.W.lo);
-    const unsigned all = Bl >= 32 ? 0xffffffffu : ((1u << Bl) - 1u);
-    const uint32_t *act = active ? active + (long long)ev * 8 : nullptr;
-    uint32_t pl[9];
-#pragma unroll
-    for (int q = 0; q < 9; q++) pl[q] = 0u;
-    auto add_votes = [&](uint32_t mk) {
-#pragma unroll
-        for (int q = 0; q < 9; q++) {
-            const uint32_t cy = pl[q] & mk;
-            pl[q] ^= mk;
-            mk = cy;
-        }
-    };
-    unsigned n_pre = 0, n_tail = 0;
-    for (int h = 0; h < nh; h++) {
-        if (act && !((act[h >> 5] >> (h & 31)) & 1u)) continue;
-        if (wguard) { add_votes(all); continue; }
-        Hit<double> hh = load_hit<double>(hs + h * 80);
-        if (mir) mirror_hit(hh);
-        MidPre pre = mid_prefix(c, m, hh);
-        n_pre++;
-        if (pre.guard) { add_votes(all); continue; }
-        uint32_t v = 0;
-#pragma unroll 1
-        for (int l = 0; l < Bl; l++)
-            if (mid_tail(pre, Lc[l], hh, c.W)) v |= 1u << l;
-        n_tail += Bl;
-        add_votes(v);
-    }
-    const long long ncell = (long long)Bd * Bp * Bw * Bz * Bl;
-    int32_t *vo = votes + (long long)e * ncell;
-    for (int l = 0; l < Bl; l++) {
-        int v = 0;
-#pragma unroll
-        for (int q = 0; q < 9; q++) v |= (int)((pl[q] >> l) & 1u) << q;
-        long long lin = d + (long long)Bd * (p + (long long)Bp * (w + (long long)Bw * (z + (long long)Bz * l)));
-        vo[lin] = v;
-        atomicAdd(&hist_s[v], 1u);
-    }
-    __syncthreads();
-    for (int i = tid; i < kHistBins && hist; i += nthr)
-        if (hist_s[i]) atomicAdd(&hist[(long long)e * kHistBins + i], hist_s[i]);
-    if (ctr) {   // work counters (diagnostics): midpoint prefixes / tails in the FP64 slots
-        unsigned long long v[2] = {n_pre, n_tail};
-#pragma unroll
-        for (int i = 0; i < 2; i++) {
-            unsigned long long x = v[i];
-            if ((int)blockDim.x - (tid & ~31) >= 32) {   // a full warp: reduce, one add per warp
-                for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-                if ((tid & 31) == 0 && x) atomicAdd(&ctr[1 + i], x);
-            } else if (x) {                               // a partial last warp
-                atomicAdd(&ctr[1 + i], x);
-            }
-        }
-    }
-}
-
-// Midpoint form on explicit cells: given keys, or the 32 children of each parent key (in
-// the order of k_vote_cells).  One cell per thread, all hits of its event.
+// One cell per thread, all hits of its event.
 __global__ void __launch_bounds__(256)
 k_vote_cells_mid(DevGeom g, const HitRecD *hd, const int32_t *n_hits, const uint32_t *active, int level,
-                 const uint64_t *keys, const uint64_t *parents, long long n_per_ev, uint64_t *out_keys,
-                 int32_t *out_votes, unsigned *status) {
+                 const uint64_t *keys, long long n_per_ev, int32_t *out_votes, unsigned *status) {
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned char *hs = smem;
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kHitCap * 80);
@@ -741,26 +631,14 @@ k_vote_cells_mid(DevGeom g, const HitRecD *hd, const int32_t *n_hits, const uint
     if (!ok) nh = 0;
     const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_per_ev) return;
-    uint64_t key;
-    if (parents) {
-        uint64_t pk = parents[(long long)ev * (n_per_ev / 32) + j / 32];
-        int idx[5], b = (int)(j % 32);
-        unpack_key(g, pk, idx);
-#pragma unroll
-        for (int a = 0; a < 5; a++) idx[a] = 2 * idx[a] + ((b >> a) & 1);
-        key = pack_key(g, idx);
-    } else {
-        key = keys[(long long)ev * n_per_ev + j];
-    }
     int idx[5];
-    unpack_key(g, key, idx);
+    unpack_key(g, keys[(long long)ev * n_per_ev + j], idx);
     const long long o = (long long)ev * n_per_ev + j;
     bool valid = true;
 #pragma unroll
     for (int a = 0; a < 5; a++) valid = valid && idx[a] < (g.bins[a] << level);
     if (!valid) {   // a key outside the grid of this level: no lookup, vote count -1
         out_votes[o] = -1;
-        if (out_keys) out_keys[o] = key;
         return;
     }
     const IV<double> Le = edge(g, 4, level, idx[4]);
@@ -779,24 +657,6 @@ k_vote_cells_mid(DevGeom g, const HitRecD *hd, const int32_t *n_hits, const uint
         v += mid_vote_pair(c, m, Lm, load_hit<double>(hs + h * 80)) ? 1 : 0;
     }
     out_votes[o] = v;
-    if (out_keys) out_keys[o] = key;
-}
-
-static void launch_coarse_mid(const DevGeom &g, int ev0, int n_ev, const HitRecD *hd, const int32_t *n_hits,
-                              const uint32_t *active, int32_t *votes, uint32_t *hist, unsigned *status,
-                              cudaStream_t s, unsigned long long *ctr) {
-    dim3 grid(g.bins[1] * g.bins[2], n_ev);
-    k_vote_coarse_mid<<<grid, g.bins[0] * g.bins[3], MidSmem::total(g.bins[4]), s>>>(
-        g, ev0, hd, n_hits, active, votes, hist, status, ctr);
-}
-
-static void launch_cells_mid(const DevGeom &g, int n_ev, const HitRecD *hd, const int32_t *n_hits,
-                             const uint32_t *active, int level, const uint64_t *keys,
-                             const uint64_t *parents, long long n_per_ev, uint64_t *out_keys,
-                             int32_t *out_votes, unsigned *status, cudaStream_t s, int block) {
-    dim3 grid((unsigned)((n_per_ev + block - 1) / block), n_ev);
-    k_vote_cells_mid<<<grid, block, kHitCap * 80 + 16, s>>>(g, hd, n_hits, active, level, keys, parents,
-                                                            n_per_ev, out_keys, out_votes, status);
 }
 
 template <int K> static void launch_coarse_cert(const DevGeom &g, int ev0, int n_ev, const HitRecD *hd,
@@ -817,7 +677,7 @@ void launch_vote_coarse(const DevGeom &g, int prec, int ev0, int n_ev, const Hit
                         const uint32_t *active, uint64_t *cand_k, int32_t *cand_v, int K) {
     if (n_ev <= 0) return;
     if (prec == APO_F64_MID) {
-        launch_coarse_mid(g, ev0, n_ev, hd, n_hits, active, votes, hist, status, s, ctr);
+        launch_coarse_cert<kMid>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K);
     } else if (prec == APO_F64_EXACT) {
         const CoarsePlan P = coarse_plan(g, true);
         k_vote_coarse_exact<<<dim3((unsigned)P.n_tiles, n_ev), P.per, ExactSmem::total(g.bins[4]), s>>>(
@@ -1038,11 +898,8 @@ __device__ __forceinline__ void children_block(const DevGeom &g, unsigned char *
         unpack_key(g, parents_e[p0 + pl], x);
 #pragma unroll
         for (int a = 0; a < 5; a++) x[a] *= 2;
-        const float e = parent_error<K>(g, edge_span(g, 0, level, x[0], x[0] + 1),
-                                        hull2(sin_phi0(g, level, x[1]), sin_phi0(g, level, x[1] + 1)),
-                                        hull2(cos_phi0(g, level, x[1]), cos_phi0(g, level, x[1] + 1)),
-                                        edge_span(g, 2, level, x[2], x[2] + 1), edge_span(g, 3, level, x[3], x[3] + 1),
-                                        edge_span(g, 4, level, x[4], x[4] + 1), hs + h * 80);
+        const int x1[5] = {x[0] + 1, x[1] + 1, x[2] + 1, x[3] + 1, x[4] + 1};
+        const float e = parent_span<K>(g, level, x, x1, hs + h * 80);
         err_s[pl * kHitCap + h] = e;
         if (!(e < 0.f)) atomicOr(&mask_s[pl * 8 + (h >> 5)], 1u << (h & 31));
     }
@@ -1056,8 +913,8 @@ __device__ __forceinline__ void children_block(const DevGeom &g, unsigned char *
                            edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
     bool guard;
     const bool mir = omega_sign<K>(c64.W, &guard);
-    const cert::CellX<0> c = cert_cell<0>(c64, mir);
-    const cert::X<0> R = cert::recip(c.W), L1 = cx<0>(edge(g, 4, level, idx[4] + 1));
+    const typename Prog<K>::CellT c = Prog<K>::cell(g, level, idx[1], c64, mir);
+    const float2 L0 = Prog<K>::tanl(c64.L), L1 = Prog<K>::tanl(edge(g, 4, level, idx[4] + 1));
     const int nw = (nh + 31) >> 5;
     int v0 = 0, v1 = 0, wd = -1;
     uint32_t m = 0;
@@ -1072,15 +929,15 @@ __device__ __forceinline__ void children_block(const DevGeom &g, unsigned char *
             const float e = err_s[pl * kHitCap + h];
             uint32_t unk = 3u;
             if (e < 1e30f) {
-                const cert::HitX<0> hx = cert_hit<0>(hs + h * 80, mir);
-                const cert::PreX<0> pre = cert::prefix(c, hx);
-                const int dir = cert_direction(pre, outgoing, e);
+                const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
+                const typename Prog<K>::Pre pre = Prog<K>::prefix(c, hx);
+                const int dir = Prog<K>::direction(pre, outgoing, e);
                 if (dir == cert::kNo) continue;
                 if (dir == cert::kYes) {
                     unk = 0;
 #pragma unroll 1
                     for (int b = 0; b < 2; b++) {
-                        const int v = cert_tail(pre, b ? L1 : c.L, hx, R, c.W, e);
+                        const int v = Prog<K>::vote(pre, b ? L1 : L0, c, hx, e);
                         if (v == cert::kYes) { if (b) v1++; else v0++; }
                         unk |= (uint32_t)(v == cert::kUnknown) << b;
                     }
@@ -1189,7 +1046,8 @@ void launch_vote_keys(const DevGeom &g, int prec, int n_ev, const HitRecD *hd, c
     if (n_ev <= 0 || n_per_ev <= 0) return;
     dim3 grid((unsigned)((n_per_ev + kCellsThreads - 1) / kCellsThreads), n_ev);
     if (prec == APO_F64_MID) {
-        launch_cells_mid(g, n_ev, hd, n_hits, active, level, keys, nullptr, n_per_ev, nullptr, votes, nullptr, s, 256);
+        k_vote_cells_mid<<<dim3((unsigned)((n_per_ev + 255) / 256), n_ev), 256, kHitCap * 80 + 16, s>>>(
+            g, hd, n_hits, active, level, keys, n_per_ev, votes, nullptr);
     } else if (prec == APO_F64_EXACT) {
         k_vote_cells_exact<<<dim3((unsigned)((n_per_ev + 255) / 256), n_ev), 256, kHitCap * 80 + 16, s>>>(
             g, hd, n_hits, active, level, keys, n_per_ev, votes, nullptr);
@@ -1218,10 +1076,10 @@ void launch_vote_children(const DevGeom &g, int prec, int n_ev, const HitRecD *h
                           int32_t *child_votes, cudaStream_t s, const uint32_t *active, int block,
                           const int32_t *n_valid) {
     if (n_ev <= 0 || n_par <= 0) return;
-    if (block != 128) block = 256;   // of the midpoint and exact-phase kernels
-    if (prec == APO_F64_MID) {   // children in the order of k_vote_children: 32 per parent
-        launch_cells_mid(g, n_ev, hd, n_hits, active, child_level, nullptr, parents, (long long)n_par * 32,
-                         child_keys, child_votes, nullptr, s, block);
+    if (block != 128) block = 256;   // of the exact-phase kernel
+    if (prec == APO_F64_MID) {
+        launch_children_cert<kMid>(g, n_ev, hd, hf, n_hits, active, child_level, parents, n_par, n_valid, child_keys,
+                                   child_votes, s);
     } else if (prec == APO_F64_EXACT) {
         const size_t sm = kHitCap * 80 + 16;
         dim3 grid((unsigned)(((long long)n_par * 16 + block - 1) / block), n_ev);
@@ -1244,6 +1102,8 @@ void launch_vote_children(const DevGeom &g, int prec, int n_ev, const HitRecD *h
 void init_kernel_attributes() {
     const int lim = 96 * 1024;   // on the current device, every time a geometry is created there
     cudaFuncSetAttribute(k_vote_coarse<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_vote_coarse<kMid>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_vote_children<kMid>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_coarse<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_coarse_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_vote_children<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
