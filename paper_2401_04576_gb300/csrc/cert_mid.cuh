@@ -31,7 +31,7 @@ APO_CERT Pt atan_pt(Pt x) {
     return {4.f * v * h};
 }
 // the interval form's enclosure holds it: its remainder only widens the range
-APO_CERT X<64> atan_pt(X<64> x) { return atanx(x); }
+template <int K> APO_CERT X<K> atan_pt(X<K> x) { return atanx(x); }
 
 // c: the mirrored voxel (its W also serves G below); m: its centre(s)
 template <int K, typename N>

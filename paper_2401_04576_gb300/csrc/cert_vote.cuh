@@ -50,67 +50,104 @@ __device__ __forceinline__ IV<double> edge_span(const DevGeom &g, int a, int lev
     return hull2(edge(g, a, level, i0), edge(g, a, level, i1));
 }
 
-// The test of one hit on a parent cell: -1 when no cell inside it gets the hit's vote, else the
-// error bound its cells share (NaN: they cannot be decided by one).  Not inlined: its registers
-// stay out of the callers' loops.
-template <int K>
-__device__ __noinline__ float parent_error(const DevGeom &g, IV<double> D, IV<double> S0, IV<double> C0,
-                                           IV<double> W, IV<double> Z, IV<double> L, const void *rec) {
+// A box of cells (a parent) as the evaluations take it: FP32 ends of the mirrored D, S0, C0, W, Z
+// and of L, and (midpoint form) the range of its phi0 centres' sin / cos (the other centres lie in
+// the box).  Made once per box and kept in shared memory: conversions from FP64 run on its pipe.
+struct CertBox {
+    float2 v[6], sc[2];
+    int mir, guard;
+};
+template <int K> __device__ __forceinline__ CertBox cert_box(const Cell<double> &c, IV<double> Sc, IV<double> Cc) {
+    CertBox b;
     bool guard;
-    const bool mir = omega_sign<K>(W, &guard);
-    if (guard) return NAN;
-    const cert::Eval<K> x = cert::eval(cert_cell<K>(Cell<double>{D, S0, C0, W, Z, L}, mir), cert_hit<K>(rec, mir));
-    const float e = cert::bound(x);
-    return cert::verdict(x, g.k.outgoing != 0, e) == cert::kNo ? -1.f : e;
+    const bool mir = omega_sign<K>(c.W, &guard);
+    auto f = [](cert::X<0> x) { return make_float2(x.lo, x.hi); };
+    b.v[0] = f(cxm<0>(c.D, mir));
+    b.v[1] = f(cxm<0>(c.S0, mir));
+    b.v[2] = f(cx<0>(c.C0));
+    b.v[3] = f(cxm<0>(c.W, mir));
+    b.v[4] = f(cx<0>(c.Z));
+    b.v[5] = f(cx<0>(c.L));
+    b.sc[0] = f(cxm<0>(Sc, mir));
+    b.sc[1] = f(cx<0>(Cc));
+    b.mir = mir;
+    b.guard = guard;
+    return b;
 }
-
-// The midpoint form's: (Sc, Cc) the sin / cos of the phi0 centres inside (their range); the other
-// centres lie in their cells.
+// The box of cells [i0, i1] per axis at `level` (ends included).
 template <int K>
-__device__ __noinline__ float parent_error_mid(IV<double> D, IV<double> S0, IV<double> C0, IV<double> W, IV<double> Z,
-                                               IV<double> L, IV<double> Sc, IV<double> Cc, const void *rec) {
-    using N = cert::X<64>;
-    bool guard;
-    const bool mir = omega_sign<64>(W, &guard);
-    if (guard) return NAN;
-    const cert::CellX<64> c = cert_cell<64>(Cell<double>{D, S0, C0, W, Z, L}, mir);
-    const cert::HitX<64> hx = cert_hit<64>(rec, mir);
-    const cert::MidHit<N> h{cert::point(hx.x0), cert::point(hx.y0), cert::point(hx.sph), cert::point(hx.cph),
-                            cert::point(hx.t), cert::point(hx.spt), cert::point(hx.cpt), cert::point(hx.t2), hx.d};
-    const cert::MidCell<N> m{c.D, cxm<64>(Sc, mir), cx<64>(Cc), c.W, c.Z, cert::recip(c.W)};
-    N Gp, Gm;
-    cert::mid_tail<64, N>(cert::mid_prefix<64, N>(c, m, h), c.L, m, h, c.W, Gp, Gm);
-    // 1 %: the FP64 program's own distance from the real values
-    const float e = (Gp.e < 1e30f && Gm.e < 1e30f) ? 1.01f * fmaxf(Gp.e, Gm.e) : NAN;
-    return cert::decide(Gp, Gm, e) == cert::kNo ? -1.f : e;
-}
-
-// The parent of cells [i0, i1] per axis at `level` (ends included).
-template <int K>
-__device__ __forceinline__ float parent_span(const DevGeom &g, int level, const int (&i0)[5], const int (&i1)[5],
-                                             const void *rec) {
-    const IV<double> D = edge_span(g, 0, level, i0[0], i1[0]), W = edge_span(g, 2, level, i0[2], i1[2]),
-                     Z = edge_span(g, 3, level, i0[3], i1[3]), L = edge_span(g, 4, level, i0[4], i1[4]),
-                     S0 = hull2(sin_phi0(g, level, i0[1]), sin_phi0(g, level, i1[1])),
-                     C0 = hull2(cos_phi0(g, level, i0[1]), cos_phi0(g, level, i1[1]));
+__device__ __forceinline__ CertBox cert_span(const DevGeom &g, int level, const int (&i0)[5], const int (&i1)[5]) {
+    double s0 = 0.0, c0 = 0.0, s1 = 0.0, c1 = 0.0;
     if constexpr (K == kMid) {
-        double s0, c0, s1, c1;
         sincos_phi0_centre(g, level, i0[1], s0, c0);
         sincos_phi0_centre(g, level, i1[1], s1, c1);
-        return parent_error_mid<K>(D, S0, C0, W, Z, L, IV<double>{mn(s0, s1), mx(s0, s1)}, IV<double>{mn(c0, c1), mx(c0, c1)},
-                                rec);
+    }
+    return cert_box<K>(Cell<double>{edge_span(g, 0, level, i0[0], i1[0]),
+                                    hull2(sin_phi0(g, level, i0[1]), sin_phi0(g, level, i1[1])),
+                                    hull2(cos_phi0(g, level, i0[1]), cos_phi0(g, level, i1[1])),
+                                    edge_span(g, 2, level, i0[2], i1[2]), edge_span(g, 3, level, i0[3], i1[3]),
+                                    edge_span(g, 4, level, i0[4], i1[4])},
+                       IV<double>{mn(s0, s1), mx(s0, s1)}, IV<double>{mn(c0, c1), mx(c0, c1)});
+}
+template <int Q> __device__ __forceinline__ cert::X<Q> xf(float2 a) {   // ends rounded from FP64
+    cert::X<Q> r;
+    r.lo = a.x;
+    r.hi = a.y;
+    r.e = Q ? cert::rnd<Q>(cert::mag2(a.x, a.y)) + cert::kTiny : 0.f;
+    return r;
+}
+
+// The test of one hit on a box: -1 when no cell inside it gets the hit's vote, else the error bound
+// its cells share (NaN: they cannot be decided by one).  Not inlined: its registers stay out of the
+// callers' loops.
+template <int K> __device__ __noinline__ float box_error(const CertBox *b, const void *rec, bool outgoing) {
+    constexpr int Q = K == kMid ? 64 : K;
+    if (b->guard) return NAN;
+    const cert::CellX<Q> c{xf<Q>(b->v[0]), xf<Q>(b->v[1]), xf<Q>(b->v[2]), xf<Q>(b->v[3]), xf<Q>(b->v[4]), xf<Q>(b->v[5])};
+    const cert::HitX<Q> hx = cert_hit<Q>(rec, b->mir);
+    if constexpr (K == kMid) {
+        using N = cert::X<64>;
+        const cert::MidHit<N> h{cert::point(hx.x0), cert::point(hx.y0), cert::point(hx.sph), cert::point(hx.cph),
+                                cert::point(hx.t), cert::point(hx.spt), cert::point(hx.cpt), cert::point(hx.t2), hx.d};
+        const cert::MidCell<N> m{c.D, xf<64>(b->sc[0]), xf<64>(b->sc[1]), c.W, c.Z, cert::recip(c.W)};
+        N Gp, Gm;
+        cert::mid_tail<64, N>(cert::mid_prefix<64, N>(c, m, h), c.L, m, h, c.W, Gp, Gm);
+        // 1 %: the FP64 program's own distance from the real values
+        const float e = (Gp.e < 1e30f && Gm.e < 1e30f) ? 1.01f * fmaxf(Gp.e, Gm.e) : NAN;
+        return cert::decide(Gp, Gm, e) == cert::kNo ? -1.f : e;
     } else {
-        return parent_error<K>(g, D, S0, C0, W, Z, L, rec);
+        const cert::Eval<K> x = cert::eval(c, hx);
+        const float e = cert::bound(x);
+        return cert::verdict(x, outgoing, e) == cert::kNo ? -1.f : e;
+    }
+}
+// Whether no cell inside the box with its tan(lambda) ends replaced by L gets the hit's vote, for an
+// error bound e of the box (the bound holds for every box inside it, so bare end points do).
+template <int K>
+__device__ __noinline__ bool box_refuses(const CertBox *b, float2 L, const void *rec, float e, bool outgoing) {
+    if (b->guard) return false;
+    const cert::CellX<0> c{xf<0>(b->v[0]), xf<0>(b->v[1]), xf<0>(b->v[2]), xf<0>(b->v[3]), xf<0>(b->v[4]), xf<0>(L)};
+    const cert::HitX<0> hx = cert_hit<0>(rec, b->mir);
+    if constexpr (K == kMid) {
+        using N = cert::X<0>;
+        const cert::MidHit<N> h{cert::point(hx.x0), cert::point(hx.y0), cert::point(hx.sph), cert::point(hx.cph),
+                                cert::point(hx.t), cert::point(hx.spt), cert::point(hx.cpt), cert::point(hx.t2), hx.d};
+        const cert::MidCell<N> m{c.D, xf<0>(b->sc[0]), xf<0>(b->sc[1]), c.W, c.Z, cert::recip(c.W)};
+        N Gp, Gm;
+        cert::mid_tail<0, N>(cert::mid_prefix<0, N>(c, m, h), c.L, m, h, c.W, Gp, Gm);
+        return cert::decide(Gp, Gm, e) == cert::kNo;
+    } else {
+        return cert::verdict(cert::eval(c, hx), outgoing, e) == cert::kNo;
     }
 }
 
-// Hits no parent could decide for a cell, one by one: the cell's own evaluation with errors,
-// then the reference program.  mask: tan(lambda) cells l0 + bit in question; returns those that
-// vote.  Not inlined: about one pair in 10^4 comes here,
-// and its registers stay out of the callers' loops.
+// Hits no parent could decide for a cell, one by one: with `own` (the parent had no bound) the
+// cell's own evaluation with errors, then the reference program.  mask: tan(lambda) cells l0 + bit
+// in question; returns those that vote.  Not inlined: about one pair in 10^4 comes here, and its
+// registers stay out of the callers' loops.
 template <int K>
 __device__ __noinline__ uint32_t resolve(const DevGeom &g, int level, int d, int p, int w, int z, int l0,
-                                         uint32_t mask, const HitRecD *hd, const HitRecF *hf) {
+                                         uint32_t mask, bool own, const HitRecD *hd, const HitRecF *hf) {
     Cell<double> c{edge(g, 0, level, d), sin_phi0(g, level, p), cos_phi0(g, level, p), edge(g, 2, level, w),
                    edge(g, 3, level, z), {0.0, 0.0}};
     uint32_t yes = 0;
@@ -135,9 +172,11 @@ __device__ __noinline__ uint32_t resolve(const DevGeom &g, int level, int d, int
             const int b = __ffs(mask) - 1;
             mask &= mask - 1;
             c.L = edge(g, 4, level, l0 + b);
-            const cert::Eval<K> ev = cert::eval(cert_cell<K>(c, mir), h);
-            int v = cert::verdict(ev, g.k.outgoing != 0, cert::bound(ev));
-            if (guard) v = cert::kUnknown;
+            int v = cert::kUnknown;
+            if (own && !guard) {
+                const cert::Eval<K> ev = cert::eval(cert_cell<K>(c, mir), h);
+                v = cert::verdict(ev, g.k.outgoing != 0, cert::bound(ev));
+            }
             if (v == cert::kUnknown) {
                 const Cell<T> ct{to_prec<T>(c.D), to_prec<T>(c.S0), to_prec<T>(c.C0),
                                  to_prec<T>(c.W), to_prec<T>(c.Z), to_prec<T>(c.L)};
@@ -174,8 +213,9 @@ __device__ __forceinline__ bool vote_single(const DevGeom &g, const Cell<double>
 }
 
 // The FP64 vote of a staged hit for one cell with its drift widened to [max(rd(d - width), 0),
-// ru(d + width)] (the hit finding), by the pair's own bound.
-__device__ __forceinline__ bool vote_widened(const DevGeom &g, const Cell<double> &c, const HitRecD *hd,
+// ru(d + width)] (the hit finding), by the pair's own bound.  Not inlined (see resolve).
+template <int K = 64>
+__device__ __noinline__ bool vote_widened(const DevGeom &g, const Cell<double> &c, const HitRecD *hd,
                                              double width) {
     Hit<double> h = load_hit<double>(hd);
     const double d = h.d.lo, dlo = __dsub_rd(d, width);
@@ -196,38 +236,51 @@ __device__ __forceinline__ bool vote_widened(const DevGeom &g, const Cell<double
     return vote_reference<double>(g, c, h);
 }
 
-// A block's undecided (thread, hit) pairs, resolved together so that whole warps do that work.
-// Threads push at most kCertStep pairs between block barriers, where the queue is drained if it
-// could overflow in the next step (and at the end); so no push is ever refused.
-constexpr int kCertStep = 4, kCertDrain = 256;
-template <int NT> struct CertQueue {
-    static constexpr int cap = kCertDrain + kCertStep * NT;
-    uint32_t n, pad[3];
-    uint32_t id[cap];     // thread | hit << 16
-    uint32_t mask[cap];   // tan(lambda) bits in question, then those that vote
-    __device__ __forceinline__ void push(int tid, int h, uint32_t m) {
-        const uint32_t s = atomicAdd(&n, 1u);
-        if (s >= (uint32_t)cap) return;   // cannot happen; never write past the arrays
-        id[s] = (uint32_t)tid | ((uint32_t)h << 16);
-        mask[s] = m;
+// A warp's undecided (lane, hit) pairs, resolved by its lanes together once 32 are waiting and at
+// the end.  Every lane calls push in step, so no atomics and no block barrier are needed (a block's
+// queue behind barriers cost a quarter of the voting kernels' time).
+struct WarpQueue {
+    uint32_t id[64];     // lane (or pair, below 256) | hit << 8 | own << 16
+    uint32_t mask[64];   // tan(lambda) bits in question, then those that vote
+    // n: entries held (below 32 on entry), the same in every lane; returns their new number
+    __device__ __forceinline__ int push(int n, int lane, int h, bool own, uint32_t m) {
+        return push(n, lane, lane, h, own, m);
+    }
+    __device__ __forceinline__ int push(int n, int pair, int lane, int h, bool own, uint32_t m) {
+        const unsigned b = __ballot_sync(0xffffffffu, m != 0u);
+        if (m) {
+            const int s = n + __popc(b & ((1u << lane) - 1u));
+            id[s] = (uint32_t)pair | ((uint32_t)h << 8) | (own ? 1u << 16 : 0u);
+            mask[s] = m;
+        }
+        return n + __popc(b);
+    }
+    // each(pair, hit, own, mask) for all n entries, one per lane
+    template <typename Each> __device__ __forceinline__ void drain(int n, int lane, Each each) {
+        __syncwarp();
+        for (int i = lane; i < n; i += 32)
+            each((int)(id[i] & 255u), (int)((id[i] >> 8) & 255u), (id[i] >> 16) != 0u, mask[i]);
+        __syncwarp();
+    }
+    // resolves all n entries (solve(lane, hit, own, mask) -> voting bits) and gives every lane its
+    // own (take(bits))
+    template <typename Solve, typename Take>
+    __device__ __forceinline__ void drain(int n, int lane, Solve solve, Take take) {
+        __syncwarp();
+        for (int i = lane; i < n; i += 32)
+            mask[i] = solve((int)(id[i] & 255u), (int)((id[i] >> 8) & 255u), (id[i] >> 16) != 0u, mask[i]);
+        __syncwarp();
+        for (int i = 0; i < n; i++)
+            if ((int)(id[i] & 255u) == lane) take(mask[i]);
+        __syncwarp();
     }
 };
 
-// The votes of one tan(lambda) interval for a prefix and error bound e: the signs of L and of
-// the wire's t are made known where they can be, by the reflection z -> -z of cell and wire,
-// which changes no end point ((L, t) -> (-L, -t)).
+// The vote of one tan(lambda) interval for a prefix and error bound e.
 __device__ __forceinline__ int cert_tail(const cert::PreX<0> &p, cert::X<0> L, const cert::HitX<0> &h,
                                          cert::X<0> R, cert::X<0> W, float e) {
     cert::X<0> Gp, Gm;
-    const bool lpos = L.lo >= 0.f;
-    if (lpos || L.hi <= 0.f) {
-        cert::HitX<0> hr = h;
-        if (!lpos) { L = cert::neg(L); hr.t = cert::neg(h.t); }
-        if (hr.t.v >= 0.f) cert::tail<1, 1>(p, L, hr, R, W, Gp, Gm);
-        else cert::tail<1, -1>(p, L, hr, R, W, Gp, Gm);
-    } else {
-        cert::tail<0, 0>(p, L, h, R, W, Gp, Gm);
-    }
+    cert::tail(p, L, h, R, W, Gp, Gm);
     return cert::decide(Gp, Gm, e);
 }
 

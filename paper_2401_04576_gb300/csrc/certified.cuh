@@ -42,9 +42,16 @@ namespace cert {
 // Documented maximum relative error 2^-23 each (PTX ISA, rcp / sqrt .approx.f32)
 APO_CERT float rcp_a(float x) { float r; asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
 APO_CERT float sqrt_a(float x) { float r; asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
+// (rsqrt: 2^-22.9)
+APO_CERT float rsqrt_a(float x) { float r; asm("rsqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
+APO_CERT float min3(float a, float b, float c) { float r; asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r; }
+APO_CERT float max3(float a, float b, float c) { float r; asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r; }
 #else
 APO_CERT float rcp_a(float x) { return 1.0f / x; }
 APO_CERT float sqrt_a(float x) { return std::sqrt(x); }
+APO_CERT float rsqrt_a(float x) { return 1.0f / std::sqrt(x); }
+APO_CERT float min3(float a, float b, float c) { return fminf(fminf(a, b), c); }
+APO_CERT float max3(float a, float b, float c) { return fmaxf(fmaxf(a, b), c); }
 #endif
 
 // Rounding of one operation, both sides together, relative to the result's magnitude: FP32 to
@@ -113,18 +120,17 @@ template <int K, typename A, typename B> APO_CERT float perr(A a, B b) {   // a 
 }
 template <int K> APO_CERT X<K> mul(X<K> a, X<K> b) {
     const float p = a.lo * b.lo, q = a.lo * b.hi, r = a.hi * b.lo, s = a.hi * b.hi;
-    return fin<K>(fminf(fminf(p, q), fminf(r, s)), fmaxf(fmaxf(p, q), fmaxf(r, s)), perr<K>(a, b));
+    return fin<K>(min3(p, q, fminf(r, s)), max3(p, q, fmaxf(r, s)), perr<K>(a, b));
 }
 // b >= 0 in the reference (its structure), both >= 0, b <= 0
 template <int K> APO_CERT X<K> mul_nn(X<K> a, X<K> b) {
     return fin<K>(fminf(a.lo * b.lo, a.lo * b.hi), fmaxf(a.hi * b.lo, a.hi * b.hi), perr<K>(a, b));
 }
 template <int K> APO_CERT X<K> mul_pp(X<K> a, X<K> b) { return fin<K>(a.lo * b.lo, a.hi * b.hi, perr<K>(a, b)); }
-// times a number: S = 1 / -1 when its sign is known (>= 0 / <= 0)
+// times a number (S = 1: known to be >= 0)
 template <int S, int K> APO_CERT X<K> muls(X<K> a, Sc<K> s) {
     const float p = a.lo * s.v, q = a.hi * s.v;
     if (S > 0) return fin<K>(p, q, perr<K>(a, s));
-    if (S < 0) return fin<K>(q, p, perr<K>(a, s));
     return fin<K>(fminf(p, q), fmaxf(p, q), perr<K>(a, s));
 }
 // (ends of a s) + c for numbers s, c: the sum's rounding and the product's
@@ -133,13 +139,8 @@ template <int K> APO_CERT X<K> axpc(X<K> a, Sc<K> s, Sc<K> c) {
     return fin<K>(fminf(p, q), fmaxf(p, q), K ? perr<K>(a, s) + rnd<K>(M(a) * M(s)) + c.e : 0.f);
 }
 template <int K> APO_CERT X<K> sqr(X<K> a) {
-    const float m = fmaxf(-a.lo, a.hi), n = fmaxf(0.f, fmaxf(a.lo, -a.hi));
+    const float m = fmaxf(-a.lo, a.hi), n = max3(0.f, a.lo, -a.hi);
     return fin<K>(n * n, m * m, K ? 2.f * M(a) * a.e + kTiny : 0.f);
-}
-template <int S, int K> APO_CERT X<K> sqrs(X<K> a) {   // square of known sign S
-    if (S > 0) return mul_pp(a, a);
-    if (S < 0) { const X<K> b = neg(a); return mul_pp(b, b); }
-    return sqr(a);
 }
 template <int K> APO_CERT X<K> clamp1(X<K> a) {
     X<K> r;
@@ -273,24 +274,17 @@ template <int K> APO_CERT PreX<K> prefix(const CellX<K> &c, const HitX<K> &h) {
     return p;
 }
 
-// a b for an interval b of known sign S (>= 0 / <= 0), S = 0: unknown
-template <int S, int K> APO_CERT X<K> mulk(X<K> a, X<K> b) {
-    if (S > 0) return mul_nn(a, b);
-    if (S < 0) return neg(mul_nn(a, neg(b)));
-    return mul(a, b);
-}
-
 // The rest for one tan(lambda) interval L (R = 1 / W): G of both drift signs,
 // G = G0 - a2 + a5 + 2 (z t rcA -+ L Q t rsA) + W (z t)^2 -+ 2 Q with z = z^St - z_ref.
-// LS: 1 when L >= 0 is known; TS: the sign of h.t when known (1 / -1).
-template <int LS, int TS, int K>
+// One copy for every sign of L and t: copies with the signs known take two minima less in six
+// products, but then a voting loop outgrows the instruction cache (level 0 of 1024 events, FP32:
+// 41.3 ms with three copies).
+template <int K>
 APO_CERT void tail(const PreX<K> &p, X<K> L, const HitX<K> &h, X<K> R, X<K> W, X<K> &Gp, X<K> &Gm) {
-    constexpr int LT = LS * TS;
-    const X<K> L2 = LS > 0 ? mul_pp(L, L) : sqr(L);
-    const X<K> Lt = muls<TS>(L, h.t);
-    const X<K> de = add(mulk<LT>(p.A1, Lt), mul_nn(p.A2, L2));
+    const X<K> L2 = sqr(L), Lt = muls<0>(L, h.t);
+    const X<K> de = add(mul(p.A1, Lt), mul_nn(p.A2, L2));
     const X<K> NL = add(p.N, mul_pp(L2, add1(p.N, 1.f)));
-    const X<K> dod = add(mulk<LT>(p.B1, Lt), mul_nn(add(mul_nn(p.pc2, L2), mul_nn(p.sin2, NL)), p.B2));
+    const X<K> dod = add(mul(p.B1, Lt), mul_nn(add(mul_nn(p.pc2, L2), mul_nn(p.sin2, NL)), p.B2));
     const X<K> dP = add(de, dod), dM = sub(de, dod);
     X<K> dh, sd, cd;
     dh.lo = fminf(dP.lo, dM.lo);
@@ -299,19 +293,16 @@ APO_CERT void tail(const PreX<K> &p, X<K> L, const HitX<K> &h, X<K> R, X<K> W, X
     sincosx(dh, sd, cd);
     const X<K> sP = clamp1(add(mul_nn(p.sPA, cd), mul(p.cPA, sd)));    // cos(delta) > 0
     const X<K> cP = clamp1(sub(mul_nn(p.cPA, cd), mul(p.sPA, sd)));
-    const X<K> u2 = add(add(add1(mulk<LT>(sP, scl(Lt, 2.f)), 1.f), muls<1>(L2, h.t2)), muls<1>(sqr(cP), h.t2));
+    const X<K> u2 = add(add(add1(mul(sP, scl(Lt, 2.f)), 1.f), muls<1>(L2, h.t2)), muls<1>(sqr(cP), h.t2));
     const X<K> Q = mul_pp(h.d, recip(sqrtx(u2)));
     const X<K> cz = mul_nn(cP, muls<1>(Q, p.tt));                      // t (cos Phi) t q
-    X<K> LQt;
-    if (LT != 0) LQt = LT > 0 ? mul_pp(Lt, Q) : neg(mul_pp(neg(Lt), Q));
-    else LQt = mul_nn(Lt, Q);
-    const X<K> LQr = mulk<LT>(p.rsA, LQt);
-    const X<K> a2 = mul_pp(W, mul_pp(Q, Q)), a5 = mul_pp(W, sqrs<LT>(LQt));
+    const X<K> LQt = mul_nn(Lt, Q), LQr = mul(p.rsA, LQt);
+    const X<K> a2 = mul_pp(W, mul_pp(Q, Q)), a5 = mul_pp(W, sqr(LQt));
     const X<K> base = add(sub(p.G0, a2), a5);
     const X<K> Q2 = scl(Q, 2.f);
 #pragma unroll
     for (int sg = 0; sg < 2; sg++) {
-        const X<K> zL = mulk<LT>(mul_nn(add(p.psi, sg ? dM : dP), R), Lt);
+        const X<K> zL = mul(mul_nn(add(p.psi, sg ? dM : dP), R), Lt);
         const X<K> zt = sg ? add(zL, cz) : sub(zL, cz);
         const X<K> zr = mul(zt, p.rcA);
         const X<K> Y = scl(sg ? add(zr, LQr) : sub(zr, LQr), 2.f);
@@ -337,7 +328,7 @@ template <int K> struct Eval { X<K> Gp, Gm, wt; };
 template <int K> APO_CERT Eval<K> eval(const CellX<K> &c, const HitX<K> &h) {
     Eval<K> r;
     const PreX<K> p = prefix(c, h);
-    tail<0, 0>(p, c.L, h, recip(c.W), c.W, r.Gp, r.Gm);
+    tail(p, c.L, h, recip(c.W), c.W, r.Gp, r.Gm);
     r.wt = p.wt;
     return r;
 }

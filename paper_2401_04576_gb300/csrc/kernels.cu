@@ -341,72 +341,118 @@ __device__ __forceinline__ void add_counts(unsigned long long *ctr, const unsign
 }
 
 // FP64 (K = 64), outward FP32 (K = 32) and midpoint-form voting, decided by certified FP32 values.
-// Phase 1: the parent test, one (tile, hit) per thread, gives the mask of hits that can vote and
-// the error bound that every cell of the tile shares.  Phase 2: the bare end points per
-// (cell, hit), bit-sliced counters; the undecided pairs are queued and resolved in whole warps.
+// Phase 1: the parent tests of the block's tiles, one (tile, hit) per thread, give the mask of hits
+// that can vote and the error bound that every cell of a tile shares; phase 2 the tan(lambda) bins
+// of a kept hit that the tile's cells can vote in, and for a hit without a bound (wide cells) one
+// from its bins' boxes; phase 3, tile by tile and without barriers,
+// the bare values per (cell, hit, bin), bit-sliced counters; undecided pairs go to the warp's queue.
 // What bounds it: FP32 issue.  The FP64 pipe (about 1.7 directed operations per clock and SM)
 // evaluated every pair before; now about one pair in 10^4 reaches it.
 //
-// A block is 128 threads.  Grids with few (d0, z0) cells put `tiles` of them in one block (full
-// votes only: the K best are kept per tile), so that its warps stay full.
-constexpr int kCoarseThreads = 128, kCoarseMaxTiles = 16;
+// A block is 128 threads and takes up to four tiles, so that phases 1 and 2, whose chains a single
+// tile cannot hide, keep all its warps busy (fewer where the launch would have too few blocks).
+// Grids with few (d0, z0) cells put `group` tiles side by side in the block (full votes only: the K
+// best are kept per tile), so that its warps stay full.
+constexpr int kCoarseThreads = 128, kCoarseMaxGroup = 8, kCoarseRounds = 4;
+constexpr int kCoarseBinCells = 64;   // fewest cells of a tile whose every kept hit is tested by bin
 struct CoarsePlan {
-    int parts, per, tiles;   // parts of a (phi0, omega) tile, cells of a part, tiles per block
+    int parts, per;          // parts of a (phi0, omega) tile's cells, cells of a part (= one tile)
+    int group, tiles;        // tiles side by side, tiles per block (group or one after another)
     long long n_tiles;       // of one event
 };
-__host__ __device__ inline CoarsePlan coarse_plan(const DevGeom &g, bool lists) {
+// n_ev: events of the launch (0: one block takes a whole event)
+__host__ __device__ inline CoarsePlan coarse_plan(const DevGeom &g, bool lists, long long n_ev) {
     CoarsePlan P;
     const int n = g.bins[0] * g.bins[3];
     P.parts = (n + kCoarseThreads - 1) / kCoarseThreads;
     P.per = (n + P.parts - 1) / P.parts;
-    const int fit = kCoarseThreads / P.per;
-    P.tiles = lists ? 1 : (fit < 1 ? 1 : (fit > kCoarseMaxTiles ? kCoarseMaxTiles : fit));
     P.n_tiles = (long long)P.parts * g.bins[1] * g.bins[2];
+    const int fit = kCoarseThreads / P.per;
+    P.group = lists || fit < 2 ? 1 : (fit > kCoarseMaxGroup ? kCoarseMaxGroup : fit);
+    P.tiles = P.group;
+    if (P.group == 1) {   // at least two waves of four blocks on 152 SMs
+        const long long r = n_ev == 0 ? kCoarseRounds : P.n_tiles * n_ev / (2 * 4 * 152);
+        P.tiles = r < 1 ? 1 : (r > kCoarseRounds ? kCoarseRounds : (int)r);
+    }
     return P;
 }
 
 struct CoarseSmem {   // of a cert coarse block; every offset a multiple of 16
     static constexpr size_t hits = 0;
     static constexpr size_t queue = kHitCap * 80;
-    static constexpr size_t hist = queue + ((sizeof(CertQueue<kCoarseThreads>) + 15) & ~size_t(15));
+    static constexpr size_t hist = queue + sizeof(WarpQueue) * (kCoarseThreads / 32);
     static constexpr size_t bar = hist + ((kHistBins * 4 + 15) & ~size_t(15));
     static constexpr size_t L = bar + 16;
     __host__ __device__ static size_t mask(int Bl) { return L + ((8 * (size_t)Bl + 15) & ~size_t(15)); }
-    __host__ __device__ static size_t err(int Bl, int tiles) { return mask(Bl) + 32 * (size_t)tiles; }
-    __host__ __device__ static size_t total(int Bl, int tiles) { return err(Bl, tiles) + sizeof(float) * kHitCap * (size_t)tiles; }
+    __host__ __device__ static size_t box(int Bl, const CoarsePlan &P) { return mask(Bl) + 32 * (size_t)P.tiles; }
+    __host__ __device__ static size_t err(int Bl, const CoarsePlan &P) {
+        return box(Bl, P) + ((sizeof(CertBox) * (size_t)P.tiles + 15) & ~size_t(15));
+    }
+    // per (tile, hit): the tan(lambda) bins in question, those without a bound; the (tile, hit)s of phase 2
+    __host__ __device__ static size_t bins(int Bl, const CoarsePlan &P) {
+        return err(Bl, P) + sizeof(float) * kHitCap * (size_t)P.tiles;
+    }
+    __host__ __device__ static size_t own(int Bl, const CoarsePlan &P) {
+        return bins(Bl, P) + sizeof(uint32_t) * kHitCap * (size_t)P.tiles;
+    }
+    __host__ __device__ static size_t list(int Bl, const CoarsePlan &P) {
+        return own(Bl, P) + sizeof(uint32_t) * kHitCap * (size_t)P.tiles;
+    }
+    __host__ __device__ static size_t total(int Bl, const CoarsePlan &P) {
+        return list(Bl, P) + 16 + sizeof(uint16_t) * kHitCap * (size_t)P.tiles;
+    }
 };
 
+// Tiles [tile0, tile0 + P.tiles) of event ev by one block of 128 threads; cand_e / cand_v: the
+// event's candidate lists, Kc per tile (null: full votes to vo).
 template <int K>
 __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan &P, int ev, long long tile0,
                                              const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
                                              const uint32_t *active, int32_t *vo, uint32_t *hist_e,
                                              unsigned *status, unsigned long long *ctr, unsigned char *smem,
                                              uint64_t *cand_k = nullptr, int32_t *cand_v = nullptr, int Kc = 0) {
-    const int Bd = g.bins[0], Bp = g.bins[1], Bz = g.bins[3], Bl = g.bins[4];
-    const int ntile = Bd * Bz, nthr = blockDim.x, tid = threadIdx.x;
+    const int Bd = g.bins[0], Bp = g.bins[1], Bw = g.bins[2], Bz = g.bins[3], Bl = g.bins[4];
+    const int ntile = Bd * Bz, nthr = kCoarseThreads, tid = threadIdx.x, lane = tid & 31;
     unsigned char *hs = smem + CoarseSmem::hits;
-    CertQueue<kCoarseThreads> &q = *reinterpret_cast<CertQueue<kCoarseThreads> *>(smem + CoarseSmem::queue);
+    WarpQueue &q = reinterpret_cast<WarpQueue *>(smem + CoarseSmem::queue)[tid >> 5];
     uint32_t *hist_s = reinterpret_cast<uint32_t *>(smem + CoarseSmem::hist);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + CoarseSmem::bar);
     float2 *Ls = reinterpret_cast<float2 *>(smem + CoarseSmem::L);
     uint32_t *mask_s = reinterpret_cast<uint32_t *>(smem + CoarseSmem::mask(Bl));
-    float *err_s = reinterpret_cast<float *>(smem + CoarseSmem::err(Bl, P.tiles));
-    const bool outgoing = g.k.outgoing != 0;
+    CertBox *box_s = reinterpret_cast<CertBox *>(smem + CoarseSmem::box(Bl, P));
+    float *err_s = reinterpret_cast<float *>(smem + CoarseSmem::err(Bl, P));
+    uint32_t *bins_s = reinterpret_cast<uint32_t *>(smem + CoarseSmem::bins(Bl, P));
+    uint32_t *own_s = reinterpret_cast<uint32_t *>(smem + CoarseSmem::own(Bl, P));
+    uint32_t *n_list = reinterpret_cast<uint32_t *>(smem + CoarseSmem::list(Bl, P));
+    uint16_t *list_s = reinterpret_cast<uint16_t *>(n_list + 4);
+    const unsigned all = Bl >= 32 ? 0xffffffffu : ((1u << Bl) - 1u);
+    const bool outgoing = g.k.outgoing != 0, single = P.group == 1;
+    const HitRecD *hd_e = hd + (long long)ev * kHitCap;
+    const HitRecF *hf_e = hf + (long long)ev * kHitCap;
 
     int nh = n_hits[ev];
     if (nh < 0) nh = 0;
     for (int i = tid; i < kHistBins; i += nthr) hist_s[i] = 0;
     for (int i = tid; i < 8 * P.tiles; i += nthr) mask_s[i] = 0;
     for (int l = tid; l < Bl; l += nthr) Ls[l] = Prog<K>::tanl(edge(g, 4, 0, l));
-    if (tid == 0) q.n = 0;
-    const bool ok = stage_to_smem(hs, hf + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr, nullptr, 0u, bar,
-                                  status);
+    if (tid == 0) *n_list = 0;
+    for (int i = tid; i < P.tiles; i += nthr) {   // the tiles' parents
+        const long long t = tile0 + i;
+        if (t >= P.n_tiles) break;
+        const int part = (int)(t % P.parts), pw = (int)(t / P.parts), p = pw % Bp, w = pw / Bp;
+        const int c0 = part * P.per, c1 = c0 + P.per < ntile ? c0 + P.per : ntile;
+        const bool row = c0 / Bd == (c1 - 1) / Bd;   // cells of one z0 bin
+        const int i0[5] = {row ? c0 % Bd : 0, p, w, c0 / Bd, 0};
+        const int i1[5] = {row ? (c1 - 1) % Bd : Bd - 1, p, w, (c1 - 1) / Bd, Bl - 1};
+        box_s[i] = cert_span<K>(g, 0, i0, i1);
+    }
+    const bool ok = stage_to_smem(hs, hf_e, (unsigned)nh * 80u, nullptr, nullptr, 0u, bar, status);
     __syncthreads();
     if (tid == 0) mbar_inval(bar);   // the barrier's memory may be set up again by a later call
     if (!ok) nh = 0;
     unsigned cnt[6] = {0, 0, 0, 0, 0, 0};
 
-    // the parent tests: a warp's 32 items are one word of one tile's hit mask
+    // phase 1: a warp's 32 items are one word of one tile's hit mask
     const uint32_t *act = active ? active + (long long)ev * 8 : nullptr;
     const int nw = (nh + 31) >> 5;
     for (int i = tid; i < P.tiles * nw * 32; i += nthr) {
@@ -415,89 +461,135 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan 
         bool keep = h < nh && t < P.n_tiles && (!act || ((act[h >> 5] >> (h & 31)) & 1u));
         float e = NAN;
         if (keep) {
-            const int part = (int)(t % P.parts), pw = (int)(t / P.parts), p = pw % Bp, w = pw / Bp;
-            const int c0 = part * P.per, c1 = c0 + P.per < ntile ? c0 + P.per : ntile;
-            const bool row = c0 / Bd == (c1 - 1) / Bd;   // cells of one z0 bin
-            const int i0[5] = {row ? c0 % Bd : 0, p, w, c0 / Bd, 0};
-            const int i1[5] = {row ? (c1 - 1) % Bd : Bd - 1, p, w, (c1 - 1) / Bd, Bl - 1};
-            e = parent_span<K>(g, 0, i0, i1, hs + h * 80);
+            e = box_error<K>(box_s + tl, hs + h * 80, outgoing);
             keep = !(e < 0.f);
             cnt[3]++;
         }
         const unsigned m = __ballot_sync(0xffffffffu, keep);
-        if ((tid & 31) == 0) mask_s[tl * 8 + (h >> 5)] = m;
-        err_s[tl * kHitCap + h] = e;
+        if (lane == 0) mask_s[tl * 8 + (h >> 5)] = m;
+        if (keep) {
+            const int x = tl * kHitCap + h;
+            const bool ok = e < 1e30f, test = !box_s[tl].guard && (!ok || P.per >= kCoarseBinCells);
+            err_s[x] = ok ? e : 0.f;
+            bins_s[x] = test ? 0u : all;
+            own_s[x] = 0u;
+            if (test) list_s[atomicAdd(n_list, 1u)] = (uint16_t)(x | (ok ? 0 : 1 << 15));
+        }
+    }
+    __syncthreads();
+    // phase 2: one (tile, hit, bin) per thread.  Of 16^5 cells' (tile, hit, bin)s a quarter of those
+    // phase 1 kept go, and with them their tails; tiles of few cells would spend more here than
+    // that, so there only the hits without a bound come: a box of one bin mostly has one.
+    {
+        const int n = (int)*n_list * Bl;
+        for (int i = tid; i < n; i += nthr) {
+            const int y = list_s[i / Bl], x = y & 0x7fff, l = i % Bl, tl = x / kHitCap;
+            const void *rec = hs + (x % kHitCap) * 80;
+            const float2 L = K == kMid ? make_float2(Ls[l].x, Ls[l].x) : Ls[l];   // its centre: a point
+            if (!(y >> 15)) {
+                if (!box_refuses<K>(box_s + tl, L, rec, err_s[x], outgoing)) atomicOr(&bins_s[x], 1u << l);
+            } else {
+                CertBox b = box_s[tl];
+                b.v[5] = L;
+                const float e = box_error<K>(&b, rec, outgoing);
+                if (!(e < 0.f)) atomicOr(e < 1e30f ? &bins_s[x] : &own_s[x], 1u << l);
+                if (e >= 0.f && e < 1e30f) atomicMax(reinterpret_cast<int *>(&err_s[x]), __float_as_int(e));
+            }
+        }
     }
     __syncthreads();
 
-    const int tl = tid / P.per;
-    const long long t = tile0 + tl;
-    const int part = (int)(t % P.parts), pw = (int)(t / P.parts);
-    const int cell = part * P.per + (tid - tl * P.per);
-    const bool has_cell = tl < P.tiles && t < P.n_tiles && cell < ntile;
-    const int p = has_cell ? pw % Bp : 0, w = has_cell ? pw / Bp : 0;
-    const int d = has_cell ? cell % Bd : 0, z = has_cell ? cell / Bd : 0;
-    VotePlanes pl;
-    pl.clear();
-    const unsigned all = Bl >= 32 ? 0xffffffffu : ((1u << Bl) - 1u);
-    const Cell<double> c64{edge(g, 0, 0, d), sin_phi0(g, 0, p), cos_phi0(g, 0, p), edge(g, 2, 0, w),
-                           edge(g, 3, 0, z), {0.0, 0.0}};
-    bool guard;
-    const bool mir = omega_sign<K>(c64.W, &guard);
-    const typename Prog<K>::CellT c = Prog<K>::cell(g, 0, p, c64, mir);
-    int wd = -1;
-    uint32_t m = 0;
-    bool left = has_cell;
-    while (__syncthreads_or(left)) {
-        for (int step = 0; step < kCertStep && left; step++) {
-            while (!m && ++wd < nw) m = mask_s[tl * 8 + wd];
-            if (!m) { left = false; break; }
-            const int h = wd * 32 + __ffs(m) - 1;
-            m &= m - 1;
-            if (guard) { pl.add(all); continue; }
-            const float e = err_s[tl * kHitCap + h];
-            uint32_t yes = 0, unk = all;
-            if (e < 1e30f) {
-                const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
-                const typename Prog<K>::Pre pre = Prog<K>::prefix(c, hx);
-                cnt[4]++;
-                const int dir = Prog<K>::direction(pre, outgoing, e);
-                if (dir == cert::kNo) continue;
-                if (dir == cert::kYes) {
-                    unk = 0;
-                    cnt[5] += Bl;
+    // phase 3
+    for (int r = 0; r < (single ? P.tiles : 1); r++) {
+        const int tl = single ? r : tid / P.per;
+        const long long t = tile0 + tl;
+        const int part = (int)(t % P.parts), pw = (int)(t / P.parts);
+        const int k = single ? tid : tid - tl * P.per, cell = part * P.per + k;
+        const bool has = tl < P.tiles && t < P.n_tiles && k < P.per && cell < ntile;
+        const int p = has ? pw % Bp : 0, w = has ? pw / Bp : 0;
+        const int d = has ? cell % Bd : 0, z = has ? cell / Bd : 0;
+        if (single && t >= P.n_tiles) break;
+        VotePlanes pl;
+        pl.clear();
+        const Cell<double> c64{edge(g, 0, 0, d), sin_phi0(g, 0, p), cos_phi0(g, 0, p), edge(g, 2, 0, w),
+                               edge(g, 3, 0, z), {0.0, 0.0}};
+        bool guard;
+        const bool mir = omega_sign<K>(c64.W, &guard);
+        const typename Prog<K>::CellT c = Prog<K>::cell(g, 0, p, c64, mir);
+        // another lane's pair: its cell from its number
+        auto solve = [&](int ol, int oh, bool own, uint32_t om) -> uint32_t {
+            const int ot = (tid & ~31) + ol, otl = single ? r : ot / P.per;
+            const long long u = tile0 + otl;
+            const int oc = (int)(u % P.parts) * P.per + (single ? ot : ot - otl * P.per), opw = (int)(u / P.parts);
+            return resolve<K>(g, 0, oc % Bd, opw % Bp, opw / Bp, oc / Bd, 0, om, own, hd_e + oh, hf_e + oh);
+        };
+        auto take = [&](uint32_t v) { pl.add(v); };
+        int nq = 0, wd = -1;
+        uint32_t m = 0;
+        for (;;) {
+            while (has && !m && ++wd < nw) m = mask_s[tl * 8 + wd];
+            const bool more = __any_sync(0xffffffffu, m != 0u);
+            uint32_t unk = 0;
+            int h = 0;
+            bool own = false;
+            if (m) {
+                h = wd * 32 + __ffs(m) - 1;
+                m &= m - 1;
+                const float e = err_s[tl * kHitCap + h];
+                uint32_t lm = bins_s[tl * kHitCap + h], yes = 0;
+                own = true;   // a level-0 cell's own bound is several times a tile's
+                if (guard) {
+                    yes = all;
+                } else {
+                    unk = own_s[tl * kHitCap + h];
+                }
+                if (!guard && lm) {
+                    const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
+                    const typename Prog<K>::Pre pre = Prog<K>::prefix(c, hx);
+                    cnt[4]++;
+                    const int dir = Prog<K>::direction(pre, outgoing, e);
+                    if (dir == cert::kNo) unk = 0;
+                    if (dir == cert::kUnknown) unk |= lm;
+                    if (dir == cert::kYes) {
+                        cnt[5] += __popc(lm);
 #pragma unroll 1
-                    for (int l = 0; l < Bl; l++) {
-                        const int v = Prog<K>::vote(pre, Ls[l], c, hx, e);
-                        yes |= (uint32_t)(v == cert::kYes) << l;
-                        unk |= (uint32_t)(v == cert::kUnknown) << l;
+                        while (lm) {
+                            const int l = __ffs(lm) - 1;
+                            lm &= lm - 1;
+                            const int v = Prog<K>::vote(pre, Ls[l], c, hx, e);
+                            yes |= (uint32_t)(v == cert::kYes) << l;
+                            unk |= (uint32_t)(v == cert::kUnknown) << l;
+                        }
                     }
                 }
-            }
-            if (unk) {
+                pl.add(yes);
                 cnt[0] += __popc(unk);
-                q.push(tid, h, unk);
             }
-            pl.add(yes);
+            if (more) nq = q.push(nq, lane, h, own, unk);
+            if (nq >= 32 || (!more && nq)) {
+                q.drain(nq, lane, solve, take);
+                nq = 0;
+            }
+            if (!more) break;
         }
-        __syncthreads();
-        const int nq = (int)q.n;
-        if (nq > kCertDrain || !__syncthreads_or(left)) {
-            for (int i = tid; i < nq; i += nthr) {   // any thread's pair: its cell from its number
-                const int ot = (int)(q.id[i] & 0xffffu), oh = (int)(q.id[i] >> 16), otl = ot / P.per;
-                const long long u = tile0 + otl;
-                const int oc = (int)(u % P.parts) * P.per + (ot - otl * P.per), opw = (int)(u / P.parts);
-                q.mask[i] = resolve<K>(g, 0, oc % Bd, opw % Bp, opw / Bp, oc / Bd, 0, q.mask[i],
-                                       hd + (long long)ev * kHitCap + oh, hf + (long long)ev * kHitCap + oh);
+        if (cand_k) {
+            coarse_output(g, pl, has, d, p, w, z, hist_s, hist_e, nullptr, cand_k + t * Kc, cand_v + t * Kc, Kc);
+            __syncthreads();
+            for (int i = tid; i < kHistBins; i += nthr) hist_s[i] = 0;
+            __syncthreads();
+        } else {
+            for (int l = 0; l < Bl && has; l++) {
+                const int v = pl.get(l);
+                vo[d + (long long)Bd * (p + (long long)Bp * (w + (long long)Bw * (z + (long long)Bz * l)))] = v;
+                atomicAdd(&hist_s[v], 1u);
             }
-            __syncthreads();
-            for (int i = 0; i < nq; i++)
-                if ((int)(q.id[i] & 0xffffu) == tid) pl.add(q.mask[i]);
-            __syncthreads();
-            if (tid == 0) q.n = 0;
         }
     }
-    coarse_output(g, pl, has_cell, d, p, w, z, hist_s, hist_e, vo, cand_k, cand_v, Kc);
+    if (!cand_k) {
+        __syncthreads();
+        for (int i = tid; i < kHistBins && hist_e; i += nthr)
+            if (hist_s[i]) atomicAdd(&hist_e[i], hist_s[i]);
+    }
     add_counts(ctr, cnt);
     __syncthreads();   // shared memory is reused by the caller's next step
 }
@@ -508,14 +600,14 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan 
 #endif
 template <int K>
 __global__ void __launch_bounds__(kCoarseThreads, APO_COARSE_MIN_BLOCKS)
-k_vote_coarse(const __grid_constant__ DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
-              const uint32_t *active, int32_t *votes, uint32_t *hist, unsigned *status,
+k_vote_coarse(const __grid_constant__ DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const HitRecF *hf,
+              const int32_t *n_hits, const uint32_t *active, int32_t *votes, uint32_t *hist, unsigned *status,
               unsigned long long *ctr, uint64_t *cand_k, int32_t *cand_v, int Kc) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int e = blockIdx.y;
     const long long ncell = (long long)g.bins[0] * g.bins[1] * g.bins[2] * g.bins[3] * g.bins[4];
-    // candidates: Kc slots per block (one tile), the blocks of an event in blockIdx.x order
-    const long long co = ((long long)e * gridDim.x + blockIdx.x) * Kc;
+    // candidates: Kc slots per tile, an event's tiles in order
+    const long long co = (long long)e * P.n_tiles * Kc;
     coarse_block<K>(g, P, ev0 + e, (long long)blockIdx.x * P.tiles, hd, hf, n_hits, active,
                     votes ? votes + (long long)e * ncell : nullptr,
                     hist ? hist + (long long)e * kHistBins : nullptr, status, ctr, smem,
@@ -663,13 +755,13 @@ template <int K> static void launch_coarse_cert(const DevGeom &g, int ev0, int n
                                                const HitRecF *hf, const int32_t *n_hits, const uint32_t *active,
                                                int32_t *votes, uint32_t *hist, unsigned *status, cudaStream_t s,
                                                unsigned long long *ctr, uint64_t *cand_k, int32_t *cand_v, int Kc) {
-    const CoarsePlan P = coarse_plan(g, cand_k != nullptr);
+    const CoarsePlan P = coarse_plan(g, cand_k != nullptr, n_ev);
     dim3 grid((unsigned)((P.n_tiles + P.tiles - 1) / P.tiles), n_ev);
-    k_vote_coarse<K><<<grid, kCoarseThreads, CoarseSmem::total(g.bins[4], P.tiles), s>>>(
+    k_vote_coarse<K><<<grid, kCoarseThreads, CoarseSmem::total(g.bins[4], P), s>>>(
         g, P, ev0, hd, hf, n_hits, active, votes, hist, status, ctr, cand_k, cand_v, Kc);
 }
 
-int coarse_lists(const DevGeom &g, int) { return (int)coarse_plan(g, true).n_tiles; }
+int coarse_lists(const DevGeom &g, int) { return (int)coarse_plan(g, true, 1).n_tiles; }
 
 void launch_vote_coarse(const DevGeom &g, int prec, int ev0, int n_ev, const HitRecD *hd,
                         const HitRecF *hf, const int32_t *n_hits, int32_t *votes, uint32_t *hist,
@@ -679,7 +771,7 @@ void launch_vote_coarse(const DevGeom &g, int prec, int ev0, int n_ev, const Hit
     if (prec == APO_F64_MID) {
         launch_coarse_cert<kMid>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K);
     } else if (prec == APO_F64_EXACT) {
-        const CoarsePlan P = coarse_plan(g, true);
+        const CoarsePlan P = coarse_plan(g, true, 1);
         k_vote_coarse_exact<<<dim3((unsigned)P.n_tiles, n_ev), P.per, ExactSmem::total(g.bins[4]), s>>>(
             g, P, ev0, hd, n_hits, active, votes, hist, status, ctr, cand_k, cand_v, K);
     } else if (prec == APO_F32) {
@@ -715,12 +807,16 @@ __device__ __forceinline__ IV<double> warp_hull(IV<double> a) {
 // of one cell, as apo_refine lists them, that cell; for scattered keys it is wide, its bound
 // decides little, and the pairs are evaluated one by one with their own bounds.
 constexpr int kCellsThreads = 128;
+struct WarpScratch {   // one warp's parent, and its queue
+    CertBox box;
+    float err[kHitCap];
+    uint32_t mask[8];
+    WarpQueue q;
+};
 struct CellsSmem {
     static constexpr size_t hits = 0;
-    static constexpr size_t queue = kHitCap * 80;
-    static constexpr size_t err = queue + ((sizeof(CertQueue<kCellsThreads>) + 15) & ~size_t(15));
-    static constexpr size_t mask = err + sizeof(float) * kHitCap * (kCellsThreads / 32);
-    static constexpr size_t bar = mask + 32 * (kCellsThreads / 32);
+    static constexpr size_t warp = kHitCap * 80;
+    static constexpr size_t bar = warp + sizeof(WarpScratch) * (kCellsThreads / 32);
     static constexpr size_t total = bar + 16;
 };
 template <int K>
@@ -730,21 +826,20 @@ k_vote_cells(const __grid_constant__ DevGeom g, const HitRecD *hd, const HitRecF
              unsigned *status) {
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned char *hs = smem + CellsSmem::hits;
-    CertQueue<kCellsThreads> &q = *reinterpret_cast<CertQueue<kCellsThreads> *>(smem + CellsSmem::queue);
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, ev = blockIdx.y;
-    float *err_w = reinterpret_cast<float *>(smem + CellsSmem::err) + wid * kHitCap;
-    uint32_t *mask_w = reinterpret_cast<uint32_t *>(smem + CellsSmem::mask) + wid * 8;
+    const int tid = threadIdx.x, lane = tid & 31, ev = blockIdx.y;
+    WarpScratch &ws = reinterpret_cast<WarpScratch *>(smem + CellsSmem::warp)[tid >> 5];
     const bool outgoing = g.k.outgoing != 0;
     int nh = n_hits[ev];
     if (nh < 0) nh = 0;
-    if (tid == 0) q.n = 0;
-    const bool ok = stage_to_smem(hs, hf + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr, nullptr, 0u,
+    const HitRecD *hd_e = hd + (long long)ev * kHitCap;
+    const HitRecF *hf_e = hf + (long long)ev * kHitCap;
+    const bool ok = stage_to_smem(hs, hf_e, (unsigned)nh * 80u, nullptr, nullptr, 0u,
                                   reinterpret_cast<uint64_t *>(smem + CellsSmem::bar), status);
     __syncthreads();
     if (!ok) nh = 0;
     const int nw = (nh + 31) >> 5;
     const uint32_t *act = active ? active + (long long)ev * 8 : nullptr;
-    const long long j0 = (long long)blockIdx.x * kCellsThreads, j = j0 + tid;
+    const long long j0 = (long long)blockIdx.x * kCellsThreads + (tid & ~31), j = j0 + lane;   // this warp's keys
     const uint64_t *keys_e = keys + (long long)ev * n_per_ev;
     const IV<double> none{1e300, -1e300};
     Cell<double> c64{none, none, none, none, none, none};
@@ -752,61 +847,63 @@ k_vote_cells(const __grid_constant__ DevGeom g, const HitRecD *hd, const HitRecF
     const bool in = j < n_per_ev, has = in && key_cell(g, level, keys_e[j], idx, c64);
     {   // the warp's parent, one hit per lane
         const bool any = __any_sync(0xffffffffu, has);
-        const IV<double> D = warp_hull(c64.D), S0 = warp_hull(c64.S0), C0 = warp_hull(c64.C0), W = warp_hull(c64.W),
-                         Z = warp_hull(c64.Z), L = warp_hull(c64.L);
+        const Cell<double> b{warp_hull(c64.D), warp_hull(c64.S0), warp_hull(c64.C0), warp_hull(c64.W),
+                             warp_hull(c64.Z), warp_hull(c64.L)};
+        if (lane == 0) ws.box = cert_box<K>(b, none, none);
+        __syncwarp();
         for (int h = lane; h < nw * 32; h += 32) {
             bool keep = any && h < nh && (!act || ((act[h >> 5] >> (h & 31)) & 1u));
             if (keep) {
-                const float e = parent_error<K>(g, D, S0, C0, W, Z, L, hs + h * 80);
-                err_w[h] = e;
+                const float e = box_error<K>(&ws.box, hs + h * 80, outgoing);
+                ws.err[h] = e;
                 keep = !(e < 0.f);
             }
             const unsigned m = __ballot_sync(0xffffffffu, keep);
-            if (lane == 0) mask_w[h >> 5] = m;
+            if (lane == 0) ws.mask[h >> 5] = m;
         }
         __syncwarp();
     }
     bool guard;
     const bool mir = omega_sign<K>(c64.W, &guard);
-    const cert::CellX<0> c = cert_cell<0>(c64, mir);
-    const cert::X<0> R = cert::recip(c.W);
-    int v = 0, wd = -1;
+    const typename Prog<K>::CellT c = Prog<K>::cell(g, level, idx[1], c64, mir);
+    const float2 L = Prog<K>::tanl(c64.L);
+    int v = 0, wd = -1, nq = 0;
+    auto solve = [&](int ol, int oh, bool own, uint32_t om) -> uint32_t {
+        int x[5];
+        unpack_key(g, keys_e[j0 + ol], x);
+        return resolve<K>(g, level, x[0], x[1], x[2], x[3], x[4], om, own, hd_e + oh, hf_e + oh);
+    };
+    auto take = [&](uint32_t b) { v += (int)b; };
     uint32_t m = 0;
-    bool left = has;
-    while (__syncthreads_or(left)) {
-        for (int step = 0; step < kCertStep && left; step++) {
-            while (!m && ++wd < nw) m = mask_w[wd];
-            if (!m) { left = false; break; }
-            const int h = wd * 32 + __ffs(m) - 1;
+    for (;;) {
+        while (has && !m && ++wd < nw) m = ws.mask[wd];
+        const bool more = __any_sync(0xffffffffu, m != 0u);
+        int h = 0, r = cert::kNo;
+        bool own = false;
+        if (m) {
+            h = wd * 32 + __ffs(m) - 1;
             m &= m - 1;
-            if (guard) { v++; continue; }
-            const float e = err_w[h];
-            int r = cert::kUnknown;
-            if (e < 1e30f) {
-                const cert::HitX<0> hx = cert_hit<0>(hs + h * 80, mir);
-                const cert::PreX<0> pre = cert::prefix(c, hx);
-                r = cert_direction(pre, outgoing, e);
-                if (r == cert::kYes) r = cert_tail(pre, c.L, hx, R, c.W, e);
+            const float e = ws.err[h];
+            if (guard) {
+                r = cert::kYes;
+            } else if (!(e < 1e30f)) {
+                r = cert::kUnknown;
+                own = true;
+            } else {
+                const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
+                const typename Prog<K>::Pre pre = Prog<K>::prefix(c, hx);
+                r = Prog<K>::direction(pre, outgoing, e);
+                if (r == cert::kYes) r = Prog<K>::vote(pre, L, c, hx, e);
+                own = true;   // the keys need not be one cell's children
             }
             v += r == cert::kYes;
-            if (r == cert::kUnknown) q.push(tid, h, 1u);
         }
-        __syncthreads();
-        const int nq = (int)q.n;
-        if (nq > kCertDrain || !__syncthreads_or(left)) {
-            for (int i = tid; i < nq; i += kCellsThreads) {
-                const int oh = (int)(q.id[i] >> 16);
-                int x[5];
-                unpack_key(g, keys_e[j0 + (q.id[i] & 0xffffu)], x);
-                q.mask[i] = resolve<K>(g, level, x[0], x[1], x[2], x[3], x[4], 1u, hd + (long long)ev * kHitCap + oh,
-                                       hf + (long long)ev * kHitCap + oh);
-            }
-            __syncthreads();
-            for (int i = 0; i < nq; i++)
-                if ((int)(q.id[i] & 0xffffu) == tid) v += q.mask[i] & 1u;
-            __syncthreads();
-            if (tid == 0) q.n = 0;
+        if (more) nq = ws.q.push(nq, lane, h, own, r == cert::kUnknown ? 1u : 0u);
+        if (nq >= 32 || (!more && nq)) {
+            ws.q.drain(nq, lane, solve, take);
+            nq = 0;
         }
+        if (!more) break;
     }
     if (in) out_votes[(long long)ev * n_per_ev + j] = has ? v : -1;   // -1: a key outside the level's grid
 }
@@ -859,113 +956,134 @@ __device__ __forceinline__ void pair_store(const DevGeom &g, const int idx[5], l
     out_votes_e[o + 16] = v1;
 }
 
-// FP64 (K = 64) and outward FP32 (K = 32) votes of the children, decided by certified FP32 end
-// points (see coarse_block): one evaluation with errors per (parent, hit) gives the bound that
-// the parent's 32 children share, and drops the hits that none of them can get.  FP32 issue
-// bounds it; before, every child hit that passed an FP32 test was evaluated on the FP64 pipe.
-// A block takes 8 parents.
-constexpr int kChildThreads = 128, kChildParents = kChildThreads / 16;
+// FP64 (K = 64), outward FP32 (K = 32) and midpoint-form votes of the children, decided by certified
+// FP32 values (see coarse_block).  A warp takes `np` parents, two at a time, and works by itself: no
+// block barrier after the hits are staged.  One evaluation with errors per (parent, hit) gives the
+// bound that the parent's 32 children share, and drops the hits that none of them can get.  Undecided
+// pairs collect over all the warp's parents.  FP32 issue and instruction fetch bound it: the
+// evaluation with errors and the reference program are long straight code, so a warp runs them
+// rarely and on as many lanes as there are (eight parents a warp; with two, 24 multi-track events took 133 ms
+// instead of 118).  Before, every child hit that passed an FP32 test was evaluated on the FP64 pipe.
+constexpr int kChildThreads = 128, kChildParents = 8;   // most parents of a warp
+struct ChildScratch {
+    CertBox box[kChildParents];
+    float err[kChildParents][kHitCap];
+    uint32_t mask[kChildParents][8];
+    WarpQueue q;
+};
 struct ChildSmem {
     static constexpr size_t hits = 0;
-    static constexpr size_t queue = kHitCap * 80;
-    static constexpr size_t err = queue + ((sizeof(CertQueue<kChildThreads>) + 15) & ~size_t(15));
-    static constexpr size_t mask = err + sizeof(float) * kHitCap * kChildParents;
-    static constexpr size_t bar = mask + 32 * kChildParents;
+    static constexpr size_t warp = kHitCap * 80;
+    static constexpr size_t bar = warp + sizeof(ChildScratch) * (kChildThreads / 32);
     static constexpr size_t total = bar + 16;
 };
+// Parents per warp (even): eight where that leaves four waves of 16 warps on each of 152 SMs, else
+// fewer (256 events x 64 parents: two a warp 2.05 ms, six 2.78 ms, FP32 levels of 1024 events).
+__device__ __forceinline__ int child_parents(long long n_par) {
+    const long long r = n_par / (4 * 152 * 16) & ~1LL;
+    return r < 2 ? 2 : (r > kChildParents ? kChildParents : (int)r);
+}
 
-// Pairs [j0, j0 + 128) of one event, those below n_pairs; hits staged at ChildSmem::hits.
+// Children of parents [p0, p0 + np) of one event, those below n_par, by one warp; hits staged at hs.
 template <int K>
-__device__ __forceinline__ void children_block(const DevGeom &g, unsigned char *smem, int nh, const uint32_t *act,
-                                               int level, const uint64_t *parents_e, long long j0, long long n_pairs,
-                                               const HitRecD *hd_e, const HitRecF *hf_e, uint64_t *out_keys_e,
-                                               int32_t *out_votes_e) {
-    unsigned char *hs = smem + ChildSmem::hits;
-    CertQueue<kChildThreads> &q = *reinterpret_cast<CertQueue<kChildThreads> *>(smem + ChildSmem::queue);
-    float *err_s = reinterpret_cast<float *>(smem + ChildSmem::err);
-    uint32_t *mask_s = reinterpret_cast<uint32_t *>(smem + ChildSmem::mask);
-    const int tid = threadIdx.x;
+__device__ __forceinline__ void children_warp(const DevGeom &g, const unsigned char *hs, ChildScratch &ws, int nh,
+                                              const uint32_t *act, int level, const uint64_t *parents_e, long long p0,
+                                              int np, long long n_par, const HitRecD *hd_e, const HitRecF *hf_e,
+                                              uint64_t *out_keys_e, int32_t *out_votes_e) {
+    const int lane = threadIdx.x & 31;
     const bool outgoing = g.k.outgoing != 0;
-    for (int i = tid; i < 8 * kChildParents; i += kChildThreads) mask_s[i] = 0u;
-    if (tid == 0) q.n = 0;
-    __syncthreads();
-    const long long p0 = j0 / 16, n_par = n_pairs / 16 - p0;   // parents from p0 on
-    const int np = n_par < kChildParents ? (int)n_par : kChildParents;
-    for (int i = tid; i < np * nh; i += kChildThreads) {
-        const int pl = i / nh, h = i - pl * nh;
-        if (act && !((act[h >> 5] >> (h & 31)) & 1u)) continue;
+    if (n_par - p0 < np) np = (int)(n_par - p0);
+    for (int i = lane; i < 8 * kChildParents; i += 32) ws.mask[i >> 3][i & 7] = 0u;
+    if (lane < np) {
         int x[5];
-        unpack_key(g, parents_e[p0 + pl], x);
+        unpack_key(g, parents_e[p0 + lane], x);
 #pragma unroll
         for (int a = 0; a < 5; a++) x[a] *= 2;
         const int x1[5] = {x[0] + 1, x[1] + 1, x[2] + 1, x[3] + 1, x[4] + 1};
-        const float e = parent_span<K>(g, level, x, x1, hs + h * 80);
-        err_s[pl * kHitCap + h] = e;
-        if (!(e < 0.f)) atomicOr(&mask_s[pl * 8 + (h >> 5)], 1u << (h & 31));
+        ws.box[lane] = cert_span<K>(g, level, x, x1);
     }
-    __syncthreads();
-    const long long j = j0 + tid;
-    const int pl = tid / 16;
-    const bool has = j < n_pairs;
-    int idx[5] = {0, 0, 0, 0, 0};
-    if (has) pair_index(g, parents_e[j / 16], (int)(j % 16), idx);
-    const Cell<double> c64{edge(g, 0, level, idx[0]), sin_phi0(g, level, idx[1]), cos_phi0(g, level, idx[1]),
-                           edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
-    bool guard;
-    const bool mir = omega_sign<K>(c64.W, &guard);
-    const typename Prog<K>::CellT c = Prog<K>::cell(g, level, idx[1], c64, mir);
-    const float2 L0 = Prog<K>::tanl(c64.L), L1 = Prog<K>::tanl(edge(g, 4, level, idx[4] + 1));
+    __syncwarp();
+    for (int i = lane; i < np * nh; i += 32) {
+        const int pl = i / nh, h = i - pl * nh;
+        if (act && !((act[h >> 5] >> (h & 31)) & 1u)) continue;
+        const float e = box_error<K>(&ws.box[pl], hs + h * 80, outgoing);
+        if (e < 0.f) continue;
+        ws.err[pl][h] = e;
+        atomicOr(&ws.mask[pl][h >> 5], 1u << (h & 31));
+    }
+    // keys, and votes from 0: counted votes and those of undecided pairs are added as they come
+    for (int i = lane; i < np * 16; i += 32) {
+        int x[5];
+        pair_index(g, parents_e[p0 + (i >> 4)], i & 15, x);
+        pair_store(g, x, p0 * 16 + i, 0, 0, out_keys_e, out_votes_e);
+    }
+    __syncwarp();
     const int nw = (nh + 31) >> 5;
-    int v0 = 0, v1 = 0, wd = -1;
-    uint32_t m = 0;
-    bool left = has;
-    while (__syncthreads_or(left)) {
-        for (int step = 0; step < kCertStep && left; step++) {
-            while (!m && ++wd < nw) m = mask_s[pl * 8 + wd];
-            if (!m) { left = false; break; }
-            const int h = wd * 32 + __ffs(m) - 1;
-            m &= m - 1;
-            if (guard) { v0++; v1++; continue; }
-            const float e = err_s[pl * kHitCap + h];
-            uint32_t unk = 3u;
-            if (e < 1e30f) {
-                const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
-                const typename Prog<K>::Pre pre = Prog<K>::prefix(c, hx);
-                const int dir = Prog<K>::direction(pre, outgoing, e);
-                if (dir == cert::kNo) continue;
-                if (dir == cert::kYes) {
-                    unk = 0;
+    int nq = 0;
+    // one undecided pair (16 parent + child bits)
+    auto finish = [&](int pair, int oh, bool own, uint32_t om) {
+        int x[5];
+        pair_index(g, parents_e[p0 + (pair >> 4)], pair & 15, x);
+        const uint32_t y = resolve<K>(g, level, x[0], x[1], x[2], x[3], x[4], om, own, hd_e + oh, hf_e + oh);
+        const long long o = (p0 + (pair >> 4)) * 32 + (pair & 15);
+        if (y & 1u) atomicAdd(&out_votes_e[o], 1);
+        if (y & 2u) atomicAdd(&out_votes_e[o + 16], 1);
+    };
 #pragma unroll 1
-                    for (int b = 0; b < 2; b++) {
-                        const int v = Prog<K>::vote(pre, b ? L1 : L0, c, hx, e);
-                        if (v == cert::kYes) { if (b) v1++; else v0++; }
-                        unk |= (uint32_t)(v == cert::kUnknown) << b;
+    for (int s = 0; s < np; s += 2) {
+        const int pl = s + (lane >> 4);
+        const bool has = pl < np;
+        int idx[5] = {0, 0, 0, 0, 0};
+        if (has) pair_index(g, parents_e[p0 + pl], lane & 15, idx);
+        const Cell<double> c64{edge(g, 0, level, idx[0]), sin_phi0(g, level, idx[1]), cos_phi0(g, level, idx[1]),
+                               edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
+        bool guard;
+        const bool mir = omega_sign<K>(c64.W, &guard);
+        const typename Prog<K>::CellT c = Prog<K>::cell(g, level, idx[1], c64, mir);
+        const float2 L0 = Prog<K>::tanl(c64.L), L1 = Prog<K>::tanl(edge(g, 4, level, idx[4] + 1));
+        int v0 = 0, v1 = 0, wd = -1;
+        uint32_t m = 0;
+        for (;;) {
+            while (has && !m && ++wd < nw) m = ws.mask[pl][wd];
+            const bool more = __any_sync(0xffffffffu, m != 0u);
+            uint32_t unk = 0;
+            int h = 0;
+            bool own = false;
+            if (m) {
+                h = wd * 32 + __ffs(m) - 1;
+                m &= m - 1;
+                const float e = ws.err[pl][h];
+                if (guard) {
+                    v0++;
+                    v1++;
+                } else if (!(e < 1e30f)) {
+                    unk = 3u;
+                    own = true;
+                } else {
+                    const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
+                    const typename Prog<K>::Pre pre = Prog<K>::prefix(c, hx);
+                    const int dir = Prog<K>::direction(pre, outgoing, e);
+                    if (dir == cert::kUnknown) unk = 3u;
+                    if (dir == cert::kYes) {
+#pragma unroll 1
+                        for (int b = 0; b < 2; b++) {
+                            const int v = Prog<K>::vote(pre, b ? L1 : L0, c, hx, e);
+                            if (v == cert::kYes) { if (b) v1++; else v0++; }
+                            unk |= (uint32_t)(v == cert::kUnknown) << b;
+                        }
                     }
                 }
             }
-            if (unk) q.push(tid, h, unk);
-        }
-        __syncthreads();
-        const int nq = (int)q.n;
-        if (nq > kCertDrain || !__syncthreads_or(left)) {
-            for (int i = tid; i < nq; i += kChildThreads) {
-                const long long oj = j0 + (q.id[i] & 0xffffu);
-                const int oh = (int)(q.id[i] >> 16);
-                int x[5];
-                pair_index(g, parents_e[oj / 16], (int)(oj % 16), x);
-                q.mask[i] = resolve<K>(g, level, x[0], x[1], x[2], x[3], x[4], q.mask[i], hd_e + oh, hf_e + oh);
+            if (more) nq = ws.q.push(nq, 16 * s + lane, lane, h, own, unk);
+            if (nq >= 32 || (!more && s + 2 >= np && nq)) {
+                ws.q.drain(nq, lane, finish);
+                nq = 0;
             }
-            __syncthreads();
-            for (int i = 0; i < nq; i++)
-                if ((int)(q.id[i] & 0xffffu) == tid) {
-                    v0 += q.mask[i] & 1u;
-                    v1 += (q.mask[i] >> 1) & 1u;
-                }
-            __syncthreads();
-            if (tid == 0) q.n = 0;
+            if (!more) break;
         }
+        if (v0) atomicAdd(&out_votes_e[(p0 + pl) * 32 + (lane & 15)], v0);
+        if (v1) atomicAdd(&out_votes_e[(p0 + pl) * 32 + (lane & 15) + 16], v1);
     }
-    if (has) pair_store(g, idx, j, v0, v1, out_keys_e, out_votes_e);
 }
 
 #ifndef APO_CHILD_MIN_BLOCKS
@@ -981,18 +1099,21 @@ k_vote_children(const __grid_constant__ DevGeom g, const HitRecD *hd, const HitR
     // n_valid (may be null): parents 0 .. n_valid[ev] - 1 of the event's n_par slots are
     // real; a block past them has nothing to do (the condition is uniform in the block)
     const long long n_here = n_valid ? (long long)n_valid[ev] : (long long)n_par;
-    const long long j0 = (long long)blockIdx.x * kChildThreads;
-    if (j0 >= n_here * 16) return;
+    const int np = child_parents(n_here * gridDim.y);
+    const long long b0 = (long long)blockIdx.x * np * (kChildThreads / 32);   // the block's first parent
+    if (b0 >= n_here) return;
     int nh = n_hits[ev];
     if (nh < 0) nh = 0;
     const bool ok = stage_to_smem(smem + ChildSmem::hits, hf + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr,
                                   nullptr, 0u, reinterpret_cast<uint64_t *>(smem + ChildSmem::bar), status);
     __syncthreads();
     if (!ok) nh = 0;
-    children_block<K>(g, smem, nh, active ? active + (long long)ev * 8 : nullptr, level,
-                      parents + (long long)ev * n_par, j0, n_here * 16, hd + (long long)ev * kHitCap,
-                      hf + (long long)ev * kHitCap, out_keys + (long long)ev * n_par * 32,
-                      out_votes + (long long)ev * n_par * 32);
+    const long long p0 = b0 + (long long)(threadIdx.x >> 5) * np;
+    if (p0 >= n_here) return;
+    children_warp<K>(g, smem + ChildSmem::hits, reinterpret_cast<ChildScratch *>(smem + ChildSmem::warp)[threadIdx.x >> 5],
+                     nh, active ? active + (long long)ev * 8 : nullptr, level, parents + (long long)ev * n_par, p0, np,
+                     n_here, hd + (long long)ev * kHitCap, hf + (long long)ev * kHitCap,
+                     out_keys + (long long)ev * n_par * 32, out_votes + (long long)ev * n_par * 32);
 }
 
 // The exact-phase program on children, FP64.  NT: threads per block, 256 or 128; the 128-thread
@@ -1065,7 +1186,7 @@ static void launch_children_cert(const DevGeom &g, int n_ev, const HitRecD *hd, 
                                  const int32_t *n_hits, const uint32_t *active, int level, const uint64_t *parents,
                                  int n_par, const int32_t *n_valid, uint64_t *out_keys, int32_t *out_votes,
                                  cudaStream_t s) {
-    dim3 grid((unsigned)(((long long)n_par + kChildParents - 1) / kChildParents), n_ev);
+    dim3 grid((unsigned)(((long long)n_par + kChildThreads / 16 - 1) / (kChildThreads / 16)), n_ev);   // two parents a warp
     k_vote_children<K><<<grid, kChildThreads, ChildSmem::total, s>>>(g, hd, hf, n_hits, active, level, parents, n_par,
                                                                      n_valid, out_keys, out_votes, nullptr);
 }
@@ -1544,7 +1665,7 @@ void launch_estimate_mask(const DevGeom &g, int n_ev, const uint64_t *keys, cons
 // ---------------------------------------------------------------------------------------
 template <int K> __device__ __noinline__ void persist_coarse(const DevGeom &g, const PersistArgs &A, int e,
                                                                 int32_t *vo, uint32_t *hist_b, unsigned char *smem) {
-    const CoarsePlan P = coarse_plan(g, false);
+    const CoarsePlan P = coarse_plan(g, false, 0);
     for (long long t = 0; t < P.n_tiles; t += P.tiles)
         coarse_block<K>(g, P, e, t, A.hd, A.hf, A.n_hits, A.active, vo, hist_b, A.status, nullptr, smem);
 }
@@ -1560,15 +1681,17 @@ template <int K> __device__ __noinline__ void persist_children(const DevGeom &g,
     if (threadIdx.x == 0) mbar_inval(bar);
     if (!ok) nh = 0;
     const int Kp = g.topk;
-    for (long long j0 = 0; j0 < (long long)Kp * 16; j0 += kChildThreads) {
-        children_block<K>(g, smem, nh, A.active + (long long)e * 8, level, A.fk + (long long)e * Kp, j0,
-                          (long long)Kp * 16, A.hd + (long long)e * kHitCap, hf_e, A.ck + (long long)e * Kp * 32,
-                          A.cv + (long long)e * Kp * 32);
-        __syncthreads();   // the masks and bounds are rewritten by the next pairs
-    }
+    ChildScratch &ws = reinterpret_cast<ChildScratch *>(smem + ChildSmem::warp)[threadIdx.x >> 5];
+    const int np = Kp / 8 < 2 ? 2 : (Kp / 8 > kChildParents ? kChildParents : Kp / 8 & ~1);   // two rounds of four warps
+    for (int p = (int)(threadIdx.x >> 5) * np; p < Kp; p += np * (kChildThreads / 32))
+        children_warp<K>(g, smem + ChildSmem::hits, ws, nh, A.active + (long long)e * 8, level,
+                         A.fk + (long long)e * Kp, p, np, Kp, A.hd + (long long)e * kHitCap, hf_e,
+                         A.ck + (long long)e * Kp * 32, A.cv + (long long)e * Kp * 32);
+    __threadfence_block();
+    __syncthreads();
 }
 
-__global__ void __launch_bounds__(128, 3) k_solve_persistent(const __grid_constant__ DevGeom g, const __grid_constant__ PersistArgs A) {
+__global__ void __launch_bounds__(128, 4) k_solve_persistent(const __grid_constant__ DevGeom g, const __grid_constant__ PersistArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_e;
     const int lv = g.levels, K = g.topk;
@@ -1608,7 +1731,7 @@ __global__ void __launch_bounds__(128, 3) k_solve_persistent(const __grid_consta
 }
 
 size_t persist_smem_bytes(const DevGeom &g) {
-    size_t a = CoarseSmem::total(g.bins[4], coarse_plan(g, false).tiles);
+    size_t a = CoarseSmem::total(g.bins[4], coarse_plan(g, false, 0));
     size_t b = ChildSmem::total;
     size_t c = kSortMax * sizeof(uint64_t) + kEstChunk * 5 * sizeof(double);
     size_t m = a > b ? a : b;

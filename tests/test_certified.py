@@ -45,25 +45,11 @@ template <int K> static float par(const double *c, const double *h, int og, int 
 extern "C" float parent(int k, const double *c, const double *h, int og, int *no) {
     return k == 64 ? par<64>(c, h, og, no) : par<32>(c, h, og, no);
 }
-// the end points with general products, then with the signs of L and t known; the vote with e
 extern "C" int child(const double *c, const double *h, float e, int og, float *out) {
     CellX<0> cc; HitX<0> hh;
     load(c, h, cc, hh);
-    const PreX<0> p = prefix(cc, hh);
-    const X<0> R = recip(cc.W);
-    X<0> a, b;
-    tail<0, 0>(p, cc.L, hh, R, cc.W, a, b);
-    Eval<0> r{a, b, p.wt};
-    const float g[4] = {a.lo, a.hi, b.lo, b.hi};
-    X<0> L = cc.L;
-    HitX<0> h2 = hh;
-    if (L.lo < 0 && L.hi <= 0) { L = neg(L); h2.t = neg(hh.t); }
-    if (L.lo >= 0) {
-        if (h2.t.v >= 0) tail<1, 1>(p, L, h2, R, cc.W, a, b);
-        else tail<1, -1>(p, L, h2, R, cc.W, a, b);
-    }
-    const float s[4] = {a.lo, a.hi, b.lo, b.hi};
-    for (int i = 0; i < 4; i++) { out[i] = g[i]; out[4 + i] = s[i]; }
+    const Eval<0> r = eval(cc, hh);
+    out[0] = r.Gp.lo; out[1] = r.Gp.hi; out[2] = r.Gm.lo; out[3] = r.Gm.hi;
     return verdict(r, og != 0, e);
 }
 """
@@ -135,12 +121,12 @@ def test_bounds_and_decisions(lib, bins, levels, k, og):
         for c in kids:
             v, ref = O.vote_pair(c, h, prec)
             assert not (no.value and v)
-            out = np.zeros(8, np.float32)
+            out = np.zeros(4, np.float32)
             d = lib.child(_p(c), _p(h), C.c_float(err), og, out.ctypes.data_as(C.POINTER(C.c_float)))
             if np.isnan(err):
                 assert d == 2
             if ref[4] == 0 and not np.isnan(err):   # evaluated by the oracle
-                assert np.abs(out.reshape(2, 4).astype(np.float64) - ref[:4]).max() <= err
+                assert np.abs(out.astype(np.float64) - ref[:4]).max() <= err
             assert d == 2 or d == v
             decided += d != 2
             undecided += d == 2
