@@ -161,16 +161,23 @@ __device__ __forceinline__ double edge4(double lo, int i, double w) { return __d
 __device__ __forceinline__ double mid4(double a, double b) { return __dmul_rn(__dadd_rn(a, b), 0.5); }
 
 // ---------------------------------------------------------------------------------------
-// Voting.  Block: a tile of kTile4 voxel columns (x_c, y_c, R) of one event.  First the
-// block tests every column of its tile against the disk pre-filter (Eq. ApoVoteDisk) and
-// the centre's validity, writes zero votes for the columns that fail, and lists the rest
-// in shared memory.  Then its 128 threads share out the listed columns: each runs every
-// active hit over its column's z0 voxels and both signs of tan(lambda), sharing the z0-
-// and sign-free part per hit, with vote counters bit-sliced over the z0 voxels.  Listing
-// first keeps the lanes of a warp on columns that all do the work; on the first
-// iteration's wide grid most warps would otherwise mix passing and failing columns.
+// Voting.  Block: a tile of 8 x 8 x depth voxel columns (x_c, y_c, R) of one event (depth 8, so that
+// the columns that pass fill whole warps, or 4 or 2 where there would be too few blocks).  First it
+// tests every column of its tile against the disk pre-filter (Eq. ApoVoteDisk) and the centre's
+// validity and writes zero votes for the columns that fail.  Then its threads take the groups of
+// 2 x 2 x 2 columns with a passing one, 16 groups at a time, a column each: every active hit
+// over the column's z0 voxels and both signs of tan(lambda), with vote counters bit-sliced over
+// the z0 voxels.
+//
+// The votes (of the program in T) are decided by certified FP32 values (cert4.cuh).  Per (group,
+// hit) one evaluation with errors over the group's columns and z0 voxels gives the bound that all
+// its pairs share, in chunks of 16 hits, one evaluation per thread (over each half of the z0 voxels
+// where the whole range decides nothing, then per column); pairs left undecided are queued by warp
+// and evaluated by the program itself.  FP32 issue bounds it; evaluating every pair was bound by the
+// FP64 pipe, and in FP32 by the instructions of correctly rounded quotients and roots.
 // ---------------------------------------------------------------------------------------
-constexpr int kTile4 = 512;
+constexpr int k4Threads = 128, k4Side = 8, k4MaxTile = k4Side * k4Side * k4Side, k4Groups = k4MaxTile / 8;
+constexpr int k4Slots = k4Threads / 8, k4Chunk = 16;
 
 template <typename T> struct Col4 {
     IV<T> X, Y, Rv;
@@ -178,11 +185,7 @@ template <typename T> struct Col4 {
 };
 
 template <typename T>
-__device__ __forceinline__ Col4<T> column4(const Iter4 &it, const double *le, const double *rf,
-                                           long long col) {
-    const int ix = (int)(col % it.n[0]);
-    const int iy = (int)((col / it.n[0]) % it.n[1]);
-    const int iR = (int)(col / ((long long)it.n[0] * it.n[1]));
+__device__ __forceinline__ Col4<T> column4(const Iter4 &it, const double *le, const double *rf, int ix, int iy, int iR) {
     const double xl = edge4(le[0], ix, it.w[0]), xh = edge4(le[0], ix + 1, it.w[0]);
     const double yl = edge4(le[1], iy, it.w[1]), yh = edge4(le[1], iy + 1, it.w[1]);
     const double rl = edge4(le[2], iR, it.w[2]), rh = edge4(le[2], iR + 1, it.w[2]);
@@ -194,16 +197,6 @@ __device__ __forceinline__ Col4<T> column4(const Iter4 &it, const double *le, co
                      rn<T>(it.p_gev), rn<T>(it.b_tesla), rn<T>(rf[0]), rn<T>(rf[1]));
     return c;
 }
-
-// ---------------------------------------------------------------------------------------
-// The votes (of the program in T) are decided by certified FP32 values (cert4.cuh).  Per
-// (column, hit) one evaluation with errors over the z0 voxels gives the bound that
-// all its (voxel, sign) pairs share (over each half of the z0 voxels where the whole range decides
-// nothing); the pairs left undecided are queued and evaluated by the program itself in whole warps.
-// FP32 issue bounds it; evaluating every pair was bound by the FP64 pipe, and in FP32 by the
-// instructions of correctly rounded quotients and roots.
-// ---------------------------------------------------------------------------------------
-constexpr int k4Threads = 128, k4Drain = 128, k4Queue = k4Drain + k4Threads;
 
 template <int K> __device__ __forceinline__ cert::X<K> wide(float v) {   // a value rounded to v
     return cert::point(cert::sc<K>(v));
@@ -217,28 +210,40 @@ template <int K> __device__ __forceinline__ cert::X<K> wide(float lo, float hi) 
 }
 template <int K> __device__ __forceinline__ cert::X<K> wide(cert::X<0> x) { return wide<K>(x.lo, x.hi); }
 
-// bound4 from the child's own FP32 values; out of the callers' registers
+// The ranges of some columns' constants (in Col4X's order) and intervals, from their FP32 values.
+struct Group4 { float2 m[8], box[3]; };
+
+// bound4 over a group's columns; out of the callers' registers
 template <int K>
-__device__ __noinline__ cert::Bound4 column_bound(cert::Col4X<cert::Pt> m, cert::Box4X<0> b, float zc0, float zc1,
-                                                  float z0, float z1, const cert::Hit4X<cert::Pt> *hp) {
+__device__ __noinline__ cert::Bound4 group_bound(const Group4 *gp, float zc0, float zc1, float z0, float z1,
+                                                 const cert::Hit4X<cert::Pt> *hp) {
     cert::Col4X<cert::X<K>> M;
     cert::Hit4X<cert::X<K>> H;
-    const cert::Pt *src = &m.xc, *hs = &hp->x0;
+    const cert::Pt *hs = &hp->x0;
     cert::X<K> *dst = &M.xc, *hd = &H.x0;
 #pragma unroll
-    for (int i = 0; i < 8; i++) dst[i] = wide<K>(src[i].v);
+    for (int i = 0; i < 8; i++) dst[i] = wide<K>(gp->m[i].x, gp->m[i].y);
 #pragma unroll
     for (int i = 0; i < 9; i++) hd[i] = wide<K>(hs[i].v);
     M.ion.e *= 2.f;   // an approximate reciprocal
-    return cert::bound4<K>(M, cert::Box4X<K>{wide<K>(b.X_), wide<K>(b.Y_), wide<K>(b.dR)}, wide<K>(zc0, zc1),
-                           wide<K>(z0, z1), H);
+    return cert::bound4<K>(M, cert::Box4X<K>{wide<K>(gp->box[0].x, gp->box[0].y), wide<K>(gp->box[1].x, gp->box[1].y),
+                                             wide<K>(gp->box[2].x, gp->box[2].y)},
+                           wide<K>(zc0, zc1), wide<K>(z0, z1), H);
+}
+
+// A column of the tile at (x0, y0, R0): k = 8 group + sub, both with x fastest.
+__device__ __forceinline__ void tile_column(int k, int x0, int y0, int r0, int &ix, int &iy, int &iR) {
+    const int gr = k >> 3, sub = k & 7;
+    ix = x0 + 2 * (gr & 3) + (sub & 1);
+    iy = y0 + 2 * ((gr >> 2) & 3) + ((sub >> 1) & 1);
+    iR = r0 + 2 * (gr >> 4) + (sub >> 2);
 }
 
 // The program's votes of one (column, hit) for the z0 voxels b0 (tan(lambda) > 0) and b1 (< 0).
 template <typename T>
-__device__ __noinline__ uint2 resolve4(const Iter4 &it, const double *le, const double *rf, long long col,
+__device__ __noinline__ uint2 resolve4(const Iter4 &it, const double *le, const double *rf, int ix, int iy, int iR,
                                        const HitRecD *rec, uint32_t b0, uint32_t b1) {
-    const Col4<T> c = column4<T>(it, le, rf, col);
+    const Col4<T> c = column4<T>(it, le, rf, ix, iy, iR);
     const HitP<T> h = hit_point<T>(*rec);
     const HitI<T> w = hit_iv<T>(*rec);
     uint2 yes = make_uint2(0u, 0u);
@@ -264,23 +269,27 @@ __device__ __noinline__ uint2 resolve4(const Iter4 &it, const double *le, const 
     return yes;
 }
 
+struct Queue4 { uint32_t id[64], b0[64], b1[64]; };   // lane | hit << 8; voxels of either sign of tan(lambda)
+
 template <typename T>
 __global__ void __launch_bounds__(k4Threads, 4)
 k4_vote(const __grid_constant__ Iter4 it, int ev0, const int32_t *n_hits, const HitRecD *hd,
-             const uint32_t *active, const double *lo, const double *ref, int32_t *votes, int32_t *vmax,
-             int sign_only) {
+        const uint32_t *active, const double *lo, const double *ref, int32_t *votes, int32_t *vmax, int sign_only, int depth) {
     constexpr int K = sizeof(T) == 8 ? 64 : 32;
     __shared__ cert::Hit4X<cert::Pt> s_h[kHitCap];
-    __shared__ unsigned char s_i[kHitCap];
+    __shared__ unsigned char s_i[kHitCap], s_grp[k4Groups];
     __shared__ float s_zc[32];
     __shared__ float2 s_z[32];
-    __shared__ short s_col[kTile4];
-    __shared__ uint32_t q_id[k4Queue], q_b0[k4Queue], q_b1[k4Queue];
-    __shared__ int s_n, s_np, s_nq, s_vmax[2];
-    const int el = blockIdx.y, e = ev0 + el, tid = threadIdx.x;
+    __shared__ uint32_t s_pass[k4MaxTile / 32];
+    __shared__ Group4 s_g[k4Slots];
+    __shared__ float s_e0[k4Slots][k4Chunk], s_e1[k4Slots][k4Chunk], s_eps[k4Slots][k4Chunk];
+    __shared__ Queue4 s_q[k4Threads / 32];
+    __shared__ int s_n, s_ng, s_vmax[2];
+    const int el = blockIdx.y, e = ev0 + el, tid = threadIdx.x, lane = tid & 31;
+    Queue4 &q = s_q[tid >> 5];
     int nh = n_hits[e];
     if (nh < 0) nh = 0;
-    if (tid == 0) { s_n = 0; s_np = 0; s_nq = 0; s_vmax[0] = s_vmax[1] = 0; }
+    if (tid == 0) { s_n = 0; s_vmax[0] = s_vmax[1] = 0; }
     __syncthreads();
     const uint32_t *act = active + (long long)e * 8;
     const HitRecD *hde = hd + (long long)e * kHitCap;
@@ -301,126 +310,198 @@ k4_vote(const __grid_constant__ Iter4 it, int ev0, const int32_t *n_hits, const 
     const double *rf = ref + (long long)e * 2;
     const int nz = it.n[3];
     int32_t *vo = votes + (long long)el * 2 * it.nvox;
-    const long long col0 = (long long)blockIdx.x * kTile4;
+    const int tx = (it.n[0] + k4Side - 1) / k4Side, ty = (it.n[1] + k4Side - 1) / k4Side;
+    const int x0 = k4Side * (blockIdx.x % tx), y0 = k4Side * (blockIdx.x / tx % ty), r0 = depth * (blockIdx.x / tx / ty);
+    const int ntile = k4Side * k4Side * depth;
     // disk pre-filter of the tile; failing columns get zero votes
-    for (int k = tid; k < kTile4; k += k4Threads) {
-        const long long col = col0 + k;
-        if (col >= it.ncol) break;
-        const Col4<T> c = column4<T>(it, le, rf, col);
-        if (disk4<T>(c.X, c.Y, c.Rv, up<T>(it.disk_radius)) && c.m.valid) {
-            s_col[atomicAdd(&s_np, 1)] = (short)k;
-        } else {
-            for (int s = 0; s < 2; s++)
-                if (sign_only < 0 || s == sign_only)
-                    for (int iz = 0; iz < nz; iz++) vo[(long long)s * it.nvox + col + it.ncol * iz] = 0;
+    for (int k = tid; k < ntile; k += k4Threads) {
+        int ix, iy, iR;
+        tile_column(k, x0, y0, r0, ix, iy, iR);
+        const bool in = ix < it.n[0] && iy < it.n[1] && iR < it.n[2];
+        bool pass = false;
+        if (in) {
+            const Col4<T> c = column4<T>(it, le, rf, ix, iy, iR);
+            pass = disk4<T>(c.X, c.Y, c.Rv, up<T>(it.disk_radius)) && c.m.valid;
+            const long long col = ix + (long long)it.n[0] * (iy + (long long)it.n[1] * iR);
+            if (!pass)
+                for (int s = 0; s < 2; s++)
+                    if (sign_only < 0 || s == sign_only)
+                        for (int iz = 0; iz < nz; iz++) vo[(long long)s * it.nvox + col + it.ncol * iz] = 0;
         }
+        const unsigned m = __ballot_sync(0xffffffffu, pass);
+        if (lane == 0) s_pass[k >> 5] = m;
     }
     __syncthreads();
-    const int na = s_n, np = s_np;
+    if (tid < 32) {   // the groups with a passing column, in order
+        int n = 0;
+        for (int g0 = 0; g0 < ntile / 8; g0 += 32) {
+            const int gr = g0 + lane;
+            const bool any = gr < ntile / 8 && ((s_pass[gr >> 2] >> (8 * (gr & 3))) & 255u) != 0u;
+            const unsigned m = __ballot_sync(0xffffffffu, any);
+            if (any) s_grp[n + __popc(m & ((1u << lane) - 1u))] = (unsigned char)gr;
+            n += __popc(m);
+        }
+        if (lane == 0) s_ng = n;
+    }
+    __syncthreads();
+    const int na = s_n, ng = s_ng, slot = tid >> 3, half = (nz + 1) >> 1;
     const uint32_t allz = nz >= 32 ? 0xffffffffu : ((1u << nz) - 1u);
     const uint32_t all0 = sign_only == 1 ? 0u : allz, all1 = sign_only == 0 ? 0u : allz;
     int mx[2] = {0, 0};
-    for (int base = 0; base < np; base += k4Threads) {
-        const bool has = base + tid < np;
-        const long long col = col0 + s_col[has ? base + tid : 0];
-        const Col4<T> cd = column4<T>(it, le, rf, col);
+    for (int g0 = 0; g0 < ng; g0 += k4Slots) {
+        const int ns = ng - g0 < k4Slots ? ng - g0 : k4Slots;
+        const int k = slot < ns ? 8 * s_grp[g0 + slot] + (tid & 7) : 0;
+        const bool has = slot < ns && ((s_pass[k >> 5] >> (k & 31)) & 1u);
+        int ix, iy, iR;
+        tile_column(k, x0, y0, r0, ix, iy, iR);
+        const Col4<T> cd = column4<T>(it, le, rf, ix, iy, iR);
         const T cR = cd.m.R;
         const cert::Col4X<cert::Pt> m{{(float)cd.m.xc}, {(float)cd.m.yc}, {(float)cR}, {(float)cd.m.aL}, {(float)cd.m.ox},
                                       {(float)cd.m.oy}, {cert::rcp_a((float)cd.m.on)}, {(float)cd.m.psi_ref}};
         const cert::Box4X<0> b{cert::mk<0>(cd.X.lo, cd.X.hi), cert::mk<0>(cd.Y.lo, cd.Y.hi),
                                cert::mk<0>((double)cd.Rv.lo - (double)cR, (double)cd.Rv.hi - (double)cR)};
         const bool guard = cd.m.guard;
+        {   // the group's ranges over its passing columns (the eight lanes of a slot)
+            const cert::Pt *src = &m.xc;
+            auto hull8 = [&](float l, float h) {
+                if (!has) { l = INFINITY; h = -INFINITY; }
+#pragma unroll
+                for (int o = 1; o < 8; o <<= 1) {
+                    l = fminf(l, __shfl_xor_sync(0xffffffffu, l, o));
+                    h = fmaxf(h, __shfl_xor_sync(0xffffffffu, h, o));
+                }
+                return make_float2(l, h);
+            };
+            __syncthreads();   // the last groups' bounds have been read
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                const float2 r = hull8(src[i].v, src[i].v);
+                if ((tid & 7) == 0) s_g[slot].m[i] = r;
+            }
+            const float2 bx = hull8(b.X_.lo, b.X_.hi), by = hull8(b.Y_.lo, b.Y_.hi), br = hull8(b.dR.lo, b.dR.hi);
+            if ((tid & 7) == 0) { s_g[slot].box[0] = bx; s_g[slot].box[1] = by; s_g[slot].box[2] = br; }
+        }
         uint32_t pl[2][9];
 #pragma unroll
         for (int s = 0; s < 2; s++)
 #pragma unroll
-            for (int q = 0; q < 9; q++) pl[s][q] = 0u;
+            for (int i = 0; i < 9; i++) pl[s][i] = 0u;
         auto add_votes = [&](int s, uint32_t v) {
 #pragma unroll
-            for (int q = 0; q < 9; q++) {
-                const uint32_t cy = pl[s][q] & v;
-                pl[s][q] ^= v;
+            for (int i = 0; i < 9; i++) {
+                const uint32_t cy = pl[s][i] & v;
+                pl[s][i] ^= v;
                 v = cy;
             }
         };
-        for (int j = 0; j < na; j++) {   // at most one queue entry per thread and hit
-            if (has) {
+        int nq = 0;
+        for (int j0 = 0; j0 < na; j0 += k4Chunk) {
+            const int nc = na - j0 < k4Chunk ? na - j0 : k4Chunk;
+            __syncthreads();
+            for (int i = tid; i < ns * nc; i += k4Threads) {
+                const int sl = i / nc, j = i - sl * nc;
+                cert::Bound4 f0 = group_bound<K>(s_g + sl, s_zc[0], s_zc[nz - 1], s_z[0].x, s_z[nz - 1].y, s_h + j0 + j), f1 = f0;
+                if (!(f0.e < 1e30f) && nz > 1) {
+                    f0 = group_bound<K>(s_g + sl, s_zc[0], s_zc[half - 1], s_z[0].x, s_z[half - 1].y, s_h + j0 + j);
+                    f1 = group_bound<K>(s_g + sl, s_zc[half], s_zc[nz - 1], s_z[half].x, s_z[nz - 1].y, s_h + j0 + j);
+                }
+                s_e0[sl][j] = f0.e;
+                s_e1[sl][j] = f1.e;
+                s_eps[sl][j] = fmaxf(f0.eps, f1.eps);
+            }
+            __syncthreads();
+            for (int j = 0; j < nc; j++) {
                 uint32_t b0 = 0, b1 = 0, u0 = 0, u1 = 0;
-                if (guard) {
+                if (has && guard) {
                     b0 = all0;
                     b1 = all1;
-                } else {
-                    const int half = (nz + 1) >> 1;
-                    cert::Bound4 e0 = column_bound<K>(m, b, s_zc[0], s_zc[nz - 1], s_z[0].x, s_z[nz - 1].y, s_h + j), e1 = e0;
-                    if (!(e0.e < 1e30f) && nz > 1) {
-                        e0 = column_bound<K>(m, b, s_zc[0], s_zc[half - 1], s_z[0].x, s_z[half - 1].y, s_h + j);
-                        e1 = column_bound<K>(m, b, s_zc[half], s_zc[nz - 1], s_z[half].x, s_z[nz - 1].y, s_h + j);
+                } else if (has) {
+                    const cert::Hit4X<cert::Pt> h = s_h[j0 + j];
+                    float e0 = s_e0[slot][j], e1 = s_e1[slot][j], eps = s_eps[slot][j];
+                    if (!(e0 < 1e30f) || !(e1 < 1e30f)) {   // the column's own bounds
+                        Group4 own;
+                        const cert::Pt *src = &m.xc;
+#pragma unroll
+                        for (int i = 0; i < 8; i++) own.m[i] = make_float2(src[i].v, src[i].v);
+                        own.box[0] = make_float2(b.X_.lo, b.X_.hi);
+                        own.box[1] = make_float2(b.Y_.lo, b.Y_.hi);
+                        own.box[2] = make_float2(b.dR.lo, b.dR.hi);
+                        const cert::Bound4 f0 = group_bound<K>(&own, s_zc[0], s_zc[half - 1], s_z[0].x, s_z[half - 1].y, s_h + j0 + j);
+                        cert::Bound4 f1 = f0;
+                        if (nz > 1)
+                            f1 = group_bound<K>(&own, s_zc[half], s_zc[nz - 1], s_z[half].x, s_z[nz - 1].y, s_h + j0 + j);
+                        e0 = f0.e;
+                        e1 = f1.e;
+                        eps = fmaxf(f0.eps, f1.eps);
                     }
-                    const cert::Hit4X<cert::Pt> h = s_h[j];
 #pragma unroll 1
                     for (int iz = 0; iz < nz; iz++) {
                         const uint32_t bit = 1u << iz;
-                        const float e = iz < half ? e0.e : e1.e, eps = iz < half ? e0.eps : e1.eps;
+                        const float e = iz < half ? e0 : e1;
                         bool bad = true;
-                        if (e < 1e30f) {
-                            cert::Pt dx, dy;
-                            cert::wire4x(m, cert::Pt{s_zc[iz]}, h, dx, dy);
-                            cert::Pre4X<cert::Pt> pre = cert::prefix4x(dx, dy, h);
-                            pre.psi = cert::psi4(m, dx, dy, pre.iRA, eps, bad);
-                            pre.Rpsi = cert::mul(m.R, pre.psi);
-                            if (!bad) {
-                                const float2 z = s_z[iz];
-                                const cert::X<0> A2 = cert::a2_4x<0, cert::Pt>(b, cert::X<0>{z.x, z.y, 0.f}, h);
-#pragma unroll 1
-                                for (int s = 0; s < 2; s++) {
-                                    if (sign_only == 1 - s) continue;
-                                    const int v = cert::vote4x(pre, m, s ? cert::neg(m.aL) : m.aL, h, A2, b.dR, e);
-                                    const uint32_t y = v == cert::kYes ? bit : 0u, u = v == cert::kUnknown ? bit : 0u;
-                                    if (s) { b1 |= y; u1 |= u; } else { b0 |= y; u0 |= u; }
-                                }
-                            }
+                        cert::Pt dx, dy;
+                        cert::wire4x(m, cert::Pt{s_zc[iz]}, h, dx, dy);
+                        cert::Pre4X<cert::Pt> pre = cert::prefix4x(dx, dy, h);
+                        pre.psi = cert::psi4(m, dx, dy, pre.iRA, eps, bad);
+                        pre.Rpsi = cert::mul(m.R, pre.psi);
+                        if (bad || !(e < 1e30f)) {
+                            u0 |= all0 & bit;
+                            u1 |= all1 & bit;
+                            continue;
                         }
-                        if (bad) { u0 |= all0 & bit; u1 |= all1 & bit; }
-                    }
-                    if (u0 | u1) {
-                        const int k = atomicAdd(&s_nq, 1);
-                        if (k < k4Queue) {   // always: the queue is drained before it could fill
-                            q_id[k] = (uint32_t)tid | ((uint32_t)j << 16);
-                            q_b0[k] = u0;
-                            q_b1[k] = u1;
+                        const float2 z = s_z[iz];
+                        const cert::X<0> A2 = cert::a2_4x<0, cert::Pt>(b, cert::X<0>{z.x, z.y, 0.f}, h);
+                        const cert::Delta4<cert::Pt> d0 = cert::delta4x(pre, m.R, m.aL, h.d, h),
+                                                     d1 = cert::delta4x(pre, m.R, m.aL, cert::neg(h.d), h);
+#pragma unroll 1
+                        for (int s = 0; s < 2; s++) {
+                            if (sign_only == 1 - s) continue;
+                            const float f = s ? 1.f : -1.f;
+                            const cert::Pt dl[2] = {{fmaf(f, d0.v.v, d0.u.v)}, {fmaf(f, d1.v.v, d1.u.v)}};
+                            const int v = cert::vote4x(pre, m, cert::Pt{-f * m.aL.v}, h, A2, b.dR, e, dl);
+                            const uint32_t y = v == cert::kYes ? bit : 0u, u = v == cert::kUnknown ? bit : 0u;
+                            if (s) { b1 |= y; u1 |= u; } else { b0 |= y; u0 |= u; }
                         }
                     }
                 }
                 add_votes(0, b0);
                 add_votes(1, b1);
-            }
-            __syncthreads();
-            const int nq = s_nq;
-            __syncthreads();
-            if (nq > k4Drain || (j + 1 == na && nq > 0)) {
-                for (int i = tid; i < nq; i += k4Threads) {
-                    const long long oc = col0 + s_col[base + (int)(q_id[i] & 0xffffu)];
-                    const uint2 y = resolve4<T>(it, le, rf, oc, hde + s_i[q_id[i] >> 16], q_b0[i], q_b1[i]);
-                    q_b0[i] = y.x;
-                    q_b1[i] = y.y;
+                const unsigned um = __ballot_sync(0xffffffffu, (u0 | u1) != 0u);
+                if (u0 | u1) {
+                    const int i = nq + __popc(um & ((1u << lane) - 1u));   // below 64: drained from 32 on
+                    q.id[i] = (uint32_t)lane | ((uint32_t)(j0 + j) << 8);
+                    q.b0[i] = u0;
+                    q.b1[i] = u1;
                 }
-                __syncthreads();
-                for (int i = 0; i < nq; i++)
-                    if ((int)(q_id[i] & 0xffffu) == tid) {
-                        add_votes(0, q_b0[i]);
-                        add_votes(1, q_b1[i]);
+                nq += __popc(um);
+                if (nq >= 32 || (nq && j0 + j + 1 == na)) {
+                    __syncwarp();
+                    for (int i = lane; i < nq; i += 32) {
+                        const int ot = (tid & ~31) + (int)(q.id[i] & 255u);
+                        int ox, oy, oR;
+                        tile_column(8 * s_grp[g0 + (ot >> 3)] + (ot & 7), x0, y0, r0, ox, oy, oR);
+                        const uint2 y = resolve4<T>(it, le, rf, ox, oy, oR, hde + s_i[q.id[i] >> 8], q.b0[i], q.b1[i]);
+                        q.b0[i] = y.x;
+                        q.b1[i] = y.y;
                     }
-                __syncthreads();
-                if (tid == 0) s_nq = 0;
-                __syncthreads();
+                    __syncwarp();
+                    for (int i = 0; i < nq; i++)
+                        if ((int)(q.id[i] & 255u) == lane) {
+                            add_votes(0, q.b0[i]);
+                            add_votes(1, q.b1[i]);
+                        }
+                    __syncwarp();
+                    nq = 0;
+                }
             }
         }
+        const long long col = ix + (long long)it.n[0] * (iy + (long long)it.n[1] * iR);
         for (int s = 0; s < 2 && has; s++) {
             if (sign_only >= 0 && s != sign_only) continue;
             for (int iz = 0; iz < nz; iz++) {
                 int v = 0;
 #pragma unroll
-                for (int q = 0; q < 9; q++) v |= (int)((pl[s][q] >> iz) & 1u) << q;
+                for (int i = 0; i < 9; i++) v |= (int)((pl[s][i] >> iz) & 1u) << i;
                 vo[(long long)s * it.nvox + col + it.ncol * iz] = v;
                 mx[s] = v > mx[s] ? v : mx[s];
             }
@@ -652,8 +733,14 @@ template <typename T>
 void launch_vote4(const Iter4 &it, int ev0, int n, const int32_t *nh, const HitRecD *hd,
                   const uint32_t *active, const double *lo, const double *ref, int32_t *votes,
                   int32_t *vmax, cudaStream_t s, int sign_only = -1) {
-    dim3 grid((unsigned)((it.ncol + kTile4 - 1) / kTile4), n);
-    k4_vote<T><<<grid, k4Threads, 0, s>>>(it, ev0, nh, hd, active, lo, ref, votes, vmax, sign_only);
+    auto tiles = [&](int depth) {
+        auto side = [&](int a, int s) { return (long long)((it.n[a] + s - 1) / s); };
+        return side(0, k4Side) * side(1, k4Side) * side(2, depth);
+    };
+    int depth = k4Side;   // four waves of four blocks on 152 SMs
+    while (depth > 2 && tiles(depth) * n < 4 * 4 * 152) depth /= 2;
+    dim3 grid((unsigned)tiles(depth), n);
+    k4_vote<T><<<grid, k4Threads, 0, s>>>(it, ev0, nh, hd, active, lo, ref, votes, vmax, sign_only, depth);
 }
 
 void launch_stats4(const Iter4 &it, int ev0, int n, const int32_t *votes, const int32_t *vmax,

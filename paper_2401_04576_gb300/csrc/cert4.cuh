@@ -53,18 +53,20 @@ APO_CERT Pt psi4(const Col4X<Pt> &m, Pt dx, Pt dy, Pt iRA, float eps, bool &bad)
     if (ph < 0.f) ph += kTwoPi;
     return {ph - m.psi_ref.v};
 }
-// The phases of a range of wire points (dx, dy): the middle's +- the largest turn; eps: the error
+// The phases of a range of wire points (dx, dy) and centres: the middle's +- the largest turn; eps: the error
 // a child's phase can have, (e_sn + e_cs) / r + AngleErr and the roundings of 2 pi and the sum.
 struct Turn4 { float ph, turn, eps; };
 template <int K> APO_CERT Turn4 turn4(const Col4X<X<K>> &m, X<K> dx, X<K> dy, X<K> iRA) {
     const X<K> sn = sub(mul(m.ox, dy), mul(m.oy, dx)), cs = add(mul(m.ox, dx), mul(m.oy, dy));
     const X<K> ir = mul(m.ion, iRA);
     const float mx = 0.5f * (dx.lo + dx.hi), my = 0.5f * (dy.lo + dy.hi);
-    const float ms = m.ox.lo * my - m.oy.lo * mx, mc = m.ox.lo * mx + m.oy.lo * my;
+    const float ux = 0.5f * (m.ox.lo + m.ox.hi), uy = 0.5f * (m.oy.lo + m.oy.hi);
     Turn4 r;
-    r.ph = angle4(ms, mc, m.ion.lo * rcp_a(sqrt_a(mx * mx + my * my)));
+    r.ph = angle4(ux * my - uy * mx, ux * mx + uy * my, rcp_a(sqrt_a(ux * ux + uy * uy) * sqrt_a(mx * mx + my * my)));
     const float hx = dx.hi - mx + 2.f * dx.e, hy = dy.hi - my + 2.f * dy.e;
-    r.turn = 1.6f * sqrt_a(hx * hx + hy * hy) * M(iRA);   // a turn below 1 rad is under 1.1 chord / radius
+    const float kx = m.ox.hi - ux + 2.f * m.ox.e, ky = m.oy.hi - uy + 2.f * m.oy.e;
+    // each vector's turn; below 1 rad it is under 1.1 chord / radius
+    r.turn = 1.6f * (sqrt_a(hx * hx + hy * hy) * M(iRA) + sqrt_a(kx * kx + ky * ky) * M(m.ion));
     const float least = ir.lo - 2.f * ir.e;   // 1 / r's own relative error turns the angle by at most that
     r.eps = when(least > 0.f, ((sn.e + cs.e) * M(ir) + ir.e / least + 8.f * Unit<K>::u + AngleErr<K>::v) * 1.01f);
     return r;
@@ -89,20 +91,26 @@ template <typename N> APO_CERT Pre4X<N> prefix4x(N dx, N dy, const Hit4X<N> &h) 
     return p;
 }
 
-// (R + d^Ax)^2 of one drift sign (ds = +-d) and tan(lambda) L: the radicand of Eq. (defdiAX_b)
-template <typename N> APO_CERT N rad4x(const Pre4X<N> &p, N R, N L, N ds, const Hit4X<N> &h) {
+// The phase correction of one drift sign (ds = +-d), even and odd in tan(lambda) = L = +-aL: for L it
+// is u - v, for -L it is u + v.
+template <typename N> struct Delta4 { N u, v; };
+template <typename N> APO_CERT Delta4<N> delta4x(const Pre4X<N> &p, N R, N L, N ds, const Hit4X<N> &h) {
     const N zA = mul(L, p.Rpsi), Lz = mul(L, zA), L2 = sqr(L);
     const N f1 = add(mul(zA, p.sPA), mul(mul(L, ds), p.cPA));            // -Phi1 RA
     const N f2 = add(sub(mul(R, Lz), mul(mul(Lz, sub(R, scl(ds, 2.f))), p.cos2)),
                      mul(add(sqr(zA), mul(ds, add(p.RA, mul(L2, sub(add(R, p.RA), ds))))), p.sin2));
-    const N dl = sub(mul(mul(f2, p.iA2), h.t2), mul(mul(f1, p.iRA), h.t));
+    return Delta4<N>{mul(mul(f2, p.iA2), h.t2), mul(mul(f1, p.iRA), h.t)};
+}
+// (R + d^Ax)^2: the radicand of Eq. (defdiAX_b) for a phase correction dl
+template <typename N> APO_CERT N rad4x(const Pre4X<N> &p, N R, N L, N ds, N dl, const Hit4X<N> &h) {
     N sd, cd;
     sincos4(dl, sd, cd);
     const N sP = add(mul(p.sPA, cd), mul(p.cPA, sd)), cP = sub(mul(p.cPA, cd), mul(p.sPA, sd));
-    const N u2 = add(add(add1(mul(scl(mul(L, h.t), 2.f), sP), 1.f), mul(L2, h.t2)), mul(sqr(cP), h.t2));
-    const N q = mul(ds, recip(sqrtx(u2)));
+    const N Lt = mul(L, h.t);
+    const N u2 = add(add(add1(mul(scl(Lt, 2.f), sP), 1.f), mul(sqr(L), h.t2)), mul(sqr(cP), h.t2));
+    const N q = mul(ds, rsqrtx(u2));
     const N zt = mul(sub(mul(L, mul(R, add(p.psi, dl))), mul(mul(q, cP), h.t)), h.t);   // z^St t
-    const N Lqt = mul(mul(L, q), h.t);
+    const N Lqt = mul(q, Lt);
     const N ct = sub(mul(zt, p.cA), mul(Lqt, p.sA));                                     // c^tau t
     return sub(sub(sub(sqr(add(R, q)), scl(ct, 2.f)), sqr(zt)), sqr(Lqt));
 }
@@ -117,7 +125,7 @@ APO_CERT X<K> a2_4x(const Box4X<K> &b, X<K> Z, const Hit4X<N> &h) {
 
 struct Bound4 { float e, eps; };   // of G and of the radicand; of a phase (e NaN: undecidable)
 
-// The errors of every child of one (column, hit): centres z and voxels Z (ranges), both signs of
+// The errors of every child of some columns and one hit: centres m, z and voxels b, Z (ranges), both signs of
 // tan(lambda) and of the drift (one evaluation over their hulls: the errors grow with magnitudes).
 // G = A2 - (s + dR)^2 with s = sqrt(rad): its error is e_A2 + e_rad (1 + dR / s), at most
 // e_A2 + 2 e_rad where s >= dR, and the roundings of s, of d^Ax = s - R, of the sum and of the
@@ -144,7 +152,8 @@ APO_CERT Bound4 bound4(const Col4X<X<K>> &m, const Box4X<K> &b, X<K> z, X<K> Z, 
         ph.e = tr.eps + rnd<K>(4.f * kTwoPi);
         p.psi = sub(ph, m.psi_ref);
         p.Rpsi = mul(m.R, p.psi);
-        const X<K> rad = rad4x(p, m.R, L, ds, h);
+        const Delta4<X<K>> dl = delta4x(p, m.R, L, ds, h);   // L and ds hold both signs
+        const X<K> rad = rad4x(p, m.R, L, ds, sub(dl.u, dl.v), h);
         const float mr = M(rad), md = M(b.dR);
         const float x = A2.e + 2.f * rad.e + 10.f * Unit<K>::ua * (mr + md * md) + 2.f * rnd<K>(M(A2)) + 4.f * b.dR.e;
         e = x < 1e30f ? fmaxf(e, x) : INFINITY;
@@ -154,14 +163,15 @@ APO_CERT Bound4 bound4(const Col4X<X<K>> &m, const Box4X<K> &b, X<K> z, X<K> Z, 
     return Bound4{ok ? e * 1.01f : NAN, tr.eps};
 }
 
-// One voxel and sign of tan(lambda): kYes / kNo / kUnknown (either drift sign; a negative radicand
-// guards, and votes).  bad: psi is undecided.
-APO_CERT int vote4x(const Pre4X<Pt> &p, const Col4X<Pt> &m, Pt L, const Hit4X<Pt> &h, X<0> A2, X<0> dR, float e) {
+// One voxel and sign of tan(lambda), L = +-aL: kYes / kNo / kUnknown (either drift sign; a negative
+// radicand guards, and votes); dl: its phase corrections for the drift signs + and -.
+APO_CERT int vote4x(const Pre4X<Pt> &p, const Col4X<Pt> &m, Pt L, const Hit4X<Pt> &h, X<0> A2, X<0> dR, float e,
+                    const Pt (&dl)[2]) {
     const float md = mag2(dR.lo, dR.hi), least = fmaxf(4.f * e, 1.01f * md * md);
     bool yes = false, no = true;
 #pragma unroll
     for (int sg = 0; sg < 2; sg++) {
-        const float rad = rad4x(p, m.R, L, sg ? neg(h.d) : h.d, h).v;
+        const float rad = rad4x(p, m.R, L, sg ? neg(h.d) : h.d, dl[sg], h).v;
         const float s = sqrt_a(rad), a = s + dR.lo, c = s + dR.hi;   // s >= |dR|: both ends >= 0
         const float lo = A2.lo - c * c, hi = A2.hi - a * a;
         const bool in = rad > least;

@@ -21,6 +21,8 @@ APO_CERT Pt add1(Pt a, float c) { return {a.v + c}; }
 APO_CERT Pt sqr(Pt a) { return {a.v * a.v}; }
 APO_CERT Pt recip(Pt a) { return {rcp_a(a.v)}; }
 APO_CERT Pt sqrtx(Pt a) { return {sqrt_a(a.v)}; }
+APO_CERT Pt rsqrtx(Pt a) { return {rsqrt_a(a.v)}; }
+template <int K> APO_CERT X<K> rsqrtx(X<K> a) { return recip(sqrtx(a)); }   // two units for rsqrt's one
 template <typename N> APO_CERT N num(double v);
 template <> APO_CERT Pt num<Pt>(double v) { return {(float)v}; }
 template <> APO_CERT X<64> num<X<64>>(double v) { return mk<64>(v, v); }

@@ -1,5 +1,5 @@
 """The point programs' certified FP32 forms (csrc/cert4.cuh, csrc/cert_mid.cuh), compiled as host
-C++, against the oracle: with the bound of a range of centres (one column's z0 voxels; a level-0
+C++, against the oracle: with the bound of a range of centres (a group of 2 x 2 x 2 columns and their z0 voxels; a level-0
 tile or a kept cell's children) every decision must be the oracle's vote, and in FP64 the end points
 of G must lie within the bound of the oracle's.  4-D: the three iterations' voxels, FP64 and FP32,
 columns that pass the disk pre-filter anywhere in the grid (hits on either side of the centre, phases
@@ -25,27 +25,24 @@ SHIM = r"""
 using namespace apo::cert;
 static float down(double x) { float f = (float)x; return (double)f > x ? std::nextafter(f, -INFINITY) : f; }
 
-// ---- 4-D: cc = x_c, y_c, R, |tan(lambda)|, phase of the reference point; box = x, y, R lo / hi ----
-template <int K> static X<K> w(double v, double scale = 1) {
+// ---- 4-D: cc = x_c, y_c, R, |tan(lambda)|, -x_c, -y_c, 1 / |(x_c, y_c)|, phase of the reference point
+// (lo / hi pairs for a group of columns); box = x, y, R - R_centre (bound) or R (child), lo / hi ----
+template <int K> static X<K> w(double a, double b) {
     X<K> r;
-    r.lo = r.hi = (float)v;
-    r.e = (float)scale * 2.f * rnd<K>(std::fabs((float)v)) + kTiny;
-    return r;
-}
-template <int K> static X<K> wr(double a, double b) {
-    X<K> r = w<K>(a), s = w<K>(b);
-    r.hi = s.hi;
-    r.e = fmaxf(r.e, s.e);
+    r.lo = (float)a;
+    r.hi = (float)b;
+    r.e = 2.f * rnd<K>(mag2(r.lo, r.hi)) + kTiny;
     return r;
 }
 template <int K> static Bound4 b4(const double *cc, const double *box, const double *z, const double *h) {
-    const double ion = 1 / std::sqrt(cc[0] * cc[0] + cc[1] * cc[1]);
-    Col4X<X<K>> m{w<K>(cc[0]), w<K>(cc[1]), w<K>(cc[2]), w<K>(cc[3]), w<K>(-cc[0]), w<K>(-cc[1]), w<K>(ion, 2), w<K>(cc[4])};
+    Col4X<X<K>> m;
     Hit4X<X<K>> x;
-    X<K> *f = &x.x0;
-    for (int i = 0; i < 9; i++) f[i] = w<K>(h[i]);
-    return bound4<K>(m, Box4X<K>{wr<K>(box[0], box[1]), wr<K>(box[2], box[3]), wr<K>(box[4] - cc[2], box[5] - cc[2])},
-                     wr<K>(z[0], z[1]), wr<K>(z[2], z[3]), x);
+    X<K> *q = &m.xc, *f = &x.x0;
+    for (int i = 0; i < 8; i++) q[i] = w<K>(cc[2 * i], cc[2 * i + 1]);
+    m.ion.e *= 2.f;
+    for (int i = 0; i < 9; i++) f[i] = w<K>(h[i], h[i]);
+    return bound4<K>(m, Box4X<K>{w<K>(box[0], box[1]), w<K>(box[2], box[3]), w<K>(box[4], box[5])}, w<K>(z[0], z[1]),
+                     w<K>(z[2], z[3]), x);
 }
 extern "C" float bound_4d(int k, const double *cc, const double *box, const double *z, const double *h, float *eps) {
     const Bound4 r = k == 64 ? b4<64>(cc, box, z, h) : b4<32>(cc, box, z, h);
@@ -54,11 +51,11 @@ extern "C" float bound_4d(int k, const double *cc, const double *box, const doub
 }
 extern "C" int child_4d(const double *cc, const double *box, const double *z, const double *h, int sign, float e,
                         float eps, float *out) {
-    const float ion = 1 / std::sqrt((float)cc[0] * (float)cc[0] + (float)cc[1] * (float)cc[1]);
-    Col4X<Pt> m{{(float)cc[0]}, {(float)cc[1]}, {(float)cc[2]}, {(float)cc[3]}, {-(float)cc[0]}, {-(float)cc[1]}, {ion},
-                {(float)cc[4]}};
+    Col4X<Pt> m;
     Hit4X<Pt> x;
-    Pt *f = &x.x0, dx, dy;
+    Pt *q = &m.xc, *f = &x.x0, dx, dy;
+    for (int i = 0; i < 8; i++) q[i].v = (float)cc[i];
+    m.ion.v = 1 / std::sqrt(m.xc.v * m.xc.v + m.yc.v * m.yc.v);
     for (int i = 0; i < 9; i++) f[i].v = (float)h[i];
     const Box4X<0> b{mk<0>(box[0], box[1]), mk<0>(box[2], box[3]), mk<0>(box[4] - cc[2], box[5] - cc[2])};
     bool bad;
@@ -67,14 +64,16 @@ extern "C" int child_4d(const double *cc, const double *box, const double *z, co
     p.psi = psi4(m, dx, dy, p.iRA, eps, bad);
     p.Rpsi = mul(m.R, p.psi);
     const X<0> A2 = a2_4x<0, Pt>(b, mk<0>(z[1], z[2]), x);
-    const Pt L = sign > 0 ? m.aL : neg(m.aL);
-    for (int s = 0; s < 2; s++) {
-        const float rad = rad4x(p, m.R, L, s ? neg(x.d) : x.d, x).v, q = std::sqrt(rad);
-        out[3 * s] = rad;
-        out[3 * s + 1] = A2.lo - (q + b.dR.hi) * (q + b.dR.hi);
-        out[3 * s + 2] = A2.hi - (q + b.dR.lo) * (q + b.dR.lo);
+    const Delta4<Pt> d0 = delta4x(p, m.R, m.aL, x.d, x), d1 = delta4x(p, m.R, m.aL, neg(x.d), x);
+    const float s = sign > 0 ? -1.f : 1.f;
+    const Pt dl[2] = {{std::fma(s, d0.v.v, d0.u.v)}, {std::fma(s, d1.v.v, d1.u.v)}}, L{-s * m.aL.v};
+    for (int i = 0; i < 2; i++) {
+        const float rad = rad4x(p, m.R, L, i ? neg(x.d) : x.d, dl[i], x).v, r = std::sqrt(rad);
+        out[3 * i] = rad;
+        out[3 * i + 1] = A2.lo - (r + b.dR.hi) * (r + b.dR.hi);
+        out[3 * i + 2] = A2.hi - (r + b.dR.lo) * (r + b.dR.lo);
     }
-    return bad ? kUnknown : vote4x(p, m, L, x, A2, b.dR, e);
+    return bad ? kUnknown : vote4x(p, m, L, x, A2, b.dR, e, dl);
 }
 
 // ---- midpoint form: c = cell12; m = lo / hi of the centres D, sin, cos, W, Z, L ----
@@ -169,45 +168,54 @@ def test_four_d(lib, it, k):
         if it == 2:
             c = comet.helix_centre(ev.tracks[e][0])
             lo = [c[a] - 0.5 * N[a] * W[a] + 0.002 for a in range(3)] + [-0.5 * N[3] * W[3]]
-        while True:
-            ix = [int(rng.integers(N[a])) for a in range(3)]
-            b = [v for a in range(3) for v in (lo[a] + ix[a] * W[a], lo[a] + (ix[a] + 1) * W[a])]
-            if O.four_disk(b):
-                break
-        x, y, R = (b[0] + b[1]) / 2, (b[2] + b[3]) / 2, (b[4] + b[5]) / 2
+        boxes = []
+        while not boxes:   # a group of 2 x 2 x 2 columns, those that pass
+            i0 = [2 * int(rng.integers(N[a] // 2)) for a in range(3)]
+            for s in range(8):
+                ix = [i0[a] + ((s >> a) & 1) for a in range(3)]
+                b = [v for a in range(3) for v in (lo[a] + ix[a] * W[a], lo[a] + (ix[a] + 1) * W[a])]
+                if O.four_disk(b) and 0.105 / (0.15 * (b[4] + b[5])) > 1.0 + 1e-5:
+                    boxes.append(b)
         ref = (0.0, 0.0) if it == 0 or k == 32 else (0.98 * h[0], 0.97 * h[1])
-        ratio = 0.105 / (0.3 * R)
-        if ratio <= 1.0 + 1e-5:
-            continue
-        if k == 32:
-            x, y, R = [float(np.float32(v)) for v in (x, y, R)]
-            cc = _a([x, y, R, O.four_vote_pair(b + [0.0, 0.07], 1, ref, h, prec=1)[1][3], 0.0])
-        else:
-            cc = _a([x, y, R, math.sqrt(ratio * ratio - 1.0), _phase(-x, -y, ref[0] - x, ref[1] - y)])
+        cc = []
+        for b in boxes:
+            x, y, R = (b[0] + b[1]) / 2, (b[2] + b[3]) / 2, (b[4] + b[5]) / 2
+            if k == 32:
+                x, y, R = [float(np.float32(v)) for v in (x, y, R)]
+                aL, ph = O.four_vote_pair(b + [0.0, 0.07], 1, ref, h, prec=1)[1][3], 0.0
+            else:
+                aL, ph = math.sqrt((0.105 / (0.3 * R)) ** 2 - 1.0), _phase(-x, -y, ref[0] - x, ref[1] - y)
+            cc.append([x, y, R, aL, -x, -y, 1.0 / math.hypot(x, y), ph])
+        cc, bb = np.array(cc), np.array(boxes)
+        group = _a(np.stack([cc.min(0), cc.max(0)], 1).ravel())
+        box = _a([bb[:, 0].min(), bb[:, 1].max(), bb[:, 2].min(), bb[:, 3].max(),
+                  (bb[:, 4] - cc[:, 2]).min(), (bb[:, 5] - cc[:, 2]).max()])
         z = [lo[3] + j * W[3] for j in range(N[3] + 1)]
-        box, eps = _a(b), C.c_float()
+        eps = C.c_float()
         zr = _a([(z[0] + z[1]) / 2, (z[-2] + z[-1]) / 2, z[0], z[-1]])
-        err = lib.bound_4d(k, _p(cc), _p(box), _p(zr), _p(h), C.byref(eps))
+        err = lib.bound_4d(k, _p(group), _p(box), _p(zr), _p(h), C.byref(eps))
+        q = int(rng.integers(len(boxes)))
+        b, ctr = boxes[q], _a(cc[q])
         for j in rng.choice(N[3], 3, replace=False):
             for sign in (1, -1):
                 v, r = O.four_vote_pair(b + [z[j], z[j + 1]], sign, ref, h, prec=0 if k == 64 else 1)
                 out = np.zeros(6, np.float32)
                 zc = _a([(z[j] + z[j + 1]) / 2, z[j], z[j + 1]])
-                d = lib.child_4d(_p(cc), _p(box), _p(zc), _p(h), sign, C.c_float(err), eps, out.ctypes.data_as(F4))
+                d = lib.child_4d(_p(ctr), _p(_a(b)), _p(zc), _p(h), sign, C.c_float(err), eps, out.ctypes.data_as(F4))
                 assert d == 2 or (d == v and not math.isnan(err))
                 decided += d != 2
                 undecided += d == 2
                 if k == 32 or d == 2:
                     continue
-                xw, yw = sorted([h[0] + z[j + q] * h[5] for q in (0, 1)]), sorted([h[1] - z[j + q] * h[6] for q in (0, 1)])
+                xw, yw = sorted([h[0] + z[j + s] * h[5] for s in (0, 1)]), sorted([h[1] - z[j + s] * h[6] for s in (0, 1)])
                 sx, sy = _sq(xw, b[0:2]), _sq(yw, b[2:4])
                 for s in (0, 1):
                     if out[3 * s] < 1e-5 or (int(r[2]) >> s) & 1:
                         continue
-                    q = sorted([(b[4] + r[s]) ** 2, (b[5] + r[s]) ** 2])
-                    assert abs(out[3 * s + 1] - (sx[0] + sy[0] - q[1])) <= err
-                    assert abs(out[3 * s + 2] - (sx[1] + sy[1] - q[0])) <= err
-    assert decided > 20 * undecided
+                    g = sorted([(b[4] + r[s]) ** 2, (b[5] + r[s]) ** 2])
+                    assert abs(out[3 * s + 1] - (sx[0] + sy[0] - g[1])) <= err
+                    assert abs(out[3 * s + 2] - (sx[1] + sy[1] - g[0])) <= err
+    assert decided > 10 * undecided
 
 
 @pytest.mark.parametrize("bins,levels", [([16] * 5, 6), ([5, 6, 6, 5, 5], 5), ([7, 6, 8, 5, 9], 2)])
