@@ -98,9 +98,11 @@ template <int Q> __device__ __forceinline__ cert::X<Q> xf(float2 a) {   // ends 
 }
 
 // The test of one hit on a box: -1 when no cell inside it gets the hit's vote, else the error bound
-// its cells share (NaN: they cannot be decided by one).  Not inlined: its registers stay out of the
-// callers' loops.
-template <int K> __device__ __noinline__ float box_error(const CertBox *b, const void *rec, bool outgoing) {
+// its cells share (NaN: they cannot be decided by one).  own: the box is one cell; -2 when it votes.
+// Not inlined: its registers stay out of the callers' loops, and one copy stays in the instruction
+// cache.
+template <int K>
+__device__ __noinline__ float box_error(const CertBox *b, const void *rec, bool outgoing, bool own = false) {
     constexpr int Q = K == kMid ? 64 : K;
     if (b->guard) return NAN;
     const cert::CellX<Q> c{xf<Q>(b->v[0]), xf<Q>(b->v[1]), xf<Q>(b->v[2]), xf<Q>(b->v[3]), xf<Q>(b->v[4]), xf<Q>(b->v[5])};
@@ -116,9 +118,10 @@ template <int K> __device__ __noinline__ float box_error(const CertBox *b, const
         const float e = (Gp.e < 1e30f && Gm.e < 1e30f) ? 1.01f * fmaxf(Gp.e, Gm.e) : NAN;
         return cert::decide(Gp, Gm, e) == cert::kNo ? -1.f : e;
     } else {
-        const cert::Eval<K> x = cert::eval(c, hx);
+        const cert::Eval<K> x = cert::eval(c, hx, own);
         const float e = cert::bound(x);
-        return cert::verdict(x, outgoing, e) == cert::kNo ? -1.f : e;
+        const int v = cert::verdict(x, outgoing, e);
+        return v == cert::kNo ? -1.f : (own && v == cert::kYes ? -2.f : e);
     }
 }
 // Whether no cell inside the box with its tan(lambda) ends replaced by L gets the hit's vote, for an
@@ -165,17 +168,18 @@ __device__ __noinline__ uint32_t resolve(const DevGeom &g, int level, int d, int
         return yes;
     } else {
         using T = typename RefOf<K>::T;
-        bool guard;
-        const bool mir = omega_sign<K>(c.W, &guard);
-        const cert::HitX<K> h = cert_hit<K>(hf, mir);
+        const IV<double> L0 = edge(g, 4, level, l0);
+        c.L = L0;
+        CertBox box = cert_box<K>(c, L0, L0);
         while (mask) {
             const int b = __ffs(mask) - 1;
             mask &= mask - 1;
             c.L = edge(g, 4, level, l0 + b);
             int v = cert::kUnknown;
-            if (own && !guard) {
-                const cert::Eval<K> ev = cert::eval(cert_cell<K>(c, mir), h);
-                v = cert::verdict(ev, g.k.outgoing != 0, cert::bound(ev));
+            if (own) {
+                box.v[5] = make_float2((float)c.L.lo, (float)c.L.hi);
+                const float e = box_error<K>(&box, hf, g.k.outgoing != 0, true);
+                v = e == -1.f ? cert::kNo : (e == -2.f ? cert::kYes : cert::kUnknown);
             }
             if (v == cert::kUnknown) {
                 const Cell<T> ct{to_prec<T>(c.D), to_prec<T>(c.S0), to_prec<T>(c.C0),
@@ -205,7 +209,7 @@ __device__ __forceinline__ bool vote_single(const DevGeom &g, const Cell<double>
     bool guard;
     const bool mir = omega_sign<K>(c.W, &guard);
     if (guard) return true;
-    const cert::Eval<K> x = cert::eval(cert_cell<K>(c, mir), cert_hit<K>(hf, mir));
+    const cert::Eval<K> x = cert::eval(cert_cell<K>(c, mir), cert_hit<K>(hf, mir), true);
     const int v = cert::verdict(x, g.k.outgoing != 0, cert::bound(x));
     if (v != cert::kUnknown) return v == cert::kYes;
     const void *rec = K == 64 ? static_cast<const void *>(hd) : static_cast<const void *>(hf);
@@ -230,7 +234,7 @@ __device__ __noinline__ bool vote_widened(const DevGeom &g, const Cell<double> &
     for (int i = 0; i < 8; i++)
         s[i] = cert::sc<64>(__double2float_rd((mir && (i == 1 || i == 3 || i == 6)) ? -f[i].lo : f[i].lo));
     hx.d = cx<64>(h.d);
-    const cert::Eval<64> x = cert::eval(cert_cell<64>(c, mir), hx);
+    const cert::Eval<64> x = cert::eval(cert_cell<64>(c, mir), hx, true);
     const int v = cert::verdict(x, g.k.outgoing != 0, cert::bound(x));
     if (v != cert::kUnknown) return v == cert::kYes;
     return vote_reference<double>(g, c, h);

@@ -203,8 +203,16 @@ template <int K> APO_CERT X<K> atanx(X<K> x) {
     return scl(fin<K>(a.lo - rem, a.hi + rem, K ? a.e + 2e-5f * x.e + 6e-12f : 0.f), 4.f);
 }
 
-// sin and cos of |d| <= 1 as in the program (series and remainder)
-template <int K> APO_CERT void sincosx(X<K> d, X<K> &s, X<K> &c) {
+// sin and cos as in the program: series and remainder for |d| <= 1, else [-1, 1].  A box whose d may
+// pass 1 has cells on either side and no bound; a single cell (own) is certainly beyond where its
+// magnitude is by more than the error.
+template <int K> APO_CERT void sincosx(X<K> d, X<K> &s, X<K> &c, bool own) {
+    if (K && own && mag2(d.lo, d.hi) - 2.f * d.e > 1.f) {
+        s.lo = c.lo = -1.f;
+        s.hi = c.hi = 1.f;
+        s.e = c.e = 0.f;
+        return;
+    }
     const X<K> y = sqr(d);
     const float c6 = (float)(1.0 / 6);
     X<K> S;
@@ -280,7 +288,7 @@ template <int K> APO_CERT PreX<K> prefix(const CellX<K> &c, const HitX<K> &h) {
 // products, but then a voting loop outgrows the instruction cache (level 0 of 1024 events, FP32:
 // 41.3 ms with three copies).
 template <int K>
-APO_CERT void tail(const PreX<K> &p, X<K> L, const HitX<K> &h, X<K> R, X<K> W, X<K> &Gp, X<K> &Gm) {
+APO_CERT void tail(const PreX<K> &p, X<K> L, const HitX<K> &h, X<K> R, X<K> W, X<K> &Gp, X<K> &Gm, bool own = false) {
     const X<K> L2 = sqr(L), Lt = muls<0>(L, h.t);
     const X<K> de = add(mul(p.A1, Lt), mul_nn(p.A2, L2));
     const X<K> NL = add(p.N, mul_pp(L2, add1(p.N, 1.f)));
@@ -290,9 +298,10 @@ APO_CERT void tail(const PreX<K> &p, X<K> L, const HitX<K> &h, X<K> R, X<K> W, X
     dh.lo = fminf(dP.lo, dM.lo);
     dh.hi = fmaxf(dP.hi, dM.hi);
     dh.e = K ? dP.e + (dM.e - dM.e) + fmaxf(dM.e - dP.e, 0.f) : 0.f;   // the larger; NaN / inf kept
-    sincosx(dh, sd, cd);
-    const X<K> sP = clamp1(add(mul_nn(p.sPA, cd), mul(p.cPA, sd)));    // cos(delta) > 0
-    const X<K> cP = clamp1(sub(mul_nn(p.cPA, cd), mul(p.sPA, sd)));
+    sincosx(dh, sd, cd, own);
+    // cos(delta) > 0 for |delta| <= 1, as where only bare end points are evaluated
+    const X<K> sP = clamp1(add(K ? mul(p.sPA, cd) : mul_nn(p.sPA, cd), mul(p.cPA, sd)));
+    const X<K> cP = clamp1(sub(K ? mul(p.cPA, cd) : mul_nn(p.cPA, cd), mul(p.sPA, sd)));
     const X<K> u2 = add(add(add1(mul(sP, scl(Lt, 2.f)), 1.f), muls<1>(L2, h.t2)), muls<1>(sqr(cP), h.t2));
     const X<K> Q = mul_pp(h.d, recip(sqrtx(u2)));
     const X<K> cz = mul_nn(cP, muls<1>(Q, p.tt));                      // t (cos Phi) t q
@@ -323,12 +332,13 @@ template <int K> APO_CERT int decide(X<K> Gp, X<K> Gm, float e) {
     return ((Gp.lo > e || Gp.hi < -e) && (Gm.lo > e || Gm.hi < -e)) ? kNo : kUnknown;
 }
 
-// One evaluation with errors: the cell's own G and direction quantity
+// One evaluation: the cell's G and direction quantity.  own: a single cell, not a box of cells whose
+// bound is wanted
 template <int K> struct Eval { X<K> Gp, Gm, wt; };
-template <int K> APO_CERT Eval<K> eval(const CellX<K> &c, const HitX<K> &h) {
+template <int K> APO_CERT Eval<K> eval(const CellX<K> &c, const HitX<K> &h, bool own = false) {
     Eval<K> r;
     const PreX<K> p = prefix(c, h);
-    tail(p, c.L, h, recip(c.W), c.W, r.Gp, r.Gm);
+    tail(p, c.L, h, recip(c.W), c.W, r.Gp, r.Gm, own);
     r.wt = p.wt;
     return r;
 }

@@ -34,6 +34,15 @@ template <int K> static void load(const double *c, const double *h, CellX<K> &cc
     for (int i = 0; i < 8; i++) s[i] = sc<K>((mir && (i == 1 || i == 3 || i == 6)) ? -down(h[i]) : down(h[i]));
     hh.d = point(sc<K>(down(h[8])));
 }
+template <int K> static int one(const double *c, const double *h, int og) {
+    CellX<K> cc; HitX<K> hh;
+    load(c, h, cc, hh);
+    const Eval<K> r = eval(cc, hh, true);
+    return verdict(r, og != 0, bound(r));
+}
+extern "C" int single(int k, const double *c, const double *h, int og) {
+    return k == 64 ? one<64>(c, h, og) : one<32>(c, h, og);
+}
 template <int K> static float par(const double *c, const double *h, int og, int *no) {
     CellX<K> cc; HitX<K> hh;
     load(c, h, cc, hh);
@@ -90,7 +99,7 @@ def test_bounds_and_decisions(lib, bins, levels, k, og):
     rng = np.random.default_rng(sum(bins) + k)
     ev = chamber.single_track_events(6, seed=17, w=w)
     prec = (0 if k == 64 else 1) | (O.OUTGOING if og else 0)
-    decided = undecided = 0
+    decided = undecided = alone = far = 0
     for n in range(500):
         e = int(rng.integers(ev.n_events))
         i = int(rng.integers(ev.offsets[e], ev.offsets[e + 1]))
@@ -130,7 +139,13 @@ def test_bounds_and_decisions(lib, bins, levels, k, og):
             assert d == 2 or d == v
             decided += d != 2
             undecided += d == 2
-    assert decided > 20 * undecided
+            d = lib.single(k, _p(c), _p(h), og)   # by its own bound, |delta| > 1 included
+            assert d == 2 or d == v
+            far += abs(ref[5:]).max() > 1.0 and d != 2
+            alone += d == 2
+    assert decided > 20 * undecided and undecided >= alone
+    if bins == [5, 6, 6, 5, 5] and not og:
+        assert far > 0
 
 
 def test_nothing_is_decided_at_a_guard_or_overflow(lib):
