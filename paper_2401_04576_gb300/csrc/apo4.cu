@@ -167,7 +167,7 @@ __device__ __forceinline__ double mid4(double a, double b) { return __dmul_rn(__
 // validity and writes zero votes for the columns that fail.  Then its threads take the groups of
 // 2 x 2 x 2 columns with a passing one, 16 groups at a time, a column each: every active hit
 // over the column's z0 voxels and both signs of tan(lambda), with vote counters bit-sliced over
-// the z0 voxels.
+// the z0 voxels; a warp (four groups) works by itself.
 //
 // The votes (of the program in T) are decided by certified FP32 values (cert4.cuh).  Per (group,
 // hit) one evaluation with errors over the group's columns and z0 voxels gives the bound that all
@@ -372,7 +372,7 @@ k4_vote(const __grid_constant__ Iter4 it, int ev0, const int32_t *n_hits, const 
                 }
                 return make_float2(l, h);
             };
-            __syncthreads();   // the last groups' bounds have been read
+            __syncwarp();   // the last groups' bounds have been read
 #pragma unroll
             for (int i = 0; i < 8; i++) {
                 const float2 r = hull8(src[i].v, src[i].v);
@@ -397,9 +397,10 @@ k4_vote(const __grid_constant__ Iter4 it, int ev0, const int32_t *n_hits, const 
         int nq = 0;
         for (int j0 = 0; j0 < na; j0 += k4Chunk) {
             const int nc = na - j0 < k4Chunk ? na - j0 : k4Chunk;
-            __syncthreads();
-            for (int i = tid; i < ns * nc; i += k4Threads) {
-                const int sl = i / nc, j = i - sl * nc;
+            __syncwarp();
+            for (int i = lane; i < 4 * nc; i += 32) {   // the warp's own four groups
+                const int sl = (tid >> 5) * 4 + i / nc, j = i % nc;
+                if (sl >= ns) continue;
                 cert::Bound4 f0 = group_bound<K>(s_g + sl, s_zc[0], s_zc[nz - 1], s_z[0].x, s_z[nz - 1].y, s_h + j0 + j), f1 = f0;
                 if (!(f0.e < 1e30f) && nz > 1) {
                     f0 = group_bound<K>(s_g + sl, s_zc[0], s_zc[half - 1], s_z[0].x, s_z[half - 1].y, s_h + j0 + j);
@@ -409,7 +410,7 @@ k4_vote(const __grid_constant__ Iter4 it, int ev0, const int32_t *n_hits, const 
                 s_e1[sl][j] = f1.e;
                 s_eps[sl][j] = fmaxf(f0.eps, f1.eps);
             }
-            __syncthreads();
+            __syncwarp();
             for (int j = 0; j < nc; j++) {
                 uint32_t b0 = 0, b1 = 0, u0 = 0, u1 = 0;
                 if (has && guard) {
