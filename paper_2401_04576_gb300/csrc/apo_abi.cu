@@ -70,7 +70,7 @@ namespace {
 // Workspace regions for a batch of n_events.
 struct Layout {
     size_t status, n_hits, hd, hf, votes, hist, fk, fv, ck, cv, mask, done, ntr, tune_tracks;
-    size_t ms_front, ms_count, ms_stop, ms_ck, ms_cv, ms_ts, ms_tcnt, p_votes, p_hist, p_next, cand_k, cand_v,
+    size_t ms_front, ms_count, ms_stop, ms_ck, ms_cv, ms_hist, ms_keep, ms_thist, ms_ts, ms_tcnt, p_votes, p_hist, p_next, cand_k, cand_v,
         end;
     int chunk, ms_chunk;
 };
@@ -83,6 +83,12 @@ int maxset_chunk(const Layout &L, int max_keep) {
     if (c < 1) c = 1;
     if (c > L.chunk) c = L.chunk;
     return (int)c;
+}
+
+// Tiles of the largest level the max-set selection sees.
+size_t maxset_event_tiles(const apo_geometry *g, int max_keep) {
+    const long long cells = (long long)max_keep * 32;
+    return (size_t)maxset_tiles(cells > g->n_coarse ? cells : g->n_coarse);
 }
 
 Layout layout(const apo_geometry *g, int n_events, const apo_solve_opts *opts = nullptr) {
@@ -117,7 +123,7 @@ Layout layout(const apo_geometry *g, int n_events, const apo_solve_opts *opts = 
     L.ntr = o; o = align256(o + sizeof(int32_t) * (size_t)n_events);
     L.tune_tracks = o; o = align256(o + sizeof(apo_track) * (size_t)n_events * APO_MAX_TRACKS);
     L.ms_chunk = 0;
-    L.ms_front = L.ms_count = L.ms_stop = L.ms_ck = L.ms_cv = L.ms_ts = L.ms_tcnt = o;
+    L.ms_front = L.ms_count = L.ms_stop = L.ms_ck = L.ms_cv = L.ms_hist = L.ms_keep = L.ms_thist = L.ms_ts = L.ms_tcnt = o;
     L.p_votes = L.p_hist = L.p_next = o;
     if (opts && opts->schedule == APO_SCHED_TOPK && opts->tune.persistent) {
         const size_t B = (size_t)(g->persist_blocks > 0 ? g->persist_blocks : 1);
@@ -134,6 +140,9 @@ Layout layout(const apo_geometry *g, int n_events, const apo_solve_opts *opts = 
         L.ms_stop = o; o = align256(o + sizeof(int32_t) * (size_t)c);
         L.ms_ck = o; o = align256(o + sizeof(uint64_t) * (size_t)c * K * 32);
         L.ms_cv = o; o = align256(o + sizeof(int32_t) * (size_t)c * K * 32);
+        L.ms_hist = o; o = align256(o + sizeof(uint32_t) * (size_t)c * kHistBins);
+        L.ms_keep = o; o = align256(o + sizeof(int32_t) * 2 * (size_t)c);   // keep_from and cells
+        L.ms_thist = o; o = align256(o + sizeof(uint16_t) * (size_t)c * maxset_event_tiles(g, opts->max_keep) * kHistBins);
         if (opts->max_tracks > 1) {   // the multi-track rounds' track step
             L.ms_ts = o; o = align256(o + sizeof(TrackStep) * (size_t)c);
             L.ms_tcnt = o; o = align256(o + maxset_smem_bytes(g->dg) * (size_t)c);
@@ -545,6 +554,12 @@ int enqueue_maxset(const apo_geometry *g, const apo_hits *hits, const apo_solve_
         A.n_coarse = g->n_coarse;
         A.front = front;
         A.count_out = count;
+        A.hist = at<uint32_t>(ws, L.ms_hist);
+        A.keep_from = at<int32_t>(ws, L.ms_keep);
+        A.cells = A.keep_from + n;
+        A.tile_hist = at<uint16_t>(ws, L.ms_thist);
+        A.tiles = (int)maxset_event_tiles(g, K);
+        CU(cudaMemsetAsync(A.hist, 0, sizeof(uint32_t) * (size_t)n * kHistBins, s));
         A.stop = stop;
         A.n_hits = nhe;
         A.tracks = tracks_out + (size_t)e0 * mt;

@@ -187,7 +187,17 @@ struct MaxsetArgs {
     TrackStep *ts;
     uint32_t *tcnt;
     int cnt_stride;
+    // selection scratch: per event the level's histogram (kHistBins, zero between uses), the votes a
+    // cell needs to be kept (INT_MAX: none is), and per tile of kMaxsetTile cells its own histogram
+    // (`tiles` of them per event); cells_in: count_in as it was before the selection
+    uint32_t *hist;
+    int32_t *keep_from;
+    uint16_t *tile_hist;
+    int tiles;
+    int32_t *cells;
 };
+constexpr int kMaxsetTile = 4096;
+__host__ __device__ inline long long maxset_tiles(long long cells) { return (cells + kMaxsetTile - 1) / kMaxsetTile; }
 // Persistent batch search (kernels.cu): the top-K schedule with multi-track rounds, every
 // event's whole search in one block, blocks pulling events from next_event (zeroed by the
 // host).  mode[L]: the votes of level L (FP32 or FP64).

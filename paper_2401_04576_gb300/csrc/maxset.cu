@@ -3,12 +3,16 @@
 // them, T >= vmax - slack; when even the vmax group does not fit, or at the last level, the
 // search ends and the estimate is taken over that level's vmax group.
 //
-// One block per event.  Pass 1 builds the histogram of vote counts (257 bins) in shared
-// memory; thread 0 picks T.  Pass 2 is an order-preserving compaction of the kept cells
-// into the frontier (4096-cell tiles, block scan), or, at the end, per-axis counters of the
-// vmax group's cell indices, from which one warp per axis sums count x centre in ascending
-// index order: the mean of the group's cell centres with a summation order fixed by the
-// indices, so the result does not depend on the order the cells arrive in.
+// Three launches.  k_maxset_hist: a block per 4096 cells counts their votes (257 bins), adds them to
+// the event's histogram and keeps the tile's own.  k_maxset_select, one block per event, picks T
+// from the histogram, or ends the search.  k_maxset_compact, a block per tile again, writes the kept
+// cells in order to the frontier; its first slot is the sum of the kept counts in the tiles before,
+// from their histograms, so no block waits for another.  At the end of a search, per-axis
+// counters of the vmax group's cell indices (tiles without such a cell are skipped), from which one warp
+// per axis sums count x centre in ascending index order: the mean of the group's cell centres with a
+// summation order fixed by the indices, so the result does not depend on the order the cells arrive
+// in.  One block per event for all of it read every vote twice by itself: 342 us of a 665 us search
+// of one event.
 //
 // Multi-track extraction (max_tracks > 1, one search per round on the hits still active):
 // the final vmax group can hold several tracks' cells (tracks with equal hit counts tie),
@@ -32,7 +36,8 @@ namespace apo {
 namespace {
 
 constexpr int kMsThreads = 1024;
-constexpr int kMsTile = 4 * kMsThreads;
+constexpr int kMsTile = kMaxsetTile;
+constexpr int kMsTileThreads = 256;
 
 // index of the j-th cell of the event at this level: level 0 in linear order, else a key
 __device__ __forceinline__ void cell_index(const DevGeom &g, const uint64_t *keys, long long j, int idx[5]) {
@@ -96,14 +101,39 @@ __device__ __forceinline__ void ordered_estimate(const DevGeom &g, int level, in
     }
 }
 
+// Cells of the event's level (0: nothing to do there).
+__device__ __forceinline__ long long level_cells(const MaxsetArgs &A, int e) {
+    if (A.stop[e] || (A.done && A.done[e]) || A.n_hits[e] < 0) return 0;
+    return A.keys ? 32LL * A.count_in[e] : A.n_coarse;
+}
+
+__global__ void __launch_bounds__(kMsTileThreads)
+k_maxset_hist(const __grid_constant__ MaxsetArgs A) {
+    __shared__ uint32_t hist[kHistBins];
+    const int e = blockIdx.y, tid = threadIdx.x;
+    const long long n = level_cells(A, e), t0 = (long long)blockIdx.x * kMsTile;
+    if (t0 >= n) return;
+    const int32_t *vo = A.votes + (long long)e * A.stride;
+    for (int i = tid; i < kHistBins; i += kMsTileThreads) hist[i] = 0;
+    __syncthreads();
+    const long long t1 = t0 + kMsTile < n ? t0 + kMsTile : n;
+    for (long long j = t0 + tid; j < t1; j += kMsTileThreads) atomicAdd(&hist[clamp_votes(vo[j])], 1u);
+    __syncthreads();
+    uint16_t *th = A.tile_hist + ((long long)e * A.tiles + blockIdx.x) * kHistBins;
+    for (int i = tid; i < kHistBins; i += kMsTileThreads) {
+        th[i] = (uint16_t)hist[i];
+        if (hist[i]) atomicAdd(&A.hist[(long long)e * kHistBins + i], hist[i]);
+    }
+}
+
 __global__ void __launch_bounds__(kMsThreads)
 k_maxset_select(const __grid_constant__ DevGeom g, const __grid_constant__ MaxsetArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t *cnt = reinterpret_cast<uint32_t *>(smem);    // per-axis index counters
     __shared__ uint32_t hist[kHistBins];
-    __shared__ int s_warp[32];
     __shared__ int s_T, s_final, s_vmax, s_kept;
     const int e = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if (tid == 0) A.keep_from[e] = INT_MAX;   // nothing to compact, unless set below
     if (A.stop[e]) return;
     const int mt = A.max_tracks;
     if (A.done && A.done[e]) {   // a later round of an event whose extraction has ended
@@ -139,9 +169,11 @@ k_maxset_select(const __grid_constant__ DevGeom g, const __grid_constant__ Maxse
     const long long n = A.keys ? 32LL * A.count_in[e] : A.n_coarse;
     const int32_t *vo = A.votes + (long long)e * A.stride;
     const uint64_t *ke = A.keys ? A.keys + (long long)e * A.stride : nullptr;
-    for (int i = tid; i < kHistBins; i += kMsThreads) hist[i] = 0;
-    __syncthreads();
-    for (long long j = tid; j < n; j += kMsThreads) atomicAdd(&hist[clamp_votes(vo[j])], 1u);
+    const uint16_t *th = A.tile_hist + (long long)e * A.tiles * kHistBins;
+    for (int i = tid; i < kHistBins; i += kMsThreads) {   // zero again for the next level
+        hist[i] = A.hist[(long long)e * kHistBins + i];
+        A.hist[(long long)e * kHistBins + i] = 0u;
+    }
     __syncthreads();
     if (tid == 0) {
         int vmax = 0;
@@ -184,12 +216,15 @@ k_maxset_select(const __grid_constant__ DevGeom g, const __grid_constant__ Maxse
             __syncthreads();
             // the seed: the group's lowest key
             unsigned long long kmin = ~0ull;
-            for (long long j = tid; j < n; j += kMsThreads) {
-                if (clamp_votes(vo[j]) != vmax) continue;
-                int idx[5];
-                cell_index(g, ke, j, idx);
-                const unsigned long long key = pack_key(g, idx);
-                kmin = key < kmin ? key : kmin;
+            for (long long t0 = 0; t0 < n; t0 += kMsTile) {
+                if (!th[t0 / kMsTile * kHistBins + vmax]) continue;
+                for (long long j = t0 + tid; j < t0 + kMsTile && j < n; j += kMsThreads) {
+                    if (clamp_votes(vo[j]) != vmax) continue;
+                    int idx[5];
+                    cell_index(g, ke, j, idx);
+                    const unsigned long long key = pack_key(g, idx);
+                    kmin = key < kmin ? key : kmin;
+                }
             }
             atomicMin(&s_seed, kmin);
             __syncthreads();
@@ -223,12 +258,15 @@ k_maxset_select(const __grid_constant__ DevGeom g, const __grid_constant__ Maxse
         for (int a = 0; a < 5; a++) off[a + 1] = off[a] + (g.bins[a] << A.level);
         for (int i = tid; i < off[5]; i += kMsThreads) cnt[i] = 0;
         __syncthreads();
-        for (long long j = tid; j < n; j += kMsThreads) {
-            if (clamp_votes(vo[j]) != vmax) continue;
-            int idx[5];
-            cell_index(g, ke, j, idx);
+        for (long long t0 = 0; t0 < n; t0 += kMsTile) {
+            if (!th[t0 / kMsTile * kHistBins + vmax]) continue;
+            for (long long j = t0 + tid; j < t0 + kMsTile && j < n; j += kMsThreads) {
+                if (clamp_votes(vo[j]) != vmax) continue;
+                int idx[5];
+                cell_index(g, ke, j, idx);
 #pragma unroll
-            for (int a = 0; a < 5; a++) atomicAdd(&cnt[off[a] + idx[a]], 1u);
+                for (int a = 0; a < 5; a++) atomicAdd(&cnt[off[a] + idx[a]], 1u);
+            }
         }
         __syncthreads();
         ordered_estimate(g, A.level, sh, off, cnt, vmax, kept, A.min_votes, t, wid, lane);
@@ -244,13 +282,44 @@ k_maxset_select(const __grid_constant__ DevGeom g, const __grid_constant__ Maxse
         }
         return;
     }
-    // ---- order-preserving compaction of {votes >= T} ----
+    if (tid == 0) {   // {votes >= T} goes to the frontier
+        A.keep_from[e] = T;
+        A.cells[e] = (int)n;
+        A.count_out[e] = kept;
+        if (A.trace_count) A.trace_count[(long long)e * (A.levels + 1) + A.level] = kept;
+    }
+}
+
+// The cells with votes >= keep_from, in order: a tile's cells follow those of the tiles before it.
+__global__ void __launch_bounds__(kMsTileThreads)
+k_maxset_compact(const __grid_constant__ DevGeom g, const __grid_constant__ MaxsetArgs A) {
+    __shared__ int s_base, s_here, s_warp[kMsTileThreads / 32];
+    const int e = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, tile = blockIdx.x;
+    const int T = A.keep_from[e];
+    if (T == INT_MAX) return;
+    const long long n = A.cells[e], t0 = (long long)tile * kMsTile;
+    if (t0 >= n) return;
+    if (tid == 0) s_base = s_here = 0;
+    __syncthreads();
+    const uint16_t *th = A.tile_hist + (long long)e * A.tiles * kHistBins;
+    int c = 0;   // this tile's kept cells, then those of the tiles before
+    for (int v = T + tid; v < kHistBins; v += kMsTileThreads) c += th[(long long)tile * kHistBins + v];
+    if (c) atomicAdd(&s_here, c);
+    __syncthreads();
+    if (!s_here) return;
+    c = 0;
+    for (int i = tid; i < tile * 32; i += kMsTileThreads)   // 32 threads a tile: its bins T, T + 32, ...
+        for (int v = T + (i & 31); v < kHistBins; v += 32) c += th[(long long)(i >> 5) * kHistBins + v];
+    if (c) atomicAdd(&s_base, c);
+    __syncthreads();
+    const int32_t *vo = A.votes + (long long)e * A.stride;
+    const uint64_t *ke = A.keys ? A.keys + (long long)e * A.stride : nullptr;
     uint64_t *fe = A.front + (long long)e * A.max_keep;
     uint64_t *tk = A.trace_keys ? A.trace_keys + ((long long)e * (A.levels + 1) + A.level) * A.max_keep : nullptr;
     int32_t *tv = A.trace_votes ? A.trace_votes + ((long long)e * (A.levels + 1) + A.level) * A.max_keep : nullptr;
-    int run = 0;
-    for (long long t0 = 0; t0 < n && run < kept; t0 += kMsTile) {
-        const long long j0 = t0 + 4LL * tid;
+    int run = s_base;
+    for (long long q0 = t0; q0 < t0 + kMsTile && q0 < n; q0 += 4 * kMsTileThreads) {
+        const long long j0 = q0 + 4LL * tid;
         int v[4], x = 0;
 #pragma unroll
         for (int r = 0; r < 4; r++) {
@@ -266,19 +335,16 @@ k_maxset_select(const __grid_constant__ DevGeom g, const __grid_constant__ Maxse
         }
         if (lane == 31) s_warp[wid] = inc;
         __syncthreads();
-        const int w = s_warp[lane];
-        int winc = w;
+        int pre = 0, total = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, winc, o);
-            if (lane >= o) winc += y;
+        for (int w = 0; w < kMsTileThreads / 32; w++) {
+            if (w < wid) pre += s_warp[w];
+            total += s_warp[w];
         }
-        const int wpre = __shfl_sync(0xffffffffu, winc - w, wid);
-        const int total = __shfl_sync(0xffffffffu, winc, 31);
-        int pos = run + wpre + inc - x;
+        int pos = run + pre + inc - x;
 #pragma unroll
         for (int r = 0; r < 4; r++) {
-            if (v[r] < T) continue;
+            if (v[r] < T || pos >= A.max_keep) continue;
             int idx[5];
             cell_index(g, ke, j0 + r, idx);
             const uint64_t key = pack_key(g, idx);
@@ -288,11 +354,7 @@ k_maxset_select(const __grid_constant__ DevGeom g, const __grid_constant__ Maxse
             pos++;
         }
         run += total;
-        __syncthreads();   // s_warp is rewritten by the next scanned tile
-    }
-    if (tid == 0) {
-        A.count_out[e] = kept;
-        if (A.trace_count) A.trace_count[(long long)e * (A.levels + 1) + A.level] = kept;
+        __syncthreads();   // s_warp is rewritten by the next cells
     }
 }
 
@@ -453,7 +515,10 @@ void init_maxset_attributes() {
 
 void launch_maxset_select(const DevGeom &g, int n_ev, const MaxsetArgs &A, cudaStream_t s) {
     if (n_ev <= 0) return;
+    const dim3 grid((unsigned)maxset_tiles(A.keys ? A.stride : A.n_coarse), n_ev);
+    k_maxset_hist<<<grid, kMsTileThreads, 0, s>>>(A);
     k_maxset_select<<<n_ev, kMsThreads, maxset_smem_bytes(g), s>>>(g, A);
+    if (A.level < A.levels) k_maxset_compact<<<grid, kMsTileThreads, 0, s>>>(g, A);
 }
 
 void launch_track_step(const DevGeom &g, int n_ev, const MaxsetArgs &A, cudaStream_t s) {
