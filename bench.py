@@ -51,9 +51,11 @@ COARSE_F64_DRAM_BYTES_PER_EVENT = 496384 / 64
 
 
 def coarse_kernel_ops(n_parent: int, n_prefix: int, n_tail: int) -> int:
-    """Algorithmic directed FP operations of the coarse vote kernel from its work counters:
-    parent-cell tests are full evaluations, each (cell, hit) prefix and each tan(lambda)
-    tail as counted."""
+    """Algorithmic end-point operations of the coarse vote kernel from its work counters:
+    tests of boxes (tiles, and their tan(lambda) bins) are full evaluations, each (cell, hit)
+    prefix and each tan(lambda) tail as counted.  One operation is one end point of an interval
+    operation of the vote program; the kernel decides in FP32, where a general product's end
+    point takes two to four products and minima."""
     return n_parent * OPS_FULL + n_prefix * OPS_PREFIX + n_tail * OPS_TAIL
 
 
@@ -755,9 +757,7 @@ def run_apo(args) -> None:
     value = pairs * world / (t_step * 1e-3)
 
     tracks64 = apo.tracks_to_numpy(tracks, ev.n_events).copy()
-    # the same FP64 search with the knobs apo_autotune picks (the FP32-first filter on the
-    # coarse grid gives the same FP64 votes): reported beside the headline, whose roofline
-    # stays the plain FP64 kernel's
+    # the same FP64 search with the knobs apo_autotune picks: reported beside the headline
     tune64, _ = apo.autotune(geom, apo.DeviceHits.from_events(ev.subset(range(256))), opts64)
     ms64t = timed(apo.solve_opts(precision=[apo.F64] * (lv + 1), tune=tune64), max(2, args.steps), 1)
     t64t = reduce_max(sum(ms64t) / len(ms64t), world)
@@ -778,7 +778,7 @@ def run_apo(args) -> None:
     rec32 = truth_recovery(g, np.full(ev.n_events, lv), tracks32["p"][:, 0, :],
                            tracks32["w"][:, 0, :], truth)
 
-    # roofline of the dominant kernel (coarse vote, in the form the search runs: each block
+    # roofline of the dominant kernel (coarse vote, in the form the search runs: each tile
     # keeps its K best cells): counted work / live launch time
     votes = apo.vote(geom, hits, precision=apo.F64, workspace=ws, stream=stream)
     votes32 = apo.vote(geom, hits, precision=apo.F32, workspace=ws, stream=stream)
@@ -796,7 +796,7 @@ def run_apo(args) -> None:
         return [int(x) for x in c.cpu().tolist()]
 
     def coarse_launch_ms(prec, n_launch, reps, full=None):
-        # full: a vote array for the full-vote form; None: each block keeps its K best cells
+        # full: a vote array for the full-vote form; None: each tile keeps its K best cells
         out = []
         for _ in range(reps):
             flush.fill_(1)
@@ -810,44 +810,40 @@ def run_apo(args) -> None:
             out.append(s0.elapsed_time(s1) / max(n_launch, 1))
         return statistics.mean(out)
 
-    n_par, n_pre, n_tail, n_launch, p32, q32, t32c, _ = coarse_counts(apo.F64)
+    n_und, _, _, n_launch, p32, q32, t32c, _ = coarse_counts(apo.F64)
     c32 = coarse_counts(apo.F32)
-    # the FP32 coarse kernel (dominant in the FP32-bulk solve): counted FP32 directed
-    # operations / live launch time, against the measured FP32 directed add/mul rate
+    # Both coarse kernels decide in FP32 (certified end points): counted end-point operations /
+    # live launch time, against the measured FP32 directed add/mul rate.  The pairs left to the
+    # FP64 (or outward FP32) program are counted beside them.
     ops32_coarse = coarse_kernel_ops(c32[4], c32[5], c32[6]) / max(c32[3], 1)
-    # in the form the tuned FP32-bulk step runs (full votes or per-block candidates)
+    # in the form the tuned FP32-bulk step runs (full votes or per-tile candidates)
     full32 = bool(tune32.coarse_full)
     k32_ms = coarse_launch_ms(apo.F32, c32[3], max(3, args.steps), full=votes if full32 else None)
     peak32 = apo.pipe_peak(apo.F32)
-    roofline32 = {"bound": "issue", "kernel": "k_vote_coarse<float>",
-                  "form": "full votes" if full32 else "per-block K best cells",
+    peak_source = ("measured: libapo directed-rounding FP32 add/mul microbenchmark "
+                   "(apo_diag_pipe_peak) on this GPU, this run")
+    roofline32 = {"bound": "issue", "kernel": "k_vote_coarse<32>",
+                  "form": "full votes" if full32 else "per-tile K best cells",
                   "achieved": ops32_coarse / (k32_ms * 1e-3) / 1e12, "peak": peak32 / 1e12,
                   "unit": "TFLOP/s", "frac": ops32_coarse / (k32_ms * 1e-3) / peak32,
                   "launch_ms": k32_ms, "ops_per_launch": ops32_coarse,
-                  "peak_source": "measured: libapo directed-rounding FP32 add/mul microbenchmark "
-                                 "(apo_diag_pipe_peak) on this GPU, this run",
-                  "work": {"fp32_parent": c32[4], "fp32_prefix": c32[5], "fp32_tail": c32[6],
+                  "peak_source": peak_source,
+                  "work": {"undecided_pairs": c32[0], "boxes": c32[4], "prefixes": c32[5], "tails": c32[6],
                            "launches": c32[3]}}
-    ops_launch = coarse_kernel_ops(n_par, n_pre, n_tail) / max(n_launch, 1)
-    ops32_launch = coarse_kernel_ops(p32, q32, t32c) / max(n_launch, 1)
+    ops_launch = coarse_kernel_ops(p32, q32, t32c) / max(n_launch, 1)
     k_ms = coarse_launch_ms(apo.F64, n_launch, max(2, args.steps))
-    peak = apo.pipe_peak(apo.F64)
     achieved = ops_launch / (k_ms * 1e-3)
     ev_per_launch = ev.n_events / max(n_launch, 1)
     traffic = (None if COARSE_F64_DRAM_BYTES_PER_EVENT is None
                else COARSE_F64_DRAM_BYTES_PER_EVENT * ev_per_launch)
-    roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12,
-                "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic,
+    roofline = {"bound": "issue", "achieved": achieved / 1e12, "peak": peak32 / 1e12,
+                "unit": "TFLOP/s", "frac": achieved / peak32, "traffic": traffic,
                 "traffic_source": "ncu dram__bytes_read+write of a 64-event launch, scaled by "
                                   "events to this launch",
-                "kernel": "k_vote_coarse<double>",
-                "peak_source": "measured: libapo directed-rounding FP64 add/mul microbenchmark "
-                               "(apo_diag_pipe_peak) on this GPU, this run",
+                "kernel": "k_vote_coarse<64>",
+                "peak_source": peak_source,
                 "ops_per_launch": ops_launch, "launch_ms": k_ms,
-                "fp32_filter_ops_per_launch": ops32_launch,
-                "fp32_filter_tflops": ops32_launch / (k_ms * 1e-3) / 1e12,
-                "work": {"fp64_parent": n_par, "fp64_prefix": n_pre, "fp64_tail": n_tail,
-                         "fp32_parent": p32, "fp32_prefix": q32, "fp32_tail": t32c,
+                "work": {"undecided_pairs": n_und, "boxes": p32, "prefixes": q32, "tails": t32c,
                          "launches": n_launch}}
 
     # midpoint form (Section 3.1: the quantities of d^Ax at the voxel centre): coarse launch
@@ -983,8 +979,8 @@ def run_apo(args) -> None:
                           "decides most of them without evaluating the pair: the exact "
                           "parent-cell test and the shared tan(lambda)-free prefix",
                   "coarse_decided_per_step": float(np.sum(nh)) * geom.n_coarse,
-                  "coarse_tails_evaluated_per_step": float(n_tail),
-                  "coarse_prefixes_evaluated_per_step": float(n_pre),
+                  "coarse_tails_evaluated_per_step": float(t32c),
+                  "coarse_prefixes_evaluated_per_step": float(q32),
                   "refine_evaluated_per_step": float(np.sum(nh)) * lv * g.topk * 32},
         "truth_recovery": rec64,
         "fp64_autotuned": {"ms_per_step": t64t, "value": pairs * world / (t64t * 1e-3),

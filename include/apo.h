@@ -46,9 +46,8 @@ typedef enum {
 } apo_status;
 
 /* interval precision of one level.  APO_F64: FP64 intervals.  APO_F32: FP32 intervals.
- * APO_F64_FILTERED: FP64 intervals evaluated only where the FP32 program votes first (FP32
- * intervals contain the FP64 ones, so the votes are exactly APO_F64's; it pays only where
- * most FP32 votes are "no").
+ * APO_F64_FILTERED: the votes of APO_F64 (kept for callers of the earlier FP32-first filter;
+ * APO_F64 itself decides nearly every pair in FP32, by certified end points).
  * APO_F64_MID: the midpoint form of Section 3.1 (last paragraph): the quantities that build
  * d^Ax (Eq. defdiAX_b) are evaluated at the voxel centre in round-to-nearest FP64, and only
  * (x^Ax - x_c)^2 + (y^Ax - y_c)^2 - (R + d^Ax)^2 keeps the voxel's FP64 intervals.  Faster
@@ -141,14 +140,13 @@ typedef struct {
  * evaluates the same interval program cell by cell); apo_autotune picks them by timing.
  * Zero means the default. */
 typedef struct {
-    int32_t coarse_filter;   /* 1: on the level-0 grid, evaluate FP64 levels only where the
-                                FP32 program votes (as APO_F64_FILTERED) */
+    int32_t coarse_filter;   /* 1: FP64 level 0 as APO_F64_FILTERED (the same kernel) */
     int32_t cells_filter;    /* 1: the same for the bisected cells of levels >= 1 */
-    int32_t cells_block;     /* threads per block of the cell-voting kernel: 128 or 256 */
+    int32_t cells_block;     /* threads per block of APO_F64_EXACT's bisected cells: 128 or 256 */
     int32_t chunk_events;    /* events per level-0 launch (at most the workspace's chunk) */
     int32_t coarse_full;     /* 1 (APO_SCHED_TOPK): level 0 writes every cell's vote and selects
-                                from them, instead of each block keeping its topk best cells
-                                (more workspace, fewer instructions per block); the same
+                                from them, instead of each tile keeping its topk best cells
+                                (more workspace, fewer instructions per tile); the same
                                 kept set either way */
     int32_t persistent;      /* 1 (APO_SCHED_TOPK only): one persistent launch for the whole
                                 batch; each block pulls the next event from a device counter
@@ -262,8 +260,8 @@ int apo_solve_batch(const apo_geometry *geom, const apo_hits *hits, const apo_so
 /* Times apo_solve_batch on `hits` (typically a sample of the batch to come) for every
  * combination of the apo_tune knobs and writes the fastest to *best (its time to *best_ms,
  * may be NULL): the launch schedule (per-level launches, or the persistent launch when
- * the options allow it), the FP32-first filters, the threads per block of the bisected
- * cells' kernel and the events per level-0 launch.  opts: as for apo_solve_batch (its tune and use_graph are ignored).
+ * the options allow it), level 0's full votes or K best cells, the threads per block of the
+ * bisected cells' kernel and the events per level-0 launch.  opts: as for apo_solve_batch (its tune and use_graph are ignored).
  * Workspace as for apo_solve_batch.  Synchronous. */
 int apo_autotune(const apo_geometry *geom, const apo_hits *hits, const apo_solve_opts *opts,
                  void *workspace, size_t workspace_bytes, void *stream, apo_tune *best,

@@ -14,13 +14,14 @@ extern "C" {
 #endif
 
 /* apo_vote on the full level-0 grid that also counts the work the coarse kernel does
- * (votes_out NULL: the form apo_solve_batch runs, each coarse block keeping only its topk
+ * (votes_out NULL: the form apo_solve_batch runs, each tile keeping only its topk
  * best cells in the workspace, instead of writing every vote; counts_out NULL: no counting,
  * the kernel exactly as the search runs it):
- * counts_out (device, 8 x uint64, zeroed by the call) receives FP64 parent-cell
- * evaluations, FP64 per-(cell, hit) prefix evaluations, FP64 tan(lambda) tail evaluations,
- * the number of coarse-kernel launches, then the same three FP32 counts.  For APO_F64_MID
- * slots 1 and 2 count the midpoint form's per-(cell, hit) prefixes and tan(lambda) tails. */
+ * counts_out (device, 8 x uint64, zeroed by the call) receives, in slot 0, the (cell, hit) pairs
+ * that the certified FP32 values left undecided; in slot 3 the number of coarse-kernel launches;
+ * in slots 4-6 the evaluations on boxes of cells (tiles, and their tan(lambda) bins), the per-(cell,
+ * hit) prefixes and the tan(lambda) tails.  APO_F64_EXACT, evaluated in FP64 throughout: parent
+ * evaluations, prefixes and tails in slots 0-2. */
 int apo_diag_vote_coarse_counts(const apo_geometry *geom, const apo_hits *hits, int32_t precision,
                                 int32_t *votes_out, unsigned long long *counts_out,
                                 void *workspace, size_t workspace_bytes, void *stream);

@@ -846,14 +846,12 @@ int apo_autotune(const apo_geometry *g, const apo_hits *hits, const apo_solve_op
     }
     for (int full = 0; full < 2; full++)
     for (int ps = 0; ps < 2; ps++)
-    for (int cf = 0; cf < 2; cf++)
-        for (int lf = 0; lf < 2; lf++)
             for (int bs = 0; bs < 2; bs++)
                 for (int ch = 0; ch < 2; ch++) {
                     if (ch == 1 && chunks[1] == 0) continue;
                     if (ps == 1 && (!try_persistent || bs == 1 || ch == 1 || full == 1)) continue;
                     if (full == 1 && o.schedule != APO_SCHED_TOPK) continue;
-                    apo_tune t{cf, lf, bs ? 128 : 256, chunks[ch], full, ps};
+                    apo_tune t{0, 1, bs ? 128 : 256, chunks[ch], full, ps};   // the filters run the same kernels
                     o.tune = t;
                     if (layout(g, hits->n_events, &o).end > ws_bytes) continue;   // needs more workspace
                     float ms = 0.f;

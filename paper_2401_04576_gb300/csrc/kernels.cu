@@ -488,6 +488,7 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan 
             const float2 L = K == kMid ? make_float2(Ls[l].x, Ls[l].x) : Ls[l];   // its centre: a point
             if (!(y >> 15)) {
                 if (!box_refuses<K>(box_s + tl, L, rec, err_s[x], outgoing)) atomicOr(&bins_s[x], 1u << l);
+                cnt[3]++;
             } else {
                 CertBox b = box_s[tl];
                 b.v[5] = L;
