@@ -712,26 +712,28 @@ int enqueue_solve(const apo_geometry *g, const apo_hits *hits, const apo_solve_o
         // one round per track: search the active hits, record, mask the track's hits
         for (int round = 0; round < o->max_tracks; round++) {
             NvtxRange range_round("apo search round");
+            const int32_t *skip = round ? done : nullptr;   // events whose extraction has ended
             CU(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (size_t)n * kHistBins, s));
             if (prec_at(0) == APO_F64_MID || o->tune.coarse_full) {   // every cell's vote, then the selection
-                launch_vote_coarse(gl[0], prec_at(0), e0, n, hd, hf, nh, votes, hist, status, s, nullptr, active);
+                launch_vote_coarse(gl[0], prec_at(0), e0, n, hd, hf, nh, votes, hist, status, s, nullptr, active, nullptr,
+                                   nullptr, 0, skip);
                 if ((rc = check_launch("vote_coarse"))) return rc;
-                launch_select_coarse(g->dg, e0, n, votes, hist, K, fk, fv, s);
+                launch_select_coarse(g->dg, e0, n, votes, hist, K, fk, fv, s, skip);
                 if ((rc = check_launch("select_coarse"))) return rc;
             } else {   // each block's K best cells, then the selection among them
                 launch_vote_coarse(gl[0], prec_at(0), e0, n, hd, hf, nh, nullptr, hist, status, s, nullptr, active,
-                                   cand_k, cand_v, K);
+                                   cand_k, cand_v, K, skip);
                 if ((rc = check_launch("vote_coarse"))) return rc;
                 launch_select_candidates(g->dg, e0, n, cand_k, cand_v, coarse_lists(gl[0], prec_at(0)), hist, K,
-                                         fk, fv, s);
+                                         fk, fv, s, skip);
                 if ((rc = check_launch("select_candidates"))) return rc;
             }
             if (round == 0 && (rc = trace_copy(o, g, e0, n, 0, fke, fve, s))) return rc;
             for (int lev = 1; lev <= lv; lev++) {
                 launch_vote_children(gl[lev], prec_at(lev), n, hde, hfe, nhe, lev, fke, K, cke, cve, s, acte,
-                                     block);
+                                     block, nullptr, skip ? skip + e0 : nullptr);
                 if ((rc = check_launch("vote_children"))) return rc;
-                launch_topk(n, cke, cve, K * 32, K, fke, fve, s);
+                launch_topk(n, cke, cve, K * 32, K, fke, fve, s, skip ? skip + e0 : nullptr);
                 if ((rc = check_launch("topk"))) return rc;
                 if (round == 0 && (rc = trace_copy(o, g, e0, n, lev, fke, fve, s))) return rc;
             }

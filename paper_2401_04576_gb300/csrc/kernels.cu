@@ -603,9 +603,10 @@ template <int K>
 __global__ void __launch_bounds__(kCoarseThreads, APO_COARSE_MIN_BLOCKS)
 k_vote_coarse(const __grid_constant__ DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const HitRecF *hf,
               const int32_t *n_hits, const uint32_t *active, int32_t *votes, uint32_t *hist, unsigned *status,
-              unsigned long long *ctr, uint64_t *cand_k, int32_t *cand_v, int Kc) {
+              unsigned long long *ctr, uint64_t *cand_k, int32_t *cand_v, int Kc, const int32_t *skip) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int e = blockIdx.y;
+    if (skip && skip[ev0 + e]) return;
     const long long ncell = (long long)g.bins[0] * g.bins[1] * g.bins[2] * g.bins[3] * g.bins[4];
     // candidates: Kc slots per tile, an event's tiles in order
     const long long co = (long long)e * P.n_tiles * Kc;
@@ -629,9 +630,10 @@ struct ExactSmem {
 __global__ void __launch_bounds__(kCoarseThreads, 3)
 k_vote_coarse_exact(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const int32_t *n_hits, const uint32_t *active,
                     int32_t *votes, uint32_t *hist, unsigned *status, unsigned long long *ctr, uint64_t *cand_k,
-                    int32_t *cand_v, int Kc) {
+                    int32_t *cand_v, int Kc, const int32_t *skip) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int e = blockIdx.y, ev = ev0 + e;
+    if (skip && skip[ev]) return;
     const int part = blockIdx.x % P.parts, pw = blockIdx.x / P.parts;
     const int Bd = g.bins[0], Bz = g.bins[3], Bl = g.bins[4], p = pw % g.bins[1], w = pw / g.bins[1];
     const int ntile = Bd * Bz, nthr = blockDim.x, tid = threadIdx.x;
@@ -755,11 +757,12 @@ k_vote_cells_mid(DevGeom g, const HitRecD *hd, const int32_t *n_hits, const uint
 template <int K> static void launch_coarse_cert(const DevGeom &g, int ev0, int n_ev, const HitRecD *hd,
                                                const HitRecF *hf, const int32_t *n_hits, const uint32_t *active,
                                                int32_t *votes, uint32_t *hist, unsigned *status, cudaStream_t s,
-                                               unsigned long long *ctr, uint64_t *cand_k, int32_t *cand_v, int Kc) {
+                                               unsigned long long *ctr, uint64_t *cand_k, int32_t *cand_v, int Kc,
+                                               const int32_t *skip) {
     const CoarsePlan P = coarse_plan(g, cand_k != nullptr, n_ev);
     dim3 grid((unsigned)((P.n_tiles + P.tiles - 1) / P.tiles), n_ev);
     k_vote_coarse<K><<<grid, kCoarseThreads, CoarseSmem::total(g.bins[4], P), s>>>(
-        g, P, ev0, hd, hf, n_hits, active, votes, hist, status, ctr, cand_k, cand_v, Kc);
+        g, P, ev0, hd, hf, n_hits, active, votes, hist, status, ctr, cand_k, cand_v, Kc, skip);
 }
 
 int coarse_lists(const DevGeom &g, int) { return (int)coarse_plan(g, true, 1).n_tiles; }
@@ -767,18 +770,18 @@ int coarse_lists(const DevGeom &g, int) { return (int)coarse_plan(g, true, 1).n_
 void launch_vote_coarse(const DevGeom &g, int prec, int ev0, int n_ev, const HitRecD *hd,
                         const HitRecF *hf, const int32_t *n_hits, int32_t *votes, uint32_t *hist,
                         unsigned *status, cudaStream_t s, unsigned long long *ctr,
-                        const uint32_t *active, uint64_t *cand_k, int32_t *cand_v, int K) {
+                        const uint32_t *active, uint64_t *cand_k, int32_t *cand_v, int K, const int32_t *skip) {
     if (n_ev <= 0) return;
     if (prec == APO_F64_MID) {
-        launch_coarse_cert<kMid>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K);
+        launch_coarse_cert<kMid>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K, skip);
     } else if (prec == APO_F64_EXACT) {
         const CoarsePlan P = coarse_plan(g, true, 1);
         k_vote_coarse_exact<<<dim3((unsigned)P.n_tiles, n_ev), P.per, ExactSmem::total(g.bins[4]), s>>>(
-            g, P, ev0, hd, n_hits, active, votes, hist, status, ctr, cand_k, cand_v, K);
+            g, P, ev0, hd, n_hits, active, votes, hist, status, ctr, cand_k, cand_v, K, skip);
     } else if (prec == APO_F32) {
-        launch_coarse_cert<32>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K);
+        launch_coarse_cert<32>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K, skip);
     } else {   // APO_F64 and APO_F64_FILTERED: the same votes, the same kernel
-        launch_coarse_cert<64>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K);
+        launch_coarse_cert<64>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K, skip);
     }
 }
 
@@ -1094,9 +1097,10 @@ template <int K>
 __global__ void __launch_bounds__(kChildThreads, APO_CHILD_MIN_BLOCKS)
 k_vote_children(const __grid_constant__ DevGeom g, const HitRecD *hd, const HitRecF *hf, const int32_t *n_hits,
                 const uint32_t *active, int level, const uint64_t *parents, int n_par,
-                const int32_t *n_valid, uint64_t *out_keys, int32_t *out_votes, unsigned *status) {
+                const int32_t *n_valid, uint64_t *out_keys, int32_t *out_votes, unsigned *status, const int32_t *skip) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int ev = blockIdx.y;
+    if (skip && skip[ev]) return;
     // n_valid (may be null): parents 0 .. n_valid[ev] - 1 of the event's n_par slots are
     // real; a block past them has nothing to do (the condition is uniform in the block)
     const long long n_here = n_valid ? (long long)n_valid[ev] : (long long)n_par;
@@ -1124,10 +1128,11 @@ template <int NT>
 __global__ void __launch_bounds__(NT, NT == 128 ? 3 : 1)
 k_vote_children_exact(DevGeom g, const HitRecD *hd, const int32_t *n_hits, const uint32_t *active, int level,
                       const uint64_t *parents, int n_par, const int32_t *n_valid, uint64_t *out_keys,
-                      int32_t *out_votes, unsigned *status) {
+                      int32_t *out_votes, unsigned *status, const int32_t *skip) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kHitCap * 80);
     const int ev = blockIdx.y;
+    if (skip && skip[ev]) return;
     const long long n_here = n_valid ? (long long)n_valid[ev] : (long long)n_par;
     if ((long long)blockIdx.x * blockDim.x >= n_here * 16) return;
     int nh = n_hits[ev];
@@ -1186,37 +1191,37 @@ template <int K>
 static void launch_children_cert(const DevGeom &g, int n_ev, const HitRecD *hd, const HitRecF *hf,
                                  const int32_t *n_hits, const uint32_t *active, int level, const uint64_t *parents,
                                  int n_par, const int32_t *n_valid, uint64_t *out_keys, int32_t *out_votes,
-                                 cudaStream_t s) {
+                                 cudaStream_t s, const int32_t *skip) {
     dim3 grid((unsigned)(((long long)n_par + kChildThreads / 16 - 1) / (kChildThreads / 16)), n_ev);   // two parents a warp
     k_vote_children<K><<<grid, kChildThreads, ChildSmem::total, s>>>(g, hd, hf, n_hits, active, level, parents, n_par,
-                                                                     n_valid, out_keys, out_votes, nullptr);
+                                                                     n_valid, out_keys, out_votes, nullptr, skip);
 }
 
 void launch_vote_children(const DevGeom &g, int prec, int n_ev, const HitRecD *hd,
                           const HitRecF *hf, const int32_t *n_hits, int child_level,
                           const uint64_t *parents, int n_par, uint64_t *child_keys,
                           int32_t *child_votes, cudaStream_t s, const uint32_t *active, int block,
-                          const int32_t *n_valid) {
+                          const int32_t *n_valid, const int32_t *skip) {
     if (n_ev <= 0 || n_par <= 0) return;
     if (block != 128) block = 256;   // of the exact-phase kernel
     if (prec == APO_F64_MID) {
         launch_children_cert<kMid>(g, n_ev, hd, hf, n_hits, active, child_level, parents, n_par, n_valid, child_keys,
-                                   child_votes, s);
+                                   child_votes, s, skip);
     } else if (prec == APO_F64_EXACT) {
         const size_t sm = kHitCap * 80 + 16;
         dim3 grid((unsigned)(((long long)n_par * 16 + block - 1) / block), n_ev);
         if (block == 128)
             k_vote_children_exact<128><<<grid, 128, sm, s>>>(g, hd, n_hits, active, child_level, parents, n_par, n_valid,
-                                                             child_keys, child_votes, nullptr);
+                                                             child_keys, child_votes, nullptr, skip);
         else
             k_vote_children_exact<256><<<grid, 256, sm, s>>>(g, hd, n_hits, active, child_level, parents, n_par, n_valid,
-                                                             child_keys, child_votes, nullptr);
+                                                             child_keys, child_votes, nullptr, skip);
     } else if (prec == APO_F32) {
         launch_children_cert<32>(g, n_ev, hd, hf, n_hits, active, child_level, parents, n_par, n_valid, child_keys,
-                                 child_votes, s);
+                                 child_votes, s, skip);
     } else {   // APO_F64 and APO_F64_FILTERED: the same votes, the same kernel
         launch_children_cert<64>(g, n_ev, hd, hf, n_hits, active, child_level, parents, n_par, n_valid, child_keys,
-                                 child_votes, s);
+                                 child_votes, s, skip);
     }
 }
 
@@ -1337,8 +1342,9 @@ __device__ __forceinline__ void select_coarse_block(const DevGeom &g, const int3
 
 __global__ void __launch_bounds__(kSelThreads)
 k_select_coarse(DevGeom g, int ev0, const int32_t *votes, const uint32_t *hist, int K,
-                uint64_t *out_keys, int32_t *out_votes) {
+                uint64_t *out_keys, int32_t *out_votes, const int32_t *skip) {
     const int e = blockIdx.x, ev = ev0 + e;
+    if (skip && skip[ev]) return;
     const long long n = (long long)g.bins[0] * g.bins[1] * g.bins[2] * g.bins[3] * g.bins[4];
     select_coarse_block(g, votes + (long long)e * n, hist + (long long)e * kHistBins, K,
                         out_keys + (long long)ev * K, out_votes + (long long)ev * K);
@@ -1351,11 +1357,12 @@ k_select_coarse(DevGeom g, int ev0, const int32_t *votes, const uint32_t *hist, 
 // merge: `need` rounds, each taking the smallest head over the lists.
 __global__ void __launch_bounds__(kSelThreads)
 k_select_candidates(int ev0, const uint64_t *cand_k, const int32_t *cand_v, int n_lists,
-                    const uint32_t *hist, int K, uint64_t *out_keys, int32_t *out_votes) {
+                    const uint32_t *hist, int K, uint64_t *out_keys, int32_t *out_votes, const int32_t *skip) {
     extern __shared__ int s_head[];          // n_lists heads
     __shared__ int s_vstar, s_need, s_above, s_nA;
     __shared__ unsigned long long s_red[32];
     const int e = blockIdx.x, ev = ev0 + e, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if (skip && skip[ev]) return;
     const uint64_t *ck = cand_k + (long long)e * n_lists * K;
     const int32_t *cv = cand_v + (long long)e * n_lists * K;
     uint64_t *ok_ = out_keys + (long long)ev * K;
@@ -1421,26 +1428,53 @@ k_select_candidates(int ev0, const uint64_t *cand_k, const int32_t *cand_v, int 
 
 void launch_select_candidates(const DevGeom &, int ev0, int n_ev, const uint64_t *cand_k,
                               const int32_t *cand_v, int n_lists, const uint32_t *hist, int K,
-                              uint64_t *out_keys, int32_t *out_votes, cudaStream_t s) {
+                              uint64_t *out_keys, int32_t *out_votes, cudaStream_t s, const int32_t *skip) {
     if (n_ev <= 0) return;
     k_select_candidates<<<n_ev, kSelThreads, sizeof(int) * (size_t)n_lists, s>>>(
-        ev0, cand_k, cand_v, n_lists, hist, K, out_keys, out_votes);
+        ev0, cand_k, cand_v, n_lists, hist, K, out_keys, out_votes, skip);
 }
 
 void launch_select_coarse(const DevGeom &g, int ev0, int n_ev, const int32_t *votes,
                           const uint32_t *hist, int K, uint64_t *out_keys, int32_t *out_votes,
-                          cudaStream_t s) {
+                          cudaStream_t s, const int32_t *skip) {
     if (n_ev <= 0) return;
-    k_select_coarse<<<n_ev, kSelThreads, 0, s>>>(g, ev0, votes, hist, K, out_keys, out_votes);
+    k_select_coarse<<<n_ev, kSelThreads, 0, s>>>(g, ev0, votes, hist, K, out_keys, out_votes, skip);
 }
 
 // ---------------------------------------------------------------------------------------
 // Per-event bitonic sort of (votes desc, key asc) packed as ((1023 - v) << 50) | key.
 // ---------------------------------------------------------------------------------------
 constexpr int kSortMax = 4096;
+// One warp sorts or merges 64 entries, two a lane, in registers: the bitonic steps of block sizes
+// size0 .. size1 with strides below 64.
+__device__ __forceinline__ void warp_sort64(uint64_t *s, int base, int size0, int size1) {
+    const int lane = threadIdx.x & 31, i = base + lane;
+    uint64_t a = s[i], b = s[i + 32];
+    for (int size = size0; size <= size1; size <<= 1) {
+        const bool ua = (i & size) == 0, ub = ((i + 32) & size) == 0;
+        if (size >= 64 && (a > b) == ua) { const uint64_t x = a; a = b; b = x; }
+        for (int st = size >= 64 ? 16 : size >> 1; st > 0; st >>= 1) {
+            const uint64_t pa = __shfl_xor_sync(0xffffffffu, a, st), pb = __shfl_xor_sync(0xffffffffu, b, st);
+            const bool low = (lane & st) == 0;
+            a = (low == ua) == (pa < a) ? pa : a;
+            b = (low == ub) == (pb < b) ? pb : b;
+        }
+    }
+    s[i] = a;
+    s[i + 32] = b;
+}
+// Ascending bitonic sort by the block (whole warps).  Steps with strides below 64 run in registers,
+// one pass per block size instead of six (2048 entries: 15 passes through shared memory and 6
+// through registers instead of 66).
 __device__ void block_sort(uint64_t *s, int n_pow2) {
-    for (int size = 2; size <= n_pow2; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+    const int wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const bool regs = n_pow2 >= 64;
+    if (regs) {
+        for (int base = 64 * wid; base < n_pow2; base += 64 * nwarps) warp_sort64(s, base, 2, 64);
+        __syncthreads();
+    }
+    for (int size = regs ? 128 : 2; size <= n_pow2; size <<= 1) {
+        for (int stride = size >> 1; stride > (regs ? 32 : 0); stride >>= 1) {
             for (int i = threadIdx.x; i < n_pow2 / 2; i += blockDim.x) {
                 int lo = 2 * i - (i & (stride - 1));
                 int hi = lo + stride;
@@ -1448,6 +1482,10 @@ __device__ void block_sort(uint64_t *s, int n_pow2) {
                 uint64_t x = s[lo], y = s[hi];
                 if ((x > y) == up) { s[lo] = y; s[hi] = x; }
             }
+            __syncthreads();
+        }
+        if (regs) {
+            for (int base = 64 * wid; base < n_pow2; base += 64 * nwarps) warp_sort64(s, base, size, size);
             __syncthreads();
         }
     }
@@ -1481,17 +1519,18 @@ __device__ __forceinline__ void topk_block(const uint64_t *keys_e, const int32_t
 
 __global__ void __launch_bounds__(1024)
 k_topk(const uint64_t *keys, const int32_t *votes, int n_in, int K, uint64_t *out_keys,
-       int32_t *out_votes) {
+       int32_t *out_votes, const int32_t *skip) {
     __shared__ uint64_t s[kSortMax];
     const int e = blockIdx.x;
+    if (skip && skip[e]) return;
     topk_block(keys + (long long)e * n_in, votes + (long long)e * n_in, n_in, K, out_keys + (long long)e * K,
                out_votes + (long long)e * K, s);
 }
 
 void launch_topk(int n_ev, const uint64_t *keys, const int32_t *votes, int n_in, int K,
-                 uint64_t *out_keys, int32_t *out_votes, cudaStream_t s) {
+                 uint64_t *out_keys, int32_t *out_votes, cudaStream_t s, const int32_t *skip) {
     if (n_ev <= 0) return;
-    k_topk<<<n_ev, 1024, 0, s>>>(keys, votes, n_in, K, out_keys, out_votes);
+    k_topk<<<n_ev, 1024, 0, s>>>(keys, votes, n_in, K, out_keys, out_votes, skip);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -99,6 +99,8 @@ __device__ __forceinline__ void unpack_key(const DevGeom &g, uint64_t k, int idx
 enum : unsigned { ST_TIMEOUT = 1u, ST_BADHIT = 2u, ST_TOOMANY = 4u, ST_BADOFFS = 8u };
 
 // ---- launch wrappers (kernels.cu) ----
+// skip (may be null): per event (launch_vote_coarse and the selections: of the whole batch, indexed
+// from ev0), nonzero leaves the event's outputs as they are: a round after its extraction ended
 // hit_track (may be null): set to -1 for every hit of the batch
 void launch_stage(const DevGeom &g, int n_events, const int32_t *offsets, const int32_t *wire_id,
                   const double *drift, HitRecD *hd, HitRecF *hf, int32_t *n_hits,
@@ -112,14 +114,15 @@ void launch_vote_coarse(const DevGeom &g, int prec, int ev0, int n_ev, const Hit
                         const HitRecF *hf, const int32_t *n_hits, int32_t *votes, uint32_t *hist,
                         unsigned *status, cudaStream_t s, unsigned long long *ctr = nullptr,
                         const uint32_t *active = nullptr, uint64_t *cand_k = nullptr,
-                        int32_t *cand_v = nullptr, int K = 0);
+                        int32_t *cand_v = nullptr, int K = 0, const int32_t *skip = nullptr);
 int coarse_lists(const DevGeom &g, int prec);   // level-0 blocks per event of a precision
 // The K best level-0 cells of each event from its blocks' candidates (n_lists x K per
 // event) and its histogram of all cells' votes, to out_keys / out_votes (K per event, in
 // no particular order; the set is that of launch_select_coarse).
 void launch_select_candidates(const DevGeom &g, int ev0, int n_ev, const uint64_t *cand_k,
                               const int32_t *cand_v, int n_lists, const uint32_t *hist, int K,
-                              uint64_t *out_keys, int32_t *out_votes, cudaStream_t s);
+                              uint64_t *out_keys, int32_t *out_votes, cudaStream_t s,
+                              const int32_t *skip = nullptr);
 void launch_vote_keys(const DevGeom &g, int prec, int n_ev, const HitRecD *hd, const HitRecF *hf,
                       const int32_t *n_hits, int level, const uint64_t *keys, long long n_per_ev,
                       int32_t *votes, cudaStream_t s, const uint32_t *active = nullptr);
@@ -127,14 +130,14 @@ void launch_vote_children(const DevGeom &g, int prec, int n_ev, const HitRecD *h
                           const HitRecF *hf, const int32_t *n_hits, int child_level,
                           const uint64_t *parents, int n_par, uint64_t *child_keys,
                           int32_t *child_votes, cudaStream_t s, const uint32_t *active = nullptr,
-                          int block = 256, const int32_t *n_valid = nullptr);
+                          int block = 256, const int32_t *n_valid = nullptr, const int32_t *skip = nullptr);
 void init_kernel_attributes();
 void launch_wait_never(long limit, unsigned *status, cudaStream_t s);
 void launch_select_coarse(const DevGeom &g, int ev0, int n_ev, const int32_t *votes,
                           const uint32_t *hist, int K, uint64_t *out_keys, int32_t *out_votes,
-                          cudaStream_t s);
+                          cudaStream_t s, const int32_t *skip = nullptr);
 void launch_topk(int n_ev, const uint64_t *keys, const int32_t *votes, int n_in, int K,
-                 uint64_t *out_keys, int32_t *out_votes, cudaStream_t s);
+                 uint64_t *out_keys, int32_t *out_votes, cudaStream_t s, const int32_t *skip = nullptr);
 // offsets / hit_track (hit_track may be null): the batch's CSR offsets of these events and
 // the per-hit track index, written for the hits this round's track takes
 void launch_estimate_mask(const DevGeom &g, int n_ev, const uint64_t *keys, const int32_t *votes,
