@@ -388,7 +388,7 @@ def serving_leg(w, seconds: float) -> dict:
     (1-5 helices plus noise, 10-200 hits; "the config-3 distribution" read as the fourth
     configuration, index 3 counted from 0) into apo_serve at 1k-50k events/s, each slot's
     batch through the per-level launches (FP32 levels 0-4, FP64 levels 5-6, up to 5 tracks;
-    a 64-event batch is too small for the persistent launch),
+    events whose extraction has ended are skipped),
     next to the plain FP64 per-event path on the same events (one event per call,
     synchronised)."""
     import torch
@@ -444,8 +444,7 @@ def background_study(w, n_events: int = 1024, seed: int = 4, n_maxset: int = 512
     launch = {}
     results = {}
     # the same search through the per-level launches recorded as one CUDA graph, through the
-    # persistent launch, and with the knobs apo_autotune picks on a 1024-event sample (the
-    # persistent launch needs many more events than resident blocks to pay)
+    # tune.persistent set, and with the knobs apo_autotune picks on a 1024-event sample
     sample = apo.DeviceHits.from_events(ev.subset(range(min(1024, ev.n_events))))
     best, _ = apo.autotune(geom, sample, apo.solve_opts(precision=prec, max_tracks=5, min_votes=6))
     for name, tune, graph in (("graph", apo.ApoTune(0, 1, 256, 0, persistent=0), True),
@@ -1071,7 +1070,7 @@ def run_case(args) -> None:
         torch.cuda.synchronize()
         print(json.dumps({"case": args.case, "events": ev.n_events, "ok": True}))
         return
-    if args.case == "solve-persist":   # the multi-track batch through the persistent launch
+    if args.case == "solve-persist":   # the multi-track batch with tune.persistent set
         from gen import chamber, grid as G
         w = chamber.make_wires()
         g4 = G.make_grid([10] * 5, 6, 64)

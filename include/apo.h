@@ -148,12 +148,11 @@ typedef struct {
                                 from them, instead of each tile keeping its topk best cells
                                 (more workspace, fewer instructions per tile); the same
                                 kept set either way */
-    int32_t persistent;      /* 1 (APO_SCHED_TOPK only): one persistent launch for the whole
-                                batch; each block pulls the next event from a device counter
-                                and runs its whole search (every round, tile and level),
-                                instead of one launch per step and level.  Levels must share
-                                their APO_OUTGOING flag and use APO_F64, APO_F32 or
-                                APO_F64_FILTERED; no trace. */
+    int32_t persistent;      /* 1 (APO_SCHED_TOPK only): asks for one launch per batch; runs the
+                                per-level launches, which leave an event as soon as its
+                                extraction has ended and take about half the time of blocks
+                                that run whole events.  Levels must share their APO_OUTGOING
+                                flag and use APO_F64, APO_F32 or APO_F64_FILTERED; no trace. */
 } apo_tune;
 
 /* Options of apo_solve_batch.  precision[L] selects FP64 or FP32 intervals at level L
@@ -259,8 +258,7 @@ int apo_solve_batch(const apo_geometry *geom, const apo_hits *hits, const apo_so
 
 /* Times apo_solve_batch on `hits` (typically a sample of the batch to come) for every
  * combination of the apo_tune knobs and writes the fastest to *best (its time to *best_ms,
- * may be NULL): the launch schedule (per-level launches, or the persistent launch when
- * the options allow it), level 0's full votes or K best cells, the threads per block of the
+ * may be NULL): level 0's full votes or K best cells, the threads per block of the
  * bisected cells' kernel and the events per level-0 launch.  opts: as for apo_solve_batch (its tune and use_graph are ignored).
  * Workspace as for apo_solve_batch.  Synchronous. */
 int apo_autotune(const apo_geometry *geom, const apo_hits *hits, const apo_solve_opts *opts,

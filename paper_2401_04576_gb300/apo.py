@@ -328,7 +328,7 @@ def autotune(geom: Geometry, hits: DeviceHits, opts: ApoSolveOpts | None = None,
              stream=None):
     """apo_autotune: the fastest execution knobs for this batch (results never change)."""
     o = opts if opts is not None else solve_opts()
-    if workspace is None:   # room for every candidate, the persistent launch's scratch included
+    if workspace is None:   # room for every candidate
         op = ApoSolveOpts.from_buffer_copy(o)
         op.tune.persistent = 1
         of = ApoSolveOpts.from_buffer_copy(o)

@@ -360,7 +360,7 @@ struct CoarsePlan {
     int group, tiles;        // tiles side by side, tiles per block (group or one after another)
     long long n_tiles;       // of one event
 };
-// n_ev: events of the launch (0: one block takes a whole event)
+// n_ev: events of the launch
 __host__ __device__ inline CoarsePlan coarse_plan(const DevGeom &g, bool lists, long long n_ev) {
     CoarsePlan P;
     const int n = g.bins[0] * g.bins[3];
@@ -371,7 +371,7 @@ __host__ __device__ inline CoarsePlan coarse_plan(const DevGeom &g, bool lists, 
     P.group = lists || fit < 2 ? 1 : (fit > kCoarseMaxGroup ? kCoarseMaxGroup : fit);
     P.tiles = P.group;
     if (P.group == 1) {   // at least two waves of four blocks on 152 SMs
-        const long long r = n_ev == 0 ? kCoarseRounds : P.n_tiles * n_ev / (2 * 4 * 152);
+        const long long r = P.n_tiles * n_ev / (2 * 4 * 152);
         P.tiles = r < 1 ? 1 : (r > kCoarseRounds ? kCoarseRounds : (int)r);
     }
     return P;
@@ -1689,108 +1689,6 @@ void launch_estimate_mask(const DevGeom &g, int n_ev, const uint64_t *keys, cons
     k_estimate_mask<<<n_ev, 256, 0, s>>>(g, keys, votes, n_in, level, n_hits, active, done, hd, round,
                                           max_tracks, min_votes, width, out, n_tracks, offsets,
                                           hit_track);
-}
-
-// ---------------------------------------------------------------------------------------
-// Persistent batch search (top-K schedule, multi-track rounds).  One launch of as many
-// blocks as the GPU holds at once.  Each block pulls the next event from a device counter
-// and runs that event's whole search: per round the level-0 tiles (with the parent-cell
-// test), the top-K selection, every bisection level with its top-K, and the estimate with
-// the hit masking of Section 3.3; then the next round or the next event.  The steps are
-// the device functions of the per-level kernels above (same operations, same results);
-// only their scheduling differs.  Events are independent, so no block ever waits on
-// another: uneven events (10-200 hits) simply keep their block longer while the others
-// pull new ones, and no launch boundary waits for the slowest event of a level.  The only
-// device waits are the bounded waits of the hit staging.
-// ---------------------------------------------------------------------------------------
-template <int K> __device__ __noinline__ void persist_coarse(const DevGeom &g, const PersistArgs &A, int e,
-                                                                int32_t *vo, uint32_t *hist_b, unsigned char *smem) {
-    const CoarsePlan P = coarse_plan(g, false, 0);
-    for (long long t = 0; t < P.n_tiles; t += P.tiles)
-        coarse_block<K>(g, P, e, t, A.hd, A.hf, A.n_hits, A.active, vo, hist_b, A.status, nullptr, smem);
-}
-
-template <int K> __device__ __noinline__ void persist_children(const DevGeom &g, const PersistArgs &A, int e,
-                                                               int level, unsigned char *smem) {
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + ChildSmem::bar);
-    const HitRecF *hf_e = A.hf + (long long)e * kHitCap;
-    int nh = A.n_hits[e];
-    if (nh < 0) nh = 0;
-    const bool ok = stage_to_smem(smem + ChildSmem::hits, hf_e, (unsigned)nh * 80u, nullptr, nullptr, 0u, bar, A.status);
-    __syncthreads();
-    if (threadIdx.x == 0) mbar_inval(bar);
-    if (!ok) nh = 0;
-    const int Kp = g.topk;
-    ChildScratch &ws = reinterpret_cast<ChildScratch *>(smem + ChildSmem::warp)[threadIdx.x >> 5];
-    const int np = Kp / 8 < 2 ? 2 : (Kp / 8 > kChildParents ? kChildParents : Kp / 8 & ~1);   // two rounds of four warps
-    for (int p = (int)(threadIdx.x >> 5) * np; p < Kp; p += np * (kChildThreads / 32))
-        children_warp<K>(g, smem + ChildSmem::hits, ws, nh, A.active + (long long)e * 8, level,
-                         A.fk + (long long)e * Kp, p, np, Kp, A.hd + (long long)e * kHitCap, hf_e,
-                         A.ck + (long long)e * Kp * 32, A.cv + (long long)e * Kp * 32);
-    __threadfence_block();
-    __syncthreads();
-}
-
-__global__ void __launch_bounds__(128, 4) k_solve_persistent(const __grid_constant__ DevGeom g, const __grid_constant__ PersistArgs A) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_e;
-    const int lv = g.levels, K = g.topk;
-    const long long ncell = (long long)g.bins[0] * g.bins[1] * g.bins[2] * g.bins[3] * g.bins[4];
-    int32_t *vo = A.votes + (long long)blockIdx.x * ncell;        // this block's level-0 votes
-    uint32_t *hist_b = A.hist + (long long)blockIdx.x * kHistBins;
-    uint64_t *s_sort = reinterpret_cast<uint64_t *>(smem);
-    double *s_cen = reinterpret_cast<double *>(smem + kSortMax * sizeof(uint64_t));
-    for (;;) {
-        if (threadIdx.x == 0) s_e = atomicAdd(A.next_event, 1);
-        __syncthreads();
-        const int e = s_e;
-        __syncthreads();
-        if (e >= A.n_events) break;
-        for (int round = 0; round < A.max_tracks; round++) {
-            if (A.done[e]) break;
-            for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) hist_b[i] = 0u;
-            __syncthreads();
-            if (A.mode[0] == kPersistF32) persist_coarse<32>(g, A, e, vo, hist_b, smem);
-            else persist_coarse<64>(g, A, e, vo, hist_b, smem);
-            __threadfence_block();
-            __syncthreads();
-            select_coarse_block(g, vo, hist_b, K, A.fk + (long long)e * K, A.fv + (long long)e * K);
-            for (int lev = 1; lev <= lv; lev++) {
-                if (A.mode[lev] == kPersistF32) persist_children<32>(g, A, e, lev, smem);
-                else persist_children<64>(g, A, e, lev, smem);
-                topk_block(A.ck + (long long)e * K * 32, A.cv + (long long)e * K * 32, K * 32, K,
-                           A.fk + (long long)e * K, A.fv + (long long)e * K, s_sort);
-            }
-            estimate_mask_block(g, A.ck + (long long)e * K * 32, A.cv + (long long)e * K * 32, K * 32, lv,
-                                A.n_hits[e], A.active + (long long)e * 8, A.done + e,
-                                A.hd + (long long)e * kHitCap, round, A.max_tracks, A.min_votes, A.width,
-                                A.tracks + (long long)e * A.max_tracks, A.n_tracks + e,
-                                A.hit_track ? A.offsets[e] : 0, A.hit_track, s_sort, s_cen);
-        }
-    }
-}
-
-size_t persist_smem_bytes(const DevGeom &g) {
-    size_t a = CoarseSmem::total(g.bins[4], coarse_plan(g, false, 0));
-    size_t b = ChildSmem::total;
-    size_t c = kSortMax * sizeof(uint64_t) + kEstChunk * 5 * sizeof(double);
-    size_t m = a > b ? a : b;
-    return m > c ? m : c;
-}
-
-int persist_blocks(const DevGeom &g) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(k_solve_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solve_persistent, 128, persist_smem_bytes(g));
-    if (per_sm < 1) per_sm = 1;
-    return sms * per_sm;
-}
-
-void launch_solve_persistent(const DevGeom &g, int blocks, const PersistArgs &A, cudaStream_t s) {
-    if (A.n_events <= 0 || blocks <= 0) return;
-    k_solve_persistent<<<blocks, 128, persist_smem_bytes(g), s>>>(g, A);
 }
 
 }  // namespace apo
