@@ -97,6 +97,27 @@ template <int Q> __device__ __forceinline__ cert::X<Q> xf(float2 a) {   // ends 
     return r;
 }
 
+// Axis quantity q (0 .. 5: d0, sin phi0, cos phi0, omega, z0, tan(lambda)) of a cell with index i on
+// that axis, in FP32.
+__device__ __forceinline__ float2 axis_float(const DevGeom &g, int level, int q, int i) {
+    const IV<double> v = q == 0 ? edge(g, 0, level, i) : q == 1 ? sin_phi0(g, level, i) : q == 2 ? cos_phi0(g, level, i)
+                       : q == 3 ? edge(g, 2, level, i) : q == 4 ? edge(g, 3, level, i) : edge(g, 4, level, i);
+    return make_float2((float)v.lo, (float)v.hi);
+}
+// The box around the two cells v[0], v[1] per quantity.  No omega cell holds 0 (apo_geometry_create);
+// an omega that FP32 rounds to 0, or a box over both signs, leaves its reciprocal without a bound.
+__device__ __forceinline__ CertBox float_box(const float2 (&v)[2][6]) {
+    CertBox b;
+    b.mir = v[0][3].y < 0.f && v[1][3].y < 0.f;
+    b.guard = 0;
+#pragma unroll
+    for (int q = 0; q < 6; q++) {
+        const float lo = fminf(v[0][q].x, v[1][q].x), hi = fmaxf(v[0][q].y, v[1][q].y);
+        b.v[q] = b.mir && (q == 0 || q == 1 || q == 3) ? make_float2(-hi, -lo) : make_float2(lo, hi);
+    }
+    return b;
+}
+
 // The test of one hit on a box: -1 when no cell inside it gets the hit's vote, else the error bound
 // its cells share (NaN: they cannot be decided by one).  own: the box is one cell; -2 when it votes.
 // Not inlined: its registers stay out of the callers' loops, and one copy stays in the instruction
@@ -303,6 +324,15 @@ template <int K> struct Prog {
     using Pre = cert::PreX<0>;
     static __device__ __forceinline__ CellT cell(const DevGeom &, int, int, const Cell<double> &c, bool mir) {
         const cert::CellX<0> x = cert_cell<0>(c, mir);
+        return CellT{x, cert::recip(x.W)};
+    }
+    // from FP32 ends (not mirrored) of its cells per axis
+    static __device__ __forceinline__ CellT cell(const float2 (&v)[2][6], const int (&bit)[4], bool mir) {
+        auto f = [&](int q, int a, bool flip) {
+            const float2 x = v[bit[a]][q];
+            return flip ? cert::X<0>{-x.y, -x.x, 0.f} : cert::X<0>{x.x, x.y, 0.f};
+        };
+        const cert::CellX<0> x{f(0, 0, mir), f(1, 1, mir), f(2, 1, false), f(3, 2, mir), f(4, 3, false), {0.f, 0.f, 0.f}};
         return CellT{x, cert::recip(x.W)};
     }
     static __device__ __forceinline__ float2 tanl(IV<double> L) { return make_float2((float)L.lo, (float)L.hi); }

@@ -971,7 +971,9 @@ __device__ __forceinline__ void pair_store(const DevGeom &g, const int idx[5], l
 constexpr int kChildThreads = 128, kChildParents = 8;   // most parents of a warp
 struct ChildScratch {
     CertBox box[kChildParents];
-    float err[kChildParents][kHitCap];
+    float2 axis[kChildParents][2][6];   // the children's ends per axis, bit 0 and 1: conversions from
+                                        // FP64, which run on its pipe, once per parent
+    uint16_t err[kChildParents][kHitCap];   // bounds as bf16 rounded up: four blocks fit an SM
     uint32_t mask[kChildParents][8];
     WarpQueue q;
 };
@@ -981,6 +983,10 @@ struct ChildSmem {
     static constexpr size_t bar = warp + sizeof(ChildScratch) * (kChildThreads / 32);
     static constexpr size_t total = bar + 16;
 };
+// A bound >= 0 (or NaN) as bf16, rounded up.
+__device__ __forceinline__ uint16_t bound_up(float e) {
+    return e < 1e30f ? (uint16_t)((__float_as_uint(e) + 0xffffu) >> 16) : (uint16_t)0x7fc0u;
+}
 // Parents per warp (even): eight where that leaves four waves of 16 warps on each of 152 SMs, else
 // fewer (256 events x 64 parents: two a warp 2.05 ms, six 2.78 ms, FP32 levels of 1024 events).
 __device__ __forceinline__ int child_parents(long long n_par) {
@@ -998,13 +1004,25 @@ __device__ __forceinline__ void children_warp(const DevGeom &g, const unsigned c
     const bool outgoing = g.k.outgoing != 0;
     if (n_par - p0 < np) np = (int)(n_par - p0);
     for (int i = lane; i < 8 * kChildParents; i += 32) ws.mask[i >> 3][i & 7] = 0u;
-    if (lane < np) {
-        int x[5];
-        unpack_key(g, parents_e[p0 + lane], x);
+    if constexpr (K == kMid) {
+        if (lane < np) {
+            int x[5];
+            unpack_key(g, parents_e[p0 + lane], x);
 #pragma unroll
-        for (int a = 0; a < 5; a++) x[a] *= 2;
-        const int x1[5] = {x[0] + 1, x[1] + 1, x[2] + 1, x[3] + 1, x[4] + 1};
-        ws.box[lane] = cert_span<K>(g, level, x, x1);
+            for (int a = 0; a < 5; a++) x[a] *= 2;
+            const int x1[5] = {x[0] + 1, x[1] + 1, x[2] + 1, x[3] + 1, x[4] + 1};
+            ws.box[lane] = cert_span<K>(g, level, x, x1);
+        }
+    } else {
+        for (int i = lane; i < np * 12; i += 32) {
+            const int pl = i / 12, q = i % 6, bit = i / 6 & 1;
+            int x[5];
+            unpack_key(g, parents_e[p0 + pl], x);
+            const int at = q == 0 ? x[0] : q < 3 ? x[1] : q == 3 ? x[2] : q == 4 ? x[3] : x[4];
+            ws.axis[pl][bit][q] = axis_float(g, level, q, 2 * at + bit);
+        }
+        __syncwarp();
+        if (lane < np) ws.box[lane] = float_box(ws.axis[lane]);
     }
     __syncwarp();
     for (int i = lane; i < np * nh; i += 32) {
@@ -1012,7 +1030,7 @@ __device__ __forceinline__ void children_warp(const DevGeom &g, const unsigned c
         if (act && !((act[h >> 5] >> (h & 31)) & 1u)) continue;
         const float e = box_error<K>(&ws.box[pl], hs + h * 80, outgoing);
         if (e < 0.f) continue;
-        ws.err[pl][h] = e;
+        ws.err[pl][h] = bound_up(e);
         atomicOr(&ws.mask[pl][h >> 5], 1u << (h & 31));
     }
     // keys, and votes from 0: counted votes and those of undecided pairs are added as they come
@@ -1037,14 +1055,25 @@ __device__ __forceinline__ void children_warp(const DevGeom &g, const unsigned c
     for (int s = 0; s < np; s += 2) {
         const int pl = s + (lane >> 4);
         const bool has = pl < np;
-        int idx[5] = {0, 0, 0, 0, 0};
-        if (has) pair_index(g, parents_e[p0 + pl], lane & 15, idx);
-        const Cell<double> c64{edge(g, 0, level, idx[0]), sin_phi0(g, level, idx[1]), cos_phi0(g, level, idx[1]),
-                               edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
-        bool guard;
-        const bool mir = omega_sign<K>(c64.W, &guard);
-        const typename Prog<K>::CellT c = Prog<K>::cell(g, level, idx[1], c64, mir);
-        const float2 L0 = Prog<K>::tanl(c64.L), L1 = Prog<K>::tanl(edge(g, 4, level, idx[4] + 1));
+        bool guard = false, mir;
+        typename Prog<K>::CellT c;
+        float2 L0, L1;
+        if constexpr (K == kMid) {
+            int idx[5] = {0, 0, 0, 0, 0};
+            if (has) pair_index(g, parents_e[p0 + pl], lane & 15, idx);
+            const Cell<double> c64{edge(g, 0, level, idx[0]), sin_phi0(g, level, idx[1]), cos_phi0(g, level, idx[1]),
+                                   edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
+            mir = omega_sign<K>(c64.W, &guard);
+            c = Prog<K>::cell(g, level, idx[1], c64, mir);
+            L0 = Prog<K>::tanl(c64.L);
+            L1 = Prog<K>::tanl(edge(g, 4, level, idx[4] + 1));
+        } else {
+            const int bit[4] = {lane & 1, lane >> 1 & 1, lane >> 2 & 1, lane >> 3 & 1}, pa = has ? pl : 0;
+            mir = ws.axis[pa][bit[2]][3].y < 0.f;
+            c = Prog<K>::cell(ws.axis[pa], bit, mir);
+            L0 = ws.axis[pa][0][5];
+            L1 = ws.axis[pa][1][5];
+        }
         int v0 = 0, v1 = 0, wd = -1;
         uint32_t m = 0;
         for (;;) {
@@ -1056,7 +1085,7 @@ __device__ __forceinline__ void children_warp(const DevGeom &g, const unsigned c
             if (m) {
                 h = wd * 32 + __ffs(m) - 1;
                 m &= m - 1;
-                const float e = ws.err[pl][h];
+                const float e = __uint_as_float((unsigned)ws.err[pl][h] << 16);
                 if (guard) {
                     v0++;
                     v1++;
