@@ -44,10 +44,10 @@ OPS_TAIL = OPS_LPART + OPS_SIGNS
 
 # DRAM bytes (read + write) of one k_vote_coarse<FP64> launch per event: an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum, --clock-control none) of one 64-event
-# launch of that kernel on the 16^5 grid, in the search's form (each block keeps its K
-# best cells), read 496,384 B and wrote 0 B; scaled by events to the benchmark's launch.
+# launch of that kernel on the 16^5 grid, in the search's form (each tile keeps its K
+# best cells), read 593,152 B and wrote 963,072 B; scaled by events to the benchmark's launch.
 # Must be re-captured (or set to None) whenever that kernel changes.
-COARSE_F64_DRAM_BYTES_PER_EVENT = 496384 / 64
+COARSE_F64_DRAM_BYTES_PER_EVENT = (593152 + 963072) / 64
 
 
 def coarse_kernel_ops(n_parent: int, n_prefix: int, n_tail: int) -> int:
