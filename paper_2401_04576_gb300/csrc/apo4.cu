@@ -174,7 +174,9 @@ __device__ __forceinline__ double mid4(double a, double b) { return __dmul_rn(__
 // its pairs share, in chunks of 16 hits, one evaluation per thread (over each half of the z0 voxels
 // where the whole range decides nothing, then per column); pairs left undecided are queued by warp
 // and evaluated by the program itself.  FP32 issue bounds it; evaluating every pair was bound by the
-// FP64 pipe, and in FP32 by the instructions of correctly rounded quotients and roots.
+// FP64 pipe, and in FP32 by the instructions of correctly rounded quotients and roots: FP32, 48
+// electrons, 380 -> 225 ms; FP64, 2 electrons, 788 -> 13.6 ms.  Blocks of one warp took the latter
+// to 21.3 ms.  Always eight columns deep: two events' search 22.8 against 16.0 ms.
 // ---------------------------------------------------------------------------------------
 constexpr int k4Threads = 128, k4Side = 8, k4MaxTile = k4Side * k4Side * k4Side, k4Groups = k4MaxTile / 8;
 constexpr int k4Slots = k4Threads / 8, k4Chunk = 16;

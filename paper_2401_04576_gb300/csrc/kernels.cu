@@ -347,10 +347,14 @@ __device__ __forceinline__ void add_counts(unsigned long long *ctr, const unsign
 // from its bins' boxes; phase 3, tile by tile and without barriers,
 // the bare values per (cell, hit, bin), bit-sliced counters; undecided pairs go to the warp's queue.
 // What bounds it: FP32 issue.  The FP64 pipe (about 1.7 directed operations per clock and SM)
-// evaluated every pair before; now about one pair in 10^4 reaches it.
+// evaluated every pair before; now about one pair in 10^4 reaches it.  256 events on 16^5 cells:
+// FP64 votes 377 -> 9.7 ms (K best per tile), midpoint form 1077 -> 5.3 ms; FP32 votes of 1024 events
+// 55.7 -> 31.5 ms.  3.1 (FP32) and 2.9 (FP64) instructions a clock and SM of 4.
 //
 // A block is 128 threads and takes up to four tiles, so that phases 1 and 2, whose chains a single
 // tile cannot hide, keep all its warps busy (fewer where the launch would have too few blocks).
+// Phase 2's bin tests take 39.5 ms to 33.4 (FP32, 1024 events); with one tile a block they cost more
+// than they gave (41.3 -> 44.4 ms).
 // Grids with few (d0, z0) cells put `group` tiles side by side in the block (full votes only: the K
 // best are kept per tile), so that its warps stay full.
 constexpr int kCoarseThreads = 128, kCoarseMaxGroup = 8, kCoarseRounds = 4;
@@ -810,6 +814,7 @@ __device__ __forceinline__ IV<double> warp_hull(IV<double> a) {
 // coarse_block).  The parent is the smallest box around the warp's 32 cells: for the 32 children
 // of one cell, as apo_refine lists them, that cell; for scattered keys it is wide, its bound
 // decides little, and the pairs are evaluated one by one with their own bounds.
+// The children of 33 kept cells of 37 events, FP64: 0.76 -> 0.055 ms.  FP32 issue bounds it.
 constexpr int kCellsThreads = 128;
 struct WarpScratch {   // one warp's parent, and its queue
     CertBox box;
@@ -967,7 +972,8 @@ __device__ __forceinline__ void pair_store(const DevGeom &g, const int idx[5], l
 // pairs collect over all the warp's parents.  FP32 issue and instruction fetch bound it: the
 // evaluation with errors and the reference program are long straight code, so a warp runs them
 // rarely and on as many lanes as there are (eight parents a warp; with two, 24 multi-track events took 133 ms
-// instead of 118).  Before, every child hit that passed an FP32 test was evaluated on the FP64 pipe.
+// instead of 118).  Before, every child hit that passed an FP32 test was evaluated on the FP64 pipe:
+// 160 events of the max-set schedule, FP64 level 366 -> 13.6 ms, the FP32 levels 21.3 -> 15.7 ms.
 constexpr int kChildThreads = 128, kChildParents = 8;   // most parents of a warp
 struct ChildScratch {
     CertBox box[kChildParents];
@@ -1494,7 +1500,7 @@ __device__ __forceinline__ void warp_sort64(uint64_t *s, int base, int size0, in
 }
 // Ascending bitonic sort by the block (whole warps).  Steps with strides below 64 run in registers,
 // one pass per block size instead of six (2048 entries: 15 passes through shared memory and 6
-// through registers instead of 66).
+// through registers instead of 66; the six levels of 1024 events 0.77 -> 0.46 ms).
 __device__ void block_sort(uint64_t *s, int n_pow2) {
     const int wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const bool regs = n_pow2 >= 64;

