@@ -814,7 +814,7 @@ __device__ __forceinline__ IV<double> warp_hull(IV<double> a) {
 // coarse_block).  The parent is the smallest box around the warp's 32 cells: for the 32 children
 // of one cell, as apo_refine lists them, that cell; for scattered keys it is wide, its bound
 // decides little, and the pairs are evaluated one by one with their own bounds.
-// The children of 33 kept cells of 37 events, FP64: 0.76 -> 0.055 ms.  FP32 issue bounds it.
+// The children of 33 kept cells of 37 events, FP64: 0.76 -> 0.055 ms.
 constexpr int kCellsThreads = 128;
 struct WarpScratch {   // one warp's parent, and its queue
     CertBox box;
