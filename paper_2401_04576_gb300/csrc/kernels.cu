@@ -192,7 +192,8 @@ void launch_stage(const DevGeom &g, int n_events, const int32_t *offsets, const 
 // ---------------------------------------------------------------------------------------
 // The end of a coarse block: each thread's Bl vote counts (its cell (d, p, w, z), every
 // tan(lambda) bin) to vo or, with cand_k, the block's K best cells; the histogram added to hist_e
-// (may be null).  hist_s: kHistBins zeros in shared memory.
+// (may be null).  hist_s: kHistBins zeros in shared memory.  The block has whole warps, and so at
+// least a thread per tan(lambda) bin.
 __device__ __forceinline__ void coarse_output(const DevGeom &g, const VotePlanes &pl, bool has_cell, int d, int p,
                                               int w, int z, uint32_t *hist_s, uint32_t *hist_e, int32_t *vo,
                                               uint64_t *cand_k, int32_t *cand_v, int K) {
@@ -216,26 +217,23 @@ __device__ __forceinline__ void coarse_output(const DevGeom &g, const VotePlanes
         // (tan(lambda) bin, thread) are in key order.  Any cell among the event's K best is
         // among its part's K best, so these candidates are all the selection needs.
         __shared__ int s_vt, s_need, s_above;
-        // warp 0 (its cw lanes: a block may have fewer than 32 threads): suffix sums of the
-        // histogram from the top, cw bins a step
-        const int cw = nthr < 32 ? nthr : 32;
-        if (tid < cw) {
-            const unsigned m0 = cw == 32 ? 0xffffffffu : ((1u << cw) - 1u);
+        // warp 0: suffix sums of the histogram from the top, 32 bins a step
+        if (tid < 32) {
             int cum = 0;
             bool found = false;
-            for (int top = kHistBins - 1; top >= 0 && !found; top -= cw) {
+            for (int top = kHistBins - 1; top >= 0 && !found; top -= 32) {
                 const int v = top - tid;
                 const int h = v >= 0 ? (int)hist_s[v] : 0;
                 int inc = h;   // cells with votes in [v, top]
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(m0, inc, o);
+                    const int y = __shfl_up_sync(0xffffffffu, inc, o);
                     if (tid >= o) inc += y;
                 }
-                const unsigned hit = __ballot_sync(m0, v >= 0 && cum + inc >= K);
+                const unsigned hit = __ballot_sync(0xffffffffu, v >= 0 && cum + inc >= K);
                 if (hit) {   // the first bin from the top where the count reaches K
                     const int b = __ffs(hit) - 1;
-                    const int incb = __shfl_sync(m0, inc, b), hb = __shfl_sync(m0, h, b);
+                    const int incb = __shfl_sync(0xffffffffu, inc, b), hb = __shfl_sync(0xffffffffu, h, b);
                     if (tid == 0) {
                         s_vt = top - b;
                         s_above = cum + incb - hb;
@@ -243,7 +241,7 @@ __device__ __forceinline__ void coarse_output(const DevGeom &g, const VotePlanes
                     }
                     found = true;
                 } else {
-                    cum += __shfl_sync(m0, inc, cw - 1);
+                    cum += __shfl_sync(0xffffffffu, inc, 31);
                 }
             }
             if (!found && tid == 0) {   // fewer than K cells in the part
@@ -254,11 +252,7 @@ __device__ __forceinline__ void coarse_output(const DevGeom &g, const VotePlanes
         }
         __syncthreads();
         const int vt = s_vt, need = s_need, above = s_above;
-        const int lane = tid & 31, wid = tid >> 5, nwarps = (nthr + 31) >> 5;
-        // the block may end in a partial warp (e.g. 100 or 50 threads): ballots over the
-        // lanes that exist (lanes 0 .. r - 1 of the last warp)
-        const int rem = nthr - (wid << 5);
-        const unsigned wmask = rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u);
+        const int lane = tid & 31, wid = tid >> 5, nwarps = nthr >> 5;
         const unsigned lt = (1u << lane) - 1u;
         // Ranks in key order ((tan(lambda) bin, thread) order): per bin and warp, counts of
         // cells above v_t / at v_t from ballots; exclusive prefixes over warps, then over
@@ -266,7 +260,7 @@ __device__ __forceinline__ void coarse_output(const DevGeom &g, const VotePlanes
         __shared__ int s_wa[8][32], s_wb[8][32], s_ba[33], s_bb[33];
         for (int l = 0; l < Bl; l++) {
             const int v = has_cell ? vote_of(l) : -1;
-            const unsigned ma = __ballot_sync(wmask, v > vt), mb = __ballot_sync(wmask, v == vt);
+            const unsigned ma = __ballot_sync(0xffffffffu, v > vt), mb = __ballot_sync(0xffffffffu, v == vt);
             if (lane == 0) { s_wa[wid][l] = __popc(ma); s_wb[wid][l] = __popc(mb); }
         }
         __syncthreads();
@@ -299,7 +293,7 @@ __device__ __forceinline__ void coarse_output(const DevGeom &g, const VotePlanes
         for (int l = 0; l < Bl; l++) {
             const int v = has_cell ? vote_of(l) : -1;
             const bool a = v > vt, b = v == vt;
-            const unsigned ma = __ballot_sync(wmask, a), mb = __ballot_sync(wmask, b);
+            const unsigned ma = __ballot_sync(0xffffffffu, a), mb = __ballot_sync(0xffffffffu, b);
             int pos = -1;
             if (a) {
                 pos = s_ba[l] + s_wa[wid][l] + __popc(ma & lt);
@@ -326,17 +320,12 @@ __device__ __forceinline__ void coarse_output(const DevGeom &g, const VotePlanes
 // certified decisions: pairs left undecided), FP64 prefixes, FP64 tails, then the FP32 ones.
 __device__ __forceinline__ void add_counts(unsigned long long *ctr, const unsigned (&cnt)[6]) {
     if (!ctr) return;
-    const int tid = threadIdx.x, nthr = blockDim.x;
     const int slot[6] = {0, 1, 2, 4, 5, 6};
 #pragma unroll
     for (int i = 0; i < 6; i++) {
         unsigned long long x = cnt[i];
-        if (nthr - (tid & ~31) >= 32) {   // a full warp: reduce, one add per warp
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-            if ((tid & 31) == 0 && x) atomicAdd(&ctr[slot[i]], x);
-        } else if (x) {                   // the lanes of a partial last warp add their own
-            atomicAdd(&ctr[slot[i]], x);
-        }
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+        if ((threadIdx.x & 31) == 0 && x) atomicAdd(&ctr[slot[i]], x);
     }
 }
 
@@ -620,16 +609,26 @@ k_vote_coarse(const __grid_constant__ DevGeom g, CoarsePlan P, int ev0, const Hi
                     cand_k ? cand_k + co : nullptr, cand_v ? cand_v + co : nullptr, Kc);
 }
 
-// The exact-phase program on the coarse grid: FP64, the same tiles in blocks of at most 128
-// threads, one tile each.
+// The exact-phase program on the coarse grid: FP64, the same tiles.  Full votes: a block takes
+// `group` tiles side by side, so that its 128 threads have a cell each; K best lists: one tile, in
+// whole warps.  Never fewer than 32 threads: the mask's words, and the bins' prefixes of
+// coarse_output, are one thread's each.
+constexpr int kExactMaxGroup = 32;
 struct ExactSmem {
     static constexpr size_t hits = 0;
     static constexpr size_t hist = kHitCap * 80;
     static constexpr size_t mask = hist + ((kHistBins * 4 + 15) & ~size_t(15));
-    static constexpr size_t bar = mask + 32;
+    static constexpr size_t bar = mask + 32 * kExactMaxGroup;
     static constexpr size_t L = bar + 16;
     __host__ __device__ static size_t total(int Bl) { return L + 16 * (size_t)Bl; }
 };
+__host__ inline CoarsePlan exact_plan(const DevGeom &g, bool lists, int *threads) {
+    CoarsePlan P = coarse_plan(g, true, 1);
+    const int fit = kCoarseThreads / P.per;
+    P.group = P.tiles = lists || fit < 2 ? 1 : (fit > kExactMaxGroup ? kExactMaxGroup : fit);
+    *threads = (P.group * P.per + 31) & ~31;
+    return P;
+}
 
 __global__ void __launch_bounds__(kCoarseThreads, 3)
 k_vote_coarse_exact(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const int32_t *n_hits, const uint32_t *active,
@@ -638,11 +637,9 @@ k_vote_coarse_exact(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const i
     extern __shared__ __align__(16) unsigned char smem[];
     const int e = blockIdx.y, ev = ev0 + e;
     if (skip && skip[ev]) return;
-    const int part = blockIdx.x % P.parts, pw = blockIdx.x / P.parts;
-    const int Bd = g.bins[0], Bz = g.bins[3], Bl = g.bins[4], p = pw % g.bins[1], w = pw / g.bins[1];
-    const int ntile = Bd * Bz, nthr = blockDim.x, tid = threadIdx.x;
-    const int c0 = part * P.per, c1 = c0 + P.per < ntile ? c0 + P.per : ntile;   // this block's cells
-    const bool has_cell = c0 + tid < c1;
+    const int Bd = g.bins[0], Bp = g.bins[1], Bz = g.bins[3], Bl = g.bins[4];
+    const int ntile = Bd * Bz, nthr = blockDim.x, tid = threadIdx.x, lane = tid & 31;
+    const long long tile0 = (long long)blockIdx.x * P.group;
     unsigned char *hs = smem + ExactSmem::hits;
     uint32_t *hist_s = reinterpret_cast<uint32_t *>(smem + ExactSmem::hist);
     uint32_t *mask_s = reinterpret_cast<uint32_t *>(smem + ExactSmem::mask);
@@ -651,38 +648,50 @@ k_vote_coarse_exact(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const i
     int nh = n_hits[ev];
     if (nh < 0) nh = 0;
     for (int i = tid; i < kHistBins; i += nthr) hist_s[i] = 0;
-    if (tid < 8) mask_s[tid] = 0;
+    for (int i = tid; i < 8 * P.group; i += nthr) mask_s[i] = 0;
     for (int l = tid; l < Bl; l += nthr) Ls[l] = edge(g, 4, 0, l);
     const bool ok = stage_to_smem(hs, hd + (long long)ev * kHitCap, (unsigned)nh * 80u, nullptr, nullptr, 0u, bar,
                                   status);
     __syncthreads();
     if (!ok) nh = 0;
     const SeriesConsts &k = g.k;
-    const IV<double> S0 = sin_phi0(g, 0, p), C0 = cos_phi0(g, 0, p), W = edge(g, 2, 0, w);
     unsigned cnt[6] = {0, 0, 0, 0, 0, 0};
     const uint32_t *act = active ? active + (long long)ev * 8 : nullptr;
-    {
-        const bool row = c0 / Bd == (c1 - 1) / Bd;   // cells of one z0 bin
-        const Cell<double> par{edge_span(g, 0, 0, row ? c0 % Bd : 0, row ? (c1 - 1) % Bd : Bd - 1), S0, C0, W,
-                               edge_span(g, 3, 0, c0 / Bd, (c1 - 1) / Bd), edge_span(g, 4, 0, 0, Bl - 1)};
-        for (int h = tid; h < nh; h += nthr) {
-            if (act && !((act[h >> 5] >> (h & 31)) & 1u)) continue;
+    const int nw = (nh + 31) >> 5;
+    // a warp's 32 items are one word of one tile's hit mask
+    for (int i = tid; i < P.group * nw * 32; i += nthr) {
+        const int tl = i / (nw * 32), h = i - tl * nw * 32;
+        const long long t = tile0 + tl;
+        bool keep = h < nh && t < P.n_tiles && (!act || ((act[h >> 5] >> (h & 31)) & 1u));
+        if (keep) {
+            const int pw = (int)(t / P.parts), p = pw % Bp, w = pw / Bp;
+            const int c0 = (int)(t % P.parts) * P.per, c1 = c0 + P.per < ntile ? c0 + P.per : ntile;
+            const bool row = c0 / Bd == (c1 - 1) / Bd;   // cells of one z0 bin
+            const Cell<double> par{edge_span(g, 0, 0, row ? c0 % Bd : 0, row ? (c1 - 1) % Bd : Bd - 1), sin_phi0(g, 0, p),
+                                   cos_phi0(g, 0, p), edge(g, 2, 0, w), edge_span(g, 3, 0, c0 / Bd, (c1 - 1) / Bd),
+                                   edge_span(g, 4, 0, 0, Bl - 1)};
             cnt[0]++;
-            if (vote_pair_exact(par, load_hit<double>(hs + h * 80), k)) atomicOr(&mask_s[h >> 5], 1u << (h & 31));
+            keep = vote_pair_exact(par, load_hit<double>(hs + h * 80), k);
         }
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        if (lane == 0) mask_s[tl * 8 + (h >> 5)] = m;
     }
     __syncthreads();
-    const int cell = has_cell ? c0 + tid : c0;   // threads past the block's cells idle
-    const int d = cell % Bd, z = cell / Bd;
-    Cell<double> c{edge(g, 0, 0, d), S0, C0, W, edge(g, 3, 0, z), Ls[0]};
+    const int tl = tid / P.per, kc = tid - tl * P.per;
+    const long long t = tile0 + tl;
+    const int part = (int)(t % P.parts), pw = (int)(t / P.parts), cell = part * P.per + kc;
+    const bool has_cell = tl < P.group && t < P.n_tiles && cell < ntile;   // other threads idle
+    const int p = has_cell ? pw % Bp : 0, w = has_cell ? pw / Bp : 0;
+    const int d = has_cell ? cell % Bd : 0, z = has_cell ? cell / Bd : 0;
+    Cell<double> c{edge(g, 0, 0, d), sin_phi0(g, 0, p), cos_phi0(g, 0, p), edge(g, 2, 0, w), edge(g, 3, 0, z), Ls[0]};
     const bool mir = mirror_cell(c);
     const bool wguard = !gt0(c.W.lo);
     const IV<double> R = recip(c.W);
     const unsigned all = Bl >= 32 ? 0xffffffffu : ((1u << Bl) - 1u);
     VotePlanes pl;
     pl.clear();
-    for (int wd = 0; wd < 8 && has_cell; wd++) {
-        uint32_t m = mask_s[wd];
+    for (int wd = 0; wd < nw && has_cell; wd++) {
+        uint32_t m = mask_s[tl * 8 + wd];
         while (m) {
             const int h = wd * 32 + __ffs(m) - 1;
             m &= m - 1;
@@ -701,8 +710,8 @@ k_vote_coarse_exact(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const i
             pl.add(v);
         }
     }
-    const long long ncell = (long long)ntile * g.bins[1] * g.bins[2] * Bl;
-    const long long co = ((long long)e * gridDim.x + blockIdx.x) * Kc;
+    const long long ncell = (long long)ntile * Bp * g.bins[2] * Bl;
+    const long long co = ((long long)e * gridDim.x + blockIdx.x) * Kc;   // lists: one tile a block
     coarse_output(g, pl, has_cell, d, p, w, z, hist_s, hist ? hist + (long long)e * kHistBins : nullptr,
                   votes ? votes + (long long)e * ncell : nullptr, cand_k ? cand_k + co : nullptr,
                   cand_v ? cand_v + co : nullptr, Kc);
@@ -779,8 +788,10 @@ void launch_vote_coarse(const DevGeom &g, int prec, int ev0, int n_ev, const Hit
     if (prec == APO_F64_MID) {
         launch_coarse_cert<kMid>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K, skip);
     } else if (prec == APO_F64_EXACT) {
-        const CoarsePlan P = coarse_plan(g, true, 1);
-        k_vote_coarse_exact<<<dim3((unsigned)P.n_tiles, n_ev), P.per, ExactSmem::total(g.bins[4]), s>>>(
+        int threads;
+        const CoarsePlan P = exact_plan(g, cand_k != nullptr, &threads);
+        dim3 grid((unsigned)((P.n_tiles + P.group - 1) / P.group), n_ev);
+        k_vote_coarse_exact<<<grid, threads, ExactSmem::total(g.bins[4]), s>>>(
             g, P, ev0, hd, n_hits, active, votes, hist, status, ctr, cand_k, cand_v, K, skip);
     } else if (prec == APO_F32) {
         launch_coarse_cert<32>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K, skip);
