@@ -165,13 +165,37 @@ __device__ __noinline__ bool box_refuses(const CertBox *b, float2 L, const void 
     }
 }
 
-// Hits no parent could decide for a cell, one by one: with `own` (the parent had no bound) the
-// cell's own evaluation with errors, then the reference program.  mask: tan(lambda) cells l0 + bit
+// The FP32 program's votes of one hit for the cells c with tan(lambda) cells l0 + bit, bits of `mask`;
+// they share its tan(lambda)-free part.  rec: the staged FP32 record.
+static __device__ __noinline__ uint32_t program_f32(const DevGeom &g, const Cell<double> &c, int level, int l0, uint32_t mask,
+                                             const void *rec) {
+    Cell<float> x{to_prec<float>(c.D), to_prec<float>(c.S0), to_prec<float>(c.C0),
+                  to_prec<float>(c.W), to_prec<float>(c.Z), IV<float>{0.f, 0.f}};
+    Hit<float> h = load_hit<float>(rec);
+    if (mirror_cell(x)) mirror_hit(h);
+    if (le0(x.W.lo)) return mask;
+    const IV<float> R = recip(x.W);
+    const Pre<float> p = prefix(x, h, g.k);
+    if (p.novote) return 0u;
+    if (p.guard) return mask;
+    uint32_t yes = 0;
+#pragma unroll 1
+    while (mask) {
+        const int b = __ffs(mask) - 1;
+        mask &= mask - 1;
+        if (tail(p, to_prec<float>(edge(g, 4, level, l0 + b)), h, R, x.W, g.k)) yes |= 1u << b;
+    }
+    return yes;
+}
+
+// Hits no parent could decide for a cell, one by one: FP64 with `own` (the parent had no bound) by the
+// cell's own evaluation with errors first, then the reference program; FP32 by the program at once, which
+// costs no more than an evaluation with errors.  mask: tan(lambda) cells l0 + bit
 // in question; returns those that vote.  Not inlined: about one pair in 10^4 comes here, and its
 // registers stay out of the callers' loops.
 template <int K>
 __device__ __noinline__ uint32_t resolve(const DevGeom &g, int level, int d, int p, int w, int z, int l0,
-                                         uint32_t mask, bool own, const HitRecD *hd, const HitRecF *hf) {
+                                         uint32_t mask, bool own, const HitRecD *hd, const void *hf) {
     Cell<double> c{edge(g, 0, level, d), sin_phi0(g, level, p), cos_phi0(g, level, p), edge(g, 2, level, w),
                    edge(g, 3, level, z), {0.0, 0.0}};
     uint32_t yes = 0;
@@ -187,8 +211,9 @@ __device__ __noinline__ uint32_t resolve(const DevGeom &g, int level, int d, int
             if (mid_vote_pair(c, m, pt::centre(edge(g, 4, level, l0 + b)), load_hit<double>(hd))) yes |= 1u << b;
         }
         return yes;
+    } else if constexpr (K == 32) {
+        return program_f32(g, c, level, l0, mask, hf);
     } else {
-        using T = typename RefOf<K>::T;
         const IV<double> L0 = edge(g, 4, level, l0);
         c.L = L0;
         CertBox box = cert_box<K>(c, L0, L0);
@@ -202,12 +227,7 @@ __device__ __noinline__ uint32_t resolve(const DevGeom &g, int level, int d, int
                 const float e = box_error<K>(&box, hf, g.k.outgoing != 0, true);
                 v = e == -1.f ? cert::kNo : (e == -2.f ? cert::kYes : cert::kUnknown);
             }
-            if (v == cert::kUnknown) {
-                const Cell<T> ct{to_prec<T>(c.D), to_prec<T>(c.S0), to_prec<T>(c.C0),
-                                 to_prec<T>(c.W), to_prec<T>(c.Z), to_prec<T>(c.L)};
-                const void *rec = K == 64 ? static_cast<const void *>(hd) : static_cast<const void *>(hf);
-                v = vote_pair<T>(ct, load_hit<T>(rec), g.k) ? cert::kYes : cert::kNo;
-            }
+            if (v == cert::kUnknown) v = vote_pair<double>(c, load_hit<double>(hd), g.k) ? cert::kYes : cert::kNo;
             if (v == cert::kYes) yes |= 1u << b;
         }
         return yes;

@@ -340,6 +340,9 @@ __device__ __forceinline__ void add_counts(unsigned long long *ctr, const unsign
 // FP64 votes 377 -> 9.7 ms (K best per tile), midpoint form 1077 -> 5.3 ms; FP32 votes of 1024 events
 // 55.7 -> 31.5 ms.  3.1 (FP32) and 2.9 (FP64) instructions a clock and SM of 4.
 //
+// FP32 pairs without a bound (wide cells) are the program's at once, all bins of a hit after one prefix: 256 events,
+// 16x3x2x16x7 cells, 1.30 -> 0.56 ms; one event, 5x6x6x5x5 cells, 0.148 -> 0.088 ms.
+//
 // A block is 128 threads and takes up to four tiles, so that phases 1 and 2, whose chains a single
 // tile cannot hide, keep all its warps busy (fewer where the launch would have too few blocks).
 // Phase 2's bin tests take 39.5 ms to 33.4 (FP32, 1024 events); with one tile a block they cost more
@@ -536,6 +539,10 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan 
                     yes = all;
                 } else {
                     unk = own_s[tl * kHitCap + h];
+                    if (K == 32 && unk) {   // the tile's lanes share the bins: no queue
+                        yes = program_f32(g, c64, 0, 0, unk, hs + h * 80);
+                        unk = 0u;
+                    }
                 }
                 if (!guard && lm) {
                     const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
@@ -907,8 +914,12 @@ k_vote_cells(const __grid_constant__ DevGeom g, const HitRecD *hd, const HitRecF
             if (guard) {
                 r = cert::kYes;
             } else if (!(e < 1e30f)) {
-                r = cert::kUnknown;
-                own = true;
+                if constexpr (K == 32) {
+                    r = program_f32(g, c64, level, idx[4], 1u, hs + h * 80) ? cert::kYes : cert::kNo;
+                } else {
+                    r = cert::kUnknown;
+                    own = true;
+                }
             } else {
                 const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
                 const typename Prog<K>::Pre pre = Prog<K>::prefix(c, hx);
@@ -1107,8 +1118,16 @@ __device__ __forceinline__ void children_warp(const DevGeom &g, const unsigned c
                     v0++;
                     v1++;
                 } else if (!(e < 1e30f)) {
-                    unk = 3u;
-                    own = true;
+                    if constexpr (K == 32) {
+                        int x[5];
+                        pair_index(g, parents_e[p0 + pl], lane & 15, x);
+                        const uint32_t y = resolve<K>(g, level, x[0], x[1], x[2], x[3], x[4], 3u, true, nullptr, hs + h * 80);
+                        v0 += y & 1u;
+                        v1 += y >> 1;
+                    } else {
+                        unk = 3u;
+                        own = true;
+                    }
                 } else {
                     const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
                     const typename Prog<K>::Pre pre = Prog<K>::prefix(c, hx);

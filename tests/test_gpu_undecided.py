@@ -1,0 +1,36 @@
+"""Pairs that no shared bound decides, GPU against oracle: level 0 and bisected cells so wide that a
+tile, a tan(lambda) bin or a parent has no bound for most hits (there the FP32 votes are the program's
+own, several bins after one prefix)."""
+import numpy as np
+import pytest
+
+from gen import chamber, grid as G
+from oracle import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2401_04576_gb300 import apo  # noqa: E402
+
+PRECS = [(apo.F64, 0), (apo.F32, 1), (apo.F64 | apo.OUTGOING, 0 | O.OUTGOING), (apo.F32 | apo.OUTGOING, 1 | O.OUTGOING)]
+
+
+@pytest.mark.parametrize("prec,oprec", PRECS)
+@pytest.mark.parametrize("bins", [[4, 4, 4, 4, 4], [5, 6, 6, 5, 5], [16, 3, 2, 16, 7], [2, 3, 2, 3, 32]])
+def test_wide_cells(bins, prec, oprec):
+    w, g = chamber.make_wires(), G.make_grid(bins, 2, 9)
+    ev = chamber.multi_track_events(2, seed=sum(bins), w=w)
+    geom, tab, hits = apo.Geometry(g, w), O.Tables(g, w), apo.DeviceHits.from_events(ev)
+    votes = apo.vote(geom, hits, precision=prec).cpu().numpy()
+    tracks, _ = apo.solve_batch(geom, hits, apo.solve_opts(precision=[prec] * 3))
+    got = apo.tracks_to_numpy(tracks, ev.n_events)
+    for e in range(ev.n_events):
+        a, b = ev.offsets[e], ev.offsets[e + 1]
+        np.testing.assert_array_equal(votes[e], O.vote_coarse(tab, ev.wire_id[a:b], ev.drift[a:b], oprec))
+        r = O.solve_event(tab, ev.wire_id[a:b], ev.drift[a:b], [oprec] * 3)
+        assert got[e, 0]["votes"] == r["votes"]
+        assert np.array_equal(got[e, 0]["p"], r["p"]) and np.array_equal(got[e, 0]["w"], r["w"])
+    geom.close()
