@@ -548,9 +548,8 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan 
                     const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
                     const typename Prog<K>::Pre pre = Prog<K>::prefix(c, hx);
                     cnt[4]++;
-                    const int dir = Prog<K>::direction(pre, outgoing, e);
+                    const int dir = settle_direction<K>(Prog<K>::direction(pre, outgoing, e), c64, hd_e + h, hs + h * 80);
                     if (dir == cert::kNo) unk = 0;
-                    if (dir == cert::kUnknown) unk |= lm;
                     if (dir == cert::kYes) {
                         cnt[5] += __popc(lm);
 #pragma unroll 1

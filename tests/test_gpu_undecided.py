@@ -34,3 +34,16 @@ def test_wide_cells(bins, prec, oprec):
         assert got[e, 0]["votes"] == r["votes"]
         assert np.array_equal(got[e, 0]["p"], r["p"]) and np.array_equal(got[e, 0]["w"], r["w"])
     geom.close()
+
+
+@pytest.mark.parametrize("prec,oprec", PRECS[2:])
+def test_direction_left_open(prec, oprec):
+    """Tiles whose bound is too wide for the direction condition of some cells, many bins each."""
+    w, g = chamber.make_wires(), G.make_grid([16, 8, 4, 16, 7], 1, 9)
+    ev = chamber.single_track_events(2, seed=9, w=w)
+    geom, tab = apo.Geometry(g, w), O.Tables(g, w)
+    votes = apo.vote(geom, apo.DeviceHits.from_events(ev), precision=prec).cpu().numpy()
+    for e in range(ev.n_events):
+        a, b = ev.offsets[e], ev.offsets[e + 1]
+        np.testing.assert_array_equal(votes[e], O.vote_coarse(tab, ev.wire_id[a:b], ev.drift[a:b], oprec))
+    geom.close()
