@@ -820,19 +820,36 @@ __device__ __forceinline__ bool key_cell(const DevGeom &g, int level, uint64_t k
                          edge(g, 2, level, idx[2]), edge(g, 3, level, idx[3]), edge(g, 4, level, idx[4])};
     return valid;
 }
-__device__ __forceinline__ IV<double> warp_hull(IV<double> a) {
+// Floats in the order of signed integers (an involution), and the smallest range around a warp's.
+__device__ __forceinline__ int fkey(float x) { const int b = __float_as_int(x); return b ^ ((b >> 31) & 0x7fffffff); }
+__device__ __forceinline__ float2 warp_range(float lo, float hi) {
+    const int l = __reduce_min_sync(0xffffffffu, fkey(lo)), h = __reduce_max_sync(0xffffffffu, fkey(hi));
+    return make_float2(__int_as_float(l ^ ((l >> 31) & 0x7fffffff)), __int_as_float(h ^ ((h >> 31) & 0x7fffffff)));
+}
+// The smallest box around the cells of the warp's lanes (`has`; at least one), from their FP32 ends v.  One
+// that reaches omega = 0 is a guard: it has no bound.
+__device__ __forceinline__ CertBox warp_box(const float2 (&v)[6], bool has) {
+    CertBox b;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        a = hull2(a, IV<double>{__shfl_xor_sync(0xffffffffu, a.lo, o), __shfl_xor_sync(0xffffffffu, a.hi, o)});
-    return a;
+    for (int q = 0; q < 6; q++) b.v[q] = warp_range(has ? v[q].x : INFINITY, has ? v[q].y : -INFINITY);
+    b.mir = b.v[3].y < 0.f;
+    b.guard = !b.mir && !(b.v[3].x > 0.f);
+    if (b.mir)
+        for (int q = 0; q < 4; q++)
+            if (q != 2) b.v[q] = make_float2(-b.v[q].y, -b.v[q].x);
+    return b;
 }
 
 // FP64 (K = 64) and outward FP32 (K = 32) votes, decided by certified FP32 end points (see
 // coarse_block).  The parent is the smallest box around the warp's 32 cells: for the 32 children
-// of one cell, as apo_refine lists them, that cell; for scattered keys it is wide, its bound
-// decides little, and the pairs are evaluated one by one with their own bounds.
-// The children of 33 kept cells of 37 events, FP64: 0.76 -> 0.055 ms.
-constexpr int kCellsThreads = 128;
+// of one cell, as apo_refine lists them, that cell; for scattered keys it is wide, or holds both signs
+// of omega, and decides little.  FP64 pairs then go one by one with their own bounds.  FP32 pairs are
+// the program's: all of them where no hit has a bound, or those of the first hit that leaves a quarter of the
+// lanes undecided and of the hits after it.
+// FP64, the children of 33 kept cells of 37 events: 0.76 -> 0.055 ms.  FP32, 8 events x 65536 keys within three
+// cells of a track's: 0.23 ms, scattered: 0.30 ms; children of 2048 cells of 16 events: 0.32 ms (the program alone,
+// one key a thread: 0.27, 0.27 and 0.49 ms; pairs one by one as in FP64: 0.30, 0.63 and 0.42 ms).
+constexpr int kCellsThreads = 128, kCellsOpen = 8;   // undecided lanes from which a warp stops certifying
 struct WarpScratch {   // one warp's parent, and its queue
     CertBox box;
     float err[kHitCap];
@@ -867,73 +884,95 @@ k_vote_cells(const __grid_constant__ DevGeom g, const HitRecD *hd, const HitRecF
     const uint32_t *act = active ? active + (long long)ev * 8 : nullptr;
     const long long j0 = (long long)blockIdx.x * kCellsThreads + (tid & ~31), j = j0 + lane;   // this warp's keys
     const uint64_t *keys_e = keys + (long long)ev * n_per_ev;
-    const IV<double> none{1e300, -1e300};
-    Cell<double> c64{none, none, none, none, none, none};
+    Cell<double> c64{};
     int idx[5] = {0, 0, 0, 0, 0};
     const bool in = j < n_per_ev, has = in && key_cell(g, level, keys_e[j], idx, c64);
-    {   // the warp's parent, one hit per lane
-        const bool any = __any_sync(0xffffffffu, has);
-        const Cell<double> b{warp_hull(c64.D), warp_hull(c64.S0), warp_hull(c64.C0), warp_hull(c64.W),
-                             warp_hull(c64.Z), warp_hull(c64.L)};
-        if (lane == 0) ws.box = cert_box<K>(b, none, none);
+    // the cell's FP32 ends: rounded to nearest, or outward for the FP32 program (converted once: conversions
+    // from FP64 run on its pipe)
+    float2 fe[6];
+    const IV<double> de[6] = {c64.D, c64.S0, c64.C0, c64.W, c64.Z, c64.L};
+#pragma unroll
+    for (int q = 0; q < 6; q++) {
+        const IV<float> o = to_prec<float>(de[q]);
+        fe[q] = K == 32 ? make_float2(o.lo, o.hi) : make_float2((float)de[q].lo, (float)de[q].hi);
+    }
+    // the warp's parent, one hit per lane; without one when the cells are on both sides of omega = 0
+    bool plain = !__any_sync(0xffffffffu, has) ||
+                 (__any_sync(0xffffffffu, has && fe[3].y < 0.f) && __any_sync(0xffffffffu, has && !(fe[3].y < 0.f)));
+    if (!plain) {
+        const CertBox box = warp_box(fe, has);
+        // a hull over more than a radian of phi0 has hardly a bound
+        plain = K == 32 && (box.v[1].y - box.v[1].x > 1.f || box.v[2].y - box.v[2].x > 1.f);
+        if (lane == 0) ws.box = box;
         __syncwarp();
+    }
+    {
+        bool open = true;
         for (int h = lane; h < nw * 32; h += 32) {
-            bool keep = any && h < nh && (!act || ((act[h >> 5] >> (h & 31)) & 1u));
-            if (keep) {
-                const float e = box_error<K>(&ws.box, hs + h * 80, outgoing);
-                ws.err[h] = e;
-                keep = !(e < 0.f);
-            }
+            bool keep = h < nh && (!act || ((act[h >> 5] >> (h & 31)) & 1u));
+            float e = NAN;
+            if (keep && !plain) e = box_error<K>(&ws.box, hs + h * 80, outgoing);
+            open = open && !(e < 1e30f);
+            keep = keep && !(e < 0.f);
+            ws.err[h] = e;
             const unsigned m = __ballot_sync(0xffffffffu, keep);
             if (lane == 0) ws.mask[h >> 5] = m;
         }
+        plain = plain || __all_sync(0xffffffffu, open);
         __syncwarp();
     }
     bool guard;
     const bool mir = omega_sign<K>(c64.W, &guard);
-    const typename Prog<K>::CellT c = Prog<K>::cell(g, level, idx[1], c64, mir);
-    const float2 L = Prog<K>::tanl(c64.L);
-    int v = 0, wd = -1, nq = 0;
+    auto flip = [&](int q) { return mir ? cert::X<0>{-fe[q].y, -fe[q].x, 0.f} : cert::X<0>{fe[q].x, fe[q].y, 0.f}; };
+    const cert::CellX<0> c{flip(0), flip(1), xf<0>(fe[2]), flip(3), xf<0>(fe[4]), xf<0>(fe[5])};
+    const cert::X<0> R = cert::recip(c.W);
+    int v = 0, nq = 0, wd = 0;
+    uint32_t m = nw ? ws.mask[0] : 0u;
+    auto next = [&]() {   // the next hit in question, the same for all lanes; -1: none left
+        while (!m && ++wd < nw) m = ws.mask[wd];
+        return m ? wd * 32 + __ffs(m) - 1 : -1;
+    };
     auto solve = [&](int ol, int oh, bool own, uint32_t om) -> uint32_t {
         int x[5];
         unpack_key(g, keys_e[j0 + ol], x);
         return resolve<K>(g, level, x[0], x[1], x[2], x[3], x[4], om, own, hd_e + oh, hf_e + oh);
     };
     auto take = [&](uint32_t b) { v += (int)b; };
-    uint32_t m = 0;
-    for (;;) {
-        while (has && !m && ++wd < nw) m = ws.mask[wd];
-        const bool more = __any_sync(0xffffffffu, m != 0u);
-        int h = 0, r = cert::kNo;
-        bool own = false;
-        if (m) {
-            h = wd * 32 + __ffs(m) - 1;
-            m &= m - 1;
-            const float e = ws.err[h];
-            if (guard) {
-                r = cert::kYes;
-            } else if (!(e < 1e30f)) {
-                if constexpr (K == 32) {
-                    r = program_f32(g, c64, level, idx[4], 1u, hs + h * 80) ? cert::kYes : cert::kNo;
-                } else {
-                    r = cert::kUnknown;
-                    own = true;
-                }
-            } else {
-                const typename Prog<K>::HitT hx = Prog<K>::hit(hs + h * 80, mir);
-                const typename Prog<K>::Pre pre = Prog<K>::prefix(c, hx);
-                r = Prog<K>::direction(pre, outgoing, e);
-                if (r == cert::kYes) r = Prog<K>::vote(pre, L, c, hx, e);
-                own = true;   // the keys need not be one cell's children
-            }
-            v += r == cert::kYes;
+    for (int h; !(K == 32 && plain) && (h = next()) >= 0; m &= m - 1) {
+        const float e = ws.err[h];
+        int r = has ? (guard ? cert::kYes : cert::kUnknown) : cert::kNo;
+        if (r == cert::kUnknown && e < 1e30f) {
+            const cert::HitX<0> hx = cert_hit<0>(hs + h * 80, mir);
+            const cert::PreX<0> pre = cert::prefix(c, hx);
+            r = cert_direction(pre, outgoing, e);
+            if (r == cert::kYes) r = cert_tail(pre, c.L, hx, R, c.W, e);
         }
-        if (more) nq = ws.q.push(nq, lane, h, own, r == cert::kUnknown ? 1u : 0u);
-        if (nq >= 32 || (!more && nq)) {
+        const unsigned open = __ballot_sync(0xffffffffu, r == cert::kUnknown);
+        if (K == 32 && __popc(open) >= kCellsOpen) break;
+        v += r == cert::kYes;
+        // the keys need not be one cell's children: their own bounds first (FP64)
+        nq = ws.q.push(nq, lane, h, true, r == cert::kUnknown ? 1u : 0u);
+        if (nq >= 32) {
             ws.q.drain(nq, lane, solve, take);
             nq = 0;
         }
-        if (!more) break;
+    }
+    if (nq) ws.q.drain(nq, lane, solve, take);
+    if constexpr (K == 32) {   // what is left
+        IV<float> f[6];
+#pragma unroll
+        for (int q = 0; q < 6; q++) f[q] = {fe[q].x, fe[q].y};
+        Cell<float> x{f[0], f[1], f[2], f[3], f[4], f[5]};
+        mirror_cell(x);
+        const bool all = le0(x.W.lo);
+        const IV<float> Rx = recip(x.W);
+        for (int h; (h = next()) >= 0; m &= m - 1) {
+            if (!has) continue;
+            Hit<float> hx = load_hit<float>(hs + h * 80);
+            if (mir) mirror_hit(hx);
+            const Pre<float> p = prefix(x, hx, g.k);
+            v += all || (!p.novote && (p.guard || tail(p, x.L, hx, Rx, x.W, g.k)));
+        }
     }
     if (in) out_votes[(long long)ev * n_per_ev + j] = has ? v : -1;   // -1: a key outside the level's grid
 }
