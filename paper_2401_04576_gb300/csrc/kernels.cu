@@ -190,17 +190,17 @@ void launch_stage(const DevGeom &g, int n_events, const int32_t *offsets, const 
 // Writes votes[e][lin], lin = d + Bd (p + Bp (w + Bw (z + Bz l))), or each tile's K best cells,
 // and the per-event histogram of vote counts.
 // ---------------------------------------------------------------------------------------
-// The end of a coarse block: each thread's Bl vote counts (its cell (d, p, w, z), every
-// tan(lambda) bin) to vo or, with cand_k, the block's K best cells; the histogram added to hist_e
+// The end of a coarse block: each thread's vote counts (its cell (d, p, w, z), tan(lambda) bins l0 .. l1 - 1)
+// to vo or, with cand_k and every bin, the block's K best cells; the histogram added to hist_e
 // (may be null).  hist_s: kHistBins zeros in shared memory.  The block has whole warps, and so at
 // least a thread per tan(lambda) bin.
 __device__ __forceinline__ void coarse_output(const DevGeom &g, const VotePlanes &pl, bool has_cell, int d, int p,
-                                              int w, int z, uint32_t *hist_s, uint32_t *hist_e, int32_t *vo,
-                                              uint64_t *cand_k, int32_t *cand_v, int K) {
+                                              int w, int z, int l0, int l1, uint32_t *hist_s, uint32_t *hist_e,
+                                              int32_t *vo, uint64_t *cand_k, int32_t *cand_v, int K) {
     const int Bd = g.bins[0], Bp = g.bins[1], Bw = g.bins[2], Bz = g.bins[3], Bl = g.bins[4];
     const int tid = threadIdx.x, nthr = blockDim.x;
     auto vote_of = [&](int l) { return pl.get(l); };
-    for (int l = 0; l < Bl && has_cell; l++) {
+    for (int l = l0; l < l1 && has_cell; l++) {
         const int v = vote_of(l);
         if (!cand_k) {
             long long lin = d + (long long)Bd * (p + (long long)Bp * (w + (long long)Bw * (z + (long long)Bz * l)));
@@ -573,7 +573,7 @@ __device__ __forceinline__ void coarse_block(const DevGeom &g, const CoarsePlan 
             if (!more) break;
         }
         if (cand_k) {
-            coarse_output(g, pl, has, d, p, w, z, hist_s, hist_e, nullptr, cand_k + t * Kc, cand_v + t * Kc, Kc);
+            coarse_output(g, pl, has, d, p, w, z, 0, Bl, hist_s, hist_e, nullptr, cand_k + t * Kc, cand_v + t * Kc, Kc);
             __syncthreads();
             for (int i = tid; i < kHistBins; i += nthr) hist_s[i] = 0;
             __syncthreads();
@@ -616,9 +616,11 @@ k_vote_coarse(const __grid_constant__ DevGeom g, CoarsePlan P, int ev0, const Hi
 }
 
 // The exact-phase program on the coarse grid: FP64, the same tiles.  Full votes: a block takes
-// `group` tiles side by side, so that its 128 threads have a cell each; K best lists: one tile, in
-// whole warps.  Never fewer than 32 threads: the mask's words, and the bins' prefixes of
-// coarse_output, are one thread's each.
+// `group` tiles side by side, so that its 128 threads have a cell each, and gridDim.z blocks share their
+// tan(lambda) bins where there are too few; K best lists: one tile, in whole warps.  Never fewer
+// than 32 threads: the mask's words, and the bins' prefixes of coarse_output, are one thread's each.
+// One event, exact phase: 10^5 cells 7.9 -> 4.3 ms with the bins shared, max-set search on 2x256x16x2x8 26.0 -> 21.8 ms
+// (23.4 with one cell per thread); 16 events of 10^5 the same.
 constexpr int kExactMaxGroup = 32;
 struct ExactSmem {
     static constexpr size_t hits = 0;
@@ -628,12 +630,21 @@ struct ExactSmem {
     static constexpr size_t L = bar + 16;
     __host__ __device__ static size_t total(int Bl) { return L + 16 * (size_t)Bl; }
 };
-__host__ inline CoarsePlan exact_plan(const DevGeom &g, bool lists, int *threads) {
-    CoarsePlan P = coarse_plan(g, true, 1);
-    const int fit = kCoarseThreads / P.per;
-    P.group = P.tiles = lists || fit < 2 ? 1 : (fit > kExactMaxGroup ? kExactMaxGroup : fit);
-    *threads = (P.group * P.per + 31) & ~31;
-    return P;
+struct ExactPlan {
+    CoarsePlan P;
+    int threads, split;
+};
+__host__ inline ExactPlan exact_plan(const DevGeom &g, bool lists, int n_ev) {
+    ExactPlan E{coarse_plan(g, true, 1), 0, 1};
+    const int fit = kCoarseThreads / E.P.per;
+    E.P.group = E.P.tiles = lists || fit < 2 ? 1 : (fit > kExactMaxGroup ? kExactMaxGroup : fit);
+    E.threads = (E.P.group * E.P.per + 31) & ~31;
+    if (!lists) {   // two waves of three blocks on 152 SMs
+        const long long blocks = (E.P.n_tiles + E.P.group - 1) / E.P.group * n_ev, want = 2 * 3 * 152;
+        E.split = blocks >= want ? 1 : (int)((want + blocks - 1) / blocks);
+        if (E.split > g.bins[4]) E.split = g.bins[4];
+    }
+    return E;
 }
 
 __global__ void __launch_bounds__(kCoarseThreads, 3)
@@ -646,6 +657,7 @@ k_vote_coarse_exact(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const i
     const int Bd = g.bins[0], Bp = g.bins[1], Bz = g.bins[3], Bl = g.bins[4];
     const int ntile = Bd * Bz, nthr = blockDim.x, tid = threadIdx.x, lane = tid & 31;
     const long long tile0 = (long long)blockIdx.x * P.group;
+    const int l0 = (int)(blockIdx.z * Bl / gridDim.z), l1 = (int)((blockIdx.z + 1) * Bl / gridDim.z);   // its bins
     unsigned char *hs = smem + ExactSmem::hits;
     uint32_t *hist_s = reinterpret_cast<uint32_t *>(smem + ExactSmem::hist);
     uint32_t *mask_s = reinterpret_cast<uint32_t *>(smem + ExactSmem::mask);
@@ -675,7 +687,7 @@ k_vote_coarse_exact(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const i
             const bool row = c0 / Bd == (c1 - 1) / Bd;   // cells of one z0 bin
             const Cell<double> par{edge_span(g, 0, 0, row ? c0 % Bd : 0, row ? (c1 - 1) % Bd : Bd - 1), sin_phi0(g, 0, p),
                                    cos_phi0(g, 0, p), edge(g, 2, 0, w), edge_span(g, 3, 0, c0 / Bd, (c1 - 1) / Bd),
-                                   edge_span(g, 4, 0, 0, Bl - 1)};
+                                   edge_span(g, 4, 0, l0, l1 - 1)};
             cnt[0]++;
             keep = vote_pair_exact(par, load_hit<double>(hs + h * 80), k);
         }
@@ -710,15 +722,15 @@ k_vote_coarse_exact(DevGeom g, CoarsePlan P, int ev0, const HitRecD *hd, const i
             if (pre.guard) { pl.add(all); continue; }
             uint32_t v = 0;
 #pragma unroll 1
-            for (int l = 0; l < Bl; l++)
+            for (int l = l0; l < l1; l++)
                 if (tail_exact(pre, Ls[l], hx, R, c.W, k)) v |= 1u << l;
-            cnt[2] += Bl;
+            cnt[2] += l1 - l0;
             pl.add(v);
         }
     }
     const long long ncell = (long long)ntile * Bp * g.bins[2] * Bl;
     const long long co = ((long long)e * gridDim.x + blockIdx.x) * Kc;   // lists: one tile a block
-    coarse_output(g, pl, has_cell, d, p, w, z, hist_s, hist ? hist + (long long)e * kHistBins : nullptr,
+    coarse_output(g, pl, has_cell, d, p, w, z, l0, l1, hist_s, hist ? hist + (long long)e * kHistBins : nullptr,
                   votes ? votes + (long long)e * ncell : nullptr, cand_k ? cand_k + co : nullptr,
                   cand_v ? cand_v + co : nullptr, Kc);
     add_counts(ctr, cnt);
@@ -794,11 +806,10 @@ void launch_vote_coarse(const DevGeom &g, int prec, int ev0, int n_ev, const Hit
     if (prec == APO_F64_MID) {
         launch_coarse_cert<kMid>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K, skip);
     } else if (prec == APO_F64_EXACT) {
-        int threads;
-        const CoarsePlan P = exact_plan(g, cand_k != nullptr, &threads);
-        dim3 grid((unsigned)((P.n_tiles + P.group - 1) / P.group), n_ev);
-        k_vote_coarse_exact<<<grid, threads, ExactSmem::total(g.bins[4]), s>>>(
-            g, P, ev0, hd, n_hits, active, votes, hist, status, ctr, cand_k, cand_v, K, skip);
+        const ExactPlan E = exact_plan(g, cand_k != nullptr, n_ev);
+        dim3 grid((unsigned)((E.P.n_tiles + E.P.group - 1) / E.P.group), n_ev, E.split);
+        k_vote_coarse_exact<<<grid, E.threads, ExactSmem::total(g.bins[4]), s>>>(
+            g, E.P, ev0, hd, n_hits, active, votes, hist, status, ctr, cand_k, cand_v, K, skip);
     } else if (prec == APO_F32) {
         launch_coarse_cert<32>(g, ev0, n_ev, hd, hf, n_hits, active, votes, hist, status, s, ctr, cand_k, cand_v, K, skip);
     } else {   // APO_F64 and APO_F64_FILTERED: the same votes, the same kernel
