@@ -443,15 +443,13 @@ def background_study(w, n_events: int = 1024, seed: int = 4, n_maxset: int = 512
     prec = [apo.F32] * 5 + [apo.F64] * 2
     launch = {}
     results = {}
-    # the same search through the per-level launches recorded as one CUDA graph, through the
-    # tune.persistent set, and with the knobs apo_autotune picks on a 1024-event sample
+    # the same search recorded as one CUDA graph, with the default knobs and with those that
+    # apo_autotune picks on a 1024-event sample
     sample = apo.DeviceHits.from_events(ev.subset(range(min(1024, ev.n_events))))
     best, _ = apo.autotune(geom, sample, apo.solve_opts(precision=prec, max_tracks=5, min_votes=6))
-    for name, tune, graph in (("graph", apo.ApoTune(0, 1, 256, 0, persistent=0), True),
-                              ("persistent", apo.ApoTune(0, 1, 256, 0, persistent=1), False),
-                              ("autotuned", best, best.persistent == 0)):
+    for name, tune in (("graph", apo.ApoTune(0, 1, 256, 0)), ("autotuned", best)):
         o = apo.solve_opts(precision=prec, max_tracks=5, min_votes=6, hit_track=ht, tune=tune,
-                           use_graph=graph)
+                           use_graph=True)
         ws = geom.workspace(ev.n_events, opts=o)
         apo.solve_batch(geom, hits, o, workspace=ws)      # warm-up (and graph recording)
         torch.cuda.synchronize()
@@ -468,8 +466,8 @@ def background_study(w, n_events: int = 1024, seed: int = 4, n_maxset: int = 512
         results[name] = (apo.tracks_to_numpy(tracks, ev.n_events, 5).copy(), nt.cpu().numpy().copy(),
                          ht.cpu().numpy().copy())
         del ws
-    same = all(np.array_equal(results["graph"][i].view(np.uint8), results[k][i].view(np.uint8))
-               for i in range(3) for k in ("persistent", "autotuned"))
+    same = all(np.array_equal(results["graph"][i].view(np.uint8), results["autotuned"][i].view(np.uint8))
+               for i in range(3))
     fastest = min(launch, key=lambda k: launch[k]["ms"])
     ms = launch[fastest]["ms"]
     tracks, nt, hts = results[fastest]
@@ -1070,20 +1068,6 @@ def run_case(args) -> None:
         torch.cuda.synchronize()
         print(json.dumps({"case": args.case, "events": ev.n_events, "ok": True}))
         return
-    if args.case == "solve-persist":   # the multi-track batch with tune.persistent set
-        from gen import chamber, grid as G
-        w = chamber.make_wires()
-        g4 = G.make_grid([10] * 5, 6, 64)
-        ev = chamber.multi_track_events(args.events, seed=4, w=w)
-        geom = apo.Geometry(g4, w)
-        o = apo.solve_opts(precision=[apo.F32] * 5 + [apo.F64] * 2, max_tracks=5, min_votes=6,
-                           tune=apo.ApoTune(0, 1, 256, 0, persistent=1))
-        hits = apo.DeviceHits.from_events(ev)
-        for _ in range(2):
-            apo.solve_batch(geom, hits, o)
-        torch.cuda.synchronize()
-        print(json.dumps({"case": args.case, "events": ev.n_events, "ok": True}))
-        return
     w, g, ev = make_inputs()
     ev = ev.subset(range(args.events))
     geom = apo.Geometry(g, w)
@@ -1137,7 +1121,7 @@ def main(argv=None):
     ap.add_argument("--serve-seconds", type=float, default=1.0)
     ap.add_argument("--case", default=None,
                     choices=["coarse-f64", "coarse-f32", "coarse-f32-full", "coarse-mid", "solve-f64",
-                             "solve-f32", "solve-bulk", "solve-maxset", "solve-maxset-multi", "solve-persist",
+                             "solve-f32", "solve-bulk", "solve-maxset", "solve-maxset-multi",
                              "four-f32", "four-f64"],
                     help="run one small profiling case instead of the benchmark")
     ap.add_argument("--events", type=int, default=64)

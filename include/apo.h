@@ -140,19 +140,19 @@ typedef struct {
  * evaluates the same interval program cell by cell); apo_autotune picks them by timing.
  * Zero means the default. */
 typedef struct {
-    int32_t coarse_filter;   /* 1: FP64 level 0 as APO_F64_FILTERED (the same kernel) */
-    int32_t cells_filter;    /* 1: the same for the bisected cells of levels >= 1 */
+    int32_t coarse_filter;   /* accepted, without effect (APO_F64_FILTERED runs APO_F64's kernels) */
+    int32_t cells_filter;    /* the same */
     int32_t cells_block;     /* threads per block of APO_F64_EXACT's bisected cells: 128 or 256 */
     int32_t chunk_events;    /* events per level-0 launch (at most the workspace's chunk) */
     int32_t coarse_full;     /* 1 (APO_SCHED_TOPK): level 0 writes every cell's vote and selects
                                 from them, instead of each tile keeping its topk best cells
                                 (more workspace, fewer instructions per tile); the same
                                 kept set either way */
-    int32_t persistent;      /* 1 (APO_SCHED_TOPK only): asks for one launch per batch; runs the
-                                per-level launches, which leave an event as soon as its
-                                extraction has ended and take about half the time of blocks
-                                that run whole events.  Levels must share their APO_OUTGOING
-                                flag and use APO_F64, APO_F32 or APO_F64_FILTERED; no trace. */
+    int32_t persistent;      /* accepted, without effect on the launches (APO_SCHED_TOPK: every
+                                round leaves the events whose extraction has ended; one launch
+                                whose blocks ran whole events took 1.5 to 3.8 times as long).
+                                When set, levels must still share their APO_OUTGOING flag and use
+                                APO_F64, APO_F32 or APO_F64_FILTERED, without a trace. */
 } apo_tune;
 
 /* Options of apo_solve_batch.  precision[L] selects FP64 or FP32 intervals at level L

@@ -329,12 +329,10 @@ def autotune(geom: Geometry, hits: DeviceHits, opts: ApoSolveOpts | None = None,
     """apo_autotune: the fastest execution knobs for this batch (results never change)."""
     o = opts if opts is not None else solve_opts()
     if workspace is None:   # room for every candidate
-        op = ApoSolveOpts.from_buffer_copy(o)
-        op.tune.persistent = 1
         of = ApoSolveOpts.from_buffer_copy(o)
         of.tune.coarse_full = 1
         torch = _torch()
-        ws = torch.empty(max(geom.workspace_bytes(hits.n_events, x) for x in (o, op, of)),
+        ws = torch.empty(max(geom.workspace_bytes(hits.n_events, x) for x in (o, of)),
                          dtype=torch.uint8, device="cuda")
     else:
         ws = workspace

@@ -475,7 +475,7 @@ int validate_solve(const apo_geometry *g, const apo_hits *hits, const apo_solve_
         if (key_bits_total(g->dg) > 50) return fail(APO_EINVAL, "APO_SCHED_TOPK needs keys of at most 50 bits");
         if ((long long)g->dg.bins[1] * g->dg.bins[2] * 2 > 8192)
             return fail(APO_EINVAL, "APO_SCHED_TOPK needs bins[1] * bins[2] <= 4096");
-        if (o->tune.persistent) {
+        if (o->tune.persistent) {   // accepted for its former launch; what that refused stays refused
             for (int i = 0; i <= lv; i++) {
                 const int p = o->precision[i] & ~APO_OUTGOING;
                 if (p != APO_F64 && p != APO_F32 && p != APO_F64_FILTERED)
@@ -642,11 +642,7 @@ int enqueue_solve(const apo_geometry *g, const apo_hits *hits, const apo_solve_o
     const double width = 3.0 * o->mask_sigma;   // round-to-nearest, as the oracle
     const int chunk = (o->tune.chunk_events > 0 && o->tune.chunk_events < L.chunk) ? o->tune.chunk_events : L.chunk;
     const int block = o->tune.cells_block ? o->tune.cells_block : 256;
-    auto prec_at = [&](int lev) {
-        int p = o->precision[lev] & ~APO_OUTGOING;
-        bool filt = lev == 0 ? o->tune.coarse_filter != 0 : o->tune.cells_filter != 0;
-        return (p == APO_F64 && filt) ? (int)APO_F64_FILTERED : p;
-    };
+    auto prec_at = [&](int lev) { return (int)(o->precision[lev] & ~APO_OUTGOING); };
     DevGeom gl[APO_MAX_LEVELS + 1];   // per level: the geometry with that level's direction flag
     for (int lev = 0; lev <= lv; lev++) gl[lev] = geom_for(g, o->precision[lev]);
     if (o->schedule == APO_SCHED_MAXSET)

@@ -23,14 +23,9 @@ APO_CERT Pt recip(Pt a) { return {rcp_a(a.v)}; }
 APO_CERT Pt sqrtx(Pt a) { return {sqrt_a(a.v)}; }
 APO_CERT Pt rsqrtx(Pt a) { return {rsqrt_a(a.v)}; }
 template <int K> APO_CERT X<K> rsqrtx(X<K> a) { return recip(sqrtx(a)); }   // two units for rsqrt's one
-template <typename N> APO_CERT N num(double v);
-template <> APO_CERT Pt num<Pt>(double v) { return {(float)v}; }
-template <> APO_CERT X<64> num<X<64>>(double v) { return mk<64>(v, v); }
-template <> APO_CERT X<32> num<X<32>>(double v) { return mk<32>(v, v); }
 template <typename N> APO_CERT N numf(float v);            // from a hit's value rounded down
 template <> APO_CERT Pt numf<Pt>(float v) { return {v}; }
 template <> APO_CERT X<64> numf<X<64>>(float v) { return point(sc<64>(v)); }
-template <> APO_CERT X<32> numf<X<32>>(float v) { return point(sc<32>(v)); }
 APO_CERT X<0> ivp(Pt a) { X<0> r; r.lo = r.hi = a.v; r.e = 0.f; return r; }
 template <int K> APO_CERT X<K> ivp(X<K> a) { return a; }
 

@@ -163,22 +163,12 @@ template <> __device__ __forceinline__ IV<float> divi<float>(IV<float> a, IV<flo
 template <typename T> __device__ __forceinline__ IV<T> mul_nn(IV<T> a, IV<T> b) {
     return {rd_mul(a.lo, nonneg_lo(a.lo) ? b.lo : b.hi), ru_mul(a.hi, nonneg_lo(a.hi) ? b.hi : b.lo)};
 }
-// a * b for b <= 0 (b.hi <= 0): a b is decreasing in a, so the ends are a.hi and a.lo, each
-// times the end of b chosen by its sign.
-template <typename T> __device__ __forceinline__ IV<T> mul_np(IV<T> a, IV<T> b) {
-    return {rd_mul(a.hi, nonneg_lo(a.hi) ? b.lo : b.hi), ru_mul(a.lo, nonneg_lo(a.lo) ? b.hi : b.lo)};
-}
-// FP32 forms of the two above with min / max instead of sign tests and selects: for
-// b >= 0 the lower end is the smaller of a.lo b.lo and a.lo b.hi, the upper end the larger
-// of a.hi b.lo and a.hi b.hi (mirrored for b <= 0); the same values, one ALU instruction
-// per end instead of two.
+// Its FP32 form with min / max instead of sign tests and selects: the lower end is the smaller
+// of a.lo b.lo and a.lo b.hi, the upper end the larger of a.hi b.lo and a.hi b.hi; the same
+// values, one ALU instruction per end instead of two.
 template <> __device__ __forceinline__ IV<float> mul_nn<float>(IV<float> a, IV<float> b) {
     return {fminf(__fmul_rd(a.lo, b.lo), __fmul_rd(a.lo, b.hi)),
             fmaxf(__fmul_ru(a.hi, b.lo), __fmul_ru(a.hi, b.hi))};
-}
-template <> __device__ __forceinline__ IV<float> mul_np<float>(IV<float> a, IV<float> b) {
-    return {fminf(__fmul_rd(a.hi, b.lo), __fmul_rd(a.hi, b.hi)),
-            fmaxf(__fmul_ru(a.lo, b.lo), __fmul_ru(a.lo, b.hi))};
 }
 // a * b for a >= 0 and b >= 0
 template <typename T> __device__ __forceinline__ IV<T> mul_pp(IV<T> a, IV<T> b) {

@@ -107,16 +107,16 @@ void launch_stage(const DevGeom &g, int n_events, const int32_t *offsets, const 
                   uint32_t *active, int32_t *done, unsigned *status, cudaStream_t s,
                   int32_t *hit_track = nullptr);
 // active: per event 8 words of hit-activity bits (nullptr: every hit active)
-// cand_k / cand_v (may be null): instead of every cell's vote, each block writes its K best
-// cells by (votes desc, key asc) (unused slots: votes -1), coarse_lists(g, prec) blocks per
-// event in order; votes is then unused.  The midpoint form takes no candidates.
+// cand_k / cand_v (may be null): instead of every cell's vote, the K best cells of each tile
+// by (votes desc, key asc) (unused slots: votes -1), coarse_lists(g, prec) tiles per
+// event in order; votes is then unused.
 void launch_vote_coarse(const DevGeom &g, int prec, int ev0, int n_ev, const HitRecD *hd,
                         const HitRecF *hf, const int32_t *n_hits, int32_t *votes, uint32_t *hist,
                         unsigned *status, cudaStream_t s, unsigned long long *ctr = nullptr,
                         const uint32_t *active = nullptr, uint64_t *cand_k = nullptr,
                         int32_t *cand_v = nullptr, int K = 0, const int32_t *skip = nullptr);
-int coarse_lists(const DevGeom &g, int prec);   // level-0 blocks per event of a precision
-// The K best level-0 cells of each event from its blocks' candidates (n_lists x K per
+int coarse_lists(const DevGeom &g, int prec);   // level-0 tiles per event
+// The K best level-0 cells of each event from its tiles' candidates (n_lists x K per
 // event) and its histogram of all cells' votes, to out_keys / out_votes (K per event, in
 // no particular order; the set is that of launch_select_coarse).
 void launch_select_candidates(const DevGeom &g, int ev0, int n_ev, const uint64_t *cand_k,
@@ -192,7 +192,8 @@ struct MaxsetArgs {
     int cnt_stride;
     // selection scratch: per event the level's histogram (kHistBins, zero between uses), the votes a
     // cell needs to be kept (INT_MAX: none is), and per tile of kMaxsetTile cells its own histogram
-    // (`tiles` of them per event); cells_in: count_in as it was before the selection
+    // (`tiles` of them per event); cells: the level's cells (count_in may be the array
+    // that the selection writes)
     uint32_t *hist;
     int32_t *keep_from;
     uint16_t *tile_hist;
