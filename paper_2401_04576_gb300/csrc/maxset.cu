@@ -11,8 +11,9 @@
 // counters of the vmax group's cell indices (tiles without such a cell are skipped), from which one warp
 // per axis sums count x centre in ascending index order: the mean of the group's cell centres with a
 // summation order fixed by the indices, so the result does not depend on the order the cells arrive
-// in.  One block per event for all of it read every vote twice by itself: 342 us of a 665 us search
-// of one event.
+// in.  One block per event for all of it read every vote twice by itself: the selections of one event's
+// search took 342 us, now 158.  Summing the tiles before is quadratic in the tiles; at the most that
+// max_keep allows, 8192 tiles with everything kept, a whole search takes 6.6 ms against 20.6 with one block.
 //
 // Multi-track extraction (max_tracks > 1, one search per round on the hits still active):
 // the final vmax group can hold several tracks' cells (tracks with equal hit counts tie),
