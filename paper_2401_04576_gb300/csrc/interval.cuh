@@ -194,6 +194,10 @@ template <typename T> __device__ __forceinline__ T mag(IV<T> a) { return mx(-a.l
 template <typename T> __device__ __forceinline__ bool contains0(IV<T> a) {
     return le0(a.lo) && ge0(a.hi);
 }
+// The same for an end of the vote program, where FP32 ends of wide cells overflow: one that became NaN (0
+// times infinity) bounds nothing.
+__device__ __forceinline__ bool may_hold0(IV<double> a) { return contains0(a); }
+__device__ __forceinline__ bool may_hold0(IV<float> a) { return !(a.lo > 0.f) && !(a.hi < 0.f); }
 template <typename T> __device__ __forceinline__ IV<T> pm(T r) { return {-r, r}; }
 
 // [rd(1/k), ru(1/k)] for an integer k > 0

@@ -226,7 +226,7 @@ __device__ __forceinline__ bool tail(const Pre<T> &p, IV<T> L, const Hit<T> &h, 
         IV<T> Arad = sub(sub(sub(add(a1, a2), a3), a4), a5);
         IV<T> G = sub(p.G0, Arad);
         if (OUT) { ends[2 * sg] = G.lo; ends[2 * sg + 1] = G.hi; }
-        vote = vote || contains0(G);
+        vote = vote || may_hold0(G);
     }
     return vote;
 }

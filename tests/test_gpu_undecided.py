@@ -47,3 +47,22 @@ def test_direction_left_open(prec, oprec):
         a, b = ev.offsets[e], ev.offsets[e + 1]
         np.testing.assert_array_equal(votes[e], O.vote_coarse(tab, ev.wire_id[a:b], ev.drift[a:b], oprec))
     geom.close()
+
+
+@pytest.mark.parametrize("og", [0, apo.OUTGOING])
+@pytest.mark.parametrize("bins", [[3, 2, 2, 3, 3], [1, 1, 2, 1, 1], [4, 3, 4, 2, 5]])
+def test_fp32_overflow_keeps_fp64_votes(bins, og):
+    """Half-turn cells and wires without stereo in every other place: FP32 ends overflow and meet exact
+    zeros; the votes are the oracle's and contain the FP64 ones."""
+    w, g = chamber.make_wires(), G.make_grid(bins, 2, 2)
+    ev = chamber.multi_track_events(3, seed=20, w=w)
+    for name in ("tan_tau", "sphi_t", "cphi_t", "t2"):
+        getattr(w, name)[::2] = 0.0
+    geom, tab, hits = apo.Geometry(g, w), O.Tables(g, w), apo.DeviceHits.from_events(ev)
+    v32, v64 = (apo.vote(geom, hits, precision=p | og).cpu().numpy() for p in (apo.F32, apo.F64))
+    assert np.all(v32 >= v64)
+    for e in range(ev.n_events):
+        a, b = ev.offsets[e], ev.offsets[e + 1]
+        np.testing.assert_array_equal(v32[e], O.vote_coarse(tab, ev.wire_id[a:b], ev.drift[a:b], 1 | og))
+        np.testing.assert_array_equal(v64[e], O.vote_coarse(tab, ev.wire_id[a:b], ev.drift[a:b], 0 | og))
+    geom.close()
